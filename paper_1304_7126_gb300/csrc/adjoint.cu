@@ -101,10 +101,10 @@ thermo_vjp_kernel(ThermoParams p, const double *__restrict__ nH, const double *_
     cc.valid = false;
     cc.rvalid = false;
     if (p.isothermal) {
-        RatesT<Dual> t;
-        get_rates<false, false>(st.T, p.case_b, kNeedH | (p.helium ? kNeedHe : 0u), kNeedH, t);
-        h_rates_from(t, iso.h);
-        if (p.helium) he_rates_from(t, iso.he);
+        TLevel L;
+        t_level(st.T.v, L);
+        h_rates<false, false>(L, st.T.d, p.case_b, nullptr, iso.h);
+        if (p.helium) he_rates<false, false>(L, st.T.d, p.case_b, nullptr, iso.he);
     }
     double t_left = p.dt, dt_tc = p.dt;
     int att = 0;

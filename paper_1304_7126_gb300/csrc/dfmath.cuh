@@ -69,6 +69,15 @@ __device__ __forceinline__ F2 add(F2 a, F2 b)
     return fast_two_sum(s.hi, __fadd_rn(s.lo, t.lo));
 }
 
+// a + b within 2^-47 (|a| + |b|): the low parts rounded once.  Commutative,
+// and b = 0 returns a normalised a.  For the arguments and sums below, whose
+// terms carry errors of that size themselves (11 instructions, add() 20).
+__device__ __forceinline__ F2 adds(F2 a, F2 b)
+{
+    const F2 s = two_sum(a.hi, b.hi);
+    return fast_two_sum(s.hi, __fadd_rn(s.lo, __fadd_rn(a.lo, b.lo)));
+}
+
 __device__ __forceinline__ F2 add(F2 a, float b)
 {
     const F2 s = two_sum(a.hi, b);
@@ -141,6 +150,102 @@ __device__ __forceinline__ double widen(float f)
 
 __device__ __forceinline__ double to_double(F2 a) { return widen(a.hi) + widen(a.lo); }
 
+// (hi + lo) 2^m as a double without the FP64 pipe: lo, at most 1.5 2^-23 of
+// hi and rounded to 2^-52 of hi's binade, is added to the bits of hi.  hi a
+// positive float of 2^-75 and more, the result a normal double.
+__device__ __forceinline__ double combine(float hi, float lo, int m = 0)
+{
+    const unsigned u = __float_as_uint(hi);
+    int L = __float2int_rn(__fmul_rn(lo, __uint_as_float((306u << 23) - (u & 0x7f800000u))));
+    if ((u & 0x7fffffu) == 0 && L < 0) L *= 2;   // below hi the binade's steps are half as long
+    const unsigned top = (u >> 3) + 0x38000000u + ((unsigned)m << 20);
+    return __longlong_as_double((long long)(((unsigned long long)top << 32) | (unsigned long long)(u << 29)) + L);
+}
+
+// any pair times 2^m, |m| below 2000 (a zero or tiny high part through the
+// FP64 pipe; results below the normal doubles are 0)
+__device__ __forceinline__ double to_double_i(F2 a, int m = 0)
+{
+    const float h = fabsf(a.hi);
+    const bool neg = a.hi < 0.0f;
+    if (!(h > 0x1p-70f && h < 0x1p120f)) return ldexp((double)a.hi + (double)a.lo, m);
+    const int e = (int)(__float_as_uint(h) >> 23) - 127 + m;
+    if (e < -1020) return 0.0;
+    const long long r = __double_as_longlong(combine(h, neg ? -a.lo : a.lo, m));
+    return __longlong_as_double(neg ? r | (1LL << 63) : r);   // (a negation may take the FP64 pipe)
+}
+
+// ---- reciprocal and quotient of doubles ----
+// The IEEE quotient takes some nine FP64 instructions, and a warp issues one
+// per 64 cycles.  Here the reciprocal of the divisor comes from float pairs
+// (an approximate FP32 reciprocal and one Newton step in pairs, 2^-45), and
+// one FP64 residual step corrects the quotient, whose error before rounding
+// is then below 2^-88: the nearest double but for one quotient in 2^35.
+// 1/b needs two FP64 instructions, a/b three.  |b| outside 2^-70 .. 2^70,
+// zero, infinite or NaN takes the IEEE quotient.
+__device__ __forceinline__ float rcp_approx(float a)
+{
+    float r;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(a));
+    return r;
+}
+
+// a double of 2^-74 .. 2^127 in magnitude as the nearest float and the rest
+__device__ __forceinline__ F2 split_near(double x)
+{
+    const unsigned long long b = (unsigned long long)__double_as_longlong(x);
+    const unsigned hw = (unsigned)(b >> 32), lw = (unsigned)b;
+    const unsigned u = __funnelshift_l(lw, hw, 3) - 0xC0000000u;   // exponent rebiased by 896, mantissa cut to 23 bits
+    const float hi = __uint_as_float(u + ((lw >> 28) & 1u));
+    const float lo = __int2float_rn((int)(lw << 3) >> 3) * __uint_as_float((u & 0x7f800000u) - (52u << 23));
+    return {hi, lo};
+}
+
+__device__ __forceinline__ bool div_range(double b)
+{
+    const unsigned h = (unsigned)((unsigned long long)__double_as_longlong(b) >> 32) & 0x7fffffffu;
+    return h - (953u << 20) < (140u << 20);
+}
+
+__device__ __forceinline__ double rcp_seed(double b)   // div_range(b)
+{
+    const F2 s = split_near(__longlong_as_double(__double_as_longlong(b) & 0x7fffffffffffffffLL));
+    const float r0 = rcp_approx(s.hi);
+    const float e = __fmaf_rn(-s.lo, r0, __fmaf_rn(-s.hi, r0, 1.0f));
+    return __longlong_as_double(__double_as_longlong(combine(r0, __fmul_rn(r0, e))) |
+                                (__double_as_longlong(b) & (1LL << 63)));
+}
+
+static __device__ __noinline__ double ieee_div(double a, double b) { return a / b; }
+
+__device__ __forceinline__ double fast_rcp(double b)
+{
+    if (!div_range(b)) return ieee_div(1.0, b);
+    const double r = rcp_seed(b);
+    return __fma_rn(__fma_rn(-b, r, 1.0), r, r);
+}
+
+__device__ __forceinline__ double fast_div(double a, double b)
+{
+    if (!div_range(b)) return ieee_div(a, b);
+    const double r = rcp_seed(b);
+    const double q = __dmul_rn(a, r);
+    return __fma_rn(__fma_rn(-q, b, a), r, q);
+}
+
+// a double as the nearest float on the integer pipe: 0 below the normal
+// floats, NaN above them (and for infinities and NaN)
+__device__ __forceinline__ float near_float(double x)
+{
+    const unsigned long long b = (unsigned long long)__double_as_longlong(x);
+    const unsigned hw = (unsigned)(b >> 32), lw = (unsigned)b;
+    const unsigned e = hw & 0x7ff00000u;
+    unsigned u = __funnelshift_l(lw, hw, 3) - 0xC0000000u + ((lw >> 28) & 1u);
+    if (e < (897u << 20)) u = 0;
+    if (e > (1149u << 20)) u = 0x7fc00000u;
+    return __uint_as_float(u | (hw & 0x80000000u));
+}
+
 // 1 / a and sqrt(a) of a positive pair: one Newton step in pair arithmetic
 // from the correctly rounded FP32 value (relative error <= 2^-24, squared by
 // the step)
@@ -174,11 +279,9 @@ __device__ __forceinline__ F2 sqrt2(F2 a)
 // minutes.  The warp path of the rates (one call site per temperature)
 // inlines exp2d_inl and log2f2_inl, the same arithmetic.
 
-// e^x of a pair; a double result (subnormal, 0 and infinity as CUDA's exp)
-__device__ __forceinline__ double exp2d_inl(F2 x)
+// e^x of a pair as y 2^m, y a pair in [0.99, 2.02); |x| below 2000
+__device__ __forceinline__ void exp_pair(F2 x, F2 &y, int &m)
 {
-    if (!(x.hi > -745.2f)) return (x.hi != x.hi) ? (double)x.hi : 0.0;
-    if (x.hi > 709.78f) return __longlong_as_double(0x7ff0000000000000LL);
     const float kf = rintf(__fmul_rn(x.hi, kDfInvL));
     const int k = (int)kf;
     // r = x - k ln2/64: k L1 exact, x.hi - k L1 exact (Sterbenz), k L2 split
@@ -194,15 +297,23 @@ __device__ __forceinline__ double exp2d_inl(F2 x)
     const float c = __fmaf_rn(rh, r.lo,
                               rh * h2.hi * __fmaf_rn(rh, __fmaf_rn(rh, 1.0f / 120.0f, 1.0f / 24.0f), 1.0f / 6.0f));
     const F2 q = fast_two_sum(0.5f * h2.hi, __fmaf_rn(0.5f, h2.lo, c));
-    const F2 p = add(r, q);
+    const F2 p = adds(r, q);
     const float2 t = __ldg(&kDfExp2Tab[k & 63]);
     const F2 T{t.x, t.y};
-    const F2 y = add(T, mul(T, p));   // 2^(j/64) e^r
-    const double yd = to_double(y);
-    const int m = k >> 6;              // floor(k / 64)
-    if (m > -1020 && m < 1020)
-        return __longlong_as_double(__double_as_longlong(yd) + ((long long)m << 52));
-    return ldexp(yd, m);
+    y = adds(T, mul(T, p));   // 2^(j/64) e^r
+    m = k >> 6;               // floor(k / 64)
+}
+
+// e^x of a pair; a double result (subnormal, 0 and infinity as CUDA's exp)
+__device__ __forceinline__ double exp2d_inl(F2 x)
+{
+    if (!(x.hi > -745.2f)) return (x.hi != x.hi) ? (double)x.hi : 0.0;
+    if (x.hi > 709.78f) return __longlong_as_double(0x7ff0000000000000LL);
+    F2 y;
+    int m;
+    exp_pair(x, y, m);
+    if (m > -1020 && m < 1020) return combine(y.hi, y.lo, m);
+    return ldexp(to_double(y), m);
 }
 
 static __device__ __noinline__ double exp2d(F2 x) { return exp2d_inl(x); }
@@ -225,16 +336,16 @@ __device__ __forceinline__ F2 log2f2_inl(F2 v)
     const F2 u3 = mul(u2, u.hi);
     const float uh = u.hi;
     const float cub = uh * __fmaf_rn(uh, __fmaf_rn(uh, -1.0f / 6.0f, 0.2f), -0.25f);
-    F2 q = add(u, F2{-0.5f * u2.hi, -0.5f * u2.lo});
-    q = add(q, mul(u3, F2{kDfThirdHi, kDfThirdLo}));
+    F2 q = adds(u, F2{-0.5f * u2.hi, -0.5f * u2.lo});
+    q = adds(q, mul(u3, F2{kDfThirdHi, kDfThirdLo}));
     q = add(q, u3.hi * cub);
     // e ln2 + ln F + q
     const float ef = (float)e;
     F2 s = two_prod(ef, kDfLn2B);
-    s = add(F2{ef * kDfLn2A, 0.0f}, s);   // e A exact
+    s = adds(F2{ef * kDfLn2A, 0.0f}, s);   // e A exact
     s = add(s, ef * kDfLn2C);
-    s = add(s, F2{L.x, L.y});
-    return add(s, q);
+    s = adds(s, F2{L.x, L.y});
+    return adds(s, q);
 }
 
 static __device__ __noinline__ F2 log2f2(F2 v) { return log2f2_inl(v); }
@@ -272,14 +383,21 @@ static __device__ __noinline__ F2 log1pd(double w)
     return add(lv, __fdividef(t.lo, v.hi));   // + c / v
 }
 
-// ln(1 + e^z) of a pair z, with its derivative 1/(1 + e^-z) as a double.
+static __device__ __noinline__ F2 softplus_far(F2 z, F2 &sig)
+{
+    const double w = exp2d(z);
+    sig = split_any(w < 1e300 ? w / (1.0 + w) : 1.0);
+    return log1pd(w);
+}
+
+// ln(1 + e^z) of a pair z, with its derivative 1/(1 + e^-z) as a pair.
 // On [-16, 16): the interpolating polynomials of kDfSoftplusTab (degree 9
 // in t = z - middle of a 1/4-wide interval, |t| <= 1/8); the terms of
 // degree 5 and up are below 2^-24 of the value, so they are summed in
 // FP32, the rest in pair arithmetic (absolute error ~1e-14 at |z| ~ 16,
 // that of the pair coefficients).  Outside (temperatures far beyond the
 // fits' range) from e^z and log1p.
-__device__ __forceinline__ F2 softplus2(F2 z, double &sig)
+__device__ __forceinline__ F2 softplus2(F2 z, F2 &sig)
 {
     if (z.hi >= (float)kDfSpLo && z.hi < -(float)kDfSpLo) {
         int k = (int)__fmul_rn(__fadd_rn(z.hi, -(float)kDfSpLo), (float)kDfSpPer);
@@ -301,15 +419,13 @@ __device__ __forceinline__ F2 softplus2(F2 z, double &sig)
 #pragma unroll
         for (int n = 4; n >= 0; --n) {
             const float2 cn = __ldg(&c[n]);
-            P = add(F2{cn.x, cn.y}, mul(P, t));
-            if (n >= 1) D = add(mul(F2{cn.x, cn.y}, (float)n), mul(D, t));
+            P = adds(F2{cn.x, cn.y}, mul(P, t));
+            if (n >= 1) D = adds(mul(F2{cn.x, cn.y}, (float)n), mul(D, t));
         }
-        sig = to_double(D);
+        sig = D;
         return P;
     }
-    const double w = exp2d(z);
-    sig = w / (1.0 + w);
-    return log1pd(w);
+    return softplus_far(z, sig);
 }
 
 }  // namespace dfm

@@ -68,6 +68,7 @@ __device__ __forceinline__ Dual rmul(const Dual &a, const Dual &b)
 }
 __device__ __forceinline__ Dual rmul(const Dual &a, double b) { return Dual(__dmul_rn(a.v, b), a.d * b); }
 __device__ __forceinline__ Dual radd(const Dual &a, const Dual &b) { return Dual(__dadd_rn(a.v, b.v), a.d + b.d); }
+__device__ __forceinline__ Dual rmul(double a, const Dual &b) { return Dual(__dmul_rn(a, b.v), a * b.d); }
 // a b + c with one rounding, as written
 __device__ __forceinline__ double rfma(double a, double b, double c) { return __fma_rn(a, b, c); }
 __device__ __forceinline__ Dual rfma(double a, const Dual &b, const Dual &c)

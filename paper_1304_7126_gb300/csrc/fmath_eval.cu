@@ -22,13 +22,13 @@ __device__ double eval_one(int fn, double v)
     case 3: return (v > 0.0 && splittable(v)) ? to_double(rcp(split(v))) : 1.0 / v;
     case 4: return (v > 0.0 && splittable(v)) ? to_double(sqrt2(split(v))) : sqrt(v);
     case 5: {   // ln(1 + e^v)
-        double sg;
-        return to_double(softplus2(split_any(v), sg));
+        F2 sg;
+        return to_double_i(softplus2(split_any(v), sg));
     }
     default: {   // 1 / (1 + e^-v)
-        double sg;
+        F2 sg;
         softplus2(split_any(v), sg);
-        return sg;
+        return to_double_i(sg);
     }
     }
 }

@@ -12,6 +12,13 @@
 // argument is formed in the double-float arithmetic of dfmath.cuh (on the
 // FP32 pipe), exponentiated by dfm::exp2d and scaled by Cc in FP64; both
 // paths run the same expressions and so give identical bits.
+//
+// What bounds them: the FP64 pipe, of which a warp gets one instruction per
+// 64 cycles (so the count of FP64 instructions sets both the length of a lone
+// cell's chain of attempts and the throughput of the lane-per-cell kernels).
+// The functions, their T-derivatives and the cooling sums therefore stay
+// float pairs until they enter the FP64 update, and enter it through integer
+// operations (dfm::combine) instead of an FP64 addition each.
 #pragma once
 
 #include <cuda_runtime.h>
@@ -21,11 +28,20 @@
 
 namespace rtgb {
 
-// Quotients of the thermochemistry (IEEE division; a double-float quotient
-// refined by an FP64 residual step was tried and its longer dependent chain
-// made every attempt slower)
-template <typename S>
-__device__ __forceinline__ S qdiv(const S &a, const S &b) { return a / b; }
+// Quotients and reciprocals of the thermochemistry (dfmath.cuh: three and
+// two FP64 instructions)
+__device__ __forceinline__ double qdiv(double a, double b) { return dfm::fast_div(a, b); }
+__device__ __forceinline__ double qrcp(double b) { return dfm::fast_rcp(b); }
+__device__ __forceinline__ Dual qdiv(const Dual &a, const Dual &b)
+{
+    const double q = dfm::fast_div(a.v, b.v);
+    return Dual(q, dfm::fast_div(a.d - q * b.d, b.v));
+}
+__device__ __forceinline__ Dual qrcp(const Dual &b)
+{
+    const double q = dfm::fast_rcp(b.v);
+    return Dual(q, -q * q * b.d);
+}
 
 // exp arguments: exp(fma(a, ln T, fma(b, 1/T, c)))
 enum {
@@ -155,8 +171,9 @@ static_assert(kNCool <= 16 && NRF <= 32, "function slots are warp lanes");
 struct RateFn {
     double Cc;
     dfm::F2 c0, c1, c2, c3, c4, c5;
-    double d1, d2, d34, d344;   // c1, c2, c3 c4, c3 c4^2 (log-derivative and its derivative)
-    float g34;                  // c3 c4 as a float (FP32 path)
+    dfm::F2 Cm, c34;            // Cc = Cm 2^ke, 1 <= Cm < 2; c3 c4
+    double d1, d2, d34, d344;   // c1, c2, c3 c4, c3 c4^2 (second derivative)
+    int ke;
 };
 struct RateFnTab {
     RateFn f[32];
@@ -166,8 +183,12 @@ constexpr double kHalfLn1e5 = 5.756462732485114;   // ln(1e5) / 2
 
 constexpr RateFn rate_fn(double Cc, double c0, double c1, double c2, double c3, double c4, double c5)
 {
+    double m = Cc;
+    int e = 0;
+    while (m >= 2.0) { m *= 0.5; ++e; }
+    while (m > 0.0 && m < 1.0) { m *= 2.0; --e; }
     return RateFn{Cc, pair_of(c0), pair_of(c1), pair_of(c2), pair_of(c3), pair_of(c4), pair_of(c5),
-                  c1, c2, c3 * c4, c3 * c4 * c4, (float)(c3 * c4)};
+                  pair_of(m), pair_of(c3 * c4), c1, c2, c3 * c4, c3 * c4 * c4, e};
 }
 constexpr RateFn cen_fn(double A, double T0) { return rate_fn(A, 0.0, 0.5, -T0, 1.0, 0.5, -kHalfLn1e5); }
 constexpr RateFn hg_fn(const RateTable &R, int j)
@@ -211,6 +232,7 @@ constexpr RateFnTab make_rate_fns(int cb)
 // uniform reads (one thread, a compile-time slot): the constant cache;
 // lane-indexed reads (a warp): global memory through the L1 cache, which
 // serves different addresses of a warp in one request
+constexpr RateFnTab kRateFnCx[2] = {make_rate_fns(0), make_rate_fns(1)};   // (compile-time queries)
 static __constant__ RateFnTab c_rate_fn[2] = {make_rate_fns(0), make_rate_fns(1)};
 static __device__ const RateFnTab g_rate_fn[2] = {make_rate_fns(0), make_rate_fns(1)};
 
@@ -218,82 +240,134 @@ static __device__ const RateFnTab g_rate_fn[2] = {make_rate_fns(0), make_rate_fn
 static __device__ const int g_cool_sp[16] = {SP_HI, SP_HI, SP_HII, SP_FF, SP_HEI, SP_HEII, SP_HEII, SP_HEII,
                                              SP_HEII, SP_HEII, SP_HEIII, 0, 0, 0, 0, 0};
 
-// ln T and 1/T of one temperature as pairs, 1/T as a double (both paths:
-// the FP32 one needs ln T and 1/T to better than a float, see rate_value_f)
+// ln T and 1/T of one temperature as pairs
 struct TLevel {
     dfm::F2 lnT, invT;
-    double invTd;
 };
-template <bool MIX, bool INL = false>
+template <bool INL = false>
 __device__ __forceinline__ void t_level(double T, TLevel &L)
 {
     using namespace dfm;
     if (!(T > 0.0) || !splittable(T)) {   // not reached by T >= 1 K below 2^60 K
-        L.invTd = 1.0 / T;
         L.lnT = split_any(log(T));
-        L.invT = split_any(L.invTd);
+        L.invT = split_any(1.0 / T);
     } else {
         const F2 T2 = split(T);
         L.lnT = INL ? log2f2_inl(T2) : log2f2(T2);
         L.invT = rcp(T2);
-        L.invTd = to_double(L.invT);
     }
 }
 // the same from 1/T as a pair
-template <bool MIX, bool INL = false>
+template <bool INL = false>
 __device__ __forceinline__ void t_level_inv(dfm::F2 invT, TLevel &L)
 {
     using namespace dfm;
     L.invT = invT;
-    L.invTd = to_double(invT);
-    if (invT.hi > 0.0f && splittable(L.invTd)) L.lnT = neg(INL ? log2f2_inl(invT) : log2f2(invT));
-    else L.lnT = split_any(-log(L.invTd));
-}
-// f(T) of one function given l = softplus(z); all FP64 products rounded as
-// written
-__device__ __forceinline__ double rate_from_l(const RateFn &q, const TLevel &L, dfm::F2 l)
-{
-    using namespace dfm;
-    const F2 arg = add(add(add(q.c0, mul(L.lnT, q.c1)), mul(L.invT, q.c2)), neg(mul(l, q.c3)));
-    return rmul(q.Cc, exp2d(arg));
-}
-__device__ __forceinline__ dfm::F2 rate_softplus(const RateFn &q, const TLevel &L, double &sig)
-{
-    using namespace dfm;
-    return softplus2(add(mul(L.lnT, q.c4), q.c5), sig);
-}
-// f(T) of one function and sigma(z)
-__device__ __forceinline__ double rate_value(const RateFn &q, const TLevel &L, double &sig)
-{
-    return rate_from_l(q, L, rate_softplus(q, L, sig));
-}
-// df/dT = f (c1 - c2/T - c3 c4 sigma) / T
-__device__ __forceinline__ double rate_deriv(const RateFn &q, double invT, double f, double sig)
-{
-    return rmul(f, rmul(rfma(-q.d34, sig, rfma(-q.d2, invT, q.d1)), invT));
+    if (invT.hi > 0x1p-60f && invT.hi < 0x1p60f) L.lnT = neg(INL ? log2f2_inl(invT) : log2f2(invT));
+    else L.lnT = split_any(-log(to_double(invT)));
 }
 
-// FP32 (the mixed-precision thermochemistry, RT_MIXED32): the argument is
-// still formed in pairs (it reaches |20-60|, where a float's rounding alone
-// is 1e-6 of the rate, and over thousands of sub-steps that moved N by 2e-4
-// of the FP64 result), but the softplus correction ln(1 + e^-|z|) < ln 2
-// and the exponential run in FP32: e^arg = e^hi (1 + lo) with the float
-// exp of the high part; the log-derivative in FP32.  Relative accuracy
-// ~2e-7.
-__device__ __forceinline__ void rate_value_f(const RateFn &q, const TLevel &L, double &f, double &df)
+// A function value y 2^m (y a normalised pair below 8, or 0) and
+// g = d ln f / d ln T as a pair
+struct RateVal {
+    dfm::F2 y, g;
+    int m;
+};
+
+// Slots by the terms of their exponent, so that one thread can leave out
+// what is zero (adding a zero pair or multiplying by one returns the same
+// normalised pair, so both paths still give the same bits).
+__host__ __device__ constexpr unsigned rf_bit(int k) { return 1u << k; }
+enum { kZeroC0, kZeroC1, kZeroC2, kZeroC3 };
+constexpr unsigned rf_zero_mask(int what)
+{
+    unsigned m = 0;
+    for (int k = 0; k < NRF; ++k) {
+        bool z = true;
+        for (int cb = 0; cb < 2; ++cb) {
+            const RateFn &q = kRateFnCx[cb].f[k];
+            const float v = what == kZeroC0 ? q.c0.hi : what == kZeroC1 ? q.c1.hi : what == kZeroC2 ? q.c2.hi : q.c3.hi;
+            z = z && v == 0.0f;
+        }
+        if (z) m |= rf_bit(k);
+    }
+    return m;
+}
+// slots whose softplus is that of u (c3 = 1, z = (ln T - ln 1e5)/2, the same in all of them)
+constexpr unsigned rf_u_mask()
+{
+    unsigned m = rf_bit(RF_BETA_HI) | rf_bit(RF_BETA_HEI) | rf_bit(RF_BETA_HEII);
+    for (int k = 0; k < kNCool; ++k)
+        if (cool_row(k).uu) m |= rf_bit(RF_COOL0 + k);
+    return m;
+}
+constexpr unsigned kC0Zero = rf_zero_mask(kZeroC0), kC1Zero = rf_zero_mask(kZeroC1), kC2Zero = rf_zero_mask(kZeroC2),
+                   kC3Zero = rf_zero_mask(kZeroC3), kSlotU = rf_u_mask();
+
+// softplus(z) and sigma(z) of one function, z = c4 ln T + c5.  MIX (the
+// mixed-precision thermochemistry, RT_MIXED32): z still in pairs, but the
+// correction ln(1 + e^-|z|) < ln 2 and sigma in FP32.
+template <bool MIX>
+__device__ __forceinline__ dfm::F2 rate_softplus(const RateFn &q, const TLevel &L, dfm::F2 &sig)
 {
     using namespace dfm;
-    const F2 z = add(mul(L.lnT, q.c4), q.c5);
-    const float e = __expf(-fabsf(z.hi));
-    const float sg = (z.hi >= 0.0f ? 1.0f : e) / (1.0f + e);
-    const F2 l = add(z.hi >= 0.0f ? z : F2{0.0f, 0.0f}, log1pf(e));   // softplus = max(z, 0) + ln(1 + e^-|z|)
-    const F2 arg = add(add(add(q.c0, mul(L.lnT, q.c1)), mul(L.invT, q.c2)), neg(mul(l, q.c3)));
-    const double eh = widen(expf(arg.hi));
-    f = rmul(q.Cc, rfma(eh, widen(arg.lo), eh));
-    const float x = L.invT.hi;
-    const float g = __fmul_rn(__fmaf_rn(-q.g34, sg, __fmaf_rn(-q.c2.hi, x, q.c1.hi)), x);
-    df = rmul(f, widen(g));
+    const F2 z = adds(mul(L.lnT, q.c4), q.c5);
+    if constexpr (MIX) {
+        const float e = __expf(-fabsf(z.hi));
+        sig = F2{(z.hi >= 0.0f ? 1.0f : e) / (1.0f + e), 0.0f};
+        return add(z.hi >= 0.0f ? z : F2{0.0f, 0.0f}, log1pf(e));   // max(z, 0) + ln(1 + e^-|z|)
+    } else {
+        return softplus2(z, sig);
+    }
 }
+
+// One function from l = softplus(z) and sigma(z).  The argument of the
+// exponential is formed in pairs on every path (it reaches |20-60|, where a
+// float's rounding alone is 1e-6 of the rate, and over thousands of
+// sub-steps that moved N by 2e-4 of the FP64 result); MIX takes the
+// exponential of the reduced argument and the log-derivative in FP32
+// (relative accuracy ~2e-7).  zero: bits kZero* of the terms known to be
+// zero (compile-time), one3: c3 = 1.
+template <bool MIX, bool DERIV>
+__device__ __forceinline__ void rate_val(const RateFn &q, const TLevel &L, dfm::F2 l, dfm::F2 sig, unsigned zero,
+                                         bool one3, RateVal &r)
+{
+    using namespace dfm;
+    const F2 nil{0.0f, 0.0f};
+    const F2 b = (zero >> kZeroC2 & 1) ? nil : mul(L.invT, q.c2);
+    F2 arg = (zero >> kZeroC1 & 1) ? nil : mul(L.lnT, q.c1);
+    if (!(zero >> kZeroC0 & 1)) arg = adds(q.c0, arg);
+    if (!(zero >> kZeroC2 & 1)) arg = adds(arg, b);
+    if (!(zero >> kZeroC3 & 1)) arg = adds(arg, neg(one3 ? l : mul(l, q.c3)));
+    if (arg.hi < -1400.0f) arg = F2{-1400.0f, 0.0f};   // 0 in every use
+    if constexpr (MIX) {
+        const float kf = rintf(__fmul_rn(arg.hi, 1.44269504f));
+        const float t = __fadd_rn(__fmaf_rn(-kf, -1.90465421e-9f, __fmaf_rn(-kf, 0.693147182f, arg.hi)), arg.lo);
+        r.y = mul(q.Cm, expf(t));
+        r.m = (int)kf + q.ke;
+        if constexpr (DERIV)
+            r.g = F2{__fmaf_rn(-q.c34.hi, sig.hi, __fmaf_rn(-q.c2.hi, L.invT.hi, q.c1.hi)), 0.0f};
+    } else {
+        int m;
+        exp_pair(arg, r.y, m);
+        r.y = mul(q.Cm, r.y);
+        r.m = m + q.ke;
+        if constexpr (DERIV) {
+            F2 g = (zero >> kZeroC1 & 1) ? nil : q.c1;
+            if (!(zero >> kZeroC2 & 1)) g = adds(g, neg(b));
+            if (!(zero >> kZeroC3 & 1)) g = adds(g, neg(mul(sig, q.c34)));
+            r.g = g;
+        }
+    }
+}
+__device__ __forceinline__ double rate_f(const RateVal &r) { return dfm::to_double_i(r.y, r.m); }
+// df/dT = f g / T
+__device__ __forceinline__ double rate_df(const RateVal &r, const TLevel &L)
+{
+    using namespace dfm;
+    return to_double_i(mul(r.y, mul(r.g, L.invT)), r.m);
+}
+
 // values (and derivatives) of several functions at one temperature
 template <typename S>
 struct RatesT {
@@ -301,7 +375,6 @@ struct RatesT {
 };
 using Rates = RatesT<double>;
 
-__host__ __device__ constexpr unsigned rf_bit(int k) { return 1u << k; }
 constexpr unsigned kNeedH = rf_bit(RF_BETA_HI) | rf_bit(RF_ALPHA_HII);   // values and derivatives
 constexpr unsigned kNeedHe = rf_bit(RF_BETA_HEI) | rf_bit(RF_BETA_HEII) | rf_bit(RF_ALPHA_HEII) |
                              rf_bit(RF_ALPHA_HEIII);
@@ -316,116 +389,101 @@ __host__ __device__ constexpr unsigned cool_mask(int he)
 }
 constexpr unsigned kNeedCoolH = cool_mask(0), kNeedCoolHe = cool_mask(1);
 
-// slots whose softplus is that of u (z = (ln T - ln 1e5)/2, the same in
-// all of them) and slots without a softplus (c3 = 0: l and sigma enter
-// multiplied by zero, exactly)
-__host__ __device__ constexpr unsigned rf_u_mask()
+// one thread: slot k (a constant once unrolled) at level L, given the
+// softplus of u
+template <bool MIX, bool DERIV>
+__device__ __forceinline__ void rate_serial(int k, const RateFnTab &R, const TLevel &L, dfm::F2 lu, dfm::F2 su,
+                                            RateVal &r, dfm::F2 &sig)
 {
-    unsigned m = rf_bit(RF_BETA_HI) | rf_bit(RF_BETA_HEI) | rf_bit(RF_BETA_HEII);
-    for (int k = 0; k < kNCool; ++k)
-        if (cool_row(k).uu) m |= rf_bit(RF_COOL0 + k);
-    return m;
-}
-__host__ __device__ constexpr unsigned rf_plain_mask()
-{
-    unsigned m = rf_bit(RF_ALPHA_HEII);
-    for (int k = 0; k < 16; ++k)
-        if (k >= kNCool || (!cool_row(k).uu && cool_row(k).hg < 0)) m |= rf_bit(RF_COOL0 + k);
-    return m;
+    const unsigned zero = (kC0Zero >> k & 1) << kZeroC0 | (kC1Zero >> k & 1) << kZeroC1 |
+                          (kC2Zero >> k & 1) << kZeroC2 | (kC3Zero >> k & 1) << kZeroC3;
+    dfm::F2 l = lu;
+    sig = su;
+    if (!(kSlotU & rf_bit(k)) && !(kC3Zero & rf_bit(k))) l = rate_softplus<MIX>(R.f[k], L, sig);
+    rate_val<MIX, DERIV>(R.f[k], L, l, sig, zero, (kSlotU & rf_bit(k)) != 0, r);
 }
 
 // one thread: the functions in needF (derivatives of those in needD); the
-// shared softplus of u once, none where it is multiplied by zero (the same
-// bits as the warp, which evaluates every slot's own)
+// shared softplus of u once
+template <bool MIX>
 __device__ __forceinline__ void rates_serial(const TLevel &L, int case_b, unsigned needF, unsigned needD, Rates &r)
 {
-    constexpr unsigned kU = rf_u_mask(), kPlain = rf_plain_mask();
     const RateFnTab &R = c_rate_fn[case_b];
-    double sgu = 0.0;
-    dfm::F2 lu{0.0f, 0.0f};
-    if (needF & kU) lu = rate_softplus(R.f[RF_BETA_HI], L, sgu);
+    dfm::F2 lu{0.0f, 0.0f}, su{0.0f, 0.0f};
+    if (needF & kSlotU) lu = rate_softplus<MIX>(R.f[RF_BETA_HI], L, su);
 #pragma unroll
     for (int k = 0; k < NRF; ++k) {
         if (needF & rf_bit(k)) {
-            double sg = 0.0;
-            if (kU & rf_bit(k)) {
-                sg = sgu;
-                r.f[k] = rate_from_l(R.f[k], L, lu);
-            } else if (kPlain & rf_bit(k)) {
-                r.f[k] = rate_from_l(R.f[k], L, dfm::F2{0.0f, 0.0f});
+            RateVal v;
+            dfm::F2 sig;
+            if (needD & rf_bit(k)) {
+                rate_serial<MIX, true>(k, R, L, lu, su, v, sig);
+                r.df[k] = rate_df(v, L);
             } else {
-                r.f[k] = rate_value(R.f[k], L, sg);
+                rate_serial<MIX, false>(k, R, L, lu, su, v, sig);
             }
-            if (needD & rf_bit(k)) r.df[k] = rate_deriv(R.f[k], L.invTd, r.f[k], sg);
-        }
-    }
-}
-__device__ __forceinline__ void rates_serial_f(const TLevel &L, int case_b, unsigned needF, unsigned needD, Rates &r)
-{
-    const RateFnTab &R = c_rate_fn[case_b];
-#pragma unroll
-    for (int k = 0; k < NRF; ++k) {
-        if (needF & rf_bit(k)) {
-            double df;
-            rate_value_f(R.f[k], L, r.f[k], df);
-            if (needD & rf_bit(k)) r.df[k] = df;
+            r.f[k] = rate_f(v);
         }
     }
 }
 
-// a full warp (all 32 lanes, the same T): lane k's function k
-template <bool MIX>
-__device__ __forceinline__ void rate_lane(const TLevel &L, int case_b, double &f, double &df)
+// a full warp (all 32 lanes, the same T): lane k's function k, its constants
+// q in registers
+template <bool MIX, bool DERIV>
+__device__ __forceinline__ void rate_lane(const RateFn &q, const TLevel &L, RateVal &r)
 {
-    const RateFn &q = g_rate_fn[case_b].f[threadIdx.x & 31];
-    if constexpr (MIX) {
-        rate_value_f(q, L, f, df);
-    } else {
-        using namespace dfm;
-        double sg;
-        const F2 l = rate_softplus(q, L, sg);
-        const F2 arg = add(add(add(q.c0, mul(L.lnT, q.c1)), mul(L.invT, q.c2)), neg(mul(l, q.c3)));
-        f = rmul(q.Cc, exp2d_inl(arg));
-        df = rate_deriv(q, L.invTd, f, sg);
-    }
+    dfm::F2 sig;
+    const dfm::F2 l = rate_softplus<MIX>(q, L, sig);
+    rate_val<MIX, DERIV>(q, L, l, sig, 0u, false, r);
 }
 // ... and the needed ones in every lane
-template <bool MIX>
-__device__ __forceinline__ void rates_warp(const TLevel &L, int case_b, unsigned needF, unsigned needD, Rates &r)
+template <bool MIX, bool DERIV>
+__device__ __forceinline__ void rates_warp(const RateFn &q, const TLevel &L, unsigned needF, unsigned needD, Rates &r)
 {
-    double f, df;
-    rate_lane<MIX>(L, case_b, f, df);
+    RateVal v;
+    rate_lane<MIX, DERIV>(q, L, v);
+    const double f = rate_f(v);
+    double df = 0.0;
+    if constexpr (DERIV) df = rate_df(v, L);
 #pragma unroll
     for (int k = 0; k < NRF; ++k) {
         if (needF & rf_bit(k)) r.f[k] = __shfl_sync(0xffffffffu, f, k);
-        if (needD & rf_bit(k)) r.df[k] = __shfl_sync(0xffffffffu, df, k);
+        if (DERIV && (needD & rf_bit(k))) r.df[k] = __shfl_sync(0xffffffffu, df, k);
     }
 }
 
-// A dual temperature (level L of its value, derivative dT): values as in
-// rates_serial (the bits of the double path); with g = c1 - c2/T - c3 c4
-// sigma, d ln f/dT = g/T and
-//     d2f/dT2 = f [(g/T)^2 + (-g + c2/T - c3 c4^2 sigma (1 - sigma)) / T^2],
-// so f carries df dT and df carries d2f dT.
+// f, df/dT and d2f/dT2 of slot k at level L (values f, df with the bits of
+// the double path): with g = c1 - c2/T - c3 c4 sigma, d ln f/dT = g/T and
+//     d2f/dT2 = f [(g/T)^2 + (-g + c2/T - c3 c4^2 sigma (1 - sigma)) / T^2].
+__device__ __forceinline__ void rate_dd(int k, const RateFnTab &R, const TLevel &L, dfm::F2 lu, dfm::F2 su, double x,
+                                        RateVal &v, double &f, double &df, double &d2f)
+{
+    dfm::F2 sig;
+    rate_serial<false, true>(k, R, L, lu, su, v, sig);
+    const RateFn &q = R.f[k];
+    const double sg = (kC3Zero & rf_bit(k)) ? 0.0 : dfm::to_double_i(sig), g = dfm::to_double_i(v.g), D = g * x;
+    f = rate_f(v);
+    df = rate_df(v, L);
+    d2f = f * (D * D + x * x * (-g + q.d2 * x - q.d344 * sg * (1.0 - sg)));
+}
+
+// A dual temperature (level L of its value, derivative dT): f carries df dT
+// and df carries d2f dT.
 __device__ __forceinline__ void rates_dual(const TLevel &L, double dT, int case_b, unsigned needF, unsigned needD,
                                            RatesT<Dual> &r)
 {
     const RateFnTab &R = c_rate_fn[case_b];
-    const double x = L.invTd;
+    const double x = dfm::to_double_i(L.invT);
+    dfm::F2 lu{0.0f, 0.0f}, su{0.0f, 0.0f};
+    if (needF & kSlotU) lu = rate_softplus<false>(R.f[RF_BETA_HI], L, su);
 #pragma unroll
     for (int k = 0; k < NRF; ++k) {
         if (needF & rf_bit(k)) {
-            const RateFn &q = R.f[k];
-            double sg;
-            const double f = rate_value(q, L, sg);
-            const double df = rate_deriv(q, x, f, sg);
+            RateVal v;
+            double f, df, d2f;
+            rate_dd(k, R, L, lu, su, x, v, f, df, d2f);
             r.f[k] = Dual(f, df * dT);
-            if (needD & rf_bit(k)) {
-                const double g = q.d1 - q.d2 * x - q.d34 * sg;
-                const double D = g * x;
-                const double d2f = f * (D * D + x * x * (-g + q.d2 * x - q.d344 * sg * (1.0 - sg)));
-                r.df[k] = Dual(df, d2f * dT);
-            }
+            if (needD & rf_bit(k)) r.df[k] = Dual(df, d2f * dT);
         }
     }
 }
@@ -459,6 +517,51 @@ __device__ __forceinline__ void he_rates_from(const RatesT<S> &t, HeRatesT<S> &r
     r.alpha_HeIII = t.f[RF_ALPHA_HEIII];
 }
 
+// The sets of functions an attempt needs at one temperature, out of line:
+// they do not depend on the group count, and inlined into every
+// instantiation of the one-thread kernels they made ptxas run for minutes.
+template <bool MIX>
+static __device__ __noinline__ HRates h_rates_serial(TLevel L, int case_b)
+{
+    Rates t;
+    HRates r;
+    rates_serial<MIX>(L, case_b, kNeedH, kNeedH, t);
+    h_rates_from(t, r);
+    return r;
+}
+template <bool MIX>
+static __device__ __noinline__ HeRates he_rates_serial(TLevel L, int case_b)
+{
+    Rates t;
+    HeRates r;
+    rates_serial<MIX>(L, case_b, kNeedHe, 0u, t);
+    he_rates_from(t, r);
+    return r;
+}
+template <bool MIX>
+static __device__ __noinline__ double2 he3_rates_serial(TLevel L, int case_b)
+{
+    Rates t;
+    rates_serial<MIX>(L, case_b, kNeedHe3, 0u, t);
+    return make_double2(t.f[RF_BETA_HEII], t.f[RF_ALPHA_HEIII]);
+}
+static __device__ __noinline__ HRatesT<Dual> h_rates_dual(TLevel L, double dT, int case_b)
+{
+    RatesT<Dual> t;
+    HRatesT<Dual> r;
+    rates_dual(L, dT, case_b, kNeedH, kNeedH, t);
+    h_rates_from(t, r);
+    return r;
+}
+static __device__ __noinline__ HeRatesT<Dual> he_rates_dual(TLevel L, double dT, int case_b)
+{
+    RatesT<Dual> t;
+    HeRatesT<Dual> r;
+    rates_dual(L, dT, case_b, kNeedHe, 0u, t);
+    he_rates_from(t, r);
+    return r;
+}
+
 // Recombination rates of HII, HeII, HeIII (the case t was evaluated with)
 template <typename S>
 __device__ __forceinline__ void recomb_alphas(const RatesT<S> &t, S a[3])
@@ -471,9 +574,14 @@ __device__ __forceinline__ void recomb_alphas(const RatesT<S> &t, S a[3])
 // Primordial cooling magnitude L (Eq. (rate_cooling), positive = cooling)
 // and dL/dT: the sum of the cooling functions (collisional ionisation and
 // excitation, recombination and dielectronic cooling, bremsstrahlung) each
-// times its density, in a fixed pairwise order, then Compton cooling.  All
-// products and sums are rounded as written (rmul, radd), so the one-thread
-// sum and the warp sum (lane k term k) give the same bits.
+// times its density, in a fixed pairwise order, then Compton cooling.  The
+// terms, scaled by 2^kCoolExp, and their sums are float pairs (2^-46, the
+// accuracy of the functions themselves is 1e-14 to 1e-12): before, 11
+// functions and derivatives entered FP64 one by one, 90 of an attempt's FP64
+// instructions.  The one-thread sum and the warp sum (lane k term k) run the
+// same operations and give the same bits.
+constexpr int kCoolExp = 80;
+
 // a[i] through selects (registers, not local memory, for a lane-dependent
 // i; a plain a[i] once unrolled with a constant i)
 template <typename T, int N>
@@ -483,18 +591,6 @@ __device__ __forceinline__ T pick(const T (&a)[N], int i)
 #pragma unroll
     for (int j = 1; j < N; ++j) r = (i == j) ? a[j] : r;
     return r;
-}
-
-// the fixed pairwise order of a 16-lane butterfly (offsets 8, 4, 2, 1)
-template <typename S>
-__device__ __forceinline__ S tree_sum16(S a[16])
-{
-#pragma unroll
-    for (int m = 8; m >= 1; m >>= 1) {
-#pragma unroll
-        for (int i = 0; i < m; ++i) a[i] = radd(a[i], a[i + m]);
-    }
-    return a[0];
 }
 
 template <typename S>
@@ -509,6 +605,27 @@ __device__ __forceinline__ void cool_densities(const S &nHI, const S &nHII, cons
     n[SP_FF] = radd(radd(nHII, nHeII), rmul(nHeIII, 4.0));
 }
 
+// a density as a pair (below 2^-70, 1e-21 of the smallest electron density
+// that matters, as 0; 2^120 and above through the FP64 pipe)
+__device__ __forceinline__ dfm::F2 split_density(double n)
+{
+    const unsigned h = (unsigned)((unsigned long long)__double_as_longlong(n) >> 32);
+    if (h < (953u << 20)) return {0.0f, 0.0f};
+    if (h >= (1143u << 20)) return dfm::split_any(n);
+    return dfm::split_near(n);
+}
+
+// a term f n (scaled) and f n g, g = d ln f/d ln T
+__device__ __forceinline__ void cool_term(const RateVal &r, dfm::F2 n, dfm::F2 &v, dfm::F2 &dv)
+{
+    using namespace dfm;
+    const int e = r.m + kCoolExp;
+    // (terms below 2^-60 of this scale, e-42 erg, are below 2^-48 of the bremsstrahlung)
+    const float sc = e < -60 ? 0.0f : pow2f(e > 100 ? 100 : e);
+    v = mul(F2{r.y.hi * sc, r.y.lo * sc}, n);
+    dv = mul(v, r.g);
+}
+
 // + Compton, varpi = comp (T - T_gamma), comp = 1.017e-37 T_gamma^4 and
 // T_gamma = 2.727/a (ThermoParams::comp, ::tg); both sums times n_e
 template <typename S>
@@ -520,58 +637,131 @@ __device__ __forceinline__ void cooling_close(double comp, double tg, const S &T
     dL = rmul(ne, radd(dLs, S(comp)));
 }
 
-// one thread
-template <typename S>
-__device__ __forceinline__ void cooling_from(const RatesT<S> &t, double comp, double tg, bool helium, const S &T,
-                                             const S &ne, const S &nHI, const S &nHII, const S &nHeI,
-                                             const S &nHeII, const S &nHeIII, S &L, S &dL)
+// the sums of 16 slots in the order of a 16-lane butterfly (offsets 8, 4, 2,
+// 1) over slots 0..10; slots 11..15 are zero and left out
+__device__ __forceinline__ dfm::F2 tree_sum11(const dfm::F2 (&a)[kNCool])
 {
-    S n[NSP];
-    cool_densities(nHI, nHII, nHeI, nHeII, nHeIII, n);
-    S a[16], b[16];
+    using dfm::adds;
+    const dfm::F2 s0 = adds(a[0], a[8]), s1 = adds(a[1], a[9]), s2 = adds(a[2], a[10]);
+    const dfm::F2 t0 = adds(s0, a[4]), t1 = adds(s1, a[5]), t2 = adds(s2, a[6]), t3 = adds(a[3], a[7]);
+    return adds(adds(t0, t2), adds(t1, t3));
+}
+
+// one thread; RV: optional, per term f, df/dT and d2f/dT2 for the tangents
+struct CoolDD {
+    double f[kNCool], df[kNCool], d2f[kNCool];
+};
+template <bool MIX, bool DD>
+__device__ __forceinline__ void cooling_sums(const TLevel &L, int case_b, bool helium, const double *n, double &Ls,
+                                             double &dLs, CoolDD *dd)
+{
+    using namespace dfm;
+    const RateFnTab &R = c_rate_fn[case_b];
+    F2 np[NSP];
 #pragma unroll
-    for (int k = 0; k < 16; ++k) {
-        a[k] = S(0.0);
-        b[k] = S(0.0);
-    }
+    for (int k = 0; k < NSP; ++k) np[k] = split_density(n[k]);
+    F2 su;
+    const F2 lu = rate_softplus<MIX>(R.f[RF_BETA_HI], L, su);
+    F2 a[kNCool], b[kNCool];
+    double x = 0.0;
+    if constexpr (DD) x = to_double_i(L.invT);
 #pragma unroll
     for (int k = 0; k < kNCool; ++k) {
         const CoolTerm q = cool_row(k);
+        a[k] = b[k] = F2{0.0f, 0.0f};
         if (helium || !q.he) {
-            a[k] = rmul(t.f[RF_COOL0 + k], n[q.sp]);
-            b[k] = rmul(t.df[RF_COOL0 + k], n[q.sp]);
+            RateVal v;
+            F2 sig;
+            if constexpr (DD) rate_dd(k, R, L, lu, su, x, v, dd->f[k], dd->df[k], dd->d2f[k]);
+            else rate_serial<MIX, true>(k, R, L, lu, su, v, sig);
+            cool_term(v, np[q.sp], a[k], b[k]);
+        } else if constexpr (DD) {
+            dd->f[k] = dd->df[k] = dd->d2f[k] = 0.0;
         }
     }
-    const S Ls = tree_sum16(a), dLs = tree_sum16(b);
+    Ls = to_double_i(tree_sum11(a), -kCoolExp);
+    dLs = to_double_i(mul(tree_sum11(b), L.invT), -kCoolExp);
+}
+
+// (out of line, as the rate sets above)
+template <bool MIX>
+static __device__ __noinline__ double2 cooling_sums_serial(int case_b, bool helium, double T, double nHI, double nHII,
+                                                           double nHeI, double nHeII, double nHeIII)
+{
+    TLevel Lv;
+    t_level(T, Lv);
+    double n[NSP], Ls, dLs;
+    cool_densities(nHI, nHII, nHeI, nHeII, nHeIII, n);
+    cooling_sums<MIX, false>(Lv, case_b, helium, n, Ls, dLs, nullptr);
+    return make_double2(Ls, dLs);
+}
+template <bool MIX>
+__device__ __forceinline__ void cooling_serial(int case_b, double comp, double tg, bool helium, double T, double ne,
+                                               double nHI, double nHII, double nHeI, double nHeII, double nHeIII,
+                                               double &L, double &dL)
+{
+    const double2 s = cooling_sums_serial<MIX>(case_b, helium, T, nHI, nHII, nHeI, nHeII, nHeIII);
+    cooling_close(comp, tg, T, ne, s.x, s.y, L, dL);
+}
+
+// dual numbers: the values of the double path, the tangents term by term
+template <bool MIX>
+static __device__ __noinline__ void cooling_serial(int case_b, double comp, double tg, bool helium, const Dual &T,
+                                                   const Dual &ne, const Dual &nHI, const Dual &nHII,
+                                                   const Dual &nHeI, const Dual &nHeII, const Dual &nHeIII, Dual &L,
+                                                   Dual &dL)
+{
+    static_assert(!MIX, "dual rates: FP64");
+    TLevel Lv;
+    t_level(T.v, Lv);
+    Dual n[NSP];
+    cool_densities(nHI, nHII, nHeI, nHeII, nHeIII, n);
+    double nv[NSP];
+#pragma unroll
+    for (int k = 0; k < NSP; ++k) nv[k] = n[k].v;
+    CoolDD dd;
+    Dual Ls(0.0), dLs(0.0);
+    cooling_sums<false, true>(Lv, case_b, helium, nv, Ls.v, dLs.v, &dd);
+#pragma unroll
+    for (int k = 0; k < kNCool; ++k) {
+        const int sp = cool_row(k).sp;
+        Ls.d += dd.f[k] * n[sp].d + dd.df[k] * T.d * n[sp].v;
+        dLs.d += dd.df[k] * n[sp].d + dd.d2f[k] * T.d * n[sp].v;
+    }
     cooling_close(comp, tg, T, ne, Ls, dLs, L, dL);
 }
 
 // a full warp (all 32 lanes, the same arguments): lane k < 16 holds term k,
 // the sums run over shuffles in the same pairwise order
-template <bool MIX>
-__device__ __forceinline__ void cooling_warp(int case_b, double comp, double tg, bool helium, double T, double ne,
-                                             double nHI, double nHII, double nHeI, double nHeII, double nHeIII,
-                                             double &L, double &dL)
+__device__ __forceinline__ dfm::F2 shfl_xor_pair(dfm::F2 a, int m)
 {
+    return {__shfl_xor_sync(0xffffffffu, a.hi, m), __shfl_xor_sync(0xffffffffu, a.lo, m)};
+}
+template <bool MIX>
+__device__ __forceinline__ void cooling_warp(const RateFn &q, double comp, double tg, bool helium, double T,
+                                             double ne, double nHI, double nHII, double nHeI, double nHeII,
+                                             double nHeIII, double &L, double &dL)
+{
+    using namespace dfm;
     TLevel Lv;
-    t_level<MIX, true>(T, Lv);
-    double f, df;
-    rate_lane<MIX>(Lv, case_b, f, df);
+    t_level<true>(T, Lv);
+    RateVal r;
+    rate_lane<MIX, true>(q, Lv, r);
     double n[NSP];
     cool_densities(nHI, nHII, nHeI, nHeII, nHeIII, n);
     const int k = threadIdx.x & 15;
-    const double nk = pick(n, g_cool_sp[k]);
-    double v = rmul(f, nk), dv = rmul(df, nk);
-    if (!helium && (cool_mask(1) & rf_bit(k))) v = dv = 0.0;
+    F2 v, dv;
+    cool_term(r, split_density(pick(n, g_cool_sp[k])), v, dv);
+    if (k >= kNCool || (!helium && (cool_mask(1) & rf_bit(k)))) v = dv = F2{0.0f, 0.0f};
 #pragma unroll
     for (int m = 8; m >= 1; m >>= 1) {
-        v = radd(v, __shfl_xor_sync(0xffffffffu, v, m));
-        dv = radd(dv, __shfl_xor_sync(0xffffffffu, dv, m));
+        v = adds(v, shfl_xor_pair(v, m));
+        dv = adds(dv, shfl_xor_pair(dv, m));
     }
     // lanes 16..31 summed other functions: every lane takes lane 0's sums
-    v = __shfl_sync(0xffffffffu, v, 0);
-    dv = __shfl_sync(0xffffffffu, dv, 0);
-    cooling_close(comp, tg, T, ne, v, dv, L, dL);
+    v = F2{__shfl_sync(0xffffffffu, v.hi, 0), __shfl_sync(0xffffffffu, v.lo, 0)};
+    dv = F2{__shfl_sync(0xffffffffu, dv.hi, 0), __shfl_sync(0xffffffffu, dv.lo, 0)};
+    cooling_close(comp, tg, T, ne, to_double_i(v, -kCoolExp), to_double_i(mul(dv, Lv.invT), -kCoolExp), L, dL);
 }
 
 }  // namespace rtgb

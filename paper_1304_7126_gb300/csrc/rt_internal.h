@@ -75,6 +75,7 @@ struct ThermoParams {
     // derived per-group terms of the photon update (derive_group_terms):
     double crs[kMaxG][3];    // c_r sigma^N_ij, the absorption coefficient per absorber
     double hq[kMaxG][3];     // egy_i sigma^E_ij - eps_j sigma^N_ij, photoheating per absorber
+    double mu_0, mu_w;       // 1/mu = X x + mu_0 + mu_w (y2 + 2 y3): X + (1 - X)/4, (1 - X)/4
     double tg;               // T_gamma = 2.727 / a, the Compton temperature
     double comp;             // 1.017e-37 T_gamma^4, Compton exchange per (T - T_gamma) n_e
 };
@@ -82,7 +83,8 @@ struct ThermoParams {
 // Fill ThermoParams::crs and ::hq from cr and gc (the photoheating term of
 // Eq. (PHeat2): each absorbed photon of group i heats by its mean energy
 // minus the ionisation energy eps_j of the absorber, 13.60, 24.59, 54.42 eV),
-// and the Compton constants from a_exp.  Call after setting cr, gc, a_exp.
+// the Compton constants from a_exp and those of mu from X.  Call after setting
+// cr, gc, a_exp, X.
 inline void derive_group_terms(ThermoParams &p)
 {
     const double ev = 1.602176634e-12;
@@ -93,6 +95,8 @@ inline void derive_group_terms(ThermoParams &p)
             p.hq[i][j] = p.gc.egy[i] * p.gc.sigE[i][j] - eps[j] * p.gc.sigN[i][j];
         }
     // Compton cooling/heating of the rate appendix, varpi = 1.017e-37 T_g^4 (T - T_g)
+    p.mu_w = 0.25 * (1.0 - p.X);
+    p.mu_0 = p.X + p.mu_w;
     p.tg = 2.727 / p.a_exp;
     p.comp = 1.017e-37 * (p.tg * p.tg * p.tg * p.tg);
 }

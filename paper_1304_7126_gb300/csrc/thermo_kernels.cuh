@@ -31,7 +31,7 @@ template <int G, bool WARP, typename P, bool R32, bool SM>
 __device__ __forceinline__ void load_cell(const ThermoParams &p, long long c, bool first, const double *xHII,
                                           const double *xHeII, const double *xHeIII, const double *T,
                                           const P *N, const P *Npre, const double *fscale, CellState<G> &st,
-                                          IsoRates<> &iso, CoolCache<> &cc)
+                                          IsoRates<> &iso, CoolCache<> &cc, const RateFn *lq = nullptr)
 {
     st.x = xHII[c];
     st.y2 = xHeII[c];
@@ -58,10 +58,10 @@ __device__ __forceinline__ void load_cell(const ThermoParams &p, long long c, bo
     cc.valid = false;
     cc.rvalid = false;
     if (p.isothermal) {
-        Rates t;
-        get_rates<WARP, R32>(st.T, p.case_b, kNeedH | (p.helium ? kNeedHe : 0u), kNeedH, t);
-        h_rates_from(t, iso.h);
-        if (p.helium) he_rates_from(t, iso.he);
+        TLevel L;
+        t_level<WARP>(st.T, L);
+        h_rates<WARP, R32>(L, 0.0, p.case_b, lq, iso.h);
+        if (p.helium) he_rates<WARP, R32>(L, 0.0, p.case_b, lq, iso.he);
     }
 }
 
@@ -255,9 +255,7 @@ thermo_drain(ThermoParams p, const double *__restrict__ nH, double *xHII, double
 // Both warps run the cell's attempts in step with identical state; in each
 // attempt that needs the cooling at T(t), warp 2k + 1 evaluates it while
 // warp 2k updates the photons (PairX exchange, thermo_step.cuh).  Warp 2k
-// takes the next queue item and posts it to its partner the same way.  A
-// wait that runs out (it cannot while both warps run the same code) sets
-// the queue status bit and ends the pair.
+// takes the next queue item and posts it to its partner the same way.
 template <int G, typename P, bool R32, bool SM>
 __global__ void __launch_bounds__(128)
 thermo_hard(ThermoParams p, const double *__restrict__ nH, double *xHII, double *xHeII, double *xHeIII,
@@ -270,28 +268,16 @@ thermo_hard(ThermoParams p, const double *__restrict__ nH, double *xHII, double 
     const int lane = threadIdx.x & 31;
     const int warp = threadIdx.x >> 5;
     const int team = warp >> 1;
-    PairCtx pc{&px[team], warp & 1, 0, false};
-    if (lane == 0) px[team].seq[pc.role] = 0;
-    __syncthreads();
+    PairCtx pc{&px[team], warp & 1, 0, 1 + team};
     PairX<G> &X = px[team];
+    const RateFn lq = lane_rate_fn(p.case_b);
     while (true) {
         // the item: taken by role 0, posted to role 1 (exchange pc.n)
         const int b = pc.n & 1;
-        const int n = ++pc.n;
-        unsigned long long it = 0;
-        if (pc.role == 0) {
-            if (lane == 0) {
-                it = atomicAdd(&q.counters[5], 1ULL);
-                X.item[b] = it;
-            }
-            it = __shfl_sync(0xffffffffu, it, 0);
-            pair_post(&X.seq[0], n);
-            if (!pair_wait(&X.seq[1], n, status)) return;
-        } else {
-            pair_post(&X.seq[1], n);
-            if (!pair_wait(&X.seq[0], n, status)) return;
-            it = X.item[b];
-        }
+        ++pc.n;
+        if (pc.role == 0 && lane == 0) X.item[b] = atomicAdd(&q.counters[5], 1ULL);
+        pair_meet(pc);
+        const unsigned long long it = X.item[b];
         if (it >= count) break;
         const long long c = q.a.cell[it];
         double t_left = q.a.t_left[it];
@@ -301,17 +287,19 @@ thermo_hard(ThermoParams p, const double *__restrict__ nH, double *xHII, double 
         CellState<G> st;
         IsoRates<> iso;
         CoolCache<> cc;
-        load_cell<G, true, P, R32, SM>(p, c, false, xHII, xHeII, xHeIII, T, N, Npre, q.fscale, st, iso, cc);
+        load_cell<G, true, P, R32, SM>(p, c, false, xHII, xHeII, xHeIII, T, N, Npre, q.fscale, st, iso, cc, &lq);
         cell_constants(p, n_h, iso);
         bool done = false;
         while (!done) {
-            done = subcycle_once<G, true, R32, double, SM, true>(p, n_h, st, t_left, dt_tc, att, iso, cc, &pc, status);
-            if (pc.failed) return;
+            done = subcycle_once<G, true, R32, double, SM, true>(p, n_h, st, t_left, dt_tc, att, iso, cc, &lq, &pc);
             if (!done && att >= p.max_sub) {
                 if (lane == 0 && pc.role == 0) atomicOr(status, kStatusSubcycle);
                 done = true;
             }
         }
+        // (the partner has read its item's state: it has met this warp since,
+        // or, with fixed rates or kept cooling, ran the same attempts)
+        pair_meet(pc);
         if (lane == 0 && pc.role == 0) {
             store_cell<G, P, SM>(p, c, false, false, xHII, xHeII, xHeIII, T, N, F, Npre, Fpre, q.fscale, st, status);
             subcycles[c] = att;

@@ -49,23 +49,36 @@ template <typename S>
 __device__ __forceinline__ void cell_constants(const ThermoParams &p, const S &nH, IsoRates<S> &iso)
 {
     iso.nHe = nH * p.he_ratio;
-    iso.K = p.kfac / nH;
+    iso.K = qdiv(S(p.kfac), nH);
     iso.nef = kNeFloor * nH;
 }
 
-// 1/mu, mu the mean particle mass in m_H (App. A)
+// y2 + 2 y3, electrons per helium nucleus
 template <typename S>
-__device__ __forceinline__ S mu_den(double X, const S &x, const S &y2, const S &y3)
+__device__ __forceinline__ S he_electrons(const S &y2, const S &y3)
 {
-    return X * (1.0 + x) + 0.25 * (1.0 - X) * (1.0 + y2 + 2.0 * y3);
+    return rfma(2.0, y3, y2);
 }
 
+// n_e given q = he_electrons
 template <typename S>
-__device__ __forceinline__ S mu_of(double X, const S &x, const S &y2, const S &y3)
+__device__ __forceinline__ S ne_of(const S &nHII, const S &q, const S &nHe)
 {
-    return qdiv(S(1.0), mu_den(X, x, y2, y3));
+    return rfma(q, nHe, nHII);
 }
 
+// 1/mu = X (1 + x) + (1 - X)(1 + y2 + 2 y3)/4, mu the mean particle mass in
+// m_H (App. A): X x + md_he(q), md_he(q) = X + (1 - X)(1 + q)/4
+template <typename S>
+__device__ __forceinline__ S md_he(const ThermoParams &p, const S &q)
+{
+    return rfma(p.mu_w, q, S(p.mu_0));
+}
+template <typename S>
+__device__ __forceinline__ S mu_den(const ThermoParams &p, const S &x, const S &mhe)
+{
+    return rfma(p.X, x, mhe);
+}
 
 // Comparisons, minima and maxima of doubles through their bit patterns, on
 // the integer pipe (a GB300 warp issues one FP64 instruction, compares and
@@ -159,54 +172,143 @@ __device__ __forceinline__ bool ratio_lt(const S &a, const S &b, double t)
     return quotient_lt<S>(a, b, t);
 }
 
+// The change of a checked quantity from `o` to `n` against its 10% and 5%
+// limits, relative to max(o, floor): in FP32 (the floats nearest to the two
+// are within 2^-24, so 1e-5 around the limits is undecided by far), and
+// there exactly as the rounded quotient decides.  An FP64 difference and two
+// products per check before.
+template <typename S>
+__device__ __noinline__ bool change_gt(S n, S o, S floor_, double t)
+{
+    return ratio_gt(fabs(n - o), max0(o, floor_), t);
+}
+template <typename S>
+__device__ __noinline__ bool change_lt(S n, S o, S floor_, double t)
+{
+    return ratio_lt(fabs(n - o), max0(o, floor_), t);
+}
+template <typename S>
+__device__ __forceinline__ bool change_ok(const S &n, const S &o, const S &floor_, bool &small)
+{
+    const float of = dfm::near_float(val(o));
+    const float d = fabsf(__fsub_rn(dfm::near_float(val(n)), of));
+    const float den = fmaxf(of, dfm::near_float(val(floor_)));
+    bool ok = d < 0.099999f * den;
+    if (!ok) {
+        if (d > 0.100001f * den) return false;
+        if (change_gt<S>(n, o, floor_, 0.1)) return false;
+    }
+    bool sm = d < 0.049999f * den;
+    if (!sm && !(d > 0.050001f * den)) sm = change_lt<S>(n, o, floor_, 0.05);
+    small = small && sm;
+    return true;
+}
+// |a| > t b for a first-order term a (b > 0)
+template <typename S>
+__device__ __noinline__ bool term_gt(S a, S b, double t)
+{
+    return ratio_gt(fabs(a), b, t);
+}
+template <typename S>
+__device__ __noinline__ bool term_lt(S a, S b, double t)
+{
+    return ratio_lt(fabs(a), b, t);
+}
+template <typename S>
+__device__ __forceinline__ bool term_ok(const S &a, const S &b)
+{
+    const float d = fabsf(dfm::near_float(val(a))), den = dfm::near_float(val(b));
+    if (d < 0.099999f * den) return true;
+    if (d > 0.100001f * den) return false;
+    return !term_gt<S>(a, b, 0.1);
+}
+template <typename S>
+__device__ __forceinline__ bool term_small(const S &a, const S &b)
+{
+    const float d = fabsf(dfm::near_float(val(a))), den = dfm::near_float(val(b));
+    if (d < 0.049999f * den) return true;
+    if (d > 0.050001f * den) return false;
+    return term_lt<S>(a, b, 0.05);
+}
+
+// Rates at one temperature level.  lq: the warp path's function of this lane.
+__device__ __forceinline__ RateFn lane_rate_fn(int case_b) { return g_rate_fn[case_b].f[threadIdx.x & 31]; }
+
 template <bool WARP, bool MIX>
-__device__ __forceinline__ void get_rates(const Dual &T, int case_b, unsigned needF, unsigned needD,
-                                          RatesT<Dual> &r)
+__device__ __forceinline__ void h_rates(const TLevel &L, double, int case_b, const RateFn *lq, HRates &r)
+{
+    if constexpr (WARP) {
+        Rates t;
+        rates_warp<MIX, true>(*lq, L, kNeedH, kNeedH, t);
+        h_rates_from(t, r);
+    } else {
+        r = h_rates_serial<MIX>(L, case_b);
+    }
+}
+template <bool WARP, bool MIX>
+__device__ __forceinline__ void he_rates(const TLevel &L, double, int case_b, const RateFn *lq, HeRates &r)
+{
+    if constexpr (WARP) {
+        Rates t;
+        rates_warp<MIX, false>(*lq, L, kNeedHe, 0u, t);
+        he_rates_from(t, r);
+    } else {
+        r = he_rates_serial<MIX>(L, case_b);
+    }
+}
+// (only beta_HeII and alpha_HeIII)
+template <bool WARP, bool MIX>
+__device__ __forceinline__ void he3_rates(const TLevel &L, double, int case_b, const RateFn *lq, HeRates &r)
+{
+    if constexpr (WARP) {
+        Rates t;
+        rates_warp<MIX, false>(*lq, L, kNeedHe3, 0u, t);
+        r.beta_HeII = t.f[RF_BETA_HEII];
+        r.alpha_HeIII = t.f[RF_ALPHA_HEIII];
+    } else {
+        const double2 t = he3_rates_serial<MIX>(L, case_b);
+        r.beta_HeII = t.x;
+        r.alpha_HeIII = t.y;
+    }
+}
+// dual numbers: the level of the value, dT the derivative of T
+template <bool WARP, bool MIX>
+__device__ __forceinline__ void h_rates(const TLevel &L, double dT, int case_b, const RateFn *, HRatesT<Dual> &r)
 {
     static_assert(!WARP && !MIX, "dual rates: one thread, FP64");
-    TLevel L;
-    t_level<false>(T.v, L);
-    rates_dual(L, T.d, case_b, needF, needD, r);
+    r = h_rates_dual(L, dT, case_b);
 }
 template <bool WARP, bool MIX>
-__device__ __forceinline__ void rates_at(const TLevel &L, int case_b, unsigned needF, unsigned needD, Rates &r)
+__device__ __forceinline__ void he_rates(const TLevel &L, double dT, int case_b, const RateFn *, HeRatesT<Dual> &r)
 {
-    if constexpr (WARP) rates_warp<MIX>(L, case_b, needF, needD, r);
-    else if constexpr (MIX) rates_serial_f(L, case_b, needF, needD, r);
-    else rates_serial(L, case_b, needF, needD, r);
+    r = he_rates_dual(L, dT, case_b);
 }
 template <bool WARP, bool MIX>
-__device__ __forceinline__ void get_rates(double T, int case_b, unsigned needF, unsigned needD, Rates &r)
+__device__ __forceinline__ void he3_rates(const TLevel &L, double dT, int case_b, const RateFn *, HeRatesT<Dual> &r)
 {
-    TLevel L;
-    t_level<MIX, WARP>(T, L);
-    rates_at<WARP, MIX>(L, case_b, needF, needD, r);
+    r = he_rates_dual(L, dT, case_b);
 }
-// Rates at T = (T/mu') mu_j given 1/mu_j = md and 1/(T/mu') = iT as a pair
-// (the helium temperatures of step 4 enter their rates only through 1/T and
-// ln T): 1/T = md iT in pair arithmetic, no FP64 quotient.  A dual T takes
-// the levels of its value and the derivative of Tmu1 / md.
+
+// The level of T = (T/mu') mu_j given 1/mu_j = md and 1/(T/mu') = iT as a
+// pair (the temperatures of steps 3 and 4 enter their rates only through
+// 1/T and ln T): 1/T = md iT in pair arithmetic; and the derivative of a
+// dual T = Tmu1 / md.
 __device__ __forceinline__ dfm::F2 inv_pair(double x)
 {
     if (!(x > 0.0) || !dfm::splittable(x)) return dfm::split_any(1.0 / x);
     return dfm::rcp2(dfm::split(x));
 }
-template <bool WARP, bool MIX>
-__device__ __forceinline__ void rates_mu(const Dual &md, dfm::F2 iT, const Dual &Tmu1, int case_b, unsigned needF,
-                                         unsigned needD, RatesT<Dual> &r)
+template <bool WARP>
+__device__ __forceinline__ double level_mu(const Dual &md, dfm::F2 iT, const Dual &Tmu1, TLevel &L)
 {
-    static_assert(!WARP && !MIX, "dual rates: one thread, FP64");
-    TLevel L;
-    t_level_inv<false>(dfm::mul(dfm::split_any(md.v), iT), L);
-    rates_dual(L, (Tmu1 / md).d, case_b, needF, needD, r);
+    t_level_inv<WARP>(dfm::mul(dfm::split_any(md.v), iT), L);
+    return qdiv(Tmu1, md).d;
 }
-template <bool WARP, bool MIX>
-__device__ __forceinline__ void rates_mu(double md, dfm::F2 iT, double, int case_b, unsigned needF,
-                                         unsigned needD, Rates &r)
+template <bool WARP>
+__device__ __forceinline__ double level_mu(double md, dfm::F2 iT, double, TLevel &L)
 {
-    TLevel L;
-    t_level_inv<MIX, WARP>(dfm::mul(dfm::split_any(md), iT), L);
-    rates_at<WARP, MIX>(L, case_b, needF, needD, r);
+    t_level_inv<WARP>(dfm::mul(dfm::split_any(md), iT), L);
+    return 0.0;
 }
 
 // (alpha^A_j - alpha^B_j) n_j n_e of HII, HeII, HeIII at temperature T
@@ -216,15 +318,22 @@ __device__ __forceinline__ void rates_mu(double md, dfm::F2 iT, double, int case
 template <bool WARP, bool MIX, typename S>
 __device__ __noinline__ void recomb_rates(S T, S nHII, S nHeII, S nHeIII, S ne, S *rj)
 {
-    S aA[3], aB[3];
+    static_assert(std::is_same<S, double>::value, "the adjoint needs the OTSA");
+    double aA[3], aB[3];
+    TLevel L;
+    t_level<WARP>(T, L);
     {
-        RatesT<S> t;
-        get_rates<WARP, MIX>(T, 0, kNeedRec, 0u, t);
+        const RateFn q = lane_rate_fn(0);
+        Rates t;
+        if constexpr (WARP) rates_warp<MIX, false>(q, L, kNeedRec, 0u, t);
+        else rates_serial<MIX>(L, 0, kNeedRec, 0u, t);
         recomb_alphas(t, aA);
     }
     {
-        RatesT<S> t;
-        get_rates<WARP, MIX>(T, 1, kNeedRec, 0u, t);
+        const RateFn q = lane_rate_fn(1);
+        Rates t;
+        if constexpr (WARP) rates_warp<MIX, false>(q, L, kNeedRec, 0u, t);
+        else rates_serial<MIX>(L, 1, kNeedRec, 0u, t);
         recomb_alphas(t, aB);
     }
     rj[0] = (aA[0] - aB[0]) * nHII * ne;
@@ -260,10 +369,10 @@ __device__ __forceinline__ void photon_group(const ThermoParams &p, int i, const
         const float Df = __fadd_rn(__fadd_rn(__fmul_rn(narrow(p.crs[i][0]), narrow(nHI)),
                                              __fmul_rn(narrow(p.crs[i][1]), narrow(nHeI))),
                                    __fmul_rn(narrow(p.crs[i][2]), narrow(nHeII)));
-        inv = qdiv(1.0, rfma(h, dfm::widen(Df), 1.0));
+        inv = qrcp(rfma(h, dfm::widen(Df), 1.0));
     } else {
         const S D = rfma(p.crs[i][2], nHeII, rfma(p.crs[i][1], nHeI, rmul(nHI, p.crs[i][0])));
-        inv = qdiv(S(1.0), rfma(h, D, S(1.0)));
+        inv = qrcp(rfma(h, D, S(1.0)));
     }
     // smoothed RT: N + h Ndot rounded step by step, so a cell growing
     // linearly from zero meets its relative changes 1/k exactly
@@ -271,9 +380,8 @@ __device__ __forceinline__ void photon_group(const ThermoParams &p, int i, const
     if constexpr (SM) Nn = rmul(radd(N, rmul(Nd + Crec, h)), inv);
     else if (p.emit) Nn = rmul(rfma(h, Crec, N), inv);
     else Nn = rmul(N, inv);
-    const S dN = fabs(radd(Nn, -N)), den = max0(N, kFloorN);
-    o.ok = !ratio_gt(dN, den, 0.1);
-    o.small = ratio_lt(dN, den, 0.05);
+    o.small = true;
+    o.ok = change_ok(Nn, N, S(kFloorN), o.small);
     o.Nn = Nn;
     o.Fs = rmul(Fs, inv);
     if constexpr (SM) o.Fb = rmul(radd(Fb, S(h)), inv);
@@ -367,51 +475,29 @@ __device__ __forceinline__ bool photons_serial(const ThermoParams &p, const Cell
 
 // The two warps of a pair of the tail kernel (thermo_hard): while one evaluates
 // the cooling at T(t) the other updates the photons; each posts its results
-// in shared memory with a sequence number and waits (bounded) for the
-// other's.  Both then hold the same values and run the rest of the attempt
-// in step.  Two buffers alternate, so a post never overwrites data the
-// partner may still be reading (every exchange is two-way).
+// in shared memory and both meet at the pair's named barrier.  Both then hold
+// the same values and run the rest of the attempt in step, so every exchange
+// is met by both.  Two buffers alternate, so a post never overwrites data the
+// partner may still be reading.  (Polled sequence numbers, with a sleep
+// between polls, made an exchange longer.)
 template <int G>
 struct PairX {
     double N[2][G], Fs[2][G], Fb[2][G], g[2][4], L[2], dL[2], m[2][3];
     int ok[2], small[2];
     unsigned long long item[2];
-    volatile int seq[2];   // last exchange posted by role 0, role 1
 };
 
 struct PairCtx {
     void *x;          // PairX<G> of the pair, shared memory
     int role;         // 0: photons, 1: cooling
     int n;            // exchanges so far (the same in both warps)
-    bool failed;      // a wait ran out (status set; the cell is abandoned)
+    int bar;          // the pair's named barrier
 };
 
-constexpr long long kPairSpinLimit = 1LL << 24;   // polls before a wait gives up
-
-// post this warp's part of exchange pc.n, then wait for the partner's
-__device__ __forceinline__ void pair_post(volatile int *seq_mine, int n)
+__device__ __forceinline__ void pair_meet(const PairCtx &pc)
 {
-    __threadfence_block();
     __syncwarp();
-    if ((threadIdx.x & 31) == 0) *seq_mine = n;
-}
-
-__device__ __forceinline__ bool pair_wait(volatile int *seq_other, int n, unsigned *status)
-{
-    bool ok = true;
-    if ((threadIdx.x & 31) == 0) {
-        long long k = 0;
-        while (*seq_other < n && k < kPairSpinLimit) {
-            __nanosleep(32);
-            ++k;
-        }
-        ok = *seq_other >= n;
-        if (!ok) atomicOr(status, kStatusQueue);
-    }
-    ok = __shfl_sync(0xffffffffu, ok, 0);
-    __syncwarp();
-    __threadfence_block();
-    return ok;
+    asm volatile("bar.sync %0, 64;" ::"r"(pc.bar) : "memory");
 }
 
 // One thermo_step over h.  Returns true and fills `o` when the 10% rule
@@ -427,19 +513,21 @@ __device__ __forceinline__ bool pair_wait(volatile int *seq_other, int n, unsign
 template <int G, bool WARP, bool MIX, typename S = double, bool SM = false, bool PAIR = false>
 __device__ __forceinline__ bool attempt(const ThermoParams &p, const S &nH, const CellState<G, S> &s, double h,
                                         const IsoRates<S> &iso, CoolCache<S> &cc, CellState<G, S> &o,
-                                        bool &small, PairCtx *pc = nullptr, unsigned *status = nullptr)
+                                        bool &small, const RateFn *lq = nullptr, PairCtx *pc = nullptr)
 {
     static_assert(!PAIR || (WARP && sizeof(S) == sizeof(double)), "pairs of warps: the warp path");
     static_assert(!MIX || sizeof(S) == sizeof(double), "the mixed path is not differentiated");
     const S nHe = iso.nHe;
     const S x = s.x, y2 = s.y2, y3 = s.y3;
-    const S nHI = nH * (1.0 - x);
-    const S nHII = nH * x;
-    const S nHeI = nHe * (1.0 - y2 - y3);
-    const S nHeII = nHe * y2;
-    const S nHeIII = nHe * y3;
-    const S ne = nHII + (y2 + 2.0 * y3) * nHe;
-    const double cr = p.cr;
+    const S q0 = he_electrons(y2, y3);
+    const S nHI = rmul(nH, radd(S(1.0), -x));
+    const S nHII = rmul(nH, x);
+    const S yI = radd(radd(S(1.0), -y2), -y3);
+    const S nHeI = rmul(nHe, yI);
+    const S nHeII = rmul(nHe, y2);
+    const S nHeIII = rmul(nHe, y3);
+    const S ne = ne_of(nHII, q0, nHe);
+    const S mhe = md_he(p, q0);
     bool sm = true;
     S gam0 = 0.0, gam1 = 0.0, gam2 = 0.0, heat = 0.0;
 
@@ -449,9 +537,11 @@ __device__ __forceinline__ bool attempt(const ThermoParams &p, const S &nH, cons
     // recombination photons without the OTSA, Eq. (cool_N_cr), at T(t) with
     // the backward abundances; group i gains C_i = sum_j [rec_g[j] == i] rj[j]
     // (before the cooling: a pair of warps updates the photons there)
-    if (p.emit && !cc.rvalid) {
-        recomb_rates<WARP, MIX>(s.T, nHII, nHeII, nHeIII, ne, cc.rj);
-        cc.rvalid = true;
+    if constexpr (std::is_same<S, double>::value) {   // (the adjoint needs the OTSA)
+        if (p.emit && !cc.rvalid) {
+            recomb_rates<WARP, MIX>(s.T, nHII, nHeII, nHeIII, ne, cc.rj);
+            cc.rvalid = true;
+        }
     }
 
     bool pair_photons = false;   // the photon stage was done in the pair exchange
@@ -463,18 +553,18 @@ __device__ __forceinline__ bool attempt(const ThermoParams &p, const S &nH, cons
             // role 1 evaluates the cooling, role 0 the photon stage, at once
             PairX<G> &X = *static_cast<PairX<G> *>(pc->x);
             const int b = pc->n & 1;
-            const int n = ++pc->n;
+            ++pc->n;
             const int lane = threadIdx.x & 31;
+            cc.valid = true;
             if (pc->role == 1) {
-                cooling_warp<MIX>(p.case_b, p.comp, p.tg, p.helium != 0, s.T, ne, nHI, nHII, nHeI, nHeII, nHeIII,
-                                  cc.L, cc.dL);
+                cooling_warp<MIX>(*lq, p.comp, p.tg, p.helium != 0, s.T, ne, nHI, nHII, nHeI, nHeII, nHeIII, cc.L,
+                                  cc.dL);
                 if (lane == 0) {
                     X.L[b] = cc.L;
                     X.dL[b] = cc.dL;
                 }
-                pair_post(&X.seq[1], n);
-                if (!pair_wait(&X.seq[0], n, status)) { pc->failed = true; return false; }
-                if (!X.ok[b]) { cc.valid = true; return false; }
+                pair_meet(*pc);
+                if (!X.ok[b]) return false;
 #pragma unroll
                 for (int i = 0; i < G; ++i) {
                     o.N[i] = X.N[b][i];
@@ -490,9 +580,9 @@ __device__ __forceinline__ bool attempt(const ThermoParams &p, const S &nH, cons
             } else {
                 const bool ok = photons_warp<G, MIX, SM>(p, s, cc, nHI, nHeI, nHeII, h, o, gam0, gam1, gam2, heat, sm);
                 // (this warp would wait for the cooling meanwhile)
-                mden = mu_den(p.X, x, y2, y3);
-                mu = qdiv(S(1.0), mden);
-                Tmu = s.T * mden;
+                mden = mu_den(p, x, mhe);
+                mu = qrcp(mden);
+                Tmu = rmul(s.T, mden);
                 if (lane == 0) {
                     X.m[b][0] = mden; X.m[b][1] = mu; X.m[b][2] = Tmu;
 #pragma unroll
@@ -505,25 +595,20 @@ __device__ __forceinline__ bool attempt(const ThermoParams &p, const S &nH, cons
                     X.ok[b] = ok;
                     X.small[b] = sm;
                 }
-                pair_post(&X.seq[0], n);
-                if (!pair_wait(&X.seq[1], n, status)) { pc->failed = true; return false; }
+                pair_meet(*pc);
                 cc.L = X.L[b];
                 cc.dL = X.dL[b];
-                if (!ok) { cc.valid = true; return false; }
+                if (!ok) return false;
             }
-            cc.valid = true;
             pair_photons = true;
             have_mu = true;
         } else {
-            if constexpr (WARP) {   // lane k evaluates cooling term k
-                cooling_warp<MIX>(p.case_b, p.comp, p.tg, p.helium != 0, s.T, ne, nHI, nHII, nHeI, nHeII, nHeIII,
-                                  cc.L, cc.dL);
-            } else {
-                const unsigned need = kNeedCoolH | (p.helium ? kNeedCoolHe : 0u);
-                RatesT<S> t;
-                get_rates<WARP, MIX>(s.T, p.case_b, need, need, t);
-                cooling_from(t, p.comp, p.tg, p.helium != 0, s.T, ne, nHI, nHII, nHeI, nHeII, nHeIII, cc.L, cc.dL);
-            }
+            if constexpr (WARP)   // lane k evaluates cooling term k
+                cooling_warp<MIX>(*lq, p.comp, p.tg, p.helium != 0, s.T, ne, nHI, nHII, nHeI, nHeII, nHeIII, cc.L,
+                                  cc.dL);
+            else
+                cooling_serial<MIX>(p.case_b, p.comp, p.tg, p.helium != 0, s.T, ne, nHI, nHII, nHeI, nHeII, nHeIII,
+                                    cc.L, cc.dL);
             cc.valid = true;
         }
     }
@@ -539,103 +624,95 @@ __device__ __forceinline__ bool attempt(const ThermoParams &p, const S &nH, cons
         else ok = photons_serial<G, MIX, SM>(p, s, cc, nHI, nHeI, nHeII, h, o, gam0, gam1, gam2, heat, sm);
         if (!ok) return false;
     }
-    if (p.isothermal) heat = 0.0;
 
     // 2. temperature: T/mu + K h (Lambda) / (1 + mu (dL/dT) K h), Lambda =
     // heating - cooling, d Lambda/d(T/mu) = -mu dL/dT
-    if (!have_mu) {
-        mden = mu_den(p.X, x, y2, y3);
-        mu = qdiv(S(1.0), mden);
-        Tmu = s.T * mden;
-    }
     S Tmu1 = 0.0;
     if (!p.isothermal) {
-        const S Kh = iso.K * h;
-        const S num = (heat - cc.L) * Kh;
-        const S dT = qdiv(num, 1.0 + (mu * cc.dL) * Kh);
-        Tmu1 = Tmu + dT;
-        S adT = fabs(dT);
-        if (ratio_gt(fabs(num), Tmu, 0.1)) return false;
-        if (ratio_gt(adT, Tmu, 0.1)) return false;
-        sm = sm && ratio_lt(adT, Tmu, 0.05);
+        if (!have_mu) {
+            mden = mu_den(p, x, mhe);
+            mu = qrcp(mden);
+            Tmu = rmul(s.T, mden);
+        }
+        const S Kh = rmul(iso.K, h);
+        const S num = rmul(radd(heat, -cc.L), Kh);
+        const S dT = qdiv(num, rfma(rmul(mu, cc.dL), Kh, S(1.0)));
+        Tmu1 = radd(Tmu, dT);
+        if (!term_ok(num, Tmu)) return false;
+        if (!term_ok(dT, Tmu)) return false;
+        sm = sm && term_small(dT, Tmu);
     }
-    // 1/(T/mu') as a pair, for the helium temperatures (T/mu') mu_j
-    const dfm::F2 iT = (p.isothermal || !p.helium) ? dfm::F2{0.0f, 0.0f} : inv_pair(val(Tmu1));
+    // 1/(T/mu') as a pair, for the temperatures (T/mu') mu_j of steps 3 and 4
+    const dfm::F2 iT = p.isothermal ? dfm::F2{0.0f, 0.0f} : inv_pair(val(Tmu1));
 
     // 3. hydrogen
     HRatesT<S> hr;
     if (p.isothermal) {
         hr = iso.h;
     } else {
-        RatesT<S> t;
-        get_rates<WARP, MIX>(Tmu1 * mu, p.case_b, kNeedH, kNeedH, t);
-        h_rates_from(t, hr);
+        TLevel L;
+        const double dT = level_mu<WARP>(mden, iT, Tmu1, L);
+        h_rates<WARP, MIX>(L, dT, p.case_b, lq, hr);
     }
-    S C = hr.beta * ne + gam0;
-    S Dd = hr.alpha * ne;
-    S dC = nH * hr.beta, dD = nH * hr.alpha;
+    const S C = rfma(hr.beta, ne, gam0);
+    const S CD = rfma(hr.alpha, ne, C);   // C + D, D = alpha n_e
+    S dC = rmul(nH, hr.beta), dD = rmul(nH, hr.alpha);
     if (!p.isothermal) {
-        S f = ne * Tmu1 * mu * mu * p.X;
-        dC -= f * hr.dbeta;
-        dD -= f * hr.dalpha;
+        // - n_e (T/mu') mu^2 X d/dT
+        const S f = rmul(rmul(ne, rmul(Tmu1, mu)), rmul(-mu, p.X));
+        dC = rfma(f, hr.dbeta, dC);
+        dD = rfma(f, hr.dalpha, dD);
     }
-    S J = dC - (C + Dd) - x * (dC + dD);
-    S xdot = C - x * (C + Dd);
-    S x1 = x + qdiv(h * xdot, 1.0 - J * h);
+    const S J = rfma(-x, radd(dC, dD), radd(dC, -CD));
+    const S hx = rmul(rfma(-x, CD, C), h);
+    S x1 = radd(x, qdiv(hx, rfma(-J, S(h), S(1.0))));
     x1 = min0(max0(x1, kXMin), 1.0);
-    {
-        S xden = max0(x, kXMin);
-        S dx = fabs(x1 - x);
-        if (ratio_gt(dx, xden, 0.1)) return false;
-        if (ratio_gt(fabs(xdot) * h, xden, 0.1)) return false;
-        sm = sm && ratio_lt(dx, xden, 0.05);
-    }
+    if (!change_ok(x1, x, S(kXMin), sm)) return false;
+    if (!term_ok(hx, max0(x, kXMin))) return false;
 
     // 4. helium
     S y2n = y2, y3n = y3;
+    const S nHII1 = rmul(x1, nH);
     if (p.helium) {
-        S yI = 1.0 - y2 - y3;
-        S ne2 = x1 * nH + (y2 + 2.0 * y3) * nHe;
+        const S ne2 = ne_of(nHII1, q0, nHe);
         HeRatesT<S> r2;
         if (p.isothermal) {
             r2 = iso.he;
         } else {
-            RatesT<S> t;
-            rates_mu<WARP, MIX>(mu_den(p.X, x1, y2, y3), iT, Tmu1, p.case_b, kNeedHe, 0u, t);
-            he_rates_from(t, r2);
+            TLevel L;
+            const double dT = level_mu<WARP>(mu_den(p, x1, mhe), iT, Tmu1, L);
+            he_rates<WARP, MIX>(L, dT, p.case_b, lq, r2);
         }
-        S C1 = y2 * r2.alpha_HeII * ne2;
-        S D1 = r2.beta_HeI * ne2 + gam1;
-        S yI1 = qdiv(yI + C1 * h, 1.0 + D1 * h);
-        S C2 = yI1 * (r2.beta_HeI * ne2 + gam1) + y3 * r2.alpha_HeIII * ne2;
-        S D2 = (r2.beta_HeII + r2.alpha_HeII) * ne2 + gam2;
-        y2n = qdiv(y2 + C2 * h, 1.0 + D2 * h);
-        S ne3 = x1 * nH + (y2n + 2.0 * y3) * nHe;
+        const S hs(h);
+        const S D1 = rfma(r2.beta_HeI, ne2, gam1);
+        const S yI1 = qdiv(rfma(rmul(rmul(y2, r2.alpha_HeII), ne2), hs, yI), rfma(D1, hs, S(1.0)));
+        const S C2 = rfma(yI1, D1, rmul(rmul(y3, r2.alpha_HeIII), ne2));
+        const S D2 = rfma(radd(r2.beta_HeII, r2.alpha_HeII), ne2, gam2);
+        y2n = qdiv(rfma(C2, hs, y2), rfma(D2, hs, S(1.0)));
+        const S q1 = he_electrons(y2n, y3);
+        const S ne3 = ne_of(nHII1, q1, nHe);
         HeRatesT<S> r3;
         if (p.isothermal) {
             r3 = iso.he;
         } else {
-            RatesT<S> t;
-            rates_mu<WARP, MIX>(mu_den(p.X, x1, y2n, y3), iT, Tmu1, p.case_b, kNeedHe3, 0u, t);
-            r3.beta_HeII = t.f[RF_BETA_HEII];
-            r3.alpha_HeIII = t.f[RF_ALPHA_HEIII];
+            TLevel L;
+            const double dT = level_mu<WARP>(mu_den(p, x1, md_he(p, q1)), iT, Tmu1, L);
+            he3_rates<WARP, MIX>(L, dT, p.case_b, lq, r3);
         }
-        S C3 = y2n * (r3.beta_HeII * ne3 + gam2);
-        S D3 = r3.alpha_HeIII * ne3;
-        y3n = qdiv(y3 + C3 * h, 1.0 + D3 * h);
-        // conservation: lower the largest fraction (HeI largest: no change)
-        if (y2n >= yI1 && y2n >= y3n) y2n = 1.0 - yI1 - y3n;
-        else if (y3n >= yI1 && y3n > y2n) y3n = 1.0 - yI1 - y2n;
+        const S C3 = rmul(y2n, rfma(r3.beta_HeII, ne3, gam2));
+        const S D3 = rmul(r3.alpha_HeIII, ne3);
+        y3n = qdiv(rfma(C3, hs, y3), rfma(D3, hs, S(1.0)));
+        // conservation: lower the largest fraction (HeI largest: no change);
+        // (the fractions are positive or zero: compared by their bits)
+        const long long bI = dbits(val(yI1)), b2 = dbits(val(y2n)), b3 = dbits(val(y3n));
+        if (b2 >= bI && b2 >= b3) y2n = radd(radd(S(1.0), -yI1), -y3n);
+        else if (b3 >= bI && b3 > b2) y3n = radd(radd(S(1.0), -yI1), -y2n);
         y2n = min0(max0(y2n, 0.0), 1.0);
         y3n = min0(max0(y3n, 0.0), 1.0);
     }
-    {
-        S ne1 = x1 * nH + (y2n + 2.0 * y3n) * nHe;
-        S dne = fabs(ne1 - ne), den = max0(ne, iso.nef);
-        if (ratio_gt(dne, den, 0.1)) return false;
-        sm = sm && ratio_lt(dne, den, 0.05);
-    }
-    S Tf = p.isothermal ? s.T : qdiv(Tmu1, mu_den(p.X, x1, y2n, y3n));
+    const S q2 = he_electrons(y2n, y3n);
+    if (!change_ok(ne_of(nHII1, q2, nHe), ne, iso.nef, sm)) return false;
+    const S Tf = p.isothermal ? s.T : qdiv(Tmu1, mu_den(p, x1, md_he(p, q2)));
     o.x = x1;
     o.y2 = y2n;
     o.y3 = y3n;
@@ -648,14 +725,14 @@ __device__ __forceinline__ bool attempt(const ThermoParams &p, const S &nH, cons
 template <int G, bool WARP, bool MIX, typename S = double, bool SM = false, bool PAIR = false>
 __device__ __forceinline__ bool subcycle_once(const ThermoParams &p, const S &nH, CellState<G, S> &st,
                                               double &t_left, double &dt_tc, int &att, const IsoRates<S> &iso,
-                                              CoolCache<S> &cc, PairCtx *pc = nullptr, unsigned *status = nullptr)
+                                              CoolCache<S> &cc, const RateFn *lq = nullptr, PairCtx *pc = nullptr)
 {
     // t_left, dt_tc > 0: compared through their bits
     double h = (dbits(dt_tc) < dbits(t_left)) ? dt_tc : t_left;
     ++att;
     CellState<G, S> o;
     bool small = false;
-    if (attempt<G, WARP, MIX, S, SM, PAIR>(p, nH, st, h, iso, cc, o, small, pc, status)) {
+    if (attempt<G, WARP, MIX, S, SM, PAIR>(p, nH, st, h, iso, cc, o, small, lq, pc)) {
         st = o;
         cc.valid = false;
         cc.rvalid = false;
