@@ -36,15 +36,15 @@ UNIT = "cell-group updates/s"
 # (oracle/make_counts.py writes tests/golden/op_counts.json): FP64 flops per
 # thermochemistry attempt and per transport cell-group, as the oracle states
 # the method.  Transport bytes: N, F read and written once per cell-group.
-# the library's default routing: attempts of the first pass, and of the
-# first lane-per-cell drain stage
+# the library's default routing: attempts of the first pass; cells past
+# LONG_ATTEMPTS in all are reported as long sub-cyclers
 PASS1_ATTEMPTS = 6
-DRAIN1_BUDGET = 128
+LONG_ATTEMPTS = 134
 # DRAM bytes (read + write) per launch, from the ncu captures of the current
 # kernels summarised in profiles/ (128^3 x 3 groups, HLL)
 TRAFFIC = {"transport": 399187712 + 192541696,
-           # the two drains and thermo_hard of one step (the phase's three kernels)
-           "thermo_drain": 830720 + 77568 + 594688 + 5888}
+           # thermo_team
+           "thermo_drain": 325376}
 
 
 def _op_counts():
@@ -218,8 +218,8 @@ def _config(w):
 
 
 # kernels each profiled phase of one RT step launches (the thermochemistry
-# drain phase: two lane-per-cell drains and the warp-per-cell kernel)
-KERNELS_PER_PHASE = {"inject": 1, "transport": 1, "thermo_pass1": 1, "thermo_drain": 3, "reduce": 1, "finalize": 1}
+# drain phase: the team-per-cell kernel)
+KERNELS_PER_PHASE = {"inject": 1, "transport": 1, "thermo_pass1": 1, "thermo_drain": 1, "reduce": 1, "finalize": 1}
 
 
 def oracle_rate(w, nthreads, max_steps, seconds=30.0, boxes=None):
@@ -394,7 +394,7 @@ def main():
         q = sub > PASS1_ATTEMPTS
         queued += int(q.sum().item())
         queued_att += int((sub[q] - PASS1_ATTEMPTS).sum().item())
-        long_cells += int((sub > PASS1_ATTEMPTS + DRAIN1_BUDGET).sum().item())
+        long_cells += int((sub > LONG_ATTEMPTS).sum().item())
         pass1_att.append(int(torch.clamp(sub, max=PASS1_ATTEMPTS).sum().item()))
     prof = sim.profile()
     sim.set_profiling(False)
@@ -443,7 +443,7 @@ def main():
         roof = {"bound": "alu", "achieved": ach, "peak": fp64_peak, "unit": "GFLOP/s",
                 "frac": ach / fp64_peak,
                 "traffic": TRAFFIC.get(dominant) if w.name == "cosmo128_s7" else None,
-                "kernel": dominant + " (two lane-per-cell drains + warp-per-cell thermo_hard)"
+                "kernel": dominant + " (thermo_team, four lanes per cell)"
                 if dominant == "thermo_drain" else dominant,
                 "peak_kind": "measured (cuBLAS DGEMM, FP64)",
                 "flop_per_attempt": fpa, "transcendental_calls_per_attempt":
@@ -726,7 +726,7 @@ def main():
                 "variants": variants,
                 "thermo_attempts": {"per_step": attempts / args.steps, "max_per_cell": att_max,
                                     "queued_cells_per_step": queued / args.steps,
-                                    "cells_past_first_drain_per_step": long_cells / args.steps,
+                                    "long_cells_per_step": long_cells / args.steps,
                                     "first_pass_attempts_by_step": pass1_att,
                                     "queued_attempts_per_step": queued_att / args.steps}}
         print(json.dumps(line), flush=True)

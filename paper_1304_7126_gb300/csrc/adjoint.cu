@@ -103,14 +103,14 @@ thermo_vjp_kernel(ThermoParams p, const double *__restrict__ nH, const double *_
     if (p.isothermal) {
         TLevel L;
         t_level(st.T.v, L);
-        h_rates<false, false>(L, st.T.d, p.case_b, nullptr, iso.h);
-        if (p.helium) he_rates<false, false>(L, st.T.d, p.case_b, nullptr, iso.he);
+        h_rates<1, false>(L, st.T.d, p.case_b, iso.h);
+        if (p.helium) he_rates<1, false>(L, st.T.d, p.case_b, iso.he);
     }
     double t_left = p.dt, dt_tc = p.dt;
     int att = 0;
     bool done = false;
     while (!done) {
-        done = subcycle_once<G, false, false, Dual>(p, n, st, t_left, dt_tc, att, iso, cc);
+        done = subcycle_once<G, 1, false, Dual>(p, n, st, t_left, dt_tc, att, iso, cc);
         if (!done && att >= p.max_sub) {
             atomicOr(status, kStatusSubcycle);
             done = true;

@@ -244,7 +244,6 @@ static __device__ const int g_cool_sp[16] = {SP_HI, SP_HI, SP_HII, SP_FF, SP_HEI
 struct TLevel {
     dfm::F2 lnT, invT;
 };
-template <bool INL = false>
 __device__ __forceinline__ void t_level(double T, TLevel &L)
 {
     using namespace dfm;
@@ -253,17 +252,16 @@ __device__ __forceinline__ void t_level(double T, TLevel &L)
         L.invT = split_any(1.0 / T);
     } else {
         const F2 T2 = split(T);
-        L.lnT = INL ? log2f2_inl(T2) : log2f2(T2);
+        L.lnT = log2f2(T2);
         L.invT = rcp(T2);
     }
 }
 // the same from 1/T as a pair
-template <bool INL = false>
 __device__ __forceinline__ void t_level_inv(dfm::F2 invT, TLevel &L)
 {
     using namespace dfm;
     L.invT = invT;
-    if (invT.hi > 0x1p-60f && invT.hi < 0x1p60f) L.lnT = neg(INL ? log2f2_inl(invT) : log2f2(invT));
+    if (invT.hi > 0x1p-60f && invT.hi < 0x1p60f) L.lnT = neg(log2f2(invT));
     else L.lnT = split_any(-log(to_double(invT)));
 }
 
@@ -427,29 +425,27 @@ __device__ __forceinline__ void rates_serial(const TLevel &L, int case_b, unsign
     }
 }
 
-// a full warp (all 32 lanes, the same T): lane k's function k, its constants
-// q in registers
-template <bool MIX, bool DERIV>
-__device__ __forceinline__ void rate_lane(const RateFn &q, const TLevel &L, RateVal &r)
+// ---- teams: TS (4 or 8) adjacent lanes of a warp work on one cell, holding
+// the same state and sharing its rate functions ----
+template <int TS>
+__device__ __forceinline__ int team_lane() { return (int)(threadIdx.x & (TS - 1)); }
+template <int TS>
+__device__ __forceinline__ unsigned team_mask()
 {
+    static_assert(TS == 1 || TS == 4 || TS == 8, "team sizes");
+    return ((1u << TS) - 1u) << (threadIdx.x & 31u & ~(TS - 1u));
+}
+template <int TS>
+__device__ __forceinline__ double team_get(unsigned m, double v, int src) { return __shfl_sync(m, v, src, TS); }
+
+// one function per lane of a team, slot k, with its own softplus
+template <bool MIX, bool DERIV>
+__device__ __forceinline__ void rate_lane(int case_b, int k, const TLevel &L, RateVal &r)
+{
+    const RateFn &q = g_rate_fn[case_b].f[k];
     dfm::F2 sig;
     const dfm::F2 l = rate_softplus<MIX>(q, L, sig);
     rate_val<MIX, DERIV>(q, L, l, sig, 0u, false, r);
-}
-// ... and the needed ones in every lane
-template <bool MIX, bool DERIV>
-__device__ __forceinline__ void rates_warp(const RateFn &q, const TLevel &L, unsigned needF, unsigned needD, Rates &r)
-{
-    RateVal v;
-    rate_lane<MIX, DERIV>(q, L, v);
-    const double f = rate_f(v);
-    double df = 0.0;
-    if constexpr (DERIV) df = rate_df(v, L);
-#pragma unroll
-    for (int k = 0; k < NRF; ++k) {
-        if (needF & rf_bit(k)) r.f[k] = __shfl_sync(0xffffffffu, f, k);
-        if (DERIV && (needD & rf_bit(k))) r.df[k] = __shfl_sync(0xffffffffu, df, k);
-    }
 }
 
 // f, df/dT and d2f/dT2 of slot k at level L (values f, df with the bits of
@@ -545,6 +541,38 @@ static __device__ __noinline__ double2 he3_rates_serial(TLevel L, int case_b)
     rates_serial<MIX>(L, case_b, kNeedHe3, 0u, t);
     return make_double2(t.f[RF_BETA_HEII], t.f[RF_ALPHA_HEIII]);
 }
+// ... and by a team: lanes 0 and 1 the two hydrogen functions, lanes 0..3
+// the four helium ones, each then in every lane
+template <int TS, bool MIX>
+static __device__ __noinline__ HRates h_rates_team(TLevel L, int case_b)
+{
+    const unsigned m = team_mask<TS>();
+    RateVal v;
+    rate_lane<MIX, true>(case_b, team_lane<TS>() == 0 ? RF_BETA_HI : RF_ALPHA_HII, L, v);
+    const double f = rate_f(v), df = rate_df(v, L);
+    HRates r;
+    r.beta = team_get<TS>(m, f, 0);
+    r.dbeta = team_get<TS>(m, df, 0);
+    r.alpha = team_get<TS>(m, f, 1);
+    r.dalpha = team_get<TS>(m, df, 1);
+    return r;
+}
+static_assert(RF_BETA_HEII == RF_BETA_HEI + 1 && RF_ALPHA_HEII == RF_BETA_HEI + 2 && RF_ALPHA_HEIII == RF_BETA_HEI + 3,
+              "the helium functions of a team's lanes");
+template <int TS, bool MIX>
+static __device__ __noinline__ HeRates he_rates_team(TLevel L, int case_b)
+{
+    const unsigned m = team_mask<TS>();
+    RateVal v;
+    rate_lane<MIX, false>(case_b, RF_BETA_HEI + (team_lane<TS>() & 3), L, v);
+    const double f = rate_f(v);
+    HeRates r;
+    r.beta_HeI = team_get<TS>(m, f, 0);
+    r.beta_HeII = team_get<TS>(m, f, 1);
+    r.alpha_HeII = team_get<TS>(m, f, 2);
+    r.alpha_HeIII = team_get<TS>(m, f, 3);
+    return r;
+}
 static __device__ __noinline__ HRatesT<Dual> h_rates_dual(TLevel L, double dT, int case_b)
 {
     RatesT<Dual> t;
@@ -637,13 +665,26 @@ __device__ __forceinline__ void cooling_close(double comp, double tg, const S &T
     dL = rmul(ne, radd(dLs, S(comp)));
 }
 
-// the sums of 16 slots in the order of a 16-lane butterfly (offsets 8, 4, 2,
-// 1) over slots 0..10; slots 11..15 are zero and left out
-__device__ __forceinline__ dfm::F2 tree_sum11(const dfm::F2 (&a)[kNCool])
+// The terms' places in the sums: place t + 4 r is lane t's term of round r in
+// a team of four (t + 8 r in one of eight), the last place empty.  The order
+// gives round 0 the two terms with a softplus of their own beside the first
+// two of u, so a team evaluates one softplus per lane.
+__host__ __device__ __forceinline__ constexpr int cool_at(int place)
+{
+    constexpr int at[12] = {0, 1, 2, 10, 4, 5, 6, 7, 8, 9, 3, -1};
+    return at[place];
+}
+static __device__ const int g_cool_at[12] = {0, 1, 2, 10, 4, 5, 6, 7, 8, 9, 3, 11};
+
+// the sum over the places in a fixed pairwise order: places 8 apart, 4
+// apart, then 2 and 1 (the empty one left out)
+__device__ __forceinline__ dfm::F2 tree_sum(const dfm::F2 (&a)[kNCool])
 {
     using dfm::adds;
-    const dfm::F2 s0 = adds(a[0], a[8]), s1 = adds(a[1], a[9]), s2 = adds(a[2], a[10]);
-    const dfm::F2 t0 = adds(s0, a[4]), t1 = adds(s1, a[5]), t2 = adds(s2, a[6]), t3 = adds(a[3], a[7]);
+    const dfm::F2 s0 = adds(a[cool_at(0)], a[cool_at(8)]), s1 = adds(a[cool_at(1)], a[cool_at(9)]),
+                  s2 = adds(a[cool_at(2)], a[cool_at(10)]);
+    const dfm::F2 t0 = adds(s0, a[cool_at(4)]), t1 = adds(s1, a[cool_at(5)]), t2 = adds(s2, a[cool_at(6)]),
+                  t3 = adds(a[cool_at(3)], a[cool_at(7)]);
     return adds(adds(t0, t2), adds(t1, t3));
 }
 
@@ -679,8 +720,8 @@ __device__ __forceinline__ void cooling_sums(const TLevel &L, int case_b, bool h
             dd->f[k] = dd->df[k] = dd->d2f[k] = 0.0;
         }
     }
-    Ls = to_double_i(tree_sum11(a), -kCoolExp);
-    dLs = to_double_i(mul(tree_sum11(b), L.invT), -kCoolExp);
+    Ls = to_double_i(tree_sum(a), -kCoolExp);
+    dLs = to_double_i(mul(tree_sum(b), L.invT), -kCoolExp);
 }
 
 // (out of line, as the rate sets above)
@@ -731,37 +772,44 @@ static __device__ __noinline__ void cooling_serial(int case_b, double comp, doub
     cooling_close(comp, tg, T, ne, Ls, dLs, L, dL);
 }
 
-// a full warp (all 32 lanes, the same arguments): lane k < 16 holds term k,
-// the sums run over shuffles in the same pairwise order
-__device__ __forceinline__ dfm::F2 shfl_xor_pair(dfm::F2 a, int m)
+// a team of four: places t, t + 4, t + 8, the last sums over shuffles, in the
+// order of tree_sum
+__device__ __forceinline__ dfm::F2 team_add(unsigned mask, dfm::F2 a, int m)
 {
-    return {__shfl_xor_sync(0xffffffffu, a.hi, m), __shfl_xor_sync(0xffffffffu, a.lo, m)};
+    return dfm::adds(a, dfm::F2{__shfl_xor_sync(mask, a.hi, m), __shfl_xor_sync(mask, a.lo, m)});
 }
 template <bool MIX>
-__device__ __forceinline__ void cooling_warp(const RateFn &q, double comp, double tg, bool helium, double T,
-                                             double ne, double nHI, double nHII, double nHeI, double nHeII,
-                                             double nHeIII, double &L, double &dL)
+static __device__ __noinline__ double2 cooling_sums_team4(int case_b, bool helium, double T, double nHI, double nHII,
+                                                          double nHeI, double nHeII, double nHeIII)
 {
     using namespace dfm;
-    TLevel Lv;
-    t_level<true>(T, Lv);
-    RateVal r;
-    rate_lane<MIX, true>(q, Lv, r);
+    const unsigned mask = team_mask<4>();
+    const int t = team_lane<4>();
+    const RateFn *R = g_rate_fn[case_b].f;
+    TLevel L;
+    t_level(T, L);
     double n[NSP];
     cool_densities(nHI, nHII, nHeI, nHeII, nHeIII, n);
-    const int k = threadIdx.x & 15;
-    F2 v, dv;
-    cool_term(r, split_density(pick(n, g_cool_sp[k])), v, dv);
-    if (k >= kNCool || (!helium && (cool_mask(1) & rf_bit(k)))) v = dv = F2{0.0f, 0.0f};
+    // round 0: lanes 0, 1 with the softplus of u, lanes 2, 3 with their own
+    F2 sig;
+    const int k0 = g_cool_at[t];
+    const F2 l = rate_softplus<MIX>(R[k0], L, sig);
+    const F2 lu{__shfl_sync(mask, l.hi, 0, 4), __shfl_sync(mask, l.lo, 0, 4)};
+    const F2 su{__shfl_sync(mask, sig.hi, 0, 4), __shfl_sync(mask, sig.lo, 0, 4)};
+    F2 v[3], dv[3];
 #pragma unroll
-    for (int m = 8; m >= 1; m >>= 1) {
-        v = adds(v, shfl_xor_pair(v, m));
-        dv = adds(dv, shfl_xor_pair(dv, m));
+    for (int r = 0; r < 3; ++r) {
+        const int k = r ? g_cool_at[t + 4 * r] : k0;
+        RateVal q;
+        // (no softplus in round 2 nor in lane 3 of round 1: c3 = c3 c4 = 0)
+        rate_val<MIX, true>(R[k], L, r ? lu : l, r ? su : sig, r == 2 ? 1u << kZeroC3 : 0u, false, q);
+        cool_term(q, split_density(pick(n, g_cool_sp[k])), v[r], dv[r]);
+        if (k >= kNCool || (!helium && (cool_mask(1) >> k & 1))) v[r] = dv[r] = F2{0.0f, 0.0f};
     }
-    // lanes 16..31 summed other functions: every lane takes lane 0's sums
-    v = F2{__shfl_sync(0xffffffffu, v.hi, 0), __shfl_sync(0xffffffffu, v.lo, 0)};
-    dv = F2{__shfl_sync(0xffffffffu, dv.hi, 0), __shfl_sync(0xffffffffu, dv.lo, 0)};
-    cooling_close(comp, tg, T, ne, to_double_i(v, -kCoolExp), to_double_i(mul(dv, Lv.invT), -kCoolExp), L, dL);
+    F2 s = adds(adds(v[0], v[2]), v[1]), ds = adds(adds(dv[0], dv[2]), dv[1]);
+    s = team_add(mask, team_add(mask, s, 2), 1);
+    ds = team_add(mask, team_add(mask, ds, 2), 1);
+    return make_double2(to_double_i(s, -kCoolExp), to_double_i(mul(ds, L.invT), -kCoolExp));
 }
 
 }  // namespace rtgb

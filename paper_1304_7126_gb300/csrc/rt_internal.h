@@ -65,10 +65,8 @@ struct ThermoParams {
     int case_b;
     int max_sub;
     int pass1_attempts;      // attempts before a cell is handed to the queue
-    int drain_budget;        // attempts a cell may spend in the first lane-per-cell drain
-    int drain2_budget;       // ... and in the second
-    long long drain2_min;    // the second drain runs only above this many queued cells
-                             // (< 0: eight per warp of the warp-per-cell kernel)
+    int lane_budget;         // attempts a cell may spend in the lane-per-cell drain
+    long long lane_min;      // the drain runs only for queues of more cells than this
     int emit;                // no OTSA: recombination photons (Sec. 3.3.2)
     int rec_g[3];            // group receiving HII, HeII, HeIII recombination photons (-1: none)
     GroupConsts gc;
@@ -107,14 +105,12 @@ inline void derive_group_terms(ThermoParams &p)
 inline void default_routing(ThermoParams &p)
 {
     p.pass1_attempts = 6;
-    p.drain_budget = 128;
-    p.drain2_budget = 128;
-    p.drain2_min = -1;
+    p.lane_budget = 256;
+    p.lane_min = 1LL << 40;
 }
 
-// Device work queues of cells whose sub-cycling outlasted the first pass
-// (a) and the lane-per-cell drain (b); queue c, the input of the
-// warp-per-cell kernel, reuses the arrays of a once a is drained.
+// Device work queues of cells whose sub-cycling outlasted the first pass (a,
+// filled from both ends) and the lane-per-cell drain (b).
 constexpr int kQueueCounters = 8;
 
 struct QueueArrays {
@@ -125,8 +121,8 @@ struct QueueArrays {
 };
 struct Queue {
     QueueArrays a, b;
-    unsigned long long *counters;   // kQueueCounters: [0] a.count, [1] a.head, [2] b.count,
-                                    // [3] b.head, [4] c.count, [5] c.head
+    unsigned long long *counters;   // kQueueCounters: [0] a.count at the front, [1] at the back,
+                                    // [2] a.head, [3] b.count, [4] items taken after the first round
     long long capacity;             // items per queue
     double *fscale;                 // [2G][nc]: a queued cell's flux scale Fs_i (rows 0..G-1) and,
                                     // smoothed RT, its Fdot weight Fb_i (rows G..2G-1)

@@ -16,25 +16,18 @@
 // cooling rate and its derivative depend only on the state at t, so a
 // rejected sub-step keeps them for the retry.
 //
-// Load balance, three kernels per RT step:
+// Load balance, per RT step:
 //   thermo_pass1  one thread per cell (coalesced), up to 6 attempts; cells
-//                 still sub-cycling go to queue A with their partial state;
-//   thermo_drain  persistent; every lane takes queue-A items one at a time,
-//                 one attempt per loop iteration, and fetches the next item
-//                 as soon as its cell completes; a cell that needs more than
-//                 ThermoParams::drain_budget attempts here moves to queue B
-//                 (a second stage with its own budget runs when queue B is
-//                 long);
-//   thermo_hard   persistent; a pair of warps per queue-C cell.  On GB300
-//                 a lone dependent chain is slow (64 cycles per FP64 FMA),
-//                 so the lanes of a warp evaluate the cell's rate and
-//                 cooling functions of one temperature in parallel (rates.cuh,
-//                 one lane each) while the scalar update runs redundantly in
-//                 all lanes, and the second warp of the pair computes the
-//                 cooling while the first updates the photons.  The
-//                 arithmetic is identical to the one-thread path, and a
-//                 queued cell carries its flux scale, so results do not
-//                 depend on which kernel finished a cell.
+//                 still sub-cycling go to queue A with their partial state,
+//                 those with many sub-steps ahead to its front;
+//   thermo_team   persistent; a team of four lanes per queued cell, eight
+//                 cells per warp: the lanes share the cell's rate and cooling
+//                 functions (rates.cuh) and its photon groups while the scalar
+//                 update runs redundantly in all four;
+//   thermo_drain  between them, only when rt_set_thermo_routing asks for it:
+//                 persistent, one lane per cell.
+// The arithmetic is the same in all of them, and a queued cell carries its
+// flux scale, so results do not depend on which kernel finished a cell.
 // Nothing waits on another thread; each kernel ends when its queue is empty.
 // The kernels live in thermo_kernels.cuh, instantiated per precision family
 // in thermo_f64.cu, thermo_mix.cu, thermo_mix32.cu and their smoothed-RT

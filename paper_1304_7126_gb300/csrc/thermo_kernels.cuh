@@ -1,5 +1,5 @@
-// Thermochemistry kernels (first pass, lane-per-cell drains, pair-of-warps
-// tail) and their launch sequence, templated on the group count G, the
+// Thermochemistry kernels (first pass, lane-per-cell drain, team-per-cell
+// kernel) and their launch sequence, templated on the group count G, the
 // photon storage type P (double: RT_FP64; float: RT_MIXED), FP32 rate
 // transcendentals R32 (RT_MIXED32) and smoothed RT SM (Sec. 3.4).  Each
 // launcher translation unit instantiates one (P, R32) family, so the
@@ -25,67 +25,79 @@ namespace {
 using namespace thermo_detail;
 
 constexpr int kPass1Block = 128;
+constexpr int kTeam = 4;            // lanes per cell of thermo_team
+constexpr double kLongSteps = 32.0; // sub-steps ahead from which a queued cell is taken early
 
-// first: the cell's first load in this RT step (thermo_pass1)
-template <int G, bool WARP, typename P, bool R32, bool SM>
+// first: the cell's first load in this RT step (thermo_pass1).  PT: 1, or the
+// lanes of the cell's team, each of which loads and stores its own groups
+template <int G, int PT, typename P, bool R32, bool SM>
 __device__ __forceinline__ void load_cell(const ThermoParams &p, long long c, bool first, const double *xHII,
                                           const double *xHeII, const double *xHeIII, const double *T,
-                                          const P *N, const P *Npre, const double *fscale, CellState<G> &st,
-                                          IsoRates<> &iso, CoolCache<> &cc, const RateFn *lq = nullptr)
+                                          const P *N, const P *Npre, const double *fscale,
+                                          CellState<lane_groups(G, PT)> &st, IsoRates<> &iso, CoolCache<> &cc)
 {
     st.x = xHII[c];
     st.y2 = xHeII[c];
     st.y3 = xHeIII[c];
     st.T = T[c];
 #pragma unroll
-    for (int i = 0; i < G; ++i) {
+    for (int r = 0; r < lane_groups(G, PT); ++r) {
+        const int i = r * PT + team_lane<PT>();
+        st.N[r] = 0.0;
+        st.Fs[r] = 1.0;
+        if constexpr (SM) st.Nd[r] = st.Fb[r] = 0.0;
+        if (PT > 1 && i >= G) continue;
         const long long k = (long long)i * p.nc + c;
         if constexpr (SM) {
             if (first) {
                 const double n0 = (double)Npre[k];
-                st.Nd[i] = ((double)N[k] - n0) / p.dt;   // Eq. (smoothrate1)
-                st.N[i] = n0;
+                st.Nd[r] = ((double)N[k] - n0) / p.dt;   // Eq. (smoothrate1)
+                st.N[r] = n0;
             } else {
-                st.N[i] = (double)N[k];
-                st.Nd[i] = (double)Npre[k];
+                st.N[r] = (double)N[k];
+                st.Nd[r] = (double)Npre[k];
             }
-            st.Fb[i] = first ? 0.0 : fscale[(long long)(G + i) * p.nc + c];
+            st.Fb[r] = first ? 0.0 : fscale[(long long)(G + i) * p.nc + c];
         } else {
-            st.N[i] = (double)N[k];
+            st.N[r] = (double)N[k];
         }
-        st.Fs[i] = first ? 1.0 : fscale[k];
+        st.Fs[r] = first ? 1.0 : fscale[k];
     }
     cc.valid = false;
     cc.rvalid = false;
     if (p.isothermal) {
         TLevel L;
-        t_level<WARP>(st.T, L);
-        h_rates<WARP, R32>(L, 0.0, p.case_b, lq, iso.h);
-        if (p.helium) he_rates<WARP, R32>(L, 0.0, p.case_b, lq, iso.he);
+        t_level(st.T, L);
+        h_rates<PT, R32>(L, 0.0, p.case_b, iso.h);
+        if (p.helium) he_rates<PT, R32>(L, 0.0, p.case_b, iso.he);
     }
 }
 
 // handoff: the cell goes to a queue unfinished.  Its flux scale (and Fdot
 // weight) then goes to fscale and F keeps F_base: the flux is formed once,
 // when the cell finishes, so it does not depend on where it sub-cycled.
-template <int G, typename P, bool SM>
+template <int G, int PT, typename P, bool SM>
 __device__ __forceinline__ void store_cell(const ThermoParams &p, long long c, bool first, bool handoff,
                                            double *xHII, double *xHeII, double *xHeIII, double *T, P *N, P *F,
-                                           P *Npre, P *Fpre, double *fscale, const CellState<G> &st,
-                                           unsigned *status)
+                                           P *Npre, P *Fpre, double *fscale,
+                                           const CellState<lane_groups(G, PT)> &st, unsigned *status)
 {
-    xHII[c] = st.x;
-    xHeII[c] = st.y2;
-    xHeIII[c] = st.y3;
-    T[c] = st.T;
+    if (team_lane<PT>() == 0) {
+        xHII[c] = st.x;
+        xHeII[c] = st.y2;
+        xHeIII[c] = st.y3;
+        T[c] = st.T;
+    }
     bool bad = !isfinite(st.x) || !isfinite(st.T);
 #pragma unroll
-    for (int i = 0; i < G; ++i) {
-        N[(long long)i * p.nc + c] = (P)st.N[i];
-        bad |= !isfinite(st.N[i]);
+    for (int r = 0; r < lane_groups(G, PT); ++r) {
+        const int i = r * PT + team_lane<PT>();
+        if (PT > 1 && i >= G) continue;
+        N[(long long)i * p.nc + c] = (P)st.N[r];
+        bad |= !isfinite(st.N[r]);
         if (handoff) {
-            fscale[(long long)i * p.nc + c] = st.Fs[i];
-            if constexpr (SM) fscale[(long long)(G + i) * p.nc + c] = st.Fb[i];
+            fscale[(long long)i * p.nc + c] = st.Fs[r];
+            if constexpr (SM) fscale[(long long)(G + i) * p.nc + c] = st.Fb[r];
         }
         if constexpr (SM) {
             if (handoff && !first) continue;
@@ -104,13 +116,13 @@ __device__ __forceinline__ void store_cell(const ThermoParams &p, long long c, b
                     F[b] = Fpre[b];
                     Fpre[b] = (P)fd;
                 } else {
-                    F[b] = (P)(st.Fs[i] * base + st.Fb[i] * fd);
+                    F[b] = (P)(st.Fs[r] * base + st.Fb[r] * fd);
                 }
             }
-            if (handoff) Npre[(long long)i * p.nc + c] = (P)st.Nd[i];
-        } else if (!handoff && st.Fs[i] != 1.0) {
+            if (handoff) Npre[(long long)i * p.nc + c] = (P)st.Nd[r];
+        } else if (!handoff && st.Fs[r] != 1.0) {
             long long b = 3LL * i * p.nc + c;
-            const P f = (P)st.Fs[i];
+            const P f = (P)st.Fs[r];
             F[b] *= f;
             F[b + p.nc] *= f;
             F[b + 2 * p.nc] *= f;
@@ -146,67 +158,63 @@ thermo_pass1(ThermoParams p, const double *__restrict__ nH, double *xHII, double
         CellState<G> st;
         IsoRates<> iso;
         CoolCache<> cc;
-        load_cell<G, false, P, R32, SM>(p, c, true, xHII, xHeII, xHeIII, T, N, Npre, q.fscale, st, iso, cc);
+        load_cell<G, 1, P, R32, SM>(p, c, true, xHII, xHeII, xHeIII, T, N, Npre, q.fscale, st, iso, cc);
         double n = nH[c];
         cell_constants(p, n, iso);
         bool done = false;
         const int lim = p.pass1_attempts < p.max_sub ? p.pass1_attempts : p.max_sub;
         for (int k = 0; k < lim && !done; ++k)
-            done = subcycle_once<G, false, R32, double, SM>(p, n, st, t_left, dt_tc, att, iso, cc);
+            done = subcycle_once<G, 1, R32, double, SM>(p, n, st, t_left, dt_tc, att, iso, cc);
         if (!done && att >= p.max_sub) {
             atomicOr(status, kStatusSubcycle);
             done = true;
         }
-        store_cell<G, P, SM>(p, c, true, !done, xHII, xHeII, xHeIII, T, N, F, Npre, Fpre, q.fscale, st, status);
+        store_cell<G, 1, P, SM>(p, c, true, !done, xHII, xHeII, xHeIII, T, N, F, Npre, Fpre, q.fscale, st, status);
         if (done) subcycles[c] = att;
         else push = true;
     }
-    // warp-aggregated append of unfinished cells to queue A
-    unsigned m = __ballot_sync(0xffffffffu, push);
-    if (m) {
-        int lane = threadIdx.x & 31;
-        int leader = __ffs(m) - 1;
+    // warp-aggregated append of unfinished cells to queue A: the ones with
+    // the most sub-steps ahead (at the present step length) from its front,
+    // to be taken first, the others from its back
+    const int lane = threadIdx.x & 31;
+#pragma unroll
+    for (int e = 0; e < 2; ++e) {
+        const bool mine = push && (t_left > kLongSteps * dt_tc) == (e == 0);
+        const unsigned m = __ballot_sync(0xffffffffu, mine);
+        if (!m) continue;
+        const int leader = __ffs(m) - 1;
         unsigned long long base = 0;
-        if (lane == leader) base = atomicAdd(&q.counters[0], (unsigned long long)__popc(m));
-        base = __shfl_sync(0xffffffffu, base, leader);
-        if (push)
-            push_item(q.a, base + __popc(m & ((1u << lane) - 1u)), q.capacity, (uint32_t)c, t_left, dt_tc, att,
-                      status);
+        if (lane == leader) base = atomicAdd(&q.counters[e], (unsigned long long)__popc(m));
+        base = __shfl_sync(0xffffffffu, base, leader) + __popc(m & ((1u << lane) - 1u));
+        if (mine)
+            push_item(q.a, e ? (unsigned long long)q.capacity - 1ULL - base : base, q.capacity, (uint32_t)c, t_left,
+                      dt_tc, att, status);
     }
 }
 
-// One lane-per-cell drain stage: cells of queue `src` (count and head in
-// counters[cnt], counters[cnt + 1]) sub-cycle here for at most `budget`
-// attempts; a cell still unfinished moves to queue `dst` (count in
-// counters[dst_cnt]).  When `src` holds no more than `pass_below` cells the
-// stage only moves them to `dst`: so few long sub-cyclers finish sooner one
-// warp each than sharing warps.
-struct DrainStage {
-    QueueArrays src, dst;
-    int cnt, dst_cnt, budget;
-    long long pass_below;
+// Item `it` of queue A: front items first, then those at the back
+struct QueueView {
+    unsigned long long front, total;
+    __device__ __forceinline__ explicit QueueView(const Queue &q)
+        : front(q.counters[0]), total(q.counters[0] + q.counters[1])
+    {
+    }
+    __device__ __forceinline__ unsigned long long slot(const Queue &q, unsigned long long it) const
+    {
+        return it < front ? it : (unsigned long long)q.capacity - 1ULL - (it - front);
+    }
 };
 
+// The lane-per-cell drain, for long queues only (more than lane_min cells):
+// cells of queue A sub-cycle here for at most lane_budget attempts, every
+// lane taking items one at a time; a cell still unfinished moves to queue B.
 template <int G, typename P, bool R32, bool SM>
 __global__ void __launch_bounds__(128)
 thermo_drain(ThermoParams p, const double *__restrict__ nH, double *xHII, double *xHeII, double *xHeIII,
-             double *T, P *N, P *F, P *Npre, P *Fpre, int32_t *subcycles, Queue q, DrainStage ds,
-             unsigned *status)
+             double *T, P *N, P *F, P *Npre, P *Fpre, int32_t *subcycles, Queue q, unsigned *status)
 {
-    unsigned long long count = q.counters[ds.cnt];
-    if (count > (unsigned long long)q.capacity) count = (unsigned long long)q.capacity;
-    if (count == 0) return;
-    if ((long long)count <= ds.pass_below) {
-        const long long gt = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-        for (long long it = gt; it < (long long)count; it += (long long)gridDim.x * blockDim.x) {
-            ds.dst.cell[it] = ds.src.cell[it];
-            ds.dst.t_left[it] = ds.src.t_left[it];
-            ds.dst.dt_tc[it] = ds.src.dt_tc[it];
-            ds.dst.attempts[it] = ds.src.attempts[it];
-        }
-        if (gt == 0) q.counters[ds.dst_cnt] = count;
-        return;
-    }
+    const QueueView qv(q);
+    if ((long long)qv.total <= p.lane_min) return;
     CellState<G> st;
     IsoRates<> iso;
     CoolCache<> cc;
@@ -215,96 +223,102 @@ thermo_drain(ThermoParams p, const double *__restrict__ nH, double *xHII, double
     long long c = -1;
     bool have = false;
     auto fetch = [&]() {
-        unsigned long long it = atomicAdd(&q.counters[ds.cnt + 1], 1ULL);
-        if (it < count) {
-            c = ds.src.cell[it];
-            t_left = ds.src.t_left[it];
-            dt_tc = ds.src.dt_tc[it];
-            att = ds.src.attempts[it];
+        const unsigned long long it = atomicAdd(&q.counters[2], 1ULL);
+        have = it < qv.total;
+        if (have) {
+            const unsigned long long sl = qv.slot(q, it);
+            c = q.a.cell[sl];
+            t_left = q.a.t_left[sl];
+            dt_tc = q.a.dt_tc[sl];
+            att = q.a.attempts[sl];
             n = nH[c];
             used = 0;
-            load_cell<G, false, P, R32, SM>(p, c, false, xHII, xHeII, xHeIII, T, N, Npre, q.fscale, st, iso, cc);
+            load_cell<G, 1, P, R32, SM>(p, c, false, xHII, xHeII, xHeIII, T, N, Npre, q.fscale, st, iso, cc);
             cell_constants(p, n, iso);
-            have = true;
-        } else {
-            have = false;
         }
     };
     fetch();
     while (have) {
-        bool done = subcycle_once<G, false, R32, double, SM>(p, n, st, t_left, dt_tc, att, iso, cc);
+        bool done = subcycle_once<G, 1, R32, double, SM>(p, n, st, t_left, dt_tc, att, iso, cc);
         if (!done && att >= p.max_sub) {
             atomicOr(status, kStatusSubcycle);
             done = true;
         }
         if (done) {
-            store_cell<G, P, SM>(p, c, false, false, xHII, xHeII, xHeIII, T, N, F, Npre, Fpre, q.fscale, st, status);
+            store_cell<G, 1, P, SM>(p, c, false, false, xHII, xHeII, xHeIII, T, N, F, Npre, Fpre, q.fscale, st, status);
             subcycles[c] = att;
             fetch();
-        } else if (++used >= ds.budget) {
-            // long sub-cycler: hand it to the next stage
-            store_cell<G, P, SM>(p, c, false, true, xHII, xHeII, xHeIII, T, N, F, Npre, Fpre, q.fscale, st, status);
-            unsigned long long slot = atomicAdd(&q.counters[ds.dst_cnt], 1ULL);
-            push_item(ds.dst, slot, q.capacity, (uint32_t)c, t_left, dt_tc, att, status);
+        } else if (++used >= p.lane_budget) {
+            // long sub-cycler: hand it to the team kernel
+            store_cell<G, 1, P, SM>(p, c, false, true, xHII, xHeII, xHeIII, T, N, F, Npre, Fpre, q.fscale, st, status);
+            const unsigned long long slot = atomicAdd(&q.counters[3], 1ULL);
+            push_item(q.b, slot, q.capacity, (uint32_t)c, t_left, dt_tc, att, status);
             fetch();
         }
     }
 }
 
-// The tail: a pair of warps per queued cell (warps 2k, 2k + 1 of a block).
-// Both warps run the cell's attempts in step with identical state; in each
-// attempt that needs the cooling at T(t), warp 2k + 1 evaluates it while
-// warp 2k updates the photons (PairX exchange, thermo_step.cuh).  Warp 2k
-// takes the next queue item and posts it to its partner the same way.
+// A team of four lanes per queued cell, eight cells per warp: the team's
+// lanes share the cell's rate functions (one softplus and exponential each
+// instead of four to eleven) and photon groups.  Bound by the length of an
+// attempt, a chain of dependent FP32 pair and FP64 operations in which a warp
+// of one cell and a warp of eight take the same time; a pair of warps per
+// cell, the kernel before, was no shorter and spent sixteen times the issue
+// slots and FP64 instructions per cell.  The first items go to different
+// warps, spread over the SMs, then each team takes the next one.
 template <int G, typename P, bool R32, bool SM>
 __global__ void __launch_bounds__(128)
-thermo_hard(ThermoParams p, const double *__restrict__ nH, double *xHII, double *xHeII, double *xHeIII,
+thermo_team(ThermoParams p, const double *__restrict__ nH, double *xHII, double *xHeII, double *xHeIII,
             double *T, P *N, P *F, P *Npre, P *Fpre, int32_t *subcycles, Queue q, unsigned *status)
 {
-    unsigned long long count = q.counters[4];
+    const QueueView qv(q);
+    const bool drained = (long long)qv.total > p.lane_min;   // the cells left are in queue B
+    unsigned long long count = drained ? q.counters[3] : qv.total;
     if (count > (unsigned long long)q.capacity) count = (unsigned long long)q.capacity;
-    if (count == 0) return;
-    __shared__ PairX<G> px[2];
-    const int lane = threadIdx.x & 31;
-    const int warp = threadIdx.x >> 5;
-    const int team = warp >> 1;
-    PairCtx pc{&px[team], warp & 1, 0, 1 + team};
-    PairX<G> &X = px[team];
-    const RateFn lq = lane_rate_fn(p.case_b);
-    while (true) {
-        // the item: taken by role 0, posted to role 1 (exchange pc.n)
-        const int b = pc.n & 1;
-        ++pc.n;
-        if (pc.role == 0 && lane == 0) X.item[b] = atomicAdd(&q.counters[5], 1ULL);
-        pair_meet(pc);
-        const unsigned long long it = X.item[b];
-        if (it >= count) break;
-        const long long c = q.a.cell[it];
-        double t_left = q.a.t_left[it];
-        double dt_tc = q.a.dt_tc[it];
-        int att = q.a.attempts[it];
-        const double n_h = nH[c];
-        CellState<G> st;
-        IsoRates<> iso;
-        CoolCache<> cc;
-        load_cell<G, true, P, R32, SM>(p, c, false, xHII, xHeII, xHeIII, T, N, Npre, q.fscale, st, iso, cc, &lq);
-        cell_constants(p, n_h, iso);
-        bool done = false;
-        while (!done) {
-            done = subcycle_once<G, true, R32, double, SM, true>(p, n_h, st, t_left, dt_tc, att, iso, cc, &lq, &pc);
-            if (!done && att >= p.max_sub) {
-                if (lane == 0 && pc.role == 0) atomicOr(status, kStatusSubcycle);
-                done = true;
+    const QueueArrays src = drained ? q.b : q.a;
+    const unsigned mask = team_mask<kTeam>();
+    const int t = team_lane<kTeam>();
+    // item order of the first round: warp 0 of every block, warp 1, ...
+    const unsigned long long warps = (unsigned long long)gridDim.x * (blockDim.x >> 5);
+    const unsigned long long first = ((threadIdx.x & 31) / kTeam) * warps + (threadIdx.x >> 5) * gridDim.x + blockIdx.x;
+    const unsigned long long teams = warps * (32 / kTeam);
+    CellState<lane_groups(G, kTeam)> st;
+    IsoRates<> iso;
+    CoolCache<> cc;
+    double t_left = 0.0, dt_tc = 0.0, n = 0.0;
+    int att = 0;
+    long long c = -1;
+    unsigned long long it = first;
+    auto load = [&]() {
+        if (it >= count) return false;
+        const unsigned long long sl = drained ? it : qv.slot(q, it);
+        c = src.cell[sl];
+        t_left = src.t_left[sl];
+        dt_tc = src.dt_tc[sl];
+        att = src.attempts[sl];
+        n = nH[c];
+        load_cell<G, kTeam, P, R32, SM>(p, c, false, xHII, xHeII, xHeIII, T, N, Npre, q.fscale, st, iso, cc);
+        cell_constants(p, n, iso);
+        return true;
+    };
+    bool have = load();
+    while (have) {
+        bool done = subcycle_once<G, kTeam, R32, double, SM>(p, n, st, t_left, dt_tc, att, iso, cc);
+        if (!done && att >= p.max_sub) {
+            if (t == 0) atomicOr(status, kStatusSubcycle);
+            done = true;
+        }
+        if (done) {
+            store_cell<G, kTeam, P, SM>(p, c, false, false, xHII, xHeII, xHeIII, T, N, F, Npre, Fpre, q.fscale, st,
+                                        status);
+            if (t == 0) subcycles[c] = att;
+            it = count;
+            if (count > teams) {
+                if (t == 0) it = teams + atomicAdd(&q.counters[4], 1ULL);
+                it = __shfl_sync(mask, it, 0, kTeam);
             }
+            have = load();
         }
-        // (the partner has read its item's state: it has met this warp since,
-        // or, with fixed rates or kept cooling, ran the same attempts)
-        pair_meet(pc);
-        if (lane == 0 && pc.role == 0) {
-            store_cell<G, P, SM>(p, c, false, false, xHII, xHeII, xHeIII, T, N, F, Npre, Fpre, q.fscale, st, status);
-            subcycles[c] = att;
-        }
-        __syncwarp();
     }
 }
 
@@ -320,37 +334,27 @@ cudaError_t launch_g(const ThermoParams &tp, const double *nH, double *xHII, dou
                                                           status);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    static int per_sm = 0;
-    if (per_sm == 0) {
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, thermo_drain<G, P, R32, SM>, 128, 0);
-        if (per_sm < 1) per_sm = 1;
+    static int per_sm[2] = {0, 0};
+    if (per_sm[0] == 0) {
+        int a = 0, b = 0;
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&a, thermo_drain<G, P, R32, SM>, 128, 0);
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, thermo_team<G, P, R32, SM>, 128, 0);
+        per_sm[1] = b < 1 ? 1 : b;
+        per_sm[0] = a < 1 ? 1 : a;
     }
-    long long grid = (long long)per_sm * n_sm;
-    long long need = (tp.nc + 127) / 128;
-    if (grid > need) grid = need;
-    if (grid < 1) grid = 1;
-    // a pair of warps per long sub-cycler: two 4-warp blocks per SM
-    long long hgrid = 2LL * n_sm;
-    long long hneed = (tp.nc + 3) / 4;
-    if (hgrid > hneed) hgrid = hneed;
-    if (hgrid < 1) hgrid = 1;
+    auto grid = [&](int k, long long cells_per_block) {
+        const long long g = (long long)per_sm[k] * n_sm, need = (tp.nc + cells_per_block - 1) / cells_per_block;
+        return (unsigned)(g < need ? g : need);
+    };
     if (ev) { cudaEventRecord(ev[1], s); cudaEventRecord(ev[2], s); }
-    DrainStage d1{q.a, q.b, 0, 2, tp.drain_budget, 0};
-    thermo_drain<G, P, R32, SM><<<(unsigned)grid, 128, 0, s>>>(tp, nH, xHII, xHeII, xHeIII, T, N, F, Npre, Fpre, sub,
-                                                              q, d1, status);
-    e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    // many more long sub-cyclers than the tail kernel has pairs: they share
-    // the FP64 pipes anyway, so a lane per cell does more per cycle; up to
-    // eight cells per tail block (four per pair), the pairs keep each
-    // cell's path short
-    DrainStage d2{q.b, q.a, 2, 4, tp.drain2_budget, tp.drain2_min < 0 ? 8 * hgrid : tp.drain2_min};
-    thermo_drain<G, P, R32, SM><<<(unsigned)grid, 128, 0, s>>>(tp, nH, xHII, xHeII, xHeIII, T, N, F, Npre, Fpre, sub,
-                                                              q, d2, status);
-    e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    thermo_hard<G, P, R32, SM><<<(unsigned)hgrid, 128, 0, s>>>(tp, nH, xHII, xHeII, xHeIII, T, N, F, Npre, Fpre, sub, q,
-                                                             status);
+    if (tp.nc > tp.lane_min) {   // (otherwise the queue cannot hold that many)
+        thermo_drain<G, P, R32, SM><<<grid(0, 128), 128, 0, s>>>(tp, nH, xHII, xHeII, xHeIII, T, N, F, Npre, Fpre, sub,
+                                                                q, status);
+        e = cudaGetLastError();
+        if (e != cudaSuccess) return e;
+    }
+    thermo_team<G, P, R32, SM><<<grid(1, 128 / kTeam), 128, 0, s>>>(tp, nH, xHII, xHeII, xHeIII, T, N, F, Npre, Fpre,
+                                                                   sub, q, status);
     if (ev) cudaEventRecord(ev[3], s);
     return cudaGetLastError();
 }

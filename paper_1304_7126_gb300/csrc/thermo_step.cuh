@@ -22,13 +22,17 @@ constexpr double kXMin = 1e-6;
 constexpr double kNeFloor = 1e-6;
 constexpr double kTFloor = 1.0;
 
-template <int G, typename S = double>
+// Photon groups a lane holds: all G of them (PT = 1), or those of its place
+// in a team of PT lanes, group r PT + t in place r.
+__host__ __device__ constexpr int lane_groups(int G, int PT) { return (G + PT - 1) / PT; }
+
+template <int NG, typename S = double>
 struct CellState {
     S x, y2, y3, T;
-    S N[G];
-    S Fs[G];          // accumulated flux scale prod 1/(1 + h D_i)
-    S Nd[G];          // smoothed RT: photon density rate Ndot_i (Sec. 3.4)
-    S Fb[G];          // smoothed RT: weight of Fdot_i in F, sum h prod 1/(1 + h D_i)
+    S N[NG];
+    S Fs[NG];         // accumulated flux scale prod 1/(1 + h D_i)
+    S Nd[NG];         // smoothed RT: photon density rate Ndot_i (Sec. 3.4)
+    S Fb[NG];         // smoothed RT: weight of Fdot_i in F, sum h prod 1/(1 + h D_i)
 };
 
 template <typename S = double>
@@ -231,40 +235,25 @@ __device__ __forceinline__ bool term_small(const S &a, const S &b)
     return term_lt<S>(a, b, 0.05);
 }
 
-// Rates at one temperature level.  lq: the warp path's function of this lane.
-__device__ __forceinline__ RateFn lane_rate_fn(int case_b) { return g_rate_fn[case_b].f[threadIdx.x & 31]; }
-
-template <bool WARP, bool MIX>
-__device__ __forceinline__ void h_rates(const TLevel &L, double, int case_b, const RateFn *lq, HRates &r)
+// Rates at one temperature level, by one thread or by a team of TS lanes
+template <int TS, bool MIX>
+__device__ __forceinline__ void h_rates(const TLevel &L, double, int case_b, HRates &r)
 {
-    if constexpr (WARP) {
-        Rates t;
-        rates_warp<MIX, true>(*lq, L, kNeedH, kNeedH, t);
-        h_rates_from(t, r);
-    } else {
-        r = h_rates_serial<MIX>(L, case_b);
-    }
+    if constexpr (TS > 1) r = h_rates_team<TS, MIX>(L, case_b);
+    else r = h_rates_serial<MIX>(L, case_b);
 }
-template <bool WARP, bool MIX>
-__device__ __forceinline__ void he_rates(const TLevel &L, double, int case_b, const RateFn *lq, HeRates &r)
+template <int TS, bool MIX>
+__device__ __forceinline__ void he_rates(const TLevel &L, double, int case_b, HeRates &r)
 {
-    if constexpr (WARP) {
-        Rates t;
-        rates_warp<MIX, false>(*lq, L, kNeedHe, 0u, t);
-        he_rates_from(t, r);
-    } else {
-        r = he_rates_serial<MIX>(L, case_b);
-    }
+    if constexpr (TS > 1) r = he_rates_team<TS, MIX>(L, case_b);
+    else r = he_rates_serial<MIX>(L, case_b);
 }
 // (only beta_HeII and alpha_HeIII)
-template <bool WARP, bool MIX>
-__device__ __forceinline__ void he3_rates(const TLevel &L, double, int case_b, const RateFn *lq, HeRates &r)
+template <int TS, bool MIX>
+__device__ __forceinline__ void he3_rates(const TLevel &L, double, int case_b, HeRates &r)
 {
-    if constexpr (WARP) {
-        Rates t;
-        rates_warp<MIX, false>(*lq, L, kNeedHe3, 0u, t);
-        r.beta_HeII = t.f[RF_BETA_HEII];
-        r.alpha_HeIII = t.f[RF_ALPHA_HEIII];
+    if constexpr (TS > 1) {
+        r = he_rates_team<TS, MIX>(L, case_b);
     } else {
         const double2 t = he3_rates_serial<MIX>(L, case_b);
         r.beta_HeII = t.x;
@@ -272,19 +261,19 @@ __device__ __forceinline__ void he3_rates(const TLevel &L, double, int case_b, c
     }
 }
 // dual numbers: the level of the value, dT the derivative of T
-template <bool WARP, bool MIX>
-__device__ __forceinline__ void h_rates(const TLevel &L, double dT, int case_b, const RateFn *, HRatesT<Dual> &r)
+template <int TS, bool MIX>
+__device__ __forceinline__ void h_rates(const TLevel &L, double dT, int case_b, HRatesT<Dual> &r)
 {
-    static_assert(!WARP && !MIX, "dual rates: one thread, FP64");
+    static_assert(TS == 1 && !MIX, "dual rates: one thread, FP64");
     r = h_rates_dual(L, dT, case_b);
 }
-template <bool WARP, bool MIX>
-__device__ __forceinline__ void he_rates(const TLevel &L, double dT, int case_b, const RateFn *, HeRatesT<Dual> &r)
+template <int TS, bool MIX>
+__device__ __forceinline__ void he_rates(const TLevel &L, double dT, int case_b, HeRatesT<Dual> &r)
 {
     r = he_rates_dual(L, dT, case_b);
 }
-template <bool WARP, bool MIX>
-__device__ __forceinline__ void he3_rates(const TLevel &L, double dT, int case_b, const RateFn *, HeRatesT<Dual> &r)
+template <int TS, bool MIX>
+__device__ __forceinline__ void he3_rates(const TLevel &L, double dT, int case_b, HeRatesT<Dual> &r)
 {
     r = he_rates_dual(L, dT, case_b);
 }
@@ -298,16 +287,14 @@ __device__ __forceinline__ dfm::F2 inv_pair(double x)
     if (!(x > 0.0) || !dfm::splittable(x)) return dfm::split_any(1.0 / x);
     return dfm::rcp2(dfm::split(x));
 }
-template <bool WARP>
 __device__ __forceinline__ double level_mu(const Dual &md, dfm::F2 iT, const Dual &Tmu1, TLevel &L)
 {
-    t_level_inv<WARP>(dfm::mul(dfm::split_any(md.v), iT), L);
+    t_level_inv(dfm::mul(dfm::split_any(md.v), iT), L);
     return qdiv(Tmu1, md).d;
 }
-template <bool WARP>
 __device__ __forceinline__ double level_mu(double md, dfm::F2 iT, double, TLevel &L)
 {
-    t_level_inv<WARP>(dfm::mul(dfm::split_any(md), iT), L);
+    t_level_inv(dfm::mul(dfm::split_any(md), iT), L);
     return 0.0;
 }
 
@@ -315,27 +302,18 @@ __device__ __forceinline__ double level_mu(double md, dfm::F2 iT, double, TLevel
 // (Eq. (cool_N_cr)); out of line: it only runs without the OTSA, and
 // inlined its two rate tables would raise the register count of every
 // kernel
-template <bool WARP, bool MIX, typename S>
-__device__ __noinline__ void recomb_rates(S T, S nHII, S nHeII, S nHeIII, S ne, S *rj)
+template <bool MIX>
+static __device__ __noinline__ void recomb_rates(double T, double nHII, double nHeII, double nHeIII, double ne,
+                                                 double *rj)
 {
-    static_assert(std::is_same<S, double>::value, "the adjoint needs the OTSA");
     double aA[3], aB[3];
     TLevel L;
-    t_level<WARP>(T, L);
-    {
-        const RateFn q = lane_rate_fn(0);
-        Rates t;
-        if constexpr (WARP) rates_warp<MIX, false>(q, L, kNeedRec, 0u, t);
-        else rates_serial<MIX>(L, 0, kNeedRec, 0u, t);
-        recomb_alphas(t, aA);
-    }
-    {
-        const RateFn q = lane_rate_fn(1);
-        Rates t;
-        if constexpr (WARP) rates_warp<MIX, false>(q, L, kNeedRec, 0u, t);
-        else rates_serial<MIX>(L, 1, kNeedRec, 0u, t);
-        recomb_alphas(t, aB);
-    }
+    t_level(T, L);
+    Rates t;
+    rates_serial<MIX>(L, 0, kNeedRec, 0u, t);
+    recomb_alphas(t, aA);
+    rates_serial<MIX>(L, 1, kNeedRec, 0u, t);
+    recomb_alphas(t, aB);
     rj[0] = (aA[0] - aB[0]) * nHII * ne;
     rj[1] = (aA[1] - aB[1]) * nHeII * ne;
     rj[2] = (aA[2] - aB[2]) * nHeIII * ne;
@@ -392,44 +370,51 @@ __device__ __forceinline__ void photon_group(const ThermoParams &p, int i, const
     o.tq = rmul(crN, rfma(p.hq[i][2], nHeII, rfma(p.hq[i][1], nHeI, rmul(nHI, p.hq[i][0]))));
 }
 
-// a double or a dual from lane `src` of the warp
-__device__ __forceinline__ double shfl_s(double v, int src) { return __shfl_sync(0xffffffffu, v, src); }
-__device__ __forceinline__ Dual shfl_s(const Dual &v, int src)
+// The photon stage of an attempt by a team of PT lanes (each with its own
+// groups), filling the lanes' new N_i and flux scales and, in every lane, the
+// photo-ionisation rates gam_j and the photoheating; false when a group
+// breaks the 10% rule.  The recombination photons C_i (without the OTSA) come
+// from cc.rj.
+template <int G, int PT, bool MIX, bool SM>
+__device__ __forceinline__ bool photons_team(const ThermoParams &p, const CellState<lane_groups(G, PT)> &s,
+                                             const CoolCache<double> &cc, double nHI, double nHeI, double nHeII,
+                                             double h, CellState<lane_groups(G, PT)> &o, double &gam0, double &gam1,
+                                             double &gam2, double &heat, bool &sm)
 {
-    return Dual(__shfl_sync(0xffffffffu, v.v, src), __shfl_sync(0xffffffffu, v.d, src));
-}
-
-// The photon stage of an attempt (group i on lane i of a warp), filling the
-// new N_i, flux scales, the photo-ionisation rates gam_j and the
-// photoheating; false when a group breaks the 10% rule.  The recombination
-// photons C_i (without the OTSA) come from cc.rj.
-template <int G, bool MIX, bool SM, typename S>
-__device__ __forceinline__ bool photons_warp(const ThermoParams &p, const CellState<G, S> &s, const CoolCache<S> &cc,
-                                             const S &nHI, const S &nHeI, const S &nHeII, double h,
-                                             CellState<G, S> &o, S &gam0, S &gam1, S &gam2, S &heat, bool &sm)
-{
-    PhotonTerms<S> pt;
-    const int lane = threadIdx.x & 31;
-    const int gi = lane < G ? lane : 0;
-    S Crec = 0.0;
-    if (p.emit) {
+    constexpr int NG = lane_groups(G, PT);
+    const unsigned mask = team_mask<PT>();
+    const int t = team_lane<PT>();
+    bool ok = true, small = true;
+    PhotonTerms<double> pt[NG];
 #pragma unroll
-        for (int j = 0; j < 3; ++j)
-            if (p.rec_g[j] == gi) Crec += cc.rj[j];
+    for (int r = 0; r < NG; ++r) {
+        const bool mine = r * PT + t < G;
+        const int gi = mine ? r * PT + t : 0;
+        double Crec = 0.0;
+        if (p.emit) {
+#pragma unroll
+            for (int j = 0; j < 3; ++j)
+                if (p.rec_g[j] == gi) Crec += cc.rj[j];
+        }
+        photon_group<MIX, SM>(p, gi, s.N[r], s.Fs[r], s.Nd[r], s.Fb[r], Crec, nHI, nHeI, nHeII, h, pt[r]);
+        if (mine) {
+            ok = ok && pt[r].ok;
+            small = small && pt[r].small;
+        }
+        o.N[r] = pt[r].Nn;
+        o.Fs[r] = pt[r].Fs;
+        if constexpr (SM) {
+            o.Fb[r] = pt[r].Fb;
+            o.Nd[r] = s.Nd[r];
+        }
     }
-    photon_group<MIX, SM>(p, gi, s.N[gi], s.Fs[gi], s.Nd[gi], s.Fb[gi], Crec, nHI, nHeI, nHeII, h, pt);
-    const unsigned full = 0xffffffffu;
-    const bool ok = !__any_sync(full, lane < G && !pt.ok);
-    sm = sm && (__all_sync(full, lane >= G || pt.small) != 0);
+    ok = __all_sync(mask, ok);
+    sm = sm && (__all_sync(mask, small) != 0);
 #pragma unroll
     for (int i = 0; i < G; ++i) {
-        o.N[i] = shfl_s(pt.Nn, i);
-        o.Fs[i] = shfl_s(pt.Fs, i);
-        if constexpr (SM) {
-            o.Fb[i] = shfl_s(pt.Fb, i);
-            o.Nd[i] = s.Nd[i];
-        }
-        const S t0 = shfl_s(pt.t0, i), t1 = shfl_s(pt.t1, i), t2 = shfl_s(pt.t2, i), tq = shfl_s(pt.tq, i);
+        const PhotonTerms<double> &q = pt[i / PT];
+        const double t0 = team_get<PT>(mask, q.t0, i % PT), t1 = team_get<PT>(mask, q.t1, i % PT),
+                     t2 = team_get<PT>(mask, q.t2, i % PT), tq = team_get<PT>(mask, q.tq, i % PT);
         if (i == 0) {
             gam0 = t0; gam1 = t1; gam2 = t2; heat = tq;
         } else {
@@ -473,33 +458,6 @@ __device__ __forceinline__ bool photons_serial(const ThermoParams &p, const Cell
     return true;
 }
 
-// The two warps of a pair of the tail kernel (thermo_hard): while one evaluates
-// the cooling at T(t) the other updates the photons; each posts its results
-// in shared memory and both meet at the pair's named barrier.  Both then hold
-// the same values and run the rest of the attempt in step, so every exchange
-// is met by both.  Two buffers alternate, so a post never overwrites data the
-// partner may still be reading.  (Polled sequence numbers, with a sleep
-// between polls, made an exchange longer.)
-template <int G>
-struct PairX {
-    double N[2][G], Fs[2][G], Fb[2][G], g[2][4], L[2], dL[2], m[2][3];
-    int ok[2], small[2];
-    unsigned long long item[2];
-};
-
-struct PairCtx {
-    void *x;          // PairX<G> of the pair, shared memory
-    int role;         // 0: photons, 1: cooling
-    int n;            // exchanges so far (the same in both warps)
-    int bar;          // the pair's named barrier
-};
-
-__device__ __forceinline__ void pair_meet(const PairCtx &pc)
-{
-    __syncwarp();
-    asm volatile("bar.sync %0, 64;" ::"r"(pc.bar) : "memory");
-}
-
 // One thermo_step over h.  Returns true and fills `o` when the 10% rule
 // holds; `small` then tells whether every checked change stayed below 5%.
 // The checks |dX| / den > 0.1 go through ratio_gt / ratio_lt (a division
@@ -510,12 +468,15 @@ __device__ __forceinline__ void pair_meet(const PairCtx &pc)
 //
 // S is double, or Dual for the adjoint's differentiated recomputation
 // (values bit-identical to the double path; MIX only with double).
-template <int G, bool WARP, bool MIX, typename S = double, bool SM = false, bool PAIR = false>
-__device__ __forceinline__ bool attempt(const ThermoParams &p, const S &nH, const CellState<G, S> &s, double h,
-                                        const IsoRates<S> &iso, CoolCache<S> &cc, CellState<G, S> &o,
-                                        bool &small, const RateFn *lq = nullptr, PairCtx *pc = nullptr)
+// TS: 1, one thread, or 4, a team of four lanes that hold the same cell,
+// share its rate functions and each update their own photon groups; the same
+// operations in the same order, so the same bits.
+template <int G, int TS, bool MIX, typename S = double, bool SM = false>
+__device__ __forceinline__ bool attempt(const ThermoParams &p, const S &nH, const CellState<lane_groups(G, TS), S> &s,
+                                        double h, const IsoRates<S> &iso, CoolCache<S> &cc,
+                                        CellState<lane_groups(G, TS), S> &o, bool &small)
 {
-    static_assert(!PAIR || (WARP && sizeof(S) == sizeof(double)), "pairs of warps: the warp path");
+    static_assert(TS == 1 || (TS == 4 && std::is_same<S, double>::value), "teams of four, FP64");
     static_assert(!MIX || sizeof(S) == sizeof(double), "the mixed path is not differentiated");
     const S nHe = iso.nHe;
     const S x = s.x, y2 = s.y2, y3 = s.y3;
@@ -536,104 +497,43 @@ __device__ __forceinline__ bool attempt(const ThermoParams &p, const S &nH, cons
     // photon update; kept over rejected attempts
     // recombination photons without the OTSA, Eq. (cool_N_cr), at T(t) with
     // the backward abundances; group i gains C_i = sum_j [rec_g[j] == i] rj[j]
-    // (before the cooling: a pair of warps updates the photons there)
     if constexpr (std::is_same<S, double>::value) {   // (the adjoint needs the OTSA)
         if (p.emit && !cc.rvalid) {
-            recomb_rates<WARP, MIX>(s.T, nHII, nHeII, nHeIII, ne, cc.rj);
+            recomb_rates<MIX>(s.T, nHII, nHeII, nHeIII, ne, cc.rj);
             cc.rvalid = true;
         }
     }
 
-    bool pair_photons = false;   // the photon stage was done in the pair exchange
-    // the parts of step 2 that depend on the state only: 1/mu, mu, T/mu
-    S mden, mu, Tmu;
-    bool have_mu = false;
     if (!p.isothermal && !cc.valid) {
-        if constexpr (PAIR) {
-            // role 1 evaluates the cooling, role 0 the photon stage, at once
-            PairX<G> &X = *static_cast<PairX<G> *>(pc->x);
-            const int b = pc->n & 1;
-            ++pc->n;
-            const int lane = threadIdx.x & 31;
-            cc.valid = true;
-            if (pc->role == 1) {
-                cooling_warp<MIX>(*lq, p.comp, p.tg, p.helium != 0, s.T, ne, nHI, nHII, nHeI, nHeII, nHeIII, cc.L,
-                                  cc.dL);
-                if (lane == 0) {
-                    X.L[b] = cc.L;
-                    X.dL[b] = cc.dL;
-                }
-                pair_meet(*pc);
-                if (!X.ok[b]) return false;
-#pragma unroll
-                for (int i = 0; i < G; ++i) {
-                    o.N[i] = X.N[b][i];
-                    o.Fs[i] = X.Fs[b][i];
-                    if constexpr (SM) {
-                        o.Fb[i] = X.Fb[b][i];
-                        o.Nd[i] = s.Nd[i];
-                    }
-                }
-                gam0 = X.g[b][0]; gam1 = X.g[b][1]; gam2 = X.g[b][2]; heat = X.g[b][3];
-                sm = X.small[b] != 0;
-                mden = X.m[b][0]; mu = X.m[b][1]; Tmu = X.m[b][2];
-            } else {
-                const bool ok = photons_warp<G, MIX, SM>(p, s, cc, nHI, nHeI, nHeII, h, o, gam0, gam1, gam2, heat, sm);
-                // (this warp would wait for the cooling meanwhile)
-                mden = mu_den(p, x, mhe);
-                mu = qrcp(mden);
-                Tmu = rmul(s.T, mden);
-                if (lane == 0) {
-                    X.m[b][0] = mden; X.m[b][1] = mu; X.m[b][2] = Tmu;
-#pragma unroll
-                    for (int i = 0; i < G; ++i) {
-                        X.N[b][i] = o.N[i];
-                        X.Fs[b][i] = o.Fs[i];
-                        if constexpr (SM) X.Fb[b][i] = o.Fb[i];
-                    }
-                    X.g[b][0] = gam0; X.g[b][1] = gam1; X.g[b][2] = gam2; X.g[b][3] = heat;
-                    X.ok[b] = ok;
-                    X.small[b] = sm;
-                }
-                pair_meet(*pc);
-                cc.L = X.L[b];
-                cc.dL = X.dL[b];
-                if (!ok) return false;
-            }
-            pair_photons = true;
-            have_mu = true;
+        if constexpr (TS > 1) {
+            const double2 c = cooling_sums_team4<MIX>(p.case_b, p.helium != 0, s.T, nHI, nHII, nHeI, nHeII, nHeIII);
+            cooling_close(p.comp, p.tg, s.T, ne, c.x, c.y, cc.L, cc.dL);
         } else {
-            if constexpr (WARP)   // lane k evaluates cooling term k
-                cooling_warp<MIX>(*lq, p.comp, p.tg, p.helium != 0, s.T, ne, nHI, nHII, nHeI, nHeII, nHeIII, cc.L,
-                                  cc.dL);
-            else
-                cooling_serial<MIX>(p.case_b, p.comp, p.tg, p.helium != 0, s.T, ne, nHI, nHII, nHeI, nHeII, nHeIII,
-                                    cc.L, cc.dL);
-            cc.valid = true;
+            cooling_serial<MIX>(p.case_b, p.comp, p.tg, p.helium != 0, s.T, ne, nHI, nHII, nHeI, nHeII, nHeIII, cc.L,
+                                cc.dL);
         }
+        cc.valid = true;
     }
 
-
-    // 1. photons: group i's update depends on no other group, so the warp
-    // path gives group i to lane i; the one-thread path loops over the
-    // groups; both call photon_group and sum the groups' terms in the same
-    // order (rounded as written), so they give the same bits
-    if (!pair_photons) {
+    // 1. photons: group i's update depends on no other group, so the lanes of
+    // a team take a group each; one thread loops over the groups; both call
+    // photon_group and sum the groups' terms in the same order (rounded as
+    // written), so they give the same bits
+    {
         bool ok;
-        if constexpr (WARP) ok = photons_warp<G, MIX, SM>(p, s, cc, nHI, nHeI, nHeII, h, o, gam0, gam1, gam2, heat, sm);
+        if constexpr (TS > 1)
+            ok = photons_team<G, TS, MIX, SM>(p, s, cc, nHI, nHeI, nHeII, h, o, gam0, gam1, gam2, heat, sm);
         else ok = photons_serial<G, MIX, SM>(p, s, cc, nHI, nHeI, nHeII, h, o, gam0, gam1, gam2, heat, sm);
         if (!ok) return false;
     }
 
     // 2. temperature: T/mu + K h (Lambda) / (1 + mu (dL/dT) K h), Lambda =
     // heating - cooling, d Lambda/d(T/mu) = -mu dL/dT
-    S Tmu1 = 0.0;
+    S mden, mu, Tmu1 = 0.0;
     if (!p.isothermal) {
-        if (!have_mu) {
-            mden = mu_den(p, x, mhe);
-            mu = qrcp(mden);
-            Tmu = rmul(s.T, mden);
-        }
+        mden = mu_den(p, x, mhe);
+        mu = qrcp(mden);
+        const S Tmu = rmul(s.T, mden);
         const S Kh = rmul(iso.K, h);
         const S num = rmul(radd(heat, -cc.L), Kh);
         const S dT = qdiv(num, rfma(rmul(mu, cc.dL), Kh, S(1.0)));
@@ -651,8 +551,8 @@ __device__ __forceinline__ bool attempt(const ThermoParams &p, const S &nH, cons
         hr = iso.h;
     } else {
         TLevel L;
-        const double dT = level_mu<WARP>(mden, iT, Tmu1, L);
-        h_rates<WARP, MIX>(L, dT, p.case_b, lq, hr);
+        const double dT = level_mu(mden, iT, Tmu1, L);
+        h_rates<TS, MIX>(L, dT, p.case_b, hr);
     }
     const S C = rfma(hr.beta, ne, gam0);
     const S CD = rfma(hr.alpha, ne, C);   // C + D, D = alpha n_e
@@ -680,8 +580,8 @@ __device__ __forceinline__ bool attempt(const ThermoParams &p, const S &nH, cons
             r2 = iso.he;
         } else {
             TLevel L;
-            const double dT = level_mu<WARP>(mu_den(p, x1, mhe), iT, Tmu1, L);
-            he_rates<WARP, MIX>(L, dT, p.case_b, lq, r2);
+            const double dT = level_mu(mu_den(p, x1, mhe), iT, Tmu1, L);
+            he_rates<TS, MIX>(L, dT, p.case_b, r2);
         }
         const S hs(h);
         const S D1 = rfma(r2.beta_HeI, ne2, gam1);
@@ -696,8 +596,8 @@ __device__ __forceinline__ bool attempt(const ThermoParams &p, const S &nH, cons
             r3 = iso.he;
         } else {
             TLevel L;
-            const double dT = level_mu<WARP>(mu_den(p, x1, md_he(p, q1)), iT, Tmu1, L);
-            he3_rates<WARP, MIX>(L, dT, p.case_b, lq, r3);
+            const double dT = level_mu(mu_den(p, x1, md_he(p, q1)), iT, Tmu1, L);
+            he3_rates<TS, MIX>(L, dT, p.case_b, r3);
         }
         const S C3 = rmul(y2n, rfma(r3.beta_HeII, ne3, gam2));
         const S D3 = rmul(r3.alpha_HeIII, ne3);
@@ -722,17 +622,17 @@ __device__ __forceinline__ bool attempt(const ThermoParams &p, const S &nH, cons
 }
 
 // One attempt of the sub-cycling loop; returns true when the cell is done.
-template <int G, bool WARP, bool MIX, typename S = double, bool SM = false, bool PAIR = false>
-__device__ __forceinline__ bool subcycle_once(const ThermoParams &p, const S &nH, CellState<G, S> &st,
-                                              double &t_left, double &dt_tc, int &att, const IsoRates<S> &iso,
-                                              CoolCache<S> &cc, const RateFn *lq = nullptr, PairCtx *pc = nullptr)
+template <int G, int TS, bool MIX, typename S = double, bool SM = false>
+__device__ __forceinline__ bool subcycle_once(const ThermoParams &p, const S &nH,
+                                              CellState<lane_groups(G, TS), S> &st, double &t_left, double &dt_tc,
+                                              int &att, const IsoRates<S> &iso, CoolCache<S> &cc)
 {
     // t_left, dt_tc > 0: compared through their bits
     double h = (dbits(dt_tc) < dbits(t_left)) ? dt_tc : t_left;
     ++att;
-    CellState<G, S> o;
+    CellState<lane_groups(G, TS), S> o;
     bool small = false;
-    if (attempt<G, WARP, MIX, S, SM, PAIR>(p, nH, st, h, iso, cc, o, small, lq, pc)) {
+    if (attempt<G, TS, MIX, S, SM>(p, nH, st, h, iso, cc, o, small)) {
         st = o;
         cc.valid = false;
         cc.rvalid = false;
