@@ -69,13 +69,32 @@ __device__ __forceinline__ F2 add(F2 a, F2 b)
     return fast_two_sum(s.hi, __fadd_rn(s.lo, t.lo));
 }
 
-// a + b within 2^-47 (|a| + |b|): the low parts rounded once.  Commutative,
-// and b = 0 returns a normalised a.  For the arguments and sums below, whose
-// terms carry errors of that size themselves (11 instructions, add() 20).
-__device__ __forceinline__ F2 adds(F2 a, F2 b)
+// Products and sums without the final normalisation: the low part stays
+// within a few ulps of the high one, which the next operation takes as well
+// (errors of 2^-46 of the operands' magnitude, what the arguments and terms
+// they are used on carry anyway).  4, 8 and 5 instructions, mul() has 7 and
+// add() 20; a pair is normalised (norm) where it is stored or converted.
+// addu is commutative, adding a zero pair or multiplying by one returns the
+// operand unchanged.
+__device__ __forceinline__ F2 norm(F2 a) { return fast_two_sum(a.hi, a.lo); }
+
+__device__ __forceinline__ F2 addu(F2 a, F2 b)
 {
     const F2 s = two_sum(a.hi, b.hi);
-    return fast_two_sum(s.hi, __fadd_rn(s.lo, __fadd_rn(a.lo, b.lo)));
+    return {s.hi, __fadd_rn(s.lo, __fadd_rn(a.lo, b.lo))};
+}
+
+// |a.hi| >= |b.hi| or a.hi == 0
+__device__ __forceinline__ F2 addf(F2 a, F2 b)
+{
+    const F2 s = fast_two_sum(a.hi, b.hi);
+    return {s.hi, __fadd_rn(s.lo, __fadd_rn(a.lo, b.lo))};
+}
+
+__device__ __forceinline__ F2 mulu(F2 a, F2 b)
+{
+    const F2 p = two_prod(a.hi, b.hi);
+    return {p.hi, __fmaf_rn(a.lo, b.hi, __fmaf_rn(a.hi, b.lo, p.lo))};
 }
 
 __device__ __forceinline__ F2 add(F2 a, float b)
@@ -257,12 +276,14 @@ __device__ __forceinline__ F2 rcp(F2 a)
     return fast_two_sum(r0, r0 * err);
 }
 
-// 1/a refined by a second Newton step in pair arithmetic (2^-47)
+// 1/a refined by a second Newton step (2^-47)
 __device__ __forceinline__ F2 rcp2(F2 a)
 {
     const F2 r = rcp(a);
-    const F2 e = add(F2{1.0f, 0.0f}, neg(mul(a, r)));
-    return add(r, mul(r, e));
+    const F2 p = two_prod(a.hi, r.hi);
+    const float e = __fsub_rn(__fsub_rn(__fsub_rn(1.0f, p.hi), p.lo),
+                              __fmaf_rn(a.hi, r.lo, __fmul_rn(a.lo, r.hi)));
+    return fast_two_sum(r.hi, __fmaf_rn(r.hi, e, r.lo));
 }
 
 __device__ __forceinline__ F2 sqrt2(F2 a)
@@ -276,10 +297,9 @@ __device__ __forceinline__ F2 sqrt2(F2 a)
 // ---- elementary functions ----
 // exp2d, log2f2 and log1pd are called out of line: inlined at every call
 // site of every thermochemistry kernel they made ptxas run for tens of
-// minutes.  The warp path of the rates (one call site per temperature)
-// inlines exp2d_inl and log2f2_inl, the same arithmetic.
+// minutes.
 
-// e^x of a pair as y 2^m, y a pair in [0.99, 2.02); |x| below 2000
+// e^x of a pair as y 2^m, y an unnormalised pair in [0.99, 2.02); |x| below 1420
 __device__ __forceinline__ void exp_pair(F2 x, F2 &y, int &m)
 {
     const float kf = rintf(__fmul_rn(x.hi, kDfInvL));
@@ -297,10 +317,10 @@ __device__ __forceinline__ void exp_pair(F2 x, F2 &y, int &m)
     const float c = __fmaf_rn(rh, r.lo,
                               rh * h2.hi * __fmaf_rn(rh, __fmaf_rn(rh, 1.0f / 120.0f, 1.0f / 24.0f), 1.0f / 6.0f));
     const F2 q = fast_two_sum(0.5f * h2.hi, __fmaf_rn(0.5f, h2.lo, c));
-    const F2 p = adds(r, q);
+    const F2 p = addf(r, q);
     const float2 t = __ldg(&kDfExp2Tab[k & 63]);
     const F2 T{t.x, t.y};
-    y = adds(T, mul(T, p));   // 2^(j/64) e^r
+    y = addf(T, mulu(T, p));   // 2^(j/64) e^r
     m = k >> 6;               // floor(k / 64)
 }
 
@@ -312,14 +332,15 @@ __device__ __forceinline__ double exp2d_inl(F2 x)
     F2 y;
     int m;
     exp_pair(x, y, m);
+    y = norm(y);
     if (m > -1020 && m < 1020) return combine(y.hi, y.lo, m);
     return ldexp(to_double(y), m);
 }
 
 static __device__ __noinline__ double exp2d(F2 x) { return exp2d_inl(x); }
 
-// ln of a positive normal pair
-__device__ __forceinline__ F2 log2f2_inl(F2 v)
+// ln(v / 2^shift) of a positive normal pair
+__device__ __forceinline__ F2 log2f2_inl(F2 v, int shift)
 {
     const unsigned bits = __float_as_uint(v.hi);
     const int e = (int)(bits >> 23) - 127;
@@ -331,31 +352,59 @@ __device__ __forceinline__ F2 log2f2_inl(F2 v)
     const F2 f{fs.hi * sc, fs.lo * sc};
     const float4 L = __ldg(&kDfLogTab[j]);
     const F2 u = mul(f, F2{L.z, L.w});   // u = f / F, |u| <= 1/256
-    // ln(1 + u) = u - u^2/2 + u^3 (1/3 - u/4 + u^2/5 - u^3/6)
-    const F2 u2 = mul(u, u);
-    const F2 u3 = mul(u2, u.hi);
+    // ln(1 + u) = u - u^2/2 + u^3 (1/3 - u/4 + u^2/5 - u^3/6), the cubic and
+    // higher terms (below 2^-25) in FP32
     const float uh = u.hi;
-    const float cub = uh * __fmaf_rn(uh, __fmaf_rn(uh, -1.0f / 6.0f, 0.2f), -0.25f);
-    F2 q = adds(u, F2{-0.5f * u2.hi, -0.5f * u2.lo});
-    q = adds(q, mul(u3, F2{kDfThirdHi, kDfThirdLo}));
-    q = add(q, u3.hi * cub);
-    // e ln2 + ln F + q
-    const float ef = (float)e;
-    F2 s = two_prod(ef, kDfLn2B);
-    s = adds(F2{ef * kDfLn2A, 0.0f}, s);   // e A exact
-    s = add(s, ef * kDfLn2C);
-    s = adds(s, F2{L.x, L.y});
-    return adds(s, q);
+    const F2 u2 = mulu(u, u);
+    const float u3 = __fmul_rn(uh, u2.hi);
+    const float c = __fmaf_rn(u3, 1.0f / 3.0f, u3 * uh * __fmaf_rn(uh, __fmaf_rn(uh, -1.0f / 6.0f, 0.2f), -0.25f));
+    F2 q = fast_two_sum(uh, -0.5f * u2.hi);
+    q.lo = __fadd_rn(q.lo, __fadd_rn(__fmaf_rn(-0.5f, u2.lo, u.lo), c));
+    // e ln2 + ln F + q; e A exact.  The two small terms first, so that only
+    // two roundings are of the size of the sum's low part.
+    const float ef = (float)(e - shift);
+    const F2 p = two_prod(ef, kDfLn2B);
+    const F2 s = fast_two_sum(ef * kDfLn2A, L.x);
+    const F2 m = two_sum(p.hi, q.hi);
+    const F2 r = two_sum(s.hi, m.hi);
+    const float lo = __fadd_rn(m.lo, __fadd_rn(__fadd_rn(__fmaf_rn(ef, kDfLn2C, p.lo), L.y), q.lo));
+    return fast_two_sum(r.hi, __fadd_rn(__fadd_rn(s.lo, r.lo), lo));
 }
 
-static __device__ __noinline__ F2 log2f2(F2 v) { return log2f2_inl(v); }
+static __device__ __noinline__ F2 log2f2(F2 v, int shift) { return log2f2_inl(v, shift); }
 
 // ln x of a double
 __device__ __forceinline__ F2 logd(double x)
 {
-    if (x > 0.0 && splittable(x)) return log2f2(split(x));
+    if (x > 0.0 && splittable(x)) return log2f2(split(x), 0);
     const double r = log(x);
     return split(r);   // out of range: CUDA's log, split (|ln x| < 746)
+}
+
+// ln of a pair above 1 with every sum in full pair precision (relative error
+// 2^-46 also where the result is small), for log1pd
+__device__ __forceinline__ F2 log2f2_rel(F2 v)
+{
+    const unsigned bits = __float_as_uint(v.hi);
+    const int e = (int)(bits >> 23) - 127;
+    const int j = (int)(((bits & 0x7fffff) + (1u << 15)) >> 16);
+    const float Fs = __uint_as_float((unsigned)(e + 127) << 23) * (1.0f + (float)j * (1.0f / 128.0f));
+    const F2 fs = two_sum(__fsub_rn(v.hi, Fs), v.lo);
+    const float sc = pow2f(-e);
+    const float4 L = __ldg(&kDfLogTab[j]);
+    const F2 u = mul(F2{fs.hi * sc, fs.lo * sc}, F2{L.z, L.w});
+    const F2 u2 = mul(u, u);
+    const F2 u3 = mul(u2, u.hi);
+    const float uh = u.hi;
+    F2 q = add(u, F2{-0.5f * u2.hi, -0.5f * u2.lo});
+    q = add(q, mul(u3, F2{kDfThirdHi, kDfThirdLo}));
+    q = add(q, u3.hi * uh * __fmaf_rn(uh, __fmaf_rn(uh, -1.0f / 6.0f, 0.2f), -0.25f));
+    const float ef = (float)e;
+    F2 s = two_prod(ef, kDfLn2B);
+    s = add(F2{ef * kDfLn2A, 0.0f}, s);
+    s = add(s, ef * kDfLn2C);
+    s = add(s, F2{L.x, L.y});
+    return add(s, q);
 }
 
 // ln(1 + w) of a double w >= 0
@@ -379,7 +428,7 @@ static __device__ __noinline__ F2 log1pd(double w)
     const F2 s = two_sum(1.0f, W.hi);
     const F2 t = two_sum(s.lo, W.lo);
     const F2 v = fast_two_sum(s.hi, t.hi);
-    const F2 lv = log2f2(v);
+    const F2 lv = log2f2_rel(v);
     return add(lv, __fdividef(t.lo, v.hi));   // + c / v
 }
 
@@ -391,39 +440,38 @@ static __device__ __noinline__ F2 softplus_far(F2 z, F2 &sig)
 }
 
 // ln(1 + e^z) of a pair z, with its derivative 1/(1 + e^-z) as a pair.
-// On [-16, 16): the interpolating polynomials of kDfSoftplusTab (degree 9
-// in t = z - middle of a 1/4-wide interval, |t| <= 1/8); the terms of
-// degree 5 and up are below 2^-24 of the value, so they are summed in
-// FP32, the rest in pair arithmetic (absolute error ~1e-14 at |z| ~ 16,
-// that of the pair coefficients).  Outside (temperatures far beyond the
-// fits' range) from e^z and log1p.
+// On [-16, 16): the interpolating polynomials of kDfSoftplusTab (degree 7
+// in t = z - middle of a 1/32-wide interval, |t| <= 1/64); the terms of
+// degree 3 and up (in the derivative beyond 3 c3 t^2) are small enough to be
+// summed in FP32, the rest in pairs (absolute error
+// ~1e-14 at |z| ~ 16, that of the pair coefficients).  80 instructions; 250
+// with 1/4-wide intervals and degree 9.  Outside (temperatures far beyond
+// the fits' range) from e^z and log1p.
 __device__ __forceinline__ F2 softplus2(F2 z, F2 &sig)
 {
     if (z.hi >= (float)kDfSpLo && z.hi < -(float)kDfSpLo) {
         int k = (int)__fmul_rn(__fadd_rn(z.hi, -(float)kDfSpLo), (float)kDfSpPer);
         k = k < kDfSpN - 1 ? k : kDfSpN - 1;
         const float mid = (float)kDfSpLo + ((float)k + 0.5f) / (float)kDfSpPer;   // exact
-        const F2 t = add(z, -mid);
+        const F2 t0 = two_sum(z.hi, -mid);
+        const F2 t = fast_two_sum(t0.hi, __fadd_rn(t0.lo, z.lo));
         const float th = t.hi;
-        const float2 *c = kDfSoftplusTab[k];
-        float r = __ldg(&c[9].x), q = 9.0f * r;
-        r = __fmaf_rn(r, th, __ldg(&c[8].x));
-        q = __fmaf_rn(q, th, 8.0f * __ldg(&c[8].x));
-        r = __fmaf_rn(r, th, __ldg(&c[7].x));
-        q = __fmaf_rn(q, th, 7.0f * __ldg(&c[7].x));
-        r = __fmaf_rn(r, th, __ldg(&c[6].x));
-        q = __fmaf_rn(q, th, 6.0f * __ldg(&c[6].x));
-        r = __fmaf_rn(r, th, __ldg(&c[5].x));
-        q = __fmaf_rn(q, th, 5.0f * __ldg(&c[5].x));
-        F2 P{r, 0.0f}, D{q, 0.0f};
-#pragma unroll
-        for (int n = 4; n >= 0; --n) {
-            const float2 cn = __ldg(&c[n]);
-            P = adds(F2{cn.x, cn.y}, mul(P, t));
-            if (n >= 1) D = adds(mul(F2{cn.x, cn.y}, (float)n), mul(D, t));
-        }
-        sig = D;
-        return P;
+        const float4 *c = reinterpret_cast<const float4 *>(kDfSoftplusTab[k]);
+        const float4 c01 = __ldg(c), c23 = __ldg(c + 1), c45 = __ldg(c + 2), c67 = __ldg(c + 3);
+        const F2 c0{c01.x, c01.y}, c1{c01.z, c01.w};
+        const float r = __fmaf_rn(th, __fmaf_rn(th, __fmaf_rn(th, c67.x, c45.z), c45.x), c23.z);   // c3 + .. + c6 t^3
+        F2 P = fast_two_sum(c23.x, __fmul_rn(th, r));
+        P.lo = __fadd_rn(P.lo, c23.y);
+        P = addf(c1, mulu(P, t));
+        P = addf(c0, mulu(P, t));
+        const float d = __fmaf_rn(th, __fmaf_rn(th, __fmaf_rn(th, 7.0f * c67.z, 6.0f * c67.x), 5.0f * c45.z),
+                                  4.0f * c45.x);
+        const F2 c3 = two_prod(3.0f, c23.z);
+        F2 D = fast_two_sum(c3.hi, __fmul_rn(th, d));
+        D.lo = __fadd_rn(D.lo, __fmaf_rn(3.0f, c23.w, c3.lo));
+        D = addf(F2{2.0f * c23.x, 2.0f * c23.y}, mulu(D, t));
+        sig = norm(addf(c1, mulu(D, t)));
+        return norm(P);
     }
     return softplus_far(z, sig);
 }

@@ -85,7 +85,7 @@ def main():
     out.append("// at the Chebyshev points of the interval: {hi, lo}")
     out.append("constexpr int kDfSpLo = %d, kDfSpPer = %d, kDfSpN = %d, kDfSpDeg = %d;"
                % (SP_LO, SP_PER, SP_N, SP_DEG))
-    out.append("static __device__ const float2 kDfSoftplusTab[%d][%d] = {" % (SP_N, SP_DEG + 1))
+    out.append("static __device__ const __align__(16) float2 kDfSoftplusTab[%d][%d] = {" % (SP_N, SP_DEG + 1))
     rows = []
     for k in range(SP_N):
         coef = softplus_coefficients(k)
@@ -95,7 +95,7 @@ def main():
     print("\n".join(out))
 
 
-SP_LO, SP_HI, SP_PER, SP_DEG = -16, 16, 4, 9
+SP_LO, SP_HI, SP_PER, SP_DEG = -16, 16, 32, 7
 SP_N = (SP_HI - SP_LO) * SP_PER
 
 

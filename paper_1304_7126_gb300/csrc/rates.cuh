@@ -168,10 +168,18 @@ enum {
 };
 static_assert(kNCool <= 16 && NRF <= 32, "function slots are warp lanes");
 
+// The kernels take ln T relative to 2^14 K, the middle of the range that
+// matters: |ln(T / 2^14 K)| is a few units where |ln T| is 9, and so are the
+// pair roundings of the exponent's terms.  c0 and the reference's share of
+// c1 ln T go into the factor, c4's into c5r.
+constexpr int kLnTRef = 14;
+constexpr double kLnTRefV = 9.704060527839234;   // 14 ln 2
+
 struct RateFn {
     double Cc;
-    dfm::F2 c0, c1, c2, c3, c4, c5;
-    dfm::F2 Cm, c34;            // Cc = Cm 2^ke, 1 <= Cm < 2; c3 c4
+    dfm::F2 c0, c5;             // (with Cc: the function in terms of ln T, for rt_rate_functions)
+    dfm::F2 c1, c2, c3, c4, c5r;
+    dfm::F2 Cm, c34;            // Cc exp(c0 + c1 14 ln 2) = Cm 2^ke, 1 <= Cm < 2; c3 c4
     double d1, d2, d34, d344;   // c1, c2, c3 c4, c3 c4^2 (second derivative)
     int ke;
 };
@@ -181,14 +189,27 @@ struct RateFnTab {
 
 constexpr double kHalfLn1e5 = 5.756462732485114;   // ln(1e5) / 2
 
+// e^x at compile time: Taylor's series of e^(x/2^7) - 1, then seven times
+// s -> (1 + s)^2 - 1 (relative error ~1e-15)
+constexpr double const_exp(double x)
+{
+    const double t = x / 128.0;
+    double term = 1.0, sum = 0.0;   // sum = e^t - 1
+    for (int n = 1; n < 24; ++n) {
+        term *= t / n;
+        sum += term;
+    }
+    for (int k = 0; k < 7; ++k) sum = sum * (2.0 + sum);   // (1 + s)^2 - 1
+    return 1.0 + sum;
+}
 constexpr RateFn rate_fn(double Cc, double c0, double c1, double c2, double c3, double c4, double c5)
 {
-    double m = Cc;
+    double m = Cc * const_exp(c0 + c1 * kLnTRefV);
     int e = 0;
     while (m >= 2.0) { m *= 0.5; ++e; }
     while (m > 0.0 && m < 1.0) { m *= 2.0; --e; }
-    return RateFn{Cc, pair_of(c0), pair_of(c1), pair_of(c2), pair_of(c3), pair_of(c4), pair_of(c5),
-                  pair_of(m), pair_of(c3 * c4), c1, c2, c3 * c4, c3 * c4 * c4, e};
+    return RateFn{Cc, pair_of(c0), pair_of(c5), pair_of(c1), pair_of(c2), pair_of(c3), pair_of(c4),
+                  pair_of(c5 + c4 * kLnTRefV), pair_of(m), pair_of(c3 * c4), c1, c2, c3 * c4, c3 * c4 * c4, e};
 }
 constexpr RateFn cen_fn(double A, double T0) { return rate_fn(A, 0.0, 0.5, -T0, 1.0, 0.5, -kHalfLn1e5); }
 constexpr RateFn hg_fn(const RateTable &R, int j)
@@ -240,7 +261,7 @@ static __device__ const RateFnTab g_rate_fn[2] = {make_rate_fns(0), make_rate_fn
 static __device__ const int g_cool_sp[16] = {SP_HI, SP_HI, SP_HII, SP_FF, SP_HEI, SP_HEII, SP_HEII, SP_HEII,
                                              SP_HEII, SP_HEII, SP_HEIII, 0, 0, 0, 0, 0};
 
-// ln T and 1/T of one temperature as pairs
+// ln(T / 2^14 K) and 1/T of one temperature as pairs
 struct TLevel {
     dfm::F2 lnT, invT;
 };
@@ -248,11 +269,11 @@ __device__ __forceinline__ void t_level(double T, TLevel &L)
 {
     using namespace dfm;
     if (!(T > 0.0) || !splittable(T)) {   // not reached by T >= 1 K below 2^60 K
-        L.lnT = split_any(log(T));
+        L.lnT = split_any(log(T) - kLnTRefV);
         L.invT = split_any(1.0 / T);
     } else {
         const F2 T2 = split(T);
-        L.lnT = log2f2(T2);
+        L.lnT = log2f2(T2, kLnTRef);
         L.invT = rcp(T2);
     }
 }
@@ -261,8 +282,8 @@ __device__ __forceinline__ void t_level_inv(dfm::F2 invT, TLevel &L)
 {
     using namespace dfm;
     L.invT = invT;
-    if (invT.hi > 0x1p-60f && invT.hi < 0x1p60f) L.lnT = neg(log2f2(invT));
-    else L.lnT = split_any(-log(to_double(invT)));
+    if (invT.hi > 0x1p-60f && invT.hi < 0x1p60f) L.lnT = neg(log2f2(invT, -kLnTRef));
+    else L.lnT = split_any(-log(to_double(invT)) - kLnTRefV);
 }
 
 // A function value y 2^m (y a normalised pair below 8, or 0) and
@@ -276,7 +297,7 @@ struct RateVal {
 // what is zero (adding a zero pair or multiplying by one returns the same
 // normalised pair, so both paths still give the same bits).
 __host__ __device__ constexpr unsigned rf_bit(int k) { return 1u << k; }
-enum { kZeroC0, kZeroC1, kZeroC2, kZeroC3 };
+enum { kZeroC1, kZeroC2, kZeroC3 };
 constexpr unsigned rf_zero_mask(int what)
 {
     unsigned m = 0;
@@ -284,7 +305,7 @@ constexpr unsigned rf_zero_mask(int what)
         bool z = true;
         for (int cb = 0; cb < 2; ++cb) {
             const RateFn &q = kRateFnCx[cb].f[k];
-            const float v = what == kZeroC0 ? q.c0.hi : what == kZeroC1 ? q.c1.hi : what == kZeroC2 ? q.c2.hi : q.c3.hi;
+            const float v = what == kZeroC1 ? q.c1.hi : what == kZeroC2 ? q.c2.hi : q.c3.hi;
             z = z && v == 0.0f;
         }
         if (z) m |= rf_bit(k);
@@ -299,17 +320,17 @@ constexpr unsigned rf_u_mask()
         if (cool_row(k).uu) m |= rf_bit(RF_COOL0 + k);
     return m;
 }
-constexpr unsigned kC0Zero = rf_zero_mask(kZeroC0), kC1Zero = rf_zero_mask(kZeroC1), kC2Zero = rf_zero_mask(kZeroC2),
-                   kC3Zero = rf_zero_mask(kZeroC3), kSlotU = rf_u_mask();
+constexpr unsigned kC1Zero = rf_zero_mask(kZeroC1), kC2Zero = rf_zero_mask(kZeroC2), kC3Zero = rf_zero_mask(kZeroC3),
+                   kSlotU = rf_u_mask();
 
-// softplus(z) and sigma(z) of one function, z = c4 ln T + c5.  MIX (the
+// softplus(z) and sigma(z) of one function, z = c4 ln(T / 2^14 K) + c5r.  MIX (the
 // mixed-precision thermochemistry, RT_MIXED32): z still in pairs, but the
 // correction ln(1 + e^-|z|) < ln 2 and sigma in FP32.
 template <bool MIX>
 __device__ __forceinline__ dfm::F2 rate_softplus(const RateFn &q, const TLevel &L, dfm::F2 &sig)
 {
     using namespace dfm;
-    const F2 z = adds(mul(L.lnT, q.c4), q.c5);
+    const F2 z = norm(addu(mulu(L.lnT, q.c4), q.c5r));
     if constexpr (MIX) {
         const float e = __expf(-fabsf(z.hi));
         sig = F2{(z.hi >= 0.0f ? 1.0f : e) / (1.0f + e), 0.0f};
@@ -332,11 +353,11 @@ __device__ __forceinline__ void rate_val(const RateFn &q, const TLevel &L, dfm::
 {
     using namespace dfm;
     const F2 nil{0.0f, 0.0f};
-    const F2 b = (zero >> kZeroC2 & 1) ? nil : mul(L.invT, q.c2);
-    F2 arg = (zero >> kZeroC1 & 1) ? nil : mul(L.lnT, q.c1);
-    if (!(zero >> kZeroC0 & 1)) arg = adds(q.c0, arg);
-    if (!(zero >> kZeroC2 & 1)) arg = adds(arg, b);
-    if (!(zero >> kZeroC3 & 1)) arg = adds(arg, neg(one3 ? l : mul(l, q.c3)));
+    const F2 b = (zero >> kZeroC2 & 1) ? nil : mulu(L.invT, q.c2);
+    F2 arg = (zero >> kZeroC1 & 1) ? nil : mulu(L.lnT, q.c1);
+    if (!(zero >> kZeroC2 & 1)) arg = addu(arg, b);
+    if (!(zero >> kZeroC3 & 1)) arg = addu(arg, neg(one3 ? l : mulu(l, q.c3)));
+    arg = norm(arg);
     if (arg.hi < -1400.0f) arg = F2{-1400.0f, 0.0f};   // 0 in every use
     if constexpr (MIX) {
         const float kf = rintf(__fmul_rn(arg.hi, 1.44269504f));
@@ -348,13 +369,13 @@ __device__ __forceinline__ void rate_val(const RateFn &q, const TLevel &L, dfm::
     } else {
         int m;
         exp_pair(arg, r.y, m);
-        r.y = mul(q.Cm, r.y);
+        r.y = norm(mulu(q.Cm, r.y));
         r.m = m + q.ke;
         if constexpr (DERIV) {
             F2 g = (zero >> kZeroC1 & 1) ? nil : q.c1;
-            if (!(zero >> kZeroC2 & 1)) g = adds(g, neg(b));
-            if (!(zero >> kZeroC3 & 1)) g = adds(g, neg(mul(sig, q.c34)));
-            r.g = g;
+            if (!(zero >> kZeroC2 & 1)) g = addu(g, neg(b));
+            if (!(zero >> kZeroC3 & 1)) g = addu(g, neg(mulu(sig, q.c34)));
+            r.g = norm(g);
         }
     }
 }
@@ -363,7 +384,7 @@ __device__ __forceinline__ double rate_f(const RateVal &r) { return dfm::to_doub
 __device__ __forceinline__ double rate_df(const RateVal &r, const TLevel &L)
 {
     using namespace dfm;
-    return to_double_i(mul(r.y, mul(r.g, L.invT)), r.m);
+    return to_double_i(norm(mulu(r.y, mulu(r.g, L.invT))), r.m);
 }
 
 // values (and derivatives) of several functions at one temperature
@@ -393,8 +414,7 @@ template <bool MIX, bool DERIV>
 __device__ __forceinline__ void rate_serial(int k, const RateFnTab &R, const TLevel &L, dfm::F2 lu, dfm::F2 su,
                                             RateVal &r, dfm::F2 &sig)
 {
-    const unsigned zero = (kC0Zero >> k & 1) << kZeroC0 | (kC1Zero >> k & 1) << kZeroC1 |
-                          (kC2Zero >> k & 1) << kZeroC2 | (kC3Zero >> k & 1) << kZeroC3;
+    const unsigned zero = (kC1Zero >> k & 1) << kZeroC1 | (kC2Zero >> k & 1) << kZeroC2 | (kC3Zero >> k & 1) << kZeroC3;
     dfm::F2 l = lu;
     sig = su;
     if (!(kSlotU & rf_bit(k)) && !(kC3Zero & rf_bit(k))) l = rate_softplus<MIX>(R.f[k], L, sig);
@@ -650,8 +670,8 @@ __device__ __forceinline__ void cool_term(const RateVal &r, dfm::F2 n, dfm::F2 &
     const int e = r.m + kCoolExp;
     // (terms below 2^-60 of this scale, e-42 erg, are below 2^-48 of the bremsstrahlung)
     const float sc = e < -60 ? 0.0f : pow2f(e > 100 ? 100 : e);
-    v = mul(F2{r.y.hi * sc, r.y.lo * sc}, n);
-    dv = mul(v, r.g);
+    v = mulu(F2{r.y.hi * sc, r.y.lo * sc}, n);
+    dv = mulu(v, r.g);
 }
 
 // + Compton, varpi = comp (T - T_gamma), comp = 1.017e-37 T_gamma^4 and
@@ -680,12 +700,12 @@ static __device__ const int g_cool_at[12] = {0, 1, 2, 10, 4, 5, 6, 7, 8, 9, 3, 1
 // apart, then 2 and 1 (the empty one left out)
 __device__ __forceinline__ dfm::F2 tree_sum(const dfm::F2 (&a)[kNCool])
 {
-    using dfm::adds;
-    const dfm::F2 s0 = adds(a[cool_at(0)], a[cool_at(8)]), s1 = adds(a[cool_at(1)], a[cool_at(9)]),
-                  s2 = adds(a[cool_at(2)], a[cool_at(10)]);
-    const dfm::F2 t0 = adds(s0, a[cool_at(4)]), t1 = adds(s1, a[cool_at(5)]), t2 = adds(s2, a[cool_at(6)]),
-                  t3 = adds(a[cool_at(3)], a[cool_at(7)]);
-    return adds(adds(t0, t2), adds(t1, t3));
+    using dfm::addu;
+    const dfm::F2 s0 = addu(a[cool_at(0)], a[cool_at(8)]), s1 = addu(a[cool_at(1)], a[cool_at(9)]),
+                  s2 = addu(a[cool_at(2)], a[cool_at(10)]);
+    const dfm::F2 t0 = addu(s0, a[cool_at(4)]), t1 = addu(s1, a[cool_at(5)]), t2 = addu(s2, a[cool_at(6)]),
+                  t3 = addu(a[cool_at(3)], a[cool_at(7)]);
+    return dfm::norm(addu(addu(t0, t2), addu(t1, t3)));
 }
 
 // one thread; RV: optional, per term f, df/dT and d2f/dT2 for the tangents
@@ -721,7 +741,7 @@ __device__ __forceinline__ void cooling_sums(const TLevel &L, int case_b, bool h
         }
     }
     Ls = to_double_i(tree_sum(a), -kCoolExp);
-    dLs = to_double_i(mul(tree_sum(b), L.invT), -kCoolExp);
+    dLs = to_double_i(norm(mulu(tree_sum(b), L.invT)), -kCoolExp);
 }
 
 // (out of line, as the rate sets above)
@@ -776,7 +796,7 @@ static __device__ __noinline__ void cooling_serial(int case_b, double comp, doub
 // order of tree_sum
 __device__ __forceinline__ dfm::F2 team_add(unsigned mask, dfm::F2 a, int m)
 {
-    return dfm::adds(a, dfm::F2{__shfl_xor_sync(mask, a.hi, m), __shfl_xor_sync(mask, a.lo, m)});
+    return dfm::addu(a, dfm::F2{__shfl_xor_sync(mask, a.hi, m), __shfl_xor_sync(mask, a.lo, m)});
 }
 template <bool MIX>
 static __device__ __noinline__ double2 cooling_sums_team4(int case_b, bool helium, double T, double nHI, double nHII,
@@ -806,10 +826,10 @@ static __device__ __noinline__ double2 cooling_sums_team4(int case_b, bool heliu
         cool_term(q, split_density(pick(n, g_cool_sp[k])), v[r], dv[r]);
         if (k >= kNCool || (!helium && (cool_mask(1) >> k & 1))) v[r] = dv[r] = F2{0.0f, 0.0f};
     }
-    F2 s = adds(adds(v[0], v[2]), v[1]), ds = adds(adds(dv[0], dv[2]), dv[1]);
-    s = team_add(mask, team_add(mask, s, 2), 1);
-    ds = team_add(mask, team_add(mask, ds, 2), 1);
-    return make_double2(to_double_i(s, -kCoolExp), to_double_i(mul(ds, L.invT), -kCoolExp));
+    F2 s = addu(addu(v[0], v[2]), v[1]), ds = addu(addu(dv[0], dv[2]), dv[1]);
+    s = norm(team_add(mask, team_add(mask, s, 2), 1));
+    ds = norm(team_add(mask, team_add(mask, ds, 2), 1));
+    return make_double2(to_double_i(s, -kCoolExp), to_double_i(norm(mulu(ds, L.invT)), -kCoolExp));
 }
 
 }  // namespace rtgb

@@ -289,12 +289,12 @@ __device__ __forceinline__ dfm::F2 inv_pair(double x)
 }
 __device__ __forceinline__ double level_mu(const Dual &md, dfm::F2 iT, const Dual &Tmu1, TLevel &L)
 {
-    t_level_inv(dfm::mul(dfm::split_any(md.v), iT), L);
+    t_level_inv(dfm::norm(dfm::mulu(dfm::split_any(md.v), iT)), L);
     return qdiv(Tmu1, md).d;
 }
 __device__ __forceinline__ double level_mu(double md, dfm::F2 iT, double, TLevel &L)
 {
-    t_level_inv(dfm::mul(dfm::split_any(md), iT), L);
+    t_level_inv(dfm::norm(dfm::mulu(dfm::split_any(md), iT)), L);
     return 0.0;
 }
 
