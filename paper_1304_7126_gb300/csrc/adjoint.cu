@@ -13,7 +13,10 @@
 // thermo_vjp differentiates the sub-cycled thermochemistry of one cell in
 // forward mode: a team of lanes per cell, lane j seeded with the unit
 // tangent of input j (N_0..N_{G-1}, x_HII, x_HeII, x_HeIII, T, n_H), runs
-// the thermo_step code of the forward kernels instantiated on dual numbers.
+// the thermo_step code of the forward kernels instantiated on dual numbers;
+// every eight lanes share the cell's rate functions, whose values are the
+// same in all of them.  Bound by the length of the longest cell's chain of
+// attempts, three FP64 instructions per forward one.
 // Its values are the bits of the forward path, so it takes the same
 // sub-cycle decisions; the derivative is that of the step sequence the
 // forward run took (the schedule is piecewise constant in the inputs).
@@ -82,7 +85,7 @@ thermo_vjp_kernel(ThermoParams p, const double *__restrict__ nH, const double *_
         }
     }
     __syncwarp();
-    if (!valid || j >= NT) return;
+    if (!valid) return;   // (the lanes past NT stay: they share the team's rate functions)
 
     CellState<G, Dual> st;
     st.x = Dual(xHII[c], j == G ? 1.0 : 0.0);
@@ -103,14 +106,14 @@ thermo_vjp_kernel(ThermoParams p, const double *__restrict__ nH, const double *_
     if (p.isothermal) {
         TLevel L;
         t_level(st.T.v, L);
-        h_rates<1, false>(L, st.T.d, p.case_b, iso.h);
-        if (p.helium) he_rates<1, false>(L, st.T.d, p.case_b, iso.he);
+        h_rates<8, false>(L, st.T.d, p.case_b, iso.h);
+        if (p.helium) he_rates<8, false>(L, st.T.d, p.case_b, iso.he);
     }
     double t_left = p.dt, dt_tc = p.dt;
     int att = 0;
     bool done = false;
     while (!done) {
-        done = subcycle_once<G, 1, false, Dual>(p, n, st, t_left, dt_tc, att, iso, cc);
+        done = subcycle_once<G, 8, false, Dual>(p, n, st, t_left, dt_tc, att, iso, cc);
         if (!done && att >= p.max_sub) {
             atomicOr(status, kStatusSubcycle);
             done = true;
@@ -120,6 +123,7 @@ thermo_vjp_kernel(ThermoParams p, const double *__restrict__ nH, const double *_
     double g = lxv * st.x.d + ly2v * st.y2.d + ly3v * st.y3.d + lTv * st.T.d;
 #pragma unroll
     for (int i = 0; i < G; ++i) g += lNv[i] * st.N[i].d + w[i] * st.Fs[i].d;
+    if (j >= NT) return;
     if (!isfinite(g)) atomicOr(status, kStatusNonFinite);
 
     if (j < G) {

@@ -179,8 +179,7 @@ struct RateFn {
     double Cc;
     dfm::F2 c0, c5;             // (with Cc: the function in terms of ln T, for rt_rate_functions)
     dfm::F2 c1, c2, c3, c4, c5r;
-    dfm::F2 Cm, c34;            // Cc exp(c0 + c1 14 ln 2) = Cm 2^ke, 1 <= Cm < 2; c3 c4
-    double d1, d2, d34, d344;   // c1, c2, c3 c4, c3 c4^2 (second derivative)
+    dfm::F2 Cm, c34, c344;      // Cc exp(c0 + c1 14 ln 2) = Cm 2^ke, 1 <= Cm < 2; c3 c4, c3 c4^2
     int ke;
 };
 struct RateFnTab {
@@ -209,7 +208,7 @@ constexpr RateFn rate_fn(double Cc, double c0, double c1, double c2, double c3, 
     while (m >= 2.0) { m *= 0.5; ++e; }
     while (m > 0.0 && m < 1.0) { m *= 2.0; --e; }
     return RateFn{Cc, pair_of(c0), pair_of(c5), pair_of(c1), pair_of(c2), pair_of(c3), pair_of(c4),
-                  pair_of(c5 + c4 * kLnTRefV), pair_of(m), pair_of(c3 * c4), c1, c2, c3 * c4, c3 * c4 * c4, e};
+                  pair_of(c5 + c4 * kLnTRefV), pair_of(m), pair_of(c3 * c4), pair_of(c3 * c4 * c4), e};
 }
 constexpr RateFn cen_fn(double A, double T0) { return rate_fn(A, 0.0, 0.5, -T0, 1.0, 0.5, -kHalfLn1e5); }
 constexpr RateFn hg_fn(const RateTable &R, int j)
@@ -286,10 +285,11 @@ __device__ __forceinline__ void t_level_inv(dfm::F2 invT, TLevel &L)
     else L.lnT = split_any(-log(to_double(invT)) - kLnTRefV);
 }
 
-// A function value y 2^m (y a normalised pair below 8, or 0) and
-// g = d ln f / d ln T as a pair
+// A function value y 2^m (y a normalised pair below 8, or 0), as pairs
+// g = d ln f / d ln T and, for the adjoint, w = T^2 f'' / f = g^2 - g + c2/T -
+// c3 c4^2 sigma (1 - sigma)
 struct RateVal {
-    dfm::F2 y, g;
+    dfm::F2 y, g, w;
     int m;
 };
 
@@ -347,7 +347,7 @@ __device__ __forceinline__ dfm::F2 rate_softplus(const RateFn &q, const TLevel &
 // exponential of the reduced argument and the log-derivative in FP32
 // (relative accuracy ~2e-7).  zero: bits kZero* of the terms known to be
 // zero (compile-time), one3: c3 = 1.
-template <bool MIX, bool DERIV>
+template <bool MIX, int DERIV>
 __device__ __forceinline__ void rate_val(const RateFn &q, const TLevel &L, dfm::F2 l, dfm::F2 sig, unsigned zero,
                                          bool one3, RateVal &r)
 {
@@ -364,18 +364,22 @@ __device__ __forceinline__ void rate_val(const RateFn &q, const TLevel &L, dfm::
         const float t = __fadd_rn(__fmaf_rn(-kf, -1.90465421e-9f, __fmaf_rn(-kf, 0.693147182f, arg.hi)), arg.lo);
         r.y = mul(q.Cm, expf(t));
         r.m = (int)kf + q.ke;
-        if constexpr (DERIV)
+        if constexpr (DERIV > 0)
             r.g = F2{__fmaf_rn(-q.c34.hi, sig.hi, __fmaf_rn(-q.c2.hi, L.invT.hi, q.c1.hi)), 0.0f};
     } else {
         int m;
         exp_pair(arg, r.y, m);
         r.y = norm(mulu(q.Cm, r.y));
         r.m = m + q.ke;
-        if constexpr (DERIV) {
+        if constexpr (DERIV > 0) {
             F2 g = (zero >> kZeroC1 & 1) ? nil : q.c1;
             if (!(zero >> kZeroC2 & 1)) g = addu(g, neg(b));
             if (!(zero >> kZeroC3 & 1)) g = addu(g, neg(mulu(sig, q.c34)));
             r.g = norm(g);
+        }
+        if constexpr (DERIV > 1) {
+            F2 w = addu(addu(mulu(r.g, r.g), neg(r.g)), b);
+            r.w = norm(addu(w, neg(mulu(q.c344, addu(sig, neg(mulu(sig, sig)))))));
         }
     }
 }
@@ -385,6 +389,12 @@ __device__ __forceinline__ double rate_df(const RateVal &r, const TLevel &L)
 {
     using namespace dfm;
     return to_double_i(norm(mulu(r.y, mulu(r.g, L.invT))), r.m);
+}
+// d2f/dT2 = f w / T^2
+__device__ __forceinline__ double rate_d2f(const RateVal &r, const TLevel &L)
+{
+    using namespace dfm;
+    return to_double_i(norm(mulu(mulu(r.y, L.invT), mulu(r.w, L.invT))), r.m);
 }
 
 // values (and derivatives) of several functions at one temperature
@@ -410,7 +420,7 @@ constexpr unsigned kNeedCoolH = cool_mask(0), kNeedCoolHe = cool_mask(1);
 
 // one thread: slot k (a constant once unrolled) at level L, given the
 // softplus of u
-template <bool MIX, bool DERIV>
+template <bool MIX, int DERIV>
 __device__ __forceinline__ void rate_serial(int k, const RateFnTab &R, const TLevel &L, dfm::F2 lu, dfm::F2 su,
                                             RateVal &r, dfm::F2 &sig)
 {
@@ -435,10 +445,10 @@ __device__ __forceinline__ void rates_serial(const TLevel &L, int case_b, unsign
             RateVal v;
             dfm::F2 sig;
             if (needD & rf_bit(k)) {
-                rate_serial<MIX, true>(k, R, L, lu, su, v, sig);
+                rate_serial<MIX, 1>(k, R, L, lu, su, v, sig);
                 r.df[k] = rate_df(v, L);
             } else {
-                rate_serial<MIX, false>(k, R, L, lu, su, v, sig);
+                rate_serial<MIX, 0>(k, R, L, lu, su, v, sig);
             }
             r.f[k] = rate_f(v);
         }
@@ -459,49 +469,13 @@ template <int TS>
 __device__ __forceinline__ double team_get(unsigned m, double v, int src) { return __shfl_sync(m, v, src, TS); }
 
 // one function per lane of a team, slot k, with its own softplus
-template <bool MIX, bool DERIV>
+template <bool MIX, int DERIV>
 __device__ __forceinline__ void rate_lane(int case_b, int k, const TLevel &L, RateVal &r)
 {
     const RateFn &q = g_rate_fn[case_b].f[k];
     dfm::F2 sig;
     const dfm::F2 l = rate_softplus<MIX>(q, L, sig);
     rate_val<MIX, DERIV>(q, L, l, sig, 0u, false, r);
-}
-
-// f, df/dT and d2f/dT2 of slot k at level L (values f, df with the bits of
-// the double path): with g = c1 - c2/T - c3 c4 sigma, d ln f/dT = g/T and
-//     d2f/dT2 = f [(g/T)^2 + (-g + c2/T - c3 c4^2 sigma (1 - sigma)) / T^2].
-__device__ __forceinline__ void rate_dd(int k, const RateFnTab &R, const TLevel &L, dfm::F2 lu, dfm::F2 su, double x,
-                                        RateVal &v, double &f, double &df, double &d2f)
-{
-    dfm::F2 sig;
-    rate_serial<false, true>(k, R, L, lu, su, v, sig);
-    const RateFn &q = R.f[k];
-    const double sg = (kC3Zero & rf_bit(k)) ? 0.0 : dfm::to_double_i(sig), g = dfm::to_double_i(v.g), D = g * x;
-    f = rate_f(v);
-    df = rate_df(v, L);
-    d2f = f * (D * D + x * x * (-g + q.d2 * x - q.d344 * sg * (1.0 - sg)));
-}
-
-// A dual temperature (level L of its value, derivative dT): f carries df dT
-// and df carries d2f dT.
-__device__ __forceinline__ void rates_dual(const TLevel &L, double dT, int case_b, unsigned needF, unsigned needD,
-                                           RatesT<Dual> &r)
-{
-    const RateFnTab &R = c_rate_fn[case_b];
-    const double x = dfm::to_double_i(L.invT);
-    dfm::F2 lu{0.0f, 0.0f}, su{0.0f, 0.0f};
-    if (needF & kSlotU) lu = rate_softplus<false>(R.f[RF_BETA_HI], L, su);
-#pragma unroll
-    for (int k = 0; k < NRF; ++k) {
-        if (needF & rf_bit(k)) {
-            RateVal v;
-            double f, df, d2f;
-            rate_dd(k, R, L, lu, su, x, v, f, df, d2f);
-            r.f[k] = Dual(f, df * dT);
-            if (needD & rf_bit(k)) r.df[k] = Dual(df, d2f * dT);
-        }
-    }
 }
 
 template <typename S>
@@ -568,7 +542,7 @@ static __device__ __noinline__ HRates h_rates_team(TLevel L, int case_b)
 {
     const unsigned m = team_mask<TS>();
     RateVal v;
-    rate_lane<MIX, true>(case_b, team_lane<TS>() == 0 ? RF_BETA_HI : RF_ALPHA_HII, L, v);
+    rate_lane<MIX, 1>(case_b, team_lane<TS>() == 0 ? RF_BETA_HI : RF_ALPHA_HII, L, v);
     const double f = rate_f(v), df = rate_df(v, L);
     HRates r;
     r.beta = team_get<TS>(m, f, 0);
@@ -584,7 +558,7 @@ static __device__ __noinline__ HeRates he_rates_team(TLevel L, int case_b)
 {
     const unsigned m = team_mask<TS>();
     RateVal v;
-    rate_lane<MIX, false>(case_b, RF_BETA_HEI + (team_lane<TS>() & 3), L, v);
+    rate_lane<MIX, 0>(case_b, RF_BETA_HEI + (team_lane<TS>() & 3), L, v);
     const double f = rate_f(v);
     HeRates r;
     r.beta_HeI = team_get<TS>(m, f, 0);
@@ -593,20 +567,34 @@ static __device__ __noinline__ HeRates he_rates_team(TLevel L, int case_b)
     r.alpha_HeIII = team_get<TS>(m, f, 3);
     return r;
 }
+// dual numbers, by a team of eight lanes that hold the same value and each
+// their own tangent (level L of the value, dT this lane's tangent of T): the
+// values are those above, f carries df/dT dT and df/dT carries d2f/dT2 dT
 static __device__ __noinline__ HRatesT<Dual> h_rates_dual(TLevel L, double dT, int case_b)
 {
-    RatesT<Dual> t;
+    const unsigned m = team_mask<8>();
+    RateVal v;
+    rate_lane<false, 2>(case_b, team_lane<8>() == 0 ? RF_BETA_HI : RF_ALPHA_HII, L, v);
+    const double f = rate_f(v), df = rate_df(v, L), d2f = rate_d2f(v, L);
     HRatesT<Dual> r;
-    rates_dual(L, dT, case_b, kNeedH, kNeedH, t);
-    h_rates_from(t, r);
+    const double b1 = team_get<8>(m, df, 0), a1 = team_get<8>(m, df, 1);
+    r.beta = Dual(team_get<8>(m, f, 0), b1 * dT);
+    r.dbeta = Dual(b1, team_get<8>(m, d2f, 0) * dT);
+    r.alpha = Dual(team_get<8>(m, f, 1), a1 * dT);
+    r.dalpha = Dual(a1, team_get<8>(m, d2f, 1) * dT);
     return r;
 }
 static __device__ __noinline__ HeRatesT<Dual> he_rates_dual(TLevel L, double dT, int case_b)
 {
-    RatesT<Dual> t;
+    const unsigned m = team_mask<8>();
+    RateVal v;
+    rate_lane<false, 1>(case_b, RF_BETA_HEI + (team_lane<8>() & 3), L, v);
+    const double f = rate_f(v), df = rate_df(v, L);
     HeRatesT<Dual> r;
-    rates_dual(L, dT, case_b, kNeedHe, 0u, t);
-    he_rates_from(t, r);
+    r.beta_HeI = Dual(team_get<8>(m, f, 0), team_get<8>(m, df, 0) * dT);
+    r.beta_HeII = Dual(team_get<8>(m, f, 1), team_get<8>(m, df, 1) * dT);
+    r.alpha_HeII = Dual(team_get<8>(m, f, 2), team_get<8>(m, df, 2) * dT);
+    r.alpha_HeIII = Dual(team_get<8>(m, f, 3), team_get<8>(m, df, 3) * dT);
     return r;
 }
 
@@ -708,13 +696,10 @@ __device__ __forceinline__ dfm::F2 tree_sum(const dfm::F2 (&a)[kNCool])
     return dfm::norm(addu(addu(t0, t2), addu(t1, t3)));
 }
 
-// one thread; RV: optional, per term f, df/dT and d2f/dT2 for the tangents
-struct CoolDD {
-    double f[kNCool], df[kNCool], d2f[kNCool];
-};
-template <bool MIX, bool DD>
+// one thread
+template <bool MIX>
 __device__ __forceinline__ void cooling_sums(const TLevel &L, int case_b, bool helium, const double *n, double &Ls,
-                                             double &dLs, CoolDD *dd)
+                                             double &dLs)
 {
     using namespace dfm;
     const RateFnTab &R = c_rate_fn[case_b];
@@ -724,8 +709,6 @@ __device__ __forceinline__ void cooling_sums(const TLevel &L, int case_b, bool h
     F2 su;
     const F2 lu = rate_softplus<MIX>(R.f[RF_BETA_HI], L, su);
     F2 a[kNCool], b[kNCool];
-    double x = 0.0;
-    if constexpr (DD) x = to_double_i(L.invT);
 #pragma unroll
     for (int k = 0; k < kNCool; ++k) {
         const CoolTerm q = cool_row(k);
@@ -733,11 +716,8 @@ __device__ __forceinline__ void cooling_sums(const TLevel &L, int case_b, bool h
         if (helium || !q.he) {
             RateVal v;
             F2 sig;
-            if constexpr (DD) rate_dd(k, R, L, lu, su, x, v, dd->f[k], dd->df[k], dd->d2f[k]);
-            else rate_serial<MIX, true>(k, R, L, lu, su, v, sig);
+            rate_serial<MIX, 1>(k, R, L, lu, su, v, sig);
             cool_term(v, np[q.sp], a[k], b[k]);
-        } else if constexpr (DD) {
-            dd->f[k] = dd->df[k] = dd->d2f[k] = 0.0;
         }
     }
     Ls = to_double_i(tree_sum(a), -kCoolExp);
@@ -753,7 +733,7 @@ static __device__ __noinline__ double2 cooling_sums_serial(int case_b, bool heli
     t_level(T, Lv);
     double n[NSP], Ls, dLs;
     cool_densities(nHI, nHII, nHeI, nHeII, nHeIII, n);
-    cooling_sums<MIX, false>(Lv, case_b, helium, n, Ls, dLs, nullptr);
+    cooling_sums<MIX>(Lv, case_b, helium, n, Ls, dLs);
     return make_double2(Ls, dLs);
 }
 template <bool MIX>
@@ -763,33 +743,6 @@ __device__ __forceinline__ void cooling_serial(int case_b, double comp, double t
 {
     const double2 s = cooling_sums_serial<MIX>(case_b, helium, T, nHI, nHII, nHeI, nHeII, nHeIII);
     cooling_close(comp, tg, T, ne, s.x, s.y, L, dL);
-}
-
-// dual numbers: the values of the double path, the tangents term by term
-template <bool MIX>
-static __device__ __noinline__ void cooling_serial(int case_b, double comp, double tg, bool helium, const Dual &T,
-                                                   const Dual &ne, const Dual &nHI, const Dual &nHII,
-                                                   const Dual &nHeI, const Dual &nHeII, const Dual &nHeIII, Dual &L,
-                                                   Dual &dL)
-{
-    static_assert(!MIX, "dual rates: FP64");
-    TLevel Lv;
-    t_level(T.v, Lv);
-    Dual n[NSP];
-    cool_densities(nHI, nHII, nHeI, nHeII, nHeIII, n);
-    double nv[NSP];
-#pragma unroll
-    for (int k = 0; k < NSP; ++k) nv[k] = n[k].v;
-    CoolDD dd;
-    Dual Ls(0.0), dLs(0.0);
-    cooling_sums<false, true>(Lv, case_b, helium, nv, Ls.v, dLs.v, &dd);
-#pragma unroll
-    for (int k = 0; k < kNCool; ++k) {
-        const int sp = cool_row(k).sp;
-        Ls.d += dd.f[k] * n[sp].d + dd.df[k] * T.d * n[sp].v;
-        dLs.d += dd.df[k] * n[sp].d + dd.d2f[k] * T.d * n[sp].v;
-    }
-    cooling_close(comp, tg, T, ne, Ls, dLs, L, dL);
 }
 
 // a team of four: places t, t + 4, t + 8, the last sums over shuffles, in the
@@ -822,7 +775,7 @@ static __device__ __noinline__ double2 cooling_sums_team4(int case_b, bool heliu
         const int k = r ? g_cool_at[t + 4 * r] : k0;
         RateVal q;
         // (no softplus in round 2 nor in lane 3 of round 1: c3 = c3 c4 = 0)
-        rate_val<MIX, true>(R[k], L, r ? lu : l, r ? su : sig, r == 2 ? 1u << kZeroC3 : 0u, false, q);
+        rate_val<MIX, 1>(R[k], L, r ? lu : l, r ? su : sig, r == 2 ? 1u << kZeroC3 : 0u, false, q);
         cool_term(q, split_density(pick(n, g_cool_sp[k])), v[r], dv[r]);
         if (k >= kNCool || (!helium && (cool_mask(1) >> k & 1))) v[r] = dv[r] = F2{0.0f, 0.0f};
     }
@@ -830,6 +783,63 @@ static __device__ __noinline__ double2 cooling_sums_team4(int case_b, bool heliu
     s = norm(team_add(mask, team_add(mask, s, 2), 1));
     ds = norm(team_add(mask, team_add(mask, ds, 2), 1));
     return make_double2(to_double_i(s, -kCoolExp), to_double_i(norm(mulu(ds, L.invT)), -kCoolExp));
+}
+
+// dual numbers, by a team of eight (same values, a tangent per lane): places
+// t and t + 8; the values as above.  With the sums over the species s of
+// F_s = sum f and their T-derivatives, the tangents are dL = sum F_s dn_s +
+// L_T dT and dL_T = sum F_s' dn_s + L_TT dT.
+static __device__ __noinline__ void cooling_dual(int case_b, double comp, double tg, bool helium, const Dual &T,
+                                                 const Dual &ne, const Dual &nHI, const Dual &nHII, const Dual &nHeI,
+                                                 const Dual &nHeII, const Dual &nHeIII, Dual &L, Dual &dL)
+{
+    using namespace dfm;
+    const unsigned mask = team_mask<8>();
+    const int t = team_lane<8>();
+    const RateFn *R = g_rate_fn[case_b].f;
+    TLevel Lv;
+    t_level(T.v, Lv);
+    Dual n[NSP];
+    cool_densities(nHI, nHII, nHeI, nHeII, nHeIII, n);
+    double nv[NSP];
+#pragma unroll
+    for (int k = 0; k < NSP; ++k) nv[k] = n[k].v;
+    F2 v[2], dv[2], d2[2];
+    double f[2], df[2];
+#pragma unroll
+    for (int r = 0; r < 2; ++r) {
+        const int k = r ? (t < 4 ? g_cool_at[t + 8] : kNCool) : g_cool_at[t];
+        F2 sig{0.0f, 0.0f}, l{0.0f, 0.0f};
+        if (r == 0) l = rate_softplus<false>(R[k], Lv, sig);   // (none in places 8 to 11)
+        RateVal q;
+        rate_val<false, 2>(R[k], Lv, l, sig, r ? 1u << kZeroC3 : 0u, false, q);
+        cool_term(q, split_density(pick(nv, g_cool_sp[k])), v[r], dv[r]);
+        d2[r] = mulu(v[r], q.w);
+        f[r] = rate_f(q);
+        df[r] = rate_df(q, Lv);
+        if (k >= kNCool || (!helium && (cool_mask(1) >> k & 1))) {
+            v[r] = dv[r] = d2[r] = F2{0.0f, 0.0f};
+            f[r] = df[r] = 0.0;
+        }
+    }
+    F2 s = addu(v[0], v[1]), ds = addu(dv[0], dv[1]), d2s = addu(d2[0], d2[1]);
+#pragma unroll
+    for (int m = 4; m >= 1; m >>= 1) {
+        s = team_add(mask, s, m);
+        ds = team_add(mask, ds, m);
+        d2s = team_add(mask, d2s, m);
+    }
+    const double Ls = to_double_i(norm(s), -kCoolExp);
+    const double dLs = to_double_i(norm(mulu(norm(ds), Lv.invT)), -kCoolExp);
+    const double d2Ls = to_double_i(norm(mulu(mulu(d2s, Lv.invT), Lv.invT)), -kCoolExp);
+    double tL = dLs * T.d, tdL = d2Ls * T.d;
+#pragma unroll
+    for (int p = 0; p < kNCool; ++p) {
+        const int sp = cool_row(cool_at(p)).sp;
+        tL = ::fma(team_get<8>(mask, f[p / 8], p % 8), n[sp].d, tL);
+        tdL = ::fma(team_get<8>(mask, df[p / 8], p % 8), n[sp].d, tdL);
+    }
+    cooling_close(comp, tg, T, ne, Dual(Ls, tL), Dual(dLs, tdL), L, dL);
 }
 
 }  // namespace rtgb

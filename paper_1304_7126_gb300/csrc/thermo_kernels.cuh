@@ -34,14 +34,14 @@ template <int G, int PT, typename P, bool R32, bool SM>
 __device__ __forceinline__ void load_cell(const ThermoParams &p, long long c, bool first, const double *xHII,
                                           const double *xHeII, const double *xHeIII, const double *T,
                                           const P *N, const P *Npre, const double *fscale,
-                                          CellState<lane_groups(G, PT)> &st, IsoRates<> &iso, CoolCache<> &cc)
+                                          CellState<lane_groups<>(G, PT)> &st, IsoRates<> &iso, CoolCache<> &cc)
 {
     st.x = xHII[c];
     st.y2 = xHeII[c];
     st.y3 = xHeIII[c];
     st.T = T[c];
 #pragma unroll
-    for (int r = 0; r < lane_groups(G, PT); ++r) {
+    for (int r = 0; r < lane_groups<>(G, PT); ++r) {
         const int i = r * PT + team_lane<PT>();
         st.N[r] = 0.0;
         st.Fs[r] = 1.0;
@@ -80,7 +80,7 @@ template <int G, int PT, typename P, bool SM>
 __device__ __forceinline__ void store_cell(const ThermoParams &p, long long c, bool first, bool handoff,
                                            double *xHII, double *xHeII, double *xHeIII, double *T, P *N, P *F,
                                            P *Npre, P *Fpre, double *fscale,
-                                           const CellState<lane_groups(G, PT)> &st, unsigned *status)
+                                           const CellState<lane_groups<>(G, PT)> &st, unsigned *status)
 {
     if (team_lane<PT>() == 0) {
         xHII[c] = st.x;
@@ -90,7 +90,7 @@ __device__ __forceinline__ void store_cell(const ThermoParams &p, long long c, b
     }
     bool bad = !isfinite(st.x) || !isfinite(st.T);
 #pragma unroll
-    for (int r = 0; r < lane_groups(G, PT); ++r) {
+    for (int r = 0; r < lane_groups<>(G, PT); ++r) {
         const int i = r * PT + team_lane<PT>();
         if (PT > 1 && i >= G) continue;
         N[(long long)i * p.nc + c] = (P)st.N[r];
@@ -282,7 +282,7 @@ thermo_team(ThermoParams p, const double *__restrict__ nH, double *xHII, double 
     const unsigned long long warps = (unsigned long long)gridDim.x * (blockDim.x >> 5);
     const unsigned long long first = ((threadIdx.x & 31) / kTeam) * warps + (threadIdx.x >> 5) * gridDim.x + blockIdx.x;
     const unsigned long long teams = warps * (32 / kTeam);
-    CellState<lane_groups(G, kTeam)> st;
+    CellState<lane_groups<>(G, kTeam)> st;
     IsoRates<> iso;
     CoolCache<> cc;
     double t_left = 0.0, dt_tc = 0.0, n = 0.0;

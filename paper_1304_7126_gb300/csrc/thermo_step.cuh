@@ -22,9 +22,13 @@ constexpr double kXMin = 1e-6;
 constexpr double kNeFloor = 1e-6;
 constexpr double kTFloor = 1.0;
 
-// Photon groups a lane holds: all G of them (PT = 1), or those of its place
-// in a team of PT lanes, group r PT + t in place r.
-__host__ __device__ constexpr int lane_groups(int G, int PT) { return (G + PT - 1) / PT; }
+// Photon groups a lane holds: all G of them (PT = 1, or dual numbers), or
+// those of its place in a team of PT lanes, group r PT + t in place r.
+template <typename S = double>
+__host__ __device__ constexpr int lane_groups(int G, int PT)
+{
+    return std::is_same<S, double>::value ? (G + PT - 1) / PT : G;
+}
 
 template <int NG, typename S = double>
 struct CellState {
@@ -260,11 +264,11 @@ __device__ __forceinline__ void he3_rates(const TLevel &L, double, int case_b, H
         r.alpha_HeIII = t.y;
     }
 }
-// dual numbers: the level of the value, dT the derivative of T
+// dual numbers, a team of eight: the level of the value, dT the tangent of T
 template <int TS, bool MIX>
 __device__ __forceinline__ void h_rates(const TLevel &L, double dT, int case_b, HRatesT<Dual> &r)
 {
-    static_assert(TS == 1 && !MIX, "dual rates: one thread, FP64");
+    static_assert(TS == 8 && !MIX, "dual rates: teams of eight, FP64");
     r = h_rates_dual(L, dT, case_b);
 }
 template <int TS, bool MIX>
@@ -376,12 +380,12 @@ __device__ __forceinline__ void photon_group(const ThermoParams &p, int i, const
 // breaks the 10% rule.  The recombination photons C_i (without the OTSA) come
 // from cc.rj.
 template <int G, int PT, bool MIX, bool SM>
-__device__ __forceinline__ bool photons_team(const ThermoParams &p, const CellState<lane_groups(G, PT)> &s,
+__device__ __forceinline__ bool photons_team(const ThermoParams &p, const CellState<lane_groups<>(G, PT)> &s,
                                              const CoolCache<double> &cc, double nHI, double nHeI, double nHeII,
-                                             double h, CellState<lane_groups(G, PT)> &o, double &gam0, double &gam1,
+                                             double h, CellState<lane_groups<>(G, PT)> &o, double &gam0, double &gam1,
                                              double &gam2, double &heat, bool &sm)
 {
-    constexpr int NG = lane_groups(G, PT);
+    constexpr int NG = lane_groups<>(G, PT);
     const unsigned mask = team_mask<PT>();
     const int t = team_lane<PT>();
     bool ok = true, small = true;
@@ -470,13 +474,15 @@ __device__ __forceinline__ bool photons_serial(const ThermoParams &p, const Cell
 // (values bit-identical to the double path; MIX only with double).
 // TS: 1, one thread, or 4, a team of four lanes that hold the same cell,
 // share its rate functions and each update their own photon groups; the same
-// operations in the same order, so the same bits.
+// operations in the same order, so the same bits.  Dual: teams of eight lanes
+// with the same values and a tangent each; they share the rate functions.
 template <int G, int TS, bool MIX, typename S = double, bool SM = false>
-__device__ __forceinline__ bool attempt(const ThermoParams &p, const S &nH, const CellState<lane_groups(G, TS), S> &s,
+__device__ __forceinline__ bool attempt(const ThermoParams &p, const S &nH, const CellState<lane_groups<S>(G, TS), S> &s,
                                         double h, const IsoRates<S> &iso, CoolCache<S> &cc,
-                                        CellState<lane_groups(G, TS), S> &o, bool &small)
+                                        CellState<lane_groups<S>(G, TS), S> &o, bool &small)
 {
-    static_assert(TS == 1 || (TS == 4 && std::is_same<S, double>::value), "teams of four, FP64");
+    constexpr bool dual = !std::is_same<S, double>::value;
+    static_assert(dual ? TS == 8 : TS == 1 || TS == 4, "team sizes");
     static_assert(!MIX || sizeof(S) == sizeof(double), "the mixed path is not differentiated");
     const S nHe = iso.nHe;
     const S x = s.x, y2 = s.y2, y3 = s.y3;
@@ -505,7 +511,9 @@ __device__ __forceinline__ bool attempt(const ThermoParams &p, const S &nH, cons
     }
 
     if (!p.isothermal && !cc.valid) {
-        if constexpr (TS > 1) {
+        if constexpr (dual) {
+            cooling_dual(p.case_b, p.comp, p.tg, p.helium != 0, s.T, ne, nHI, nHII, nHeI, nHeII, nHeIII, cc.L, cc.dL);
+        } else if constexpr (TS > 1) {
             const double2 c = cooling_sums_team4<MIX>(p.case_b, p.helium != 0, s.T, nHI, nHII, nHeI, nHeII, nHeIII);
             cooling_close(p.comp, p.tg, s.T, ne, c.x, c.y, cc.L, cc.dL);
         } else {
@@ -521,7 +529,7 @@ __device__ __forceinline__ bool attempt(const ThermoParams &p, const S &nH, cons
     // written), so they give the same bits
     {
         bool ok;
-        if constexpr (TS > 1)
+        if constexpr (TS > 1 && !dual)
             ok = photons_team<G, TS, MIX, SM>(p, s, cc, nHI, nHeI, nHeII, h, o, gam0, gam1, gam2, heat, sm);
         else ok = photons_serial<G, MIX, SM>(p, s, cc, nHI, nHeI, nHeII, h, o, gam0, gam1, gam2, heat, sm);
         if (!ok) return false;
@@ -624,13 +632,13 @@ __device__ __forceinline__ bool attempt(const ThermoParams &p, const S &nH, cons
 // One attempt of the sub-cycling loop; returns true when the cell is done.
 template <int G, int TS, bool MIX, typename S = double, bool SM = false>
 __device__ __forceinline__ bool subcycle_once(const ThermoParams &p, const S &nH,
-                                              CellState<lane_groups(G, TS), S> &st, double &t_left, double &dt_tc,
+                                              CellState<lane_groups<S>(G, TS), S> &st, double &t_left, double &dt_tc,
                                               int &att, const IsoRates<S> &iso, CoolCache<S> &cc)
 {
     // t_left, dt_tc > 0: compared through their bits
     double h = (dbits(dt_tc) < dbits(t_left)) ? dt_tc : t_left;
     ++att;
-    CellState<lane_groups(G, TS), S> o;
+    CellState<lane_groups<S>(G, TS), S> o;
     bool small = false;
     if (attempt<G, TS, MIX, S, SM>(p, nH, st, h, iso, cc, o, small)) {
         st = o;
