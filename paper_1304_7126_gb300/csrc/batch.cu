@@ -137,7 +137,7 @@ struct rt_batch {
     int *d_bg_box = nullptr, *d_bg_grp = nullptr, *d_bg_item0 = nullptr, *d_bg_nitem = nullptr, *d_bg_stride = nullptr;
     std::vector<int> bg_first;      // first box-group index of each box
     double *d_red = nullptr, *d_budget = nullptr, *d_emitted = nullptr;
-    double *hll = nullptr;
+    long long *hllq = nullptr;     // fixed point, FP64 transport
     float *hllf = nullptr;
     unsigned *status = nullptr;
     unsigned *status_host = nullptr;
@@ -188,7 +188,7 @@ void bfree_all(rt_batch *b)
     }
     void *ptrs[] = {b->d_boxes, b->d_items, b->d_Ncls[0], b->d_Ncls[1], b->d_Fcls[0], b->d_Fcls[1], b->d_pin,
                     b->d_pout, b->d_bg_box, b->d_bg_grp, b->d_bg_item0, b->d_bg_nitem, b->d_bg_stride, b->d_red,
-                    b->d_budget, b->d_emitted, b->hll, b->hllf, b->status};
+                    b->d_budget, b->d_emitted, b->hllq, b->hllf, b->status};
     for (void *p : ptrs)
         if (p) cudaFree(p);
     if (b->status_host) cudaFreeHost(b->status_host);
@@ -299,7 +299,7 @@ int enqueue_batch_step(rt_batch *b, double dt)
         if (e != cudaSuccess) return bcuda(b, e, "inject");
     }
     const int nxt = 1 - b->cur;
-    const void *tab = f32 ? (const void *)b->hllf : (const void *)b->hll;
+    const void *tab = f32 ? (const void *)b->hllf : (const void *)b->hllq;
     e = launch_transport_batch_all(b->d_items, b->d_boxes, b->n_items_shape0, b->n_items, f32, b->opt.flux, b->cr,
                                    dt, b->dx, (const void *const *)b->d_Ncls[b->cur],
                                    (const void *const *)b->d_Fcls[b->cur], b->d_Ncls[nxt], b->d_Fcls[nxt], tab,
@@ -530,7 +530,7 @@ int rt_batch_create(int n_boxes, const rt_grid *grids, const int *n_groups, cons
             (rc = balloc(b, &b->d_bg_nitem, b->nbg)) || (rc = balloc(b, &b->d_bg_stride, b->nbg)) ||
             (rc = balloc(b, &b->d_red, b->nbg)) || (rc = balloc(b, &b->d_budget, 4 * (size_t)b->nbg)) ||
             (rc = balloc(b, &b->d_emitted, b->nbg)) || (rc = balloc(b, &b->status, 1)) ||
-            (rc = balloc(b, &b->hll, (size_t)kHllNF * kHllNMU * 2)) || (rc = balloc(b, &b->d_Ncls[0], ncls)) ||
+            (rc = balloc(b, &b->d_Ncls[0], ncls)) ||
             (rc = balloc(b, &b->d_Ncls[1], ncls)) || (rc = balloc(b, &b->d_Fcls[0], ncls)) ||
             (rc = balloc(b, &b->d_Fcls[1], ncls)))
             goto bad;
@@ -550,8 +550,11 @@ int rt_batch_create(int n_boxes, const rt_grid *grids, const int *n_groups, cons
         }
         std::vector<double> tab((size_t)kHllNF * kHllNMU * 2);
         rtgb::hll_table(kHllNF, kHllNMU, tab.data());
-        cudaMemcpy(b->hll, tab.data(), tab.size() * sizeof(double), cudaMemcpyHostToDevice);
-        if (b->mixed) {
+        if (!b->mixed) {
+            const std::vector<long long> tq = hll_fix_table(tab);
+            if ((rc = balloc(b, &b->hllq, tq.size()))) goto bad;
+            cudaMemcpy(b->hllq, tq.data(), tq.size() * sizeof(long long), cudaMemcpyHostToDevice);
+        } else {
             std::vector<float> tf(tab.begin(), tab.end());
             if ((rc = balloc(b, &b->hllf, tf.size()))) goto bad;
             cudaMemcpy(b->hllf, tf.data(), tf.size() * sizeof(float), cudaMemcpyHostToDevice);
@@ -803,7 +806,7 @@ int rt_batch_autotune(rt_batch *b, int trials)
     cudaEvent_t e0, e1;
     B_CUDA(b, cudaEventCreate(&e0));
     B_CUDA(b, cudaEventCreate(&e1));
-    const void *tab = b->mixed ? (const void *)b->hllf : (const void *)b->hll;
+    const void *tab = b->mixed ? (const void *)b->hllf : (const void *)b->hllq;
     std::vector<BoxHost> saved = b->box;
     for (auto &kv : by_side) {
         float best = 1e30f;

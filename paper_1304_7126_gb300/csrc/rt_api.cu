@@ -38,7 +38,8 @@ struct rt_handle {
     float *inflow_f = nullptr;
     bool mixed = false;
     int cur = 0;
-    double *hll = nullptr;
+    double *hll = nullptr;         // (the adjoint's)
+    long long *hllq = nullptr;     // fixed point, FP64 transport
     float *hllf = nullptr;
     int32_t *subcycles = nullptr;
     Queue q{};
@@ -124,7 +125,7 @@ void free_all(rt_handle *h)
     for (cudaEvent_t e : h->pending) cudaEventDestroy(e);
     h->pending.clear();
     void *ptrs[] = {h->nH, h->xHII, h->xHeII, h->xHeIII, h->T, h->N[0], h->N[1], h->F[0], h->F[1],
-                    h->Nf[0], h->Nf[1], h->Ff[0], h->Ff[1], h->hllf, h->hll, h->subcycles, h->q.a.cell, h->q.a.t_left, h->q.a.dt_tc, h->q.a.attempts,
+                    h->Nf[0], h->Nf[1], h->Ff[0], h->Ff[1], h->hllf, h->hll, h->hllq, h->subcycles, h->q.a.cell, h->q.a.t_left, h->q.a.dt_tc, h->q.a.attempts,
                     h->q.b.cell, h->q.b.t_left, h->q.b.dt_tc, h->q.b.attempts, h->q.counters, h->q.fscale, h->part.tr_inbox, h->part.tr_outflow, h->part.th_inbox,
                     h->budget, h->status, h->src_cell, h->src_L, h->src_cell_orig, h->adj, h->adj_sub, h->Npre, h->Fpre, h->inflow_d, h->inflow_f,
                     h->adj_count};
@@ -229,7 +230,7 @@ int enqueue_step(rt_handle *h, double dt, bool capturing = false)
                                  h->Ff[nxt], h->hllf, h->inflow_f, h->part, h->stream);
     else
         e = launch_transport(h->g, h->G, h->opt.flux, h->cr, dt, h->N[h->cur], h->F[h->cur], h->N[nxt],
-                             h->F[nxt], h->hll, h->inflow_d, h->part, h->stream);
+                             h->F[nxt], h->hllq, h->inflow_d, h->part, h->stream);
     if (e != cudaSuccess) return cuda_fail(h, e, "transport");
     if (prof) cudaEventRecord(b, h->stream);
     h->cur = nxt;
@@ -320,7 +321,7 @@ int enqueue_vjp(rt_handle *h, double dt, double *lx, double *ly2, double *ly3, d
         e = launch_inject(h->nsrc, G, nc, h->src_cell, h->src_L, dt / V, NA, st);
         if (e != cudaSuccess) return cuda_fail(h, e, "inject");
     }
-    e = launch_transport(h->g, G, h->opt.flux, h->cr, dt, NA, FA, NB, FB, h->hll, h->inflow_d, h->part, st);
+    e = launch_transport(h->g, G, h->opt.flux, h->cr, dt, NA, FA, NB, FB, h->hllq, h->inflow_d, h->part, st);
     if (e != cudaSuccess) return cuda_fail(h, e, "transport");
     ThermoParams tp = thermo_params(h, dt);
     int32_t *sub_adj = check ? h->adj_sub : nullptr;
@@ -499,6 +500,14 @@ int rt_create(const rt_grid *grid, int n_groups, const rt_options *opt, double c
         rtgb::hll_table(kHllNF, kHllNMU, tab.data());
         if ((e = cudaMemcpy(h->hll, tab.data(), tab.size() * sizeof(double), cudaMemcpyHostToDevice)) != cudaSuccess) {
             rc = cuda_fail(h, e, "hll copy"); goto bad;
+        }
+        if (!h->mixed) {
+            const std::vector<long long> tabq = hll_fix_table(tab);
+            if ((rc = dalloc(h, &h->hllq, tabq.size()))) goto bad;
+            if ((e = cudaMemcpy(h->hllq, tabq.data(), tabq.size() * sizeof(long long), cudaMemcpyHostToDevice)) !=
+                cudaSuccess) {
+                rc = cuda_fail(h, e, "hll copy"); goto bad;
+            }
         }
         if (h->mixed) {
             std::vector<float> tabf(tab.begin(), tab.end());

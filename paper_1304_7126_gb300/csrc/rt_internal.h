@@ -6,6 +6,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <cmath>
 #include <string>
 #include <vector>
 
@@ -138,11 +139,12 @@ struct Partials {
 };
 
 // ---- launchers (defined in the .cu files) ----
-// transport: reads N0/F0, writes N1/F1 for all groups.  inflow: NULL, or
+// transport: reads N0/F0, writes N1/F1 for all groups; the HLL table as fixed
+// point (hll_fix_table).  inflow: NULL, or
 // the ghost states [G][6 faces][N, Fx, Fy, Fz] of RT_BC_INFLOW faces.
 cudaError_t launch_transport(const GridDev &g, int G, int flux, double cr, double dt,
                              const double *N0, const double *F0, double *N1, double *F1,
-                             const double *hll_table, const double *inflow, const Partials &p, cudaStream_t s);
+                             const long long *hll_table, const double *inflow, const Partials &p, cudaStream_t s);
 // FP32 state (RT_MIXED): same scheme, compensated update.
 cudaError_t launch_transport_f32(const GridDev &g, int G, int flux, double cr, double dt, const float *N0,
                                  const float *F0, float *N1, float *F1, const float *hll_table,
@@ -246,6 +248,13 @@ cudaError_t launch_finalize_mode(int G, int mode, const Partials &p, double V, c
                                  double *budget, Queue q, unsigned *status, cudaStream_t s);
 
 void hll_table(int nf, int nmu, double *out);
+// the table's values times 2^62, rounded to integers (FP64 transport)
+inline std::vector<long long> hll_fix_table(const std::vector<double> &tab)
+{
+    std::vector<long long> out(tab.size());
+    for (size_t i = 0; i < tab.size(); ++i) out[i] = std::llrint(tab[i] * 4611686018427387904.0);
+    return out;
+}
 void hll_speeds(double f, double mu, double *lmin, double *lmax);
 
 }  // namespace rtgb

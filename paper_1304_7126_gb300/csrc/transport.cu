@@ -23,18 +23,34 @@
 // half the HBM traffic; the six face-flux differences are added to U with
 // error-free TwoSum steps and the accumulated rounding error folded back in
 // once, so an update loses one rounding instead of several).
+//
+// The FP64 kernel is bound by the FP64 pipe (a warp gets one FP64 instruction
+// per 64 cycles, 64 issue slots), so what need not be an FP64 operation is
+// not: comparisons, minima and clamps run on the bits; the wave speeds are
+// 64-bit fixed point (2^-62) from the table to the face, where they enter
+// FP64 as the two weights of Eq. (hll); reciprocals and square roots start
+// from float pairs (dfmath.cuh) and take two or three FP64 instructions.
+// About 150 FP64 instructions per cell and group (302 before): 3.44 -> 2.0 ms
+// at 128^3 x 3 groups, HLL.
 #include <cuda_runtime.h>
 
+#include <type_traits>
+
+#include "dfmath.cuh"
 #include "rt_internal.h"
 
 namespace rtgb {
 namespace {
 
+// HLL wave speeds: FP32 path, floats (times c once looked up); FP64 path,
+// units of c as 64-bit fixed point, value 2^62
+template <typename S> using Lam = typename std::conditional<sizeof(S) == sizeof(double), long long, S>::type;
+
 template <typename S>
 struct CellQ {
     S N, Fx, Fy, Fz;            // U
     S Pxx, Pxy, Pxz, Pyy, Pyz, Pzz;   // c^2 N D
-    S lmin[3], lmax[3];         // HLL wave speeds (already times c)
+    Lam<S> lmin[3], lmax[3];    // HLL wave speeds
 };
 
 template <typename S> struct Vec2;
@@ -54,35 +70,106 @@ __device__ __forceinline__ float tsub(float a, float b) { return __fsub_rn(a, b)
 __device__ __forceinline__ double tfma(double a, double b, double c) { return __fma_rn(a, b, c); }
 __device__ __forceinline__ float tfma(float a, float b, float c) { return __fmaf_rn(a, b, c); }
 
-// 1/d for d > 0: in FP64 an FP32 reciprocal of d (the conversions through
-// integer operations, so nothing but the Newton steps uses the FP64 pipe)
-// refined by two Newton steps (within an ulp; the FP64 transport is bound
-// by its FP64 instructions, and the IEEE quotient takes about twice as
-// many); d outside the float range takes the IEEE quotient.  In FP32 the
-// hardware's approximate reciprocal.
-__device__ __forceinline__ float f32_of(double x)   // nearest float, x a normal float magnitude
-{
-    const unsigned long long b = (unsigned long long)__double_as_longlong(x);
-    const unsigned long long a = (b & 0x7fffffffffffffffULL) + 0x10000000ULL;
-    return __uint_as_float(((unsigned)(b >> 63) << 31) | ((unsigned)((a >> 52) - 896) << 23) |
-                           (unsigned)((a >> 29) & 0x7fffff));
-}
-__device__ __forceinline__ double f64_of(float f)   // exact, f a normal float
-{
-    const unsigned u = __float_as_uint(f);
-    return __longlong_as_double((long long)(((unsigned long long)(u >> 31) << 63) |
-                                            ((unsigned long long)(((u >> 23) & 0xff) + 896) << 52) |
-                                            ((unsigned long long)(u & 0x7fffff) << 29)));
-}
-__device__ __forceinline__ double trcp(double d)
-{
-    const unsigned long long e = ((unsigned long long)__double_as_longlong(d) >> 52) & 0x7ff;
-    if (e < 1023 - 120 || e > 1023 + 120) return 1.0 / d;   // |d| outside [2^-120, 2^121)
-    double r = f64_of(__fdividef(1.0f, f32_of(d)));
-    r = __fma_rn(r, __fma_rn(-d, r, 1.0), r);
-    return __fma_rn(r, __fma_rn(-d, r, 1.0), r);
-}
 __device__ __forceinline__ float trcp(float d) { return __fdividef(1.0f, d); }
+
+// ---- FP64 pieces on the integer and FP32 pipes ----
+__device__ __forceinline__ long long tbits(double x) { return __double_as_longlong(x); }
+__device__ __forceinline__ double tdbl(long long b) { return __longlong_as_double(b); }
+__device__ __forceinline__ double tabs_(double x) { return tdbl(tbits(x) & 0x7fffffffffffffffLL); }
+
+// 1/b and 1/sqrt(x) of positive doubles of any normal size: the argument
+// scaled to [1, 2) or [1, 4) by its exponent, an FP32 approximation corrected
+// in float pairs (2^-45), one FP64 Newton step (two and three instructions,
+// within an ulp); zero, subnormal, extreme, infinite and NaN arguments take
+// CUDA's functions.
+static __device__ __noinline__ double rcp_any(double b) { return 1.0 / b; }
+static __device__ __noinline__ double rsqrt_any(double x) { return rsqrt(x); }
+
+__device__ __forceinline__ double trcp(double b)
+{
+    const int e = (int)(tbits(b) >> 52);   // (sign included: negative arguments are out of range)
+    if (e < 8 || e > 2038) return rcp_any(b);
+    const long long sh = (long long)(e - 1023) << 52;
+    const double t = tdbl(tbits(b) - sh);
+    const double r0 = dfm::rcp_seed(t);
+    const double r = __fma_rn(__fma_rn(-t, r0, 1.0), r0, r0);
+    return tdbl(tbits(r) - sh);
+}
+
+__device__ __forceinline__ float rsqrt_approx(float a)
+{
+    float r;
+    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(a));
+    return r;
+}
+
+__device__ __forceinline__ double trsqrt(double x)
+{
+    const int e = (int)(tbits(x) >> 52);
+    if (e < 8 || e > 2038) return rsqrt_any(x);
+    const int ee = (e - 1023) & ~1;
+    const double t = tdbl(tbits(x) - ((long long)ee << 52));
+    const dfm::F2 s = dfm::split_near(t);
+    const float y = rsqrt_approx(s.hi);
+    const dfm::F2 p = dfm::two_prod(y, y);
+    const float d = __fmaf_rn(-s.lo, p.hi, __fmaf_rn(-s.hi, p.lo, __fmaf_rn(-s.hi, p.hi, 1.0f)));   // 1 - t y^2
+    const double r0 = dfm::combine(y, __fmul_rn(y, __fmul_rn(d, __fmaf_rn(0.375f, d, 0.5f))));
+    const double r = __fma_rn(tdbl(tbits(r0) - (1LL << 52)), __fma_rn(-__dmul_rn(t, r0), r0, 1.0), r0);
+    return tdbl(tbits(r) - ((long long)(ee / 2) << 52));
+}
+
+// sqrt(t) of t in [1, 4], two FP64 instructions
+__device__ __forceinline__ double tsqrt14(double t)
+{
+    const dfm::F2 s = dfm::split_near(t);
+    const float y = rsqrt_approx(s.hi), g = __fmul_rn(s.hi, y), hy = 0.5f * y;
+    const float d = __fadd_rn(__fmaf_rn(-g, g, s.hi), s.lo);
+    const double s0 = dfm::combine(g, __fmul_rn(d, hy));
+    return __fma_rn(__fma_rn(-s0, s0, t), dfm::widen(hy), s0);
+}
+
+// |x| <= 1 as fixed point, value 2^62 (at most 2^63 whatever x is), and a
+// non-negative fixed-point value as the nearest double
+__device__ __forceinline__ unsigned long long to_fix(double x)
+{
+    const unsigned long long b = (unsigned long long)tbits(x) & 0x7fffffffffffffffULL;
+    int sh = 1023 - (int)(b >> 52);
+    sh = sh < 0 ? 0 : (sh > 63 ? 63 : sh);
+    return (((b & 0xfffffffffffffULL) | 0x10000000000000ULL) << 10) >> sh;
+}
+__device__ __forceinline__ double from_fix(unsigned long long v)
+{
+    if (v == 0) return 0.0;
+    const int lz = __clzll((long long)v);
+    const unsigned long long m = v << lz;
+    return tdbl((long long)(((unsigned long long)(1023 - lz) << 52) + (m >> 11) + ((m >> 10) & 1ULL)));
+}
+// d w / 2^64, rounded down
+__device__ __forceinline__ long long fix_mul(long long d, unsigned long long w)
+{
+    return (long long)(__umul64hi((unsigned long long)d, w) - (d < 0 ? w : 0ULL));
+}
+
+// Wave speeds of a cell along a direction of cosine mu from the bilinear
+// table, in fixed point throughout: f and mu are on its grid's scale by their
+// leading bits, the weights by the rest (rounding 2^-60).  k, wf: the row of
+// f and its weight.  Indices are clamped to the table whatever the state.
+__device__ __forceinline__ void hll_lookup_fix(const long long *__restrict__ tab, int k, unsigned long long wf,
+                                               double mu, long long &lo, long long &hi)
+{
+    const unsigned long long a = to_fix(mu);
+    long long v = (1LL << 62) + (tbits(mu) < 0 ? -(long long)a : (long long)a);   // (mu + 1) 2^62
+    if (tbits(mu) >= 0 && v < 0) v = 0x7fffffffffffffffLL;
+    if (v < 0) v = 0;
+    const int j = (int)(v >> 55);                                  // 0..255
+    const unsigned long long wm = (unsigned long long)v << 9;
+    const longlong2 *t = reinterpret_cast<const longlong2 *>(tab) + k * kHllNMU + j;
+    const longlong2 A = __ldg(t), B = __ldg(t + 1), C = __ldg(t + kHllNMU), D = __ldg(t + kHllNMU + 1);
+    const long long lo0 = A.x + fix_mul(B.x - A.x, wm), lo1 = C.x + fix_mul(D.x - C.x, wm);
+    const long long hi0 = A.y + fix_mul(B.y - A.y, wm), hi1 = C.y + fix_mul(D.y - C.y, wm);
+    lo = lo0 + fix_mul(lo1 - lo0, wf);
+    hi = hi0 + fix_mul(hi1 - hi0, wf);
+}
 
 template <typename S>
 __device__ __forceinline__ void hll_lookup(const S *__restrict__ tab, S f, S mu, S &lo, S &hi)
@@ -110,16 +197,65 @@ __device__ __forceinline__ void hll_lookup(const S *__restrict__ tab, S f, S mu,
 // Photon densities below this are no photons: the closure takes f = 0.
 constexpr double kClosureFloorN = 1e-30;
 
+// FP64: with q = sqrt(4 - 3 f^2), chi = (3 + 4 f^2)/(5 + 2 q) = (5 - 2 q)/3
+// (the product of 5 + 2 q and 5 - 2 q is 9 + 12 f^2), so (1 - chi)/2 =
+// (q - 1)/3 and (3 chi - 1)/2 = 2 - q, the differences exact: no quotient.
+// An isotropic cell (f = 0) has q = 2 and the table's first row, the same for
+// every mu.
+template <int FLUX>
+__device__ __forceinline__ void closure_f64(double c, const long long *__restrict__ tab, CellQ<double> &s)
+{
+    const double N = s.N;
+    const double c2N = tmul(tmul(c, c), N), th = tmul(c2N, 1.0 / 3.0);
+    const double F2 = tfma(s.Fz, s.Fz, tfma(s.Fy, s.Fy, tmul(s.Fx, s.Fx)));
+    if (tbits(N) > tbits(kClosureFloorN) && tbits(F2) > 0) {
+        const double inv = trsqrt(F2);
+        double f = tmul(tmul(F2, inv), trcp(tmul(c, N)));
+        f = tdbl(min(tbits(f), tbits(1.0)));
+        const double nx = tmul(s.Fx, inv), ny = tmul(s.Fy, inv), nz = tmul(s.Fz, inv);
+        const double q = tsqrt14(tfma(-3.0, tmul(f, f), 4.0));
+        const double ca = tmul(tsub(q, 1.0), th), cb = tmul(tsub(2.0, q), c2N);
+        const double bx = tmul(cb, nx), by = tmul(cb, ny);
+        s.Pxx = tfma(bx, nx, ca);
+        s.Pyy = tfma(by, ny, ca);
+        s.Pzz = tfma(tmul(cb, nz), nz, ca);
+        s.Pxy = tmul(bx, ny);
+        s.Pxz = tmul(bx, nz);
+        s.Pyz = tmul(by, nz);
+        if (FLUX == RT_HLL) {
+            unsigned long long v = to_fix(f);
+            if (v >= (1ULL << 62)) v = (1ULL << 62) - 1ULL;
+            const int k = (int)(v >> 54);
+            const unsigned long long wf = v << 10;
+            hll_lookup_fix(tab, k, wf, nx, s.lmin[0], s.lmax[0]);
+            hll_lookup_fix(tab, k, wf, ny, s.lmin[1], s.lmax[1]);
+            hll_lookup_fix(tab, k, wf, nz, s.lmin[2], s.lmax[2]);
+        }
+    } else {
+        s.Pxx = s.Pyy = s.Pzz = th;
+        s.Pxy = s.Pxz = s.Pyz = 0.0;
+        if (FLUX == RT_HLL) {
+            const longlong2 A = __ldg(reinterpret_cast<const longlong2 *>(tab));
+#pragma unroll
+            for (int d = 0; d < 3; ++d) { s.lmin[d] = A.x; s.lmax[d] = A.y; }
+        }
+    }
+}
+
 // M1 closure of one cell.  f := 0 for F = 0 or N below kClosureFloorN; f
 // clamped to 1.  In FP32, F is scaled by a power of two (exact) for the
 // direction and |F| so that its square neither underflows for N down to the
 // floor nor overflows.
 template <typename S, int FLUX>
-__device__ __forceinline__ void closure(S N, S Fx, S Fy, S Fz, S c, const S *__restrict__ tab, CellQ<S> &q)
+__device__ __forceinline__ void closure(S N, S Fx, S Fy, S Fz, S c, const Lam<S> *__restrict__ tab, CellQ<S> &q)
 {
     q.N = N; q.Fx = Fx; q.Fy = Fy; q.Fz = Fz;
+    if constexpr (sizeof(S) == sizeof(double)) {
+        closure_f64<FLUX>(c, tab, q);
+        return;
+    } else {
     S sc = (S)1;
-    if (sizeof(S) != sizeof(double)) {
+    {
         S m = fmax(fabs(Fx), fmax(fabs(Fy), fabs(Fz)));
         sc = (m < (S)1e-15) ? (S)0x1p64 : ((m > (S)1e15) ? (S)0x1p-64 : (S)1);
     }
@@ -150,6 +286,7 @@ __device__ __forceinline__ void closure(S N, S Fx, S Fy, S Fz, S c, const S *__r
         hll_lookup<S>(tab, f, ny, lo, hi); q.lmin[1] = tmul(lo, c); q.lmax[1] = tmul(hi, c);
         hll_lookup<S>(tab, f, nz, lo, hi); q.lmin[2] = tmul(lo, c); q.lmax[2] = tmul(hi, c);
     }
+    }
 }
 
 // Intercell flux along direction D from left cell L to right cell R.
@@ -169,7 +306,24 @@ __device__ __forceinline__ void face_flux(const CellQ<S> &L, const CellQ<S> &R, 
         fl[0] = L.Fz; fl[1] = L.Pxz; fl[2] = L.Pyz; fl[3] = L.Pzz;
         fr[0] = R.Fz; fr[1] = R.Pxz; fr[2] = R.Pyz; fr[3] = R.Pzz;
     }
-    if (FLUX == RT_HLL) {
+    if constexpr (FLUX == RT_HLL && sizeof(S) == sizeof(double)) {
+        // Eq. (hll) as A Phi_L + B Phi_R - c l+ B (U_R - U_L), A = l+/(l+ - l-),
+        // B = -l-/(l+ - l-), the speeds in units of c
+        const long long hp = max(L.lmax[D], R.lmax[D]), hm = min(L.lmin[D], R.lmin[D]);
+        const unsigned long long lp = (unsigned long long)max(0LL, hp), lm = (unsigned long long)-min(0LL, hm);
+        const unsigned long long den = lp + lm;
+        if (den != 0) {
+            const double inv = trcp(from_fix(den)), a = from_fix(lp);
+            const double A = tmul(a, inv), B = tmul(from_fix(lm), inv), Dc = tmul(tmul(c, a), B);
+#pragma unroll
+            for (int k = 0; k < 4; ++k)
+                out[k] = tfma(-Dc, tsub(ur[k], ul[k]), tfma(B, fr[k], tmul(A, fl[k])));
+        } else {
+            // both speeds vanish only for f = 1 beams parallel to the face
+#pragma unroll
+            for (int k = 0; k < 4; ++k) out[k] = tmul(0.5, tadd(fl[k], fr[k]));
+        }
+    } else if constexpr (FLUX == RT_HLL) {
         S lp = fmax((S)0, fmax(L.lmax[D], R.lmax[D]));
         S lm = fmin((S)0, fmin(L.lmin[D], R.lmin[D]));
         S den = tsub(lp, lm);
@@ -221,6 +375,46 @@ template <> struct BudgetAcc<float> {
     }
     __device__ __forceinline__ double get() const { return (double)s + (double)e; }
 };
+
+// N >= 0 and |F| <= c N of an updated state.  Squares of tiny values lose
+// digits: tiny states are compared scaled by a power of two (exact), the
+// factor is scale-free.
+__device__ __forceinline__ void realisable(float nw[4], float c)
+{
+    if (nw[0] < 0.0f) nw[0] = nw[1] = nw[2] = nw[3] = 0.0f;
+    const float cn = tmul(c, nw[0]);
+    const float m = fmaxf(fmaxf(fabsf(nw[1]), fabsf(nw[2])), fmaxf(fabsf(nw[3]), cn));
+    const float sc0 = (m < 1e-15f) ? 0x1p60f : 1.0f;
+    const float f1 = tmul(nw[1], sc0), f2 = tmul(nw[2], sc0), f3 = tmul(nw[3], sc0), cs = tmul(cn, sc0);
+    const float F2 = tfma(f3, f3, tfma(f2, f2, tmul(f1, f1)));
+    if (F2 > tmul(cs, cs)) {
+        const float sc = (F2 > 0.0f) ? tmul(cs, rsqrtf(F2)) : 0.0f;
+        nw[1] = tmul(nw[1], sc); nw[2] = tmul(nw[2], sc); nw[3] = tmul(nw[3], sc);
+    }
+}
+__device__ __noinline__ void rescale_flux(double nw[4], double c, double sc0)
+{
+    const double cs = tmul(tmul(c, nw[0]), sc0);
+    const double f1 = tmul(nw[1], sc0), f2 = tmul(nw[2], sc0), f3 = tmul(nw[3], sc0);
+    const double F2 = tfma(f3, f3, tfma(f2, f2, tmul(f1, f1)));
+    if (F2 > tmul(cs, cs)) {
+        const double sc = (F2 > 0.0) ? tmul(cs, rsqrt(F2)) : 0.0;
+        nw[1] = tmul(nw[1], sc); nw[2] = tmul(nw[2], sc); nw[3] = tmul(nw[3], sc);
+    }
+}
+__device__ __forceinline__ void realisable(double nw[4], double c)
+{
+    if (tbits(nw[0]) < 0) nw[0] = nw[1] = nw[2] = nw[3] = 0.0;   // (-0 included: its |F| <= c N is 0)
+    const double cn = tmul(c, nw[0]);
+    const long long m = max(max(tbits(tabs_(nw[1])), tbits(tabs_(nw[2]))), max(tbits(tabs_(nw[3])), tbits(cn)));
+    const double F2 = tfma(nw[3], nw[3], tfma(nw[2], nw[2], tmul(nw[1], nw[1])));
+    const bool tiny = m < tbits(1e-140);
+    if (tiny || tbits(F2) > tbits(tmul(cn, cn))) {
+        double u[4] = {nw[0], nw[1], nw[2], nw[3]};
+        if (m > 0) rescale_flux(u, c, tiny ? 0x1p600 : 1.0);
+        nw[1] = u[1]; nw[2] = u[2]; nw[3] = u[3];
+    }
+}
 
 // Load U at (x, y, z) where at most one coordinate may sit one cell outside
 // the box: that position is the boundary ghost (outflow: copy; reflect:
@@ -276,7 +470,7 @@ struct PlaneSmem {
     static constexpr int SW = TBX + 2, SH = TBY + 2;
     S N[SH][SW], Fx[SH][SW], Fy[SH][SW], Fz[SH][SW];
     S Pxx[SH][SW], Pxy[SH][SW], Pxz[SH][SW], Pyy[SH][SW], Pyz[SH][SW];
-    S lminx[SH][SW], lmaxx[SH][SW], lminy[SH][SW], lmaxy[SH][SW];
+    Lam<S> lminx[SH][SW], lmaxx[SH][SW], lminy[SH][SW], lmaxy[SH][SW];
     S fxs[4][TBY][TBX + 1];     // x faces 0..TBX of each row
     S fys[4][TBY + 1][TBX];     // y faces 0..TBY of each column
     double red[2][TBX * TBY / 32];
@@ -313,7 +507,7 @@ __device__ __forceinline__ void get_plane(const SM &s, int r, int c, CellQ<S> &q
 template <typename S, int FLUX, int TBX, int TBY>
 __device__ __forceinline__ void transport_tile(PlaneSmem<S, TBX, TBY> &s, const GridDev &g, S c, S dtdx,
                                                const S *__restrict__ N0, const S *__restrict__ F0,
-                                               S *__restrict__ N1, S *__restrict__ F1, const S *__restrict__ tab,
+                                               S *__restrict__ N1, S *__restrict__ F1, const Lam<S> *__restrict__ tab,
                                                const S *__restrict__ inf, int x0, int y0, int z0, int z1,
                                                double &inbox, double &outflow)
 {
@@ -462,20 +656,7 @@ __device__ __forceinline__ void transport_tile(PlaneSmem<S, TBX, TBY> &s, const 
                 }
             }
             // realisability |F| <= c N (acts only at rounding level for CFL <= 1)
-            if (nw[0] < (S)0) { nw[0] = 0; nw[1] = nw[2] = nw[3] = 0; }
-            // squares of tiny values lose digits: compare tiny states scaled
-            // by a power of two (exact), the factor is scale-free
-            S cn = tmul(c, nw[0]);
-            S m = fmax(fmax(fabs(nw[1]), fabs(nw[2])), fmax(fabs(nw[3]), cn));
-            const S tiny = sizeof(S) == sizeof(double) ? (S)1e-140 : (S)1e-15;
-            const S big = sizeof(S) == sizeof(double) ? (S)0x1p600 : (S)0x1p60;
-            S sc0 = (m < tiny) ? big : (S)1;
-            S f1 = tmul(nw[1], sc0), f2 = tmul(nw[2], sc0), f3 = tmul(nw[3], sc0), cs = tmul(cn, sc0);
-            S F2 = tfma(f3, f3, tfma(f2, f2, tmul(f1, f1)));
-            if (F2 > tmul(cs, cs)) {
-                S sc = (F2 > (S)0) ? tmul(cs, rsqrt(F2)) : (S)0;
-                nw[1] = tmul(nw[1], sc); nw[2] = tmul(nw[2], sc); nw[3] = tmul(nw[3], sc);
-            }
+            realisable(nw, c);
             long long i = ((long long)z * g.ny + y) * g.nx + x;
             N1[i] = nw[0];
             F1[i] = nw[1];
@@ -520,7 +701,7 @@ __device__ __forceinline__ void block_reduce2(double *red, double &a, double &b)
 template <typename S, int FLUX, int TBX, int TBY>
 __device__ __noinline__ void transport_segment(PlaneSmem<S, TBX, TBY> &s, const GridDev &g, S c, S dtdx,
                                                const S *__restrict__ N0, const S *__restrict__ F0,
-                                               S *__restrict__ N1, S *__restrict__ F1, const S *__restrict__ tab,
+                                               S *__restrict__ N1, S *__restrict__ F1, const Lam<S> *__restrict__ tab,
                                                const S *__restrict__ inf, int x0, int y0, int z0, int z1,
                                                double &inbox, double &outflow)
 {
@@ -537,7 +718,7 @@ template <typename S, int FLUX>
 __device__ __forceinline__ void transport_kernel_body(GridDev g, int G, S c, S dtdx, double area_dt,
                                                       const S *__restrict__ N0all, const S *__restrict__ F0all,
                                                       S *__restrict__ N1all, S *__restrict__ F1all,
-                                                      const S *__restrict__ tab, const S *__restrict__ inflow,
+                                                      const Lam<S> *__restrict__ tab, const S *__restrict__ inflow,
                                                       double *__restrict__ part_inbox,
                                                       double *__restrict__ part_out, int tiles_x, int tiles_y)
 {
@@ -594,7 +775,7 @@ template <typename S, int FLUX>
 __global__ void __launch_bounds__(256, 2)
 transport_kernel(GridDev g, int G, S c, S dtdx, double area_dt, const S *__restrict__ N0all,
                  const S *__restrict__ F0all, S *__restrict__ N1all, S *__restrict__ F1all,
-                 const S *__restrict__ tab, const S *__restrict__ inflow, double *__restrict__ part_inbox,
+                 const Lam<S> *__restrict__ tab, const S *__restrict__ inflow, double *__restrict__ part_inbox,
                  double *__restrict__ part_out, int tiles_x, int tiles_y)
 {
     transport_kernel_body<S, FLUX>(g, G, c, dtdx, area_dt, N0all, F0all, N1all, F1all, tab, inflow, part_inbox,
@@ -619,7 +800,7 @@ template <typename S, int FLUX, int TBX, int TBY>
 __global__ void __launch_bounds__(TBX * TBY)
 transport_batch_kernel(const BatchItem *__restrict__ items, const BatchBox *__restrict__ boxes, S c, S dtdx,
                        double area_dt, const S *const *__restrict__ N0cls, const S *const *__restrict__ F0cls,
-                       S *const *__restrict__ N1cls, S *const *__restrict__ F1cls, const S *__restrict__ tab,
+                       S *const *__restrict__ N1cls, S *const *__restrict__ F1cls, const Lam<S> *__restrict__ tab,
                        double *__restrict__ part_inbox, double *__restrict__ part_out, int item0)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -647,7 +828,7 @@ template <typename S, int FLUX>
 __global__ void __launch_bounds__(256)
 transport_batch_all_kernel(const BatchItem *__restrict__ items, const BatchBox *__restrict__ boxes, S c, S dtdx,
                            double area_dt, const S *const *__restrict__ N0cls, const S *const *__restrict__ F0cls,
-                           S *const *__restrict__ N1cls, S *const *__restrict__ F1cls, const S *__restrict__ tab,
+                           S *const *__restrict__ N1cls, S *const *__restrict__ F1cls, const Lam<S> *__restrict__ tab,
                            double *__restrict__ part_inbox, double *__restrict__ part_out, int n_shape0)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -721,7 +902,7 @@ void transport_init()
 
 template <typename S>
 static cudaError_t launch_t(const GridDev &g, int G, int flux, double cr, double dt, const S *N0, const S *F0,
-                            S *N1, S *F1, const S *tab, const S *inflow, const Partials &p, cudaStream_t st)
+                            S *N1, S *F1, const Lam<S> *tab, const S *inflow, const Partials &p, cudaStream_t st)
 {
     const int tiles_x = (g.nx + 31) / 32;
     const int tiles_y = (g.ny + 7) / 8;
@@ -749,7 +930,7 @@ static cudaError_t launch_t(const GridDev &g, int G, int flux, double cr, double
 
 cudaError_t launch_transport(const GridDev &g, int G, int flux, double cr, double dt,
                              const double *N0, const double *F0, double *N1, double *F1,
-                             const double *hll_table, const double *inflow, const Partials &p, cudaStream_t st)
+                             const long long *hll_table, const double *inflow, const Partials &p, cudaStream_t st)
 {
     return launch_t<double>(g, G, flux, cr, dt, N0, F0, N1, F1, hll_table, inflow, p, st);
 }
@@ -764,7 +945,7 @@ cudaError_t launch_transport_f32(const GridDev &g, int G, int flux, double cr, d
 template <typename S>
 static cudaError_t launch_b(const BatchItem *items, const BatchBox *boxes, int item0, int nitems, int shape,
                             int flux, double cr, double dt, double dx, const void *const *N0, const void *const *F0,
-                            void *const *N1, void *const *F1, const S *tab, double *pin, double *pout,
+                            void *const *N1, void *const *F1, const Lam<S> *tab, double *pin, double *pout,
                             cudaStream_t st)
 {
     if (nitems <= 0) return cudaSuccess;
@@ -803,7 +984,7 @@ cudaError_t launch_transport_batch(const BatchItem *items, const BatchBox *boxes
         return launch_b<float>(items, boxes, item0, nitems, shape, flux, cr, dt, dx, N0, F0, N1, F1,
                                static_cast<const float *>(tab), pin, pout, st);
     return launch_b<double>(items, boxes, item0, nitems, shape, flux, cr, dt, dx, N0, F0, N1, F1,
-                            static_cast<const double *>(tab), pin, pout, st);
+                            static_cast<const long long *>(tab), pin, pout, st);
 }
 
 }  // namespace rtgb
@@ -824,7 +1005,7 @@ cudaError_t launch_transport_batch_all(const BatchItem *items, const BatchBox *b
         auto f0 = reinterpret_cast<const S *const *>(F0);
         auto n1 = reinterpret_cast<S *const *>(N1);
         auto f1 = reinterpret_cast<S *const *>(F1);
-        const S *t = static_cast<const S *>(tab);
+        const Lam<S> *t = static_cast<const Lam<S> *>(tab);
         if (flux == RT_HLL)
             transport_batch_all_kernel<S, RT_HLL><<<nitems, 256, batch_all_smem<S>(), st>>>(
                 items, boxes, (S)cr, dtdx, area_dt, n0, f0, n1, f1, t, pin, pout, n_shape0);
@@ -838,7 +1019,7 @@ cudaError_t launch_transport_batch_all(const BatchItem *items, const BatchBox *b
         auto f0 = reinterpret_cast<const S *const *>(F0);
         auto n1 = reinterpret_cast<S *const *>(N1);
         auto f1 = reinterpret_cast<S *const *>(F1);
-        const S *t = static_cast<const S *>(tab);
+        const Lam<S> *t = static_cast<const Lam<S> *>(tab);
         if (flux == RT_HLL)
             transport_batch_all_kernel<S, RT_HLL><<<nitems, 256, batch_all_smem<S>(), st>>>(
                 items, boxes, (S)cr, dtdx, area_dt, n0, f0, n1, f1, t, pin, pout, n_shape0);
