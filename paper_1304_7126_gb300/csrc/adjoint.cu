@@ -105,9 +105,10 @@ thermo_vjp_kernel(ThermoParams p, const double *__restrict__ nH, const double *_
     cc.rvalid = false;
     if (p.isothermal) {
         TLevel L;
-        t_level(st.T.v, L);
-        h_rates<8, false>(L, st.T.d, p.case_b, iso.h);
-        if (p.helium) he_rates<8, false>(L, st.T.d, p.case_b, iso.he);
+        dfm::Exact e;
+        t_level(st.T.v, L, e);
+        h_rates<8, false>(L, st.T.d, p.case_b, iso.h, e);
+        if (p.helium) he_rates<8, false>(L, st.T.d, p.case_b, iso.he, e);
     }
     double t_left = p.dt, dt_tc = p.dt;
     int att = 0;

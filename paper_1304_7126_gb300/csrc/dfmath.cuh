@@ -194,6 +194,34 @@ __device__ __forceinline__ double to_double_i(F2 a, int m = 0)
     return __longlong_as_double(neg ? r | (1LL << 63) : r);   // (a negation may take the FP64 pipe)
 }
 
+// Two ways to deal with arguments outside an operation's range.  Exact: a
+// branch to the general form there.  Fast: no branch; `odd` is set and the
+// value is of no use, and the caller repeats the whole computation the exact
+// way (the team kernel's attempts, a single basic block that the compiler
+// can interleave).  In range both give the same bits.
+struct Exact {
+    static constexpr bool fast = false;
+};
+struct Fast {
+    static constexpr bool fast = true;
+    bool odd = false, reject = false;
+};
+
+template <class CTL>
+__device__ __forceinline__ double to_double_c(F2 a, int m, CTL &ctl)
+{
+    if constexpr (!CTL::fast) {
+        return to_double_i(a, m);
+    } else {
+        const float h = fabsf(a.hi);
+        const bool neg = a.hi < 0.0f, in = h > 0x1p-70f && h < 0x1p120f;
+        ctl.odd |= !in && a.hi != 0.0f;   // (a NaN compares unequal)
+        const int e = (int)(__float_as_uint(h) >> 23) - 127 + m;
+        const long long r = __double_as_longlong(combine(in ? h : 1.0f, neg ? -a.lo : a.lo, m));
+        return __longlong_as_double(!in || e < -1020 ? 0LL : neg ? r | (1LL << 63) : r);
+    }
+}
+
 // ---- reciprocal and quotient of doubles ----
 // The IEEE quotient takes some nine FP64 instructions, and a warp issues one
 // per 64 cycles.  Here the reciprocal of the divisor comes from float pairs
@@ -250,6 +278,30 @@ __device__ __forceinline__ double fast_div(double a, double b)
     const double r = rcp_seed(b);
     const double q = __dmul_rn(a, r);
     return __fma_rn(__fma_rn(-q, b, a), r, q);
+}
+
+template <class CTL>
+__device__ __forceinline__ double rcp_c(double b, CTL &ctl)
+{
+    if constexpr (!CTL::fast) {
+        return fast_rcp(b);
+    } else {
+        ctl.odd |= !div_range(b);
+        const double r = rcp_seed(b);
+        return __fma_rn(__fma_rn(-b, r, 1.0), r, r);
+    }
+}
+template <class CTL>
+__device__ __forceinline__ double div_c(double a, double b, CTL &ctl)
+{
+    if constexpr (!CTL::fast) {
+        return fast_div(a, b);
+    } else {
+        ctl.odd |= !div_range(b);
+        const double r = rcp_seed(b);
+        const double q = __dmul_rn(a, r);
+        return __fma_rn(__fma_rn(-q, b, a), r, q);
+    }
 }
 
 // a double as the nearest float on the integer pipe: 0 below the normal
@@ -447,11 +499,15 @@ static __device__ __noinline__ F2 softplus_far(F2 z, F2 &sig)
 // ~1e-14 at |z| ~ 16, that of the pair coefficients).  80 instructions; 250
 // with 1/4-wide intervals and degree 9.  Outside (temperatures far beyond
 // the fits' range) from e^z and log1p.
-__device__ __forceinline__ F2 softplus2(F2 z, F2 &sig)
+template <class CTL>
+__device__ __forceinline__ F2 softplus2(F2 z, F2 &sig, CTL &ctl)
 {
-    if (z.hi >= (float)kDfSpLo && z.hi < -(float)kDfSpLo) {
+    const bool in = z.hi >= (float)kDfSpLo && z.hi < -(float)kDfSpLo;
+    if constexpr (CTL::fast) ctl.odd |= !in;
+    if (CTL::fast || in) {
         int k = (int)__fmul_rn(__fadd_rn(z.hi, -(float)kDfSpLo), (float)kDfSpPer);
         k = k < kDfSpN - 1 ? k : kDfSpN - 1;
+        if (CTL::fast) k = k < 0 ? 0 : k;
         const float mid = (float)kDfSpLo + ((float)k + 0.5f) / (float)kDfSpPer;   // exact
         const F2 t0 = two_sum(z.hi, -mid);
         const F2 t = fast_two_sum(t0.hi, __fadd_rn(t0.lo, z.lo));
@@ -474,6 +530,11 @@ __device__ __forceinline__ F2 softplus2(F2 z, F2 &sig)
         return norm(P);
     }
     return softplus_far(z, sig);
+}
+__device__ __forceinline__ F2 softplus2(F2 z, F2 &sig)
+{
+    Exact e;
+    return softplus2(z, sig, e);
 }
 
 }  // namespace dfm

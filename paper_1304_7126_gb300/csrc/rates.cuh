@@ -264,10 +264,17 @@ static __device__ const int g_cool_sp[16] = {SP_HI, SP_HI, SP_HII, SP_FF, SP_HEI
 struct TLevel {
     dfm::F2 lnT, invT;
 };
-__device__ __forceinline__ void t_level(double T, TLevel &L)
+// (the logarithm inline on the fast path)
+template <class CTL>
+__device__ __forceinline__ void t_level(double T, TLevel &L, CTL &ctl)
 {
     using namespace dfm;
-    if (!(T > 0.0) || !splittable(T)) {   // not reached by T >= 1 K below 2^60 K
+    if constexpr (CTL::fast) {
+        ctl.odd |= !(T > 0.0) || !splittable(T);
+        const F2 T2 = split(T);
+        L.lnT = log2f2_inl(T2, kLnTRef);
+        L.invT = rcp(T2);
+    } else if (!(T > 0.0) || !splittable(T)) {   // not reached by T >= 1 K below 2^60 K
         L.lnT = split_any(log(T) - kLnTRefV);
         L.invT = split_any(1.0 / T);
     } else {
@@ -277,12 +284,20 @@ __device__ __forceinline__ void t_level(double T, TLevel &L)
     }
 }
 // the same from 1/T as a pair
-__device__ __forceinline__ void t_level_inv(dfm::F2 invT, TLevel &L)
+template <class CTL>
+__device__ __forceinline__ void t_level_inv(dfm::F2 invT, TLevel &L, CTL &ctl)
 {
     using namespace dfm;
     L.invT = invT;
-    if (invT.hi > 0x1p-60f && invT.hi < 0x1p60f) L.lnT = neg(log2f2(invT, -kLnTRef));
-    else L.lnT = split_any(-log(to_double(invT)) - kLnTRefV);
+    const bool in = invT.hi > 0x1p-60f && invT.hi < 0x1p60f;
+    if constexpr (CTL::fast) {
+        ctl.odd |= !in;
+        L.lnT = neg(log2f2_inl(in ? invT : F2{1.0f, 0.0f}, -kLnTRef));
+    } else if (in) {
+        L.lnT = neg(log2f2(invT, -kLnTRef));
+    } else {
+        L.lnT = split_any(-log(to_double(invT)) - kLnTRefV);
+    }
 }
 
 // A function value y 2^m (y a normalised pair below 8, or 0), as pairs
@@ -326,8 +341,8 @@ constexpr unsigned kC1Zero = rf_zero_mask(kZeroC1), kC2Zero = rf_zero_mask(kZero
 // softplus(z) and sigma(z) of one function, z = c4 ln(T / 2^14 K) + c5r.  MIX (the
 // mixed-precision thermochemistry, RT_MIXED32): z still in pairs, but the
 // correction ln(1 + e^-|z|) < ln 2 and sigma in FP32.
-template <bool MIX>
-__device__ __forceinline__ dfm::F2 rate_softplus(const RateFn &q, const TLevel &L, dfm::F2 &sig)
+template <bool MIX, class CTL>
+__device__ __forceinline__ dfm::F2 rate_softplus(const RateFn &q, const TLevel &L, dfm::F2 &sig, CTL &ctl)
 {
     using namespace dfm;
     const F2 z = norm(addu(mulu(L.lnT, q.c4), q.c5r));
@@ -336,8 +351,15 @@ __device__ __forceinline__ dfm::F2 rate_softplus(const RateFn &q, const TLevel &
         sig = F2{(z.hi >= 0.0f ? 1.0f : e) / (1.0f + e), 0.0f};
         return add(z.hi >= 0.0f ? z : F2{0.0f, 0.0f}, log1pf(e));   // max(z, 0) + ln(1 + e^-|z|)
     } else {
-        return softplus2(z, sig);
+        return softplus2(z, sig, ctl);
     }
+}
+
+template <bool MIX>
+__device__ __forceinline__ dfm::F2 rate_softplus(const RateFn &q, const TLevel &L, dfm::F2 &sig)
+{
+    dfm::Exact e;
+    return rate_softplus<MIX>(q, L, sig, e);
 }
 
 // One function from l = softplus(z) and sigma(z).  The argument of the
@@ -383,12 +405,20 @@ __device__ __forceinline__ void rate_val(const RateFn &q, const TLevel &L, dfm::
         }
     }
 }
+template <class CTL>
+__device__ __forceinline__ double rate_f(const RateVal &r, CTL &ctl) { return dfm::to_double_c(r.y, r.m, ctl); }
 __device__ __forceinline__ double rate_f(const RateVal &r) { return dfm::to_double_i(r.y, r.m); }
 // df/dT = f g / T
-__device__ __forceinline__ double rate_df(const RateVal &r, const TLevel &L)
+template <class CTL>
+__device__ __forceinline__ double rate_df(const RateVal &r, const TLevel &L, CTL &ctl)
 {
     using namespace dfm;
-    return to_double_i(norm(mulu(r.y, mulu(r.g, L.invT))), r.m);
+    return to_double_c(norm(mulu(r.y, mulu(r.g, L.invT))), r.m, ctl);
+}
+__device__ __forceinline__ double rate_df(const RateVal &r, const TLevel &L)
+{
+    dfm::Exact e;
+    return rate_df(r, L, e);
 }
 // d2f/dT2 = f w / T^2
 __device__ __forceinline__ double rate_d2f(const RateVal &r, const TLevel &L)
@@ -469,12 +499,12 @@ template <int TS>
 __device__ __forceinline__ double team_get(unsigned m, double v, int src) { return __shfl_sync(m, v, src, TS); }
 
 // one function per lane of a team, slot k, with its own softplus
-template <bool MIX, int DERIV>
-__device__ __forceinline__ void rate_lane(int case_b, int k, const TLevel &L, RateVal &r)
+template <bool MIX, int DERIV, class CTL>
+__device__ __forceinline__ void rate_lane(int case_b, int k, const TLevel &L, RateVal &r, CTL &ctl)
 {
     const RateFn &q = g_rate_fn[case_b].f[k];
     dfm::F2 sig;
-    const dfm::F2 l = rate_softplus<MIX>(q, L, sig);
+    const dfm::F2 l = rate_softplus<MIX>(q, L, sig, ctl);
     rate_val<MIX, DERIV>(q, L, l, sig, 0u, false, r);
 }
 
@@ -537,13 +567,13 @@ static __device__ __noinline__ double2 he3_rates_serial(TLevel L, int case_b)
 }
 // ... and by a team: lanes 0 and 1 the two hydrogen functions, lanes 0..3
 // the four helium ones, each then in every lane
-template <int TS, bool MIX>
-static __device__ __noinline__ HRates h_rates_team(TLevel L, int case_b)
+template <int TS, bool MIX, class CTL>
+__device__ __forceinline__ HRates h_rates_team(const TLevel &L, int case_b, CTL &ctl)
 {
     const unsigned m = team_mask<TS>();
     RateVal v;
-    rate_lane<MIX, 1>(case_b, team_lane<TS>() == 0 ? RF_BETA_HI : RF_ALPHA_HII, L, v);
-    const double f = rate_f(v), df = rate_df(v, L);
+    rate_lane<MIX, 1>(case_b, team_lane<TS>() == 0 ? RF_BETA_HI : RF_ALPHA_HII, L, v, ctl);
+    const double f = rate_f(v, ctl), df = rate_df(v, L, ctl);
     HRates r;
     r.beta = team_get<TS>(m, f, 0);
     r.dbeta = team_get<TS>(m, df, 0);
@@ -553,13 +583,13 @@ static __device__ __noinline__ HRates h_rates_team(TLevel L, int case_b)
 }
 static_assert(RF_BETA_HEII == RF_BETA_HEI + 1 && RF_ALPHA_HEII == RF_BETA_HEI + 2 && RF_ALPHA_HEIII == RF_BETA_HEI + 3,
               "the helium functions of a team's lanes");
-template <int TS, bool MIX>
-static __device__ __noinline__ HeRates he_rates_team(TLevel L, int case_b)
+template <int TS, bool MIX, class CTL>
+__device__ __forceinline__ HeRates he_rates_team(const TLevel &L, int case_b, CTL &ctl)
 {
     const unsigned m = team_mask<TS>();
     RateVal v;
-    rate_lane<MIX, 0>(case_b, RF_BETA_HEI + (team_lane<TS>() & 3), L, v);
-    const double f = rate_f(v);
+    rate_lane<MIX, 0>(case_b, RF_BETA_HEI + (team_lane<TS>() & 3), L, v, ctl);
+    const double f = rate_f(v, ctl);
     HeRates r;
     r.beta_HeI = team_get<TS>(m, f, 0);
     r.beta_HeII = team_get<TS>(m, f, 1);
@@ -574,7 +604,8 @@ static __device__ __noinline__ HRatesT<Dual> h_rates_dual(TLevel L, double dT, i
 {
     const unsigned m = team_mask<8>();
     RateVal v;
-    rate_lane<false, 2>(case_b, team_lane<8>() == 0 ? RF_BETA_HI : RF_ALPHA_HII, L, v);
+    dfm::Exact e;
+    rate_lane<false, 2>(case_b, team_lane<8>() == 0 ? RF_BETA_HI : RF_ALPHA_HII, L, v, e);
     const double f = rate_f(v), df = rate_df(v, L), d2f = rate_d2f(v, L);
     HRatesT<Dual> r;
     const double b1 = team_get<8>(m, df, 0), a1 = team_get<8>(m, df, 1);
@@ -588,7 +619,8 @@ static __device__ __noinline__ HeRatesT<Dual> he_rates_dual(TLevel L, double dT,
 {
     const unsigned m = team_mask<8>();
     RateVal v;
-    rate_lane<false, 1>(case_b, RF_BETA_HEI + (team_lane<8>() & 3), L, v);
+    dfm::Exact e;
+    rate_lane<false, 1>(case_b, RF_BETA_HEI + (team_lane<8>() & 3), L, v, e);
     const double f = rate_f(v), df = rate_df(v, L);
     HeRatesT<Dual> r;
     r.beta_HeI = Dual(team_get<8>(m, f, 0), team_get<8>(m, df, 0) * dT);
@@ -643,6 +675,19 @@ __device__ __forceinline__ void cool_densities(const S &nHI, const S &nHII, cons
 
 // a density as a pair (below 2^-70, 1e-21 of the smallest electron density
 // that matters, as 0; 2^120 and above through the FP64 pipe)
+__device__ __forceinline__ dfm::F2 split_density(double n);
+template <class CTL>
+__device__ __forceinline__ dfm::F2 split_density(double n, CTL &ctl)
+{
+    if constexpr (CTL::fast) {
+        const unsigned h = (unsigned)((unsigned long long)__double_as_longlong(n) >> 32);
+        ctl.odd |= h >= (1143u << 20);
+        const dfm::F2 s = dfm::split_near(n);
+        return h < (953u << 20) ? dfm::F2{0.0f, 0.0f} : s;
+    } else {
+        return split_density(n);
+    }
+}
 __device__ __forceinline__ dfm::F2 split_density(double n)
 {
     const unsigned h = (unsigned)((unsigned long long)__double_as_longlong(n) >> 32);
@@ -730,7 +775,8 @@ static __device__ __noinline__ double2 cooling_sums_serial(int case_b, bool heli
                                                            double nHeI, double nHeII, double nHeIII)
 {
     TLevel Lv;
-    t_level(T, Lv);
+    dfm::Exact e;
+    t_level(T, Lv, e);
     double n[NSP], Ls, dLs;
     cool_densities(nHI, nHII, nHeI, nHeII, nHeIII, n);
     cooling_sums<MIX>(Lv, case_b, helium, n, Ls, dLs);
@@ -751,22 +797,22 @@ __device__ __forceinline__ dfm::F2 team_add(unsigned mask, dfm::F2 a, int m)
 {
     return dfm::addu(a, dfm::F2{__shfl_xor_sync(mask, a.hi, m), __shfl_xor_sync(mask, a.lo, m)});
 }
-template <bool MIX>
-static __device__ __noinline__ double2 cooling_sums_team4(int case_b, bool helium, double T, double nHI, double nHII,
-                                                          double nHeI, double nHeII, double nHeIII)
+template <bool MIX, class CTL>
+__device__ __forceinline__ double2 cooling_sums_team4(int case_b, bool helium, double T, double nHI, double nHII,
+                                                          double nHeI, double nHeII, double nHeIII, CTL &ctl)
 {
     using namespace dfm;
     const unsigned mask = team_mask<4>();
     const int t = team_lane<4>();
     const RateFn *R = g_rate_fn[case_b].f;
     TLevel L;
-    t_level(T, L);
+    t_level(T, L, ctl);
     double n[NSP];
     cool_densities(nHI, nHII, nHeI, nHeII, nHeIII, n);
     // round 0: lanes 0, 1 with the softplus of u, lanes 2, 3 with their own
     F2 sig;
     const int k0 = g_cool_at[t];
-    const F2 l = rate_softplus<MIX>(R[k0], L, sig);
+    const F2 l = rate_softplus<MIX>(R[k0], L, sig, ctl);
     const F2 lu{__shfl_sync(mask, l.hi, 0, 4), __shfl_sync(mask, l.lo, 0, 4)};
     const F2 su{__shfl_sync(mask, sig.hi, 0, 4), __shfl_sync(mask, sig.lo, 0, 4)};
     F2 v[3], dv[3];
@@ -776,13 +822,13 @@ static __device__ __noinline__ double2 cooling_sums_team4(int case_b, bool heliu
         RateVal q;
         // (no softplus in round 2 nor in lane 3 of round 1: c3 = c3 c4 = 0)
         rate_val<MIX, 1>(R[k], L, r ? lu : l, r ? su : sig, r == 2 ? 1u << kZeroC3 : 0u, false, q);
-        cool_term(q, split_density(pick(n, g_cool_sp[k])), v[r], dv[r]);
+        cool_term(q, split_density(pick(n, g_cool_sp[k]), ctl), v[r], dv[r]);
         if (k >= kNCool || (!helium && (cool_mask(1) >> k & 1))) v[r] = dv[r] = F2{0.0f, 0.0f};
     }
     F2 s = addu(addu(v[0], v[2]), v[1]), ds = addu(addu(dv[0], dv[2]), dv[1]);
     s = norm(team_add(mask, team_add(mask, s, 2), 1));
     ds = norm(team_add(mask, team_add(mask, ds, 2), 1));
-    return make_double2(to_double_i(s, -kCoolExp), to_double_i(norm(mulu(ds, L.invT)), -kCoolExp));
+    return make_double2(to_double_c(s, -kCoolExp, ctl), to_double_c(norm(mulu(ds, L.invT)), -kCoolExp, ctl));
 }
 
 // dual numbers, by a team of eight (same values, a tangent per lane): places
@@ -798,7 +844,8 @@ static __device__ __noinline__ void cooling_dual(int case_b, double comp, double
     const int t = team_lane<8>();
     const RateFn *R = g_rate_fn[case_b].f;
     TLevel Lv;
-    t_level(T.v, Lv);
+    Exact e;
+    t_level(T.v, Lv, e);
     Dual n[NSP];
     cool_densities(nHI, nHII, nHeI, nHeII, nHeIII, n);
     double nv[NSP];

@@ -67,9 +67,10 @@ __device__ __forceinline__ void load_cell(const ThermoParams &p, long long c, bo
     cc.rvalid = false;
     if (p.isothermal) {
         TLevel L;
-        t_level(st.T, L);
-        h_rates<PT, R32>(L, 0.0, p.case_b, iso.h);
-        if (p.helium) he_rates<PT, R32>(L, 0.0, p.case_b, iso.he);
+        dfm::Exact e;
+        t_level(st.T, L, e);
+        h_rates<PT, R32>(L, 0.0, p.case_b, iso.h, e);
+        if (p.helium) he_rates<PT, R32>(L, 0.0, p.case_b, iso.he, e);
     }
 }
 

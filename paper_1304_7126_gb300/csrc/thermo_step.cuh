@@ -195,21 +195,28 @@ __device__ __noinline__ bool change_lt(S n, S o, S floor_, double t)
 {
     return ratio_lt(fabs(n - o), max0(o, floor_), t);
 }
-template <typename S>
-__device__ __forceinline__ bool change_ok(const S &n, const S &o, const S &floor_, bool &small)
+// (the fast path only notes what it cannot decide, and a broken limit)
+template <typename S, class CTL>
+__device__ __forceinline__ bool change_ok(const S &n, const S &o, const S &floor_, bool &small, CTL &ctl)
 {
     const float of = dfm::near_float(val(o));
     const float d = fabsf(__fsub_rn(dfm::near_float(val(n)), of));
     const float den = fmaxf(of, dfm::near_float(val(floor_)));
-    bool ok = d < 0.099999f * den;
-    if (!ok) {
-        if (d > 0.100001f * den) return false;
-        if (change_gt<S>(n, o, floor_, 0.1)) return false;
+    const bool ok = d < 0.099999f * den, bad = d > 0.100001f * den;
+    const bool sm = d < 0.049999f * den, not_sm = d > 0.050001f * den;
+    if constexpr (CTL::fast) {
+        ctl.reject |= bad;
+        ctl.odd |= !(ok || bad) || !(sm || not_sm);
+        small = small && sm;
+        return true;
+    } else {
+        if (!ok) {
+            if (bad) return false;
+            if (change_gt<S>(n, o, floor_, 0.1)) return false;
+        }
+        small = small && (sm || (!not_sm && change_lt<S>(n, o, floor_, 0.05)));
+        return true;
     }
-    bool sm = d < 0.049999f * den;
-    if (!sm && !(d > 0.050001f * den)) sm = change_lt<S>(n, o, floor_, 0.05);
-    small = small && sm;
-    return true;
 }
 // |a| > t b for a first-order term a (b > 0)
 template <typename S>
@@ -222,42 +229,44 @@ __device__ __noinline__ bool term_lt(S a, S b, double t)
 {
     return ratio_lt(fabs(a), b, t);
 }
-template <typename S>
-__device__ __forceinline__ bool term_ok(const S &a, const S &b)
+// |a| <= 0.1 b, and with `small` also whether |a| < 0.05 b
+template <typename S, class CTL>
+__device__ __forceinline__ bool term_ok(const S &a, const S &b, CTL &ctl, bool *small = nullptr)
 {
     const float d = fabsf(dfm::near_float(val(a))), den = dfm::near_float(val(b));
-    if (d < 0.099999f * den) return true;
-    if (d > 0.100001f * den) return false;
-    return !term_gt<S>(a, b, 0.1);
-}
-template <typename S>
-__device__ __forceinline__ bool term_small(const S &a, const S &b)
-{
-    const float d = fabsf(dfm::near_float(val(a))), den = dfm::near_float(val(b));
-    if (d < 0.049999f * den) return true;
-    if (d > 0.050001f * den) return false;
-    return term_lt<S>(a, b, 0.05);
+    const bool ok = d < 0.099999f * den, bad = d > 0.100001f * den;
+    const bool sm = d < 0.049999f * den, not_sm = d > 0.050001f * den;
+    if constexpr (CTL::fast) {
+        ctl.reject |= bad;
+        ctl.odd |= !(ok || bad) || (small && !(sm || not_sm));
+        if (small) *small = *small && sm;
+        return true;
+    } else {
+        if (!ok && (bad || term_gt<S>(a, b, 0.1))) return false;
+        if (small) *small = *small && (sm || (!not_sm && term_lt<S>(a, b, 0.05)));
+        return true;
+    }
 }
 
 // Rates at one temperature level, by one thread or by a team of TS lanes
-template <int TS, bool MIX>
-__device__ __forceinline__ void h_rates(const TLevel &L, double, int case_b, HRates &r)
+template <int TS, bool MIX, class CTL>
+__device__ __forceinline__ void h_rates(const TLevel &L, double, int case_b, HRates &r, CTL &ctl)
 {
-    if constexpr (TS > 1) r = h_rates_team<TS, MIX>(L, case_b);
+    if constexpr (TS > 1) r = h_rates_team<TS, MIX>(L, case_b, ctl);
     else r = h_rates_serial<MIX>(L, case_b);
 }
-template <int TS, bool MIX>
-__device__ __forceinline__ void he_rates(const TLevel &L, double, int case_b, HeRates &r)
+template <int TS, bool MIX, class CTL>
+__device__ __forceinline__ void he_rates(const TLevel &L, double, int case_b, HeRates &r, CTL &ctl)
 {
-    if constexpr (TS > 1) r = he_rates_team<TS, MIX>(L, case_b);
+    if constexpr (TS > 1) r = he_rates_team<TS, MIX>(L, case_b, ctl);
     else r = he_rates_serial<MIX>(L, case_b);
 }
 // (only beta_HeII and alpha_HeIII)
-template <int TS, bool MIX>
-__device__ __forceinline__ void he3_rates(const TLevel &L, double, int case_b, HeRates &r)
+template <int TS, bool MIX, class CTL>
+__device__ __forceinline__ void he3_rates(const TLevel &L, double, int case_b, HeRates &r, CTL &ctl)
 {
     if constexpr (TS > 1) {
-        r = he_rates_team<TS, MIX>(L, case_b);
+        r = he_rates_team<TS, MIX>(L, case_b, ctl);
     } else {
         const double2 t = he3_rates_serial<MIX>(L, case_b);
         r.beta_HeII = t.x;
@@ -265,19 +274,19 @@ __device__ __forceinline__ void he3_rates(const TLevel &L, double, int case_b, H
     }
 }
 // dual numbers, a team of eight: the level of the value, dT the tangent of T
-template <int TS, bool MIX>
-__device__ __forceinline__ void h_rates(const TLevel &L, double dT, int case_b, HRatesT<Dual> &r)
+template <int TS, bool MIX, class CTL>
+__device__ __forceinline__ void h_rates(const TLevel &L, double dT, int case_b, HRatesT<Dual> &r, CTL &)
 {
     static_assert(TS == 8 && !MIX, "dual rates: teams of eight, FP64");
     r = h_rates_dual(L, dT, case_b);
 }
-template <int TS, bool MIX>
-__device__ __forceinline__ void he_rates(const TLevel &L, double dT, int case_b, HeRatesT<Dual> &r)
+template <int TS, bool MIX, class CTL>
+__device__ __forceinline__ void he_rates(const TLevel &L, double dT, int case_b, HeRatesT<Dual> &r, CTL &)
 {
     r = he_rates_dual(L, dT, case_b);
 }
-template <int TS, bool MIX>
-__device__ __forceinline__ void he3_rates(const TLevel &L, double dT, int case_b, HeRatesT<Dual> &r)
+template <int TS, bool MIX, class CTL>
+__device__ __forceinline__ void he3_rates(const TLevel &L, double dT, int case_b, HeRatesT<Dual> &r, CTL &)
 {
     r = he_rates_dual(L, dT, case_b);
 }
@@ -286,21 +295,50 @@ __device__ __forceinline__ void he3_rates(const TLevel &L, double dT, int case_b
 // pair (the temperatures of steps 3 and 4 enter their rates only through
 // 1/T and ln T): 1/T = md iT in pair arithmetic; and the derivative of a
 // dual T = Tmu1 / md.
-__device__ __forceinline__ dfm::F2 inv_pair(double x)
+template <class CTL>
+__device__ __forceinline__ dfm::F2 inv_pair(double x, CTL &ctl)
 {
-    if (!(x > 0.0) || !dfm::splittable(x)) return dfm::split_any(1.0 / x);
-    return dfm::rcp2(dfm::split(x));
+    const bool in = (x > 0.0) && dfm::splittable(x);
+    if constexpr (CTL::fast) {
+        ctl.odd |= !in;
+        return dfm::rcp2(dfm::split(x));
+    } else {
+        if (!in) return dfm::split_any(1.0 / x);
+        return dfm::rcp2(dfm::split(x));
+    }
 }
-__device__ __forceinline__ double level_mu(const Dual &md, dfm::F2 iT, const Dual &Tmu1, TLevel &L)
+template <class CTL>
+__device__ __forceinline__ dfm::F2 md_pair(double md, CTL &ctl)
 {
-    t_level_inv(dfm::norm(dfm::mulu(dfm::split_any(md.v), iT)), L);
+    if constexpr (CTL::fast) {
+        ctl.odd |= !dfm::splittable(md);
+        return dfm::split(md);
+    } else {
+        return dfm::split_any(md);
+    }
+}
+template <class CTL>
+__device__ __forceinline__ double level_mu(const Dual &md, dfm::F2 iT, const Dual &Tmu1, TLevel &L, CTL &ctl)
+{
+    t_level_inv(dfm::norm(dfm::mulu(md_pair(md.v, ctl), iT)), L, ctl);
     return qdiv(Tmu1, md).d;
 }
-__device__ __forceinline__ double level_mu(double md, dfm::F2 iT, double, TLevel &L)
+template <class CTL>
+__device__ __forceinline__ double level_mu(double md, dfm::F2 iT, double, TLevel &L, CTL &ctl)
 {
-    t_level_inv(dfm::norm(dfm::mulu(dfm::split_any(md), iT)), L);
+    t_level_inv(dfm::norm(dfm::mulu(md_pair(md, ctl), iT)), L, ctl);
     return 0.0;
 }
+
+// quotient and reciprocal (dual numbers: always the exact way)
+template <class CTL>
+__device__ __forceinline__ double cdiv(double a, double b, CTL &ctl) { return dfm::div_c(a, b, ctl); }
+template <class CTL>
+__device__ __forceinline__ double crcp(double b, CTL &ctl) { return dfm::rcp_c(b, ctl); }
+template <class CTL>
+__device__ __forceinline__ Dual cdiv(const Dual &a, const Dual &b, CTL &) { return qdiv(a, b); }
+template <class CTL>
+__device__ __forceinline__ Dual crcp(const Dual &b, CTL &) { return qrcp(b); }
 
 // (alpha^A_j - alpha^B_j) n_j n_e of HII, HeII, HeIII at temperature T
 // (Eq. (cool_N_cr)); out of line: it only runs without the OTSA, and
@@ -312,7 +350,8 @@ static __device__ __noinline__ void recomb_rates(double T, double nHII, double n
 {
     double aA[3], aB[3];
     TLevel L;
-    t_level(T, L);
+    dfm::Exact e;
+    t_level(T, L, e);
     Rates t;
     rates_serial<MIX>(L, 0, kNeedRec, 0u, t);
     recomb_alphas(t, aA);
@@ -336,10 +375,10 @@ struct PhotonTerms {
     bool ok, small;
 };
 
-template <bool MIX, bool SM, typename S>
+template <bool MIX, bool SM, typename S, class CTL>
 __device__ __forceinline__ void photon_group(const ThermoParams &p, int i, const S &N, const S &Fs, const S &Nd,
                                              const S &Fb, const S &Crec, const S &nHI, const S &nHeI,
-                                             const S &nHeII, double h, PhotonTerms<S> &o)
+                                             const S &nHeII, double h, PhotonTerms<S> &o, CTL &ctl)
 {
     S inv;
     if constexpr (MIX) {
@@ -351,10 +390,10 @@ __device__ __forceinline__ void photon_group(const ThermoParams &p, int i, const
         const float Df = __fadd_rn(__fadd_rn(__fmul_rn(narrow(p.crs[i][0]), narrow(nHI)),
                                              __fmul_rn(narrow(p.crs[i][1]), narrow(nHeI))),
                                    __fmul_rn(narrow(p.crs[i][2]), narrow(nHeII)));
-        inv = qrcp(rfma(h, dfm::widen(Df), 1.0));
+        inv = crcp(rfma(h, dfm::widen(Df), 1.0), ctl);
     } else {
         const S D = rfma(p.crs[i][2], nHeII, rfma(p.crs[i][1], nHeI, rmul(nHI, p.crs[i][0])));
-        inv = qrcp(rfma(h, D, S(1.0)));
+        inv = crcp(rfma(h, D, S(1.0)), ctl);
     }
     // smoothed RT: N + h Ndot rounded step by step, so a cell growing
     // linearly from zero meets its relative changes 1/k exactly
@@ -363,7 +402,7 @@ __device__ __forceinline__ void photon_group(const ThermoParams &p, int i, const
     else if (p.emit) Nn = rmul(rfma(h, Crec, N), inv);
     else Nn = rmul(N, inv);
     o.small = true;
-    o.ok = change_ok(Nn, N, S(kFloorN), o.small);
+    o.ok = change_ok(Nn, N, S(kFloorN), o.small, ctl);
     o.Nn = Nn;
     o.Fs = rmul(Fs, inv);
     if constexpr (SM) o.Fb = rmul(radd(Fb, S(h)), inv);
@@ -379,11 +418,11 @@ __device__ __forceinline__ void photon_group(const ThermoParams &p, int i, const
 // photo-ionisation rates gam_j and the photoheating; false when a group
 // breaks the 10% rule.  The recombination photons C_i (without the OTSA) come
 // from cc.rj.
-template <int G, int PT, bool MIX, bool SM>
+template <int G, int PT, bool MIX, bool SM, class CTL>
 __device__ __forceinline__ bool photons_team(const ThermoParams &p, const CellState<lane_groups<>(G, PT)> &s,
                                              const CoolCache<double> &cc, double nHI, double nHeI, double nHeII,
                                              double h, CellState<lane_groups<>(G, PT)> &o, double &gam0, double &gam1,
-                                             double &gam2, double &heat, bool &sm)
+                                             double &gam2, double &heat, bool &sm, CTL &ctl)
 {
     constexpr int NG = lane_groups<>(G, PT);
     const unsigned mask = team_mask<PT>();
@@ -400,11 +439,10 @@ __device__ __forceinline__ bool photons_team(const ThermoParams &p, const CellSt
             for (int j = 0; j < 3; ++j)
                 if (p.rec_g[j] == gi) Crec += cc.rj[j];
         }
-        photon_group<MIX, SM>(p, gi, s.N[r], s.Fs[r], s.Nd[r], s.Fb[r], Crec, nHI, nHeI, nHeII, h, pt[r]);
-        if (mine) {
-            ok = ok && pt[r].ok;
-            small = small && pt[r].small;
-        }
+        // (a lane without a group of this round runs group 0 on zeros, which changes nothing)
+        photon_group<MIX, SM>(p, gi, s.N[r], s.Fs[r], s.Nd[r], s.Fb[r], Crec, nHI, nHeI, nHeII, h, pt[r], ctl);
+        ok = ok && (pt[r].ok || !mine);
+        small = small && (pt[r].small || !mine);
         o.N[r] = pt[r].Nn;
         o.Fs[r] = pt[r].Fs;
         if constexpr (SM) {
@@ -412,8 +450,12 @@ __device__ __forceinline__ bool photons_team(const ThermoParams &p, const CellSt
             o.Nd[r] = s.Nd[r];
         }
     }
-    ok = __all_sync(mask, ok);
-    sm = sm && (__all_sync(mask, small) != 0);
+    if constexpr (CTL::fast) {   // (decided for the whole team at the end)
+        sm = sm && small;
+    } else {
+        ok = __all_sync(mask, ok);
+        sm = sm && (__all_sync(mask, small) != 0);
+    }
 #pragma unroll
     for (int i = 0; i < G; ++i) {
         const PhotonTerms<double> &q = pt[i / PT];
@@ -443,7 +485,8 @@ __device__ __forceinline__ bool photons_serial(const ThermoParams &p, const Cell
             for (int j = 0; j < 3; ++j)
                 if (p.rec_g[j] == i) Crec += cc.rj[j];
         }
-        photon_group<MIX, SM>(p, i, s.N[i], s.Fs[i], s.Nd[i], s.Fb[i], Crec, nHI, nHeI, nHeII, h, pt);
+        dfm::Exact e;
+        photon_group<MIX, SM>(p, i, s.N[i], s.Fs[i], s.Nd[i], s.Fb[i], Crec, nHI, nHeI, nHeII, h, pt, e);
         if (!pt.ok) return false;
         sm = sm && pt.small;
         o.N[i] = pt.Nn;
@@ -476,11 +519,15 @@ __device__ __forceinline__ bool photons_serial(const ThermoParams &p, const Cell
 // share its rate functions and each update their own photon groups; the same
 // operations in the same order, so the same bits.  Dual: teams of eight lanes
 // with the same values and a tangent each; they share the rate functions.
-template <int G, int TS, bool MIX, typename S = double, bool SM = false>
+// CTL: Exact, or Fast (teams, OTSA, evolving T, with helium): no branches; the
+// result counts unless ctl.odd or ctl.reject is set in a lane of the team.
+template <int G, int TS, bool MIX, typename S, bool SM, class CTL>
 __device__ __forceinline__ bool attempt(const ThermoParams &p, const S &nH, const CellState<lane_groups<S>(G, TS), S> &s,
                                         double h, const IsoRates<S> &iso, CoolCache<S> &cc,
-                                        CellState<lane_groups<S>(G, TS), S> &o, bool &small)
+                                        CellState<lane_groups<S>(G, TS), S> &o, bool &small, CTL &ctl)
 {
+    constexpr bool fast = CTL::fast;
+    const bool isothermal = !fast && p.isothermal, helium = fast || p.helium;
     constexpr bool dual = !std::is_same<S, double>::value;
     static_assert(dual ? TS == 8 : TS == 1 || TS == 4, "team sizes");
     static_assert(!MIX || sizeof(S) == sizeof(double), "the mixed path is not differentiated");
@@ -503,21 +550,21 @@ __device__ __forceinline__ bool attempt(const ThermoParams &p, const S &nH, cons
     // photon update; kept over rejected attempts
     // recombination photons without the OTSA, Eq. (cool_N_cr), at T(t) with
     // the backward abundances; group i gains C_i = sum_j [rec_g[j] == i] rj[j]
-    if constexpr (std::is_same<S, double>::value) {   // (the adjoint needs the OTSA)
+    if constexpr (!dual && !fast) {   // (the adjoint needs the OTSA)
         if (p.emit && !cc.rvalid) {
             recomb_rates<MIX>(s.T, nHII, nHeII, nHeIII, ne, cc.rj);
             cc.rvalid = true;
         }
     }
 
-    if (!p.isothermal && !cc.valid) {
+    if (fast || (!isothermal && !cc.valid)) {
         if constexpr (dual) {
-            cooling_dual(p.case_b, p.comp, p.tg, p.helium != 0, s.T, ne, nHI, nHII, nHeI, nHeII, nHeIII, cc.L, cc.dL);
+            cooling_dual(p.case_b, p.comp, p.tg, helium, s.T, ne, nHI, nHII, nHeI, nHeII, nHeIII, cc.L, cc.dL);
         } else if constexpr (TS > 1) {
-            const double2 c = cooling_sums_team4<MIX>(p.case_b, p.helium != 0, s.T, nHI, nHII, nHeI, nHeII, nHeIII);
+            const double2 c = cooling_sums_team4<MIX>(p.case_b, helium, s.T, nHI, nHII, nHeI, nHeII, nHeIII, ctl);
             cooling_close(p.comp, p.tg, s.T, ne, c.x, c.y, cc.L, cc.dL);
         } else {
-            cooling_serial<MIX>(p.case_b, p.comp, p.tg, p.helium != 0, s.T, ne, nHI, nHII, nHeI, nHeII, nHeIII, cc.L,
+            cooling_serial<MIX>(p.case_b, p.comp, p.tg, helium, s.T, ne, nHI, nHII, nHeI, nHeII, nHeIII, cc.L,
                                 cc.dL);
         }
         cc.valid = true;
@@ -530,7 +577,7 @@ __device__ __forceinline__ bool attempt(const ThermoParams &p, const S &nH, cons
     {
         bool ok;
         if constexpr (TS > 1 && !dual)
-            ok = photons_team<G, TS, MIX, SM>(p, s, cc, nHI, nHeI, nHeII, h, o, gam0, gam1, gam2, heat, sm);
+            ok = photons_team<G, TS, MIX, SM>(p, s, cc, nHI, nHeI, nHeII, h, o, gam0, gam1, gam2, heat, sm, ctl);
         else ok = photons_serial<G, MIX, SM>(p, s, cc, nHI, nHeI, nHeII, h, o, gam0, gam1, gam2, heat, sm);
         if (!ok) return false;
     }
@@ -538,34 +585,33 @@ __device__ __forceinline__ bool attempt(const ThermoParams &p, const S &nH, cons
     // 2. temperature: T/mu + K h (Lambda) / (1 + mu (dL/dT) K h), Lambda =
     // heating - cooling, d Lambda/d(T/mu) = -mu dL/dT
     S mden, mu, Tmu1 = 0.0;
-    if (!p.isothermal) {
+    if (!isothermal) {
         mden = mu_den(p, x, mhe);
-        mu = qrcp(mden);
+        mu = crcp(mden, ctl);
         const S Tmu = rmul(s.T, mden);
         const S Kh = rmul(iso.K, h);
         const S num = rmul(radd(heat, -cc.L), Kh);
-        const S dT = qdiv(num, rfma(rmul(mu, cc.dL), Kh, S(1.0)));
+        const S dT = cdiv(num, rfma(rmul(mu, cc.dL), Kh, S(1.0)), ctl);
         Tmu1 = radd(Tmu, dT);
-        if (!term_ok(num, Tmu)) return false;
-        if (!term_ok(dT, Tmu)) return false;
-        sm = sm && term_small(dT, Tmu);
+        if (!term_ok(num, Tmu, ctl)) return false;
+        if (!term_ok(dT, Tmu, ctl, &sm)) return false;
     }
     // 1/(T/mu') as a pair, for the temperatures (T/mu') mu_j of steps 3 and 4
-    const dfm::F2 iT = p.isothermal ? dfm::F2{0.0f, 0.0f} : inv_pair(val(Tmu1));
+    const dfm::F2 iT = isothermal ? dfm::F2{0.0f, 0.0f} : inv_pair(val(Tmu1), ctl);
 
     // 3. hydrogen
     HRatesT<S> hr;
-    if (p.isothermal) {
+    if (isothermal) {
         hr = iso.h;
     } else {
         TLevel L;
-        const double dT = level_mu(mden, iT, Tmu1, L);
-        h_rates<TS, MIX>(L, dT, p.case_b, hr);
+        const double dT = level_mu(mden, iT, Tmu1, L, ctl);
+        h_rates<TS, MIX>(L, dT, p.case_b, hr, ctl);
     }
     const S C = rfma(hr.beta, ne, gam0);
     const S CD = rfma(hr.alpha, ne, C);   // C + D, D = alpha n_e
     S dC = rmul(nH, hr.beta), dD = rmul(nH, hr.alpha);
-    if (!p.isothermal) {
+    if (!isothermal) {
         // - n_e (T/mu') mu^2 X d/dT
         const S f = rmul(rmul(ne, rmul(Tmu1, mu)), rmul(-mu, p.X));
         dC = rfma(f, hr.dbeta, dC);
@@ -573,54 +619,56 @@ __device__ __forceinline__ bool attempt(const ThermoParams &p, const S &nH, cons
     }
     const S J = rfma(-x, radd(dC, dD), radd(dC, -CD));
     const S hx = rmul(rfma(-x, CD, C), h);
-    S x1 = radd(x, qdiv(hx, rfma(-J, S(h), S(1.0))));
+    S x1 = radd(x, cdiv(hx, rfma(-J, S(h), S(1.0)), ctl));
     x1 = min0(max0(x1, kXMin), 1.0);
-    if (!change_ok(x1, x, S(kXMin), sm)) return false;
-    if (!term_ok(hx, max0(x, kXMin))) return false;
+    if (!change_ok(x1, x, S(kXMin), sm, ctl)) return false;
+    if (!term_ok(hx, max0(x, kXMin), ctl)) return false;
 
     // 4. helium
     S y2n = y2, y3n = y3;
     const S nHII1 = rmul(x1, nH);
-    if (p.helium) {
+    if (helium) {
         const S ne2 = ne_of(nHII1, q0, nHe);
         HeRatesT<S> r2;
-        if (p.isothermal) {
+        if (isothermal) {
             r2 = iso.he;
         } else {
             TLevel L;
-            const double dT = level_mu(mu_den(p, x1, mhe), iT, Tmu1, L);
-            he_rates<TS, MIX>(L, dT, p.case_b, r2);
+            const double dT = level_mu(mu_den(p, x1, mhe), iT, Tmu1, L, ctl);
+            he_rates<TS, MIX>(L, dT, p.case_b, r2, ctl);
         }
         const S hs(h);
         const S D1 = rfma(r2.beta_HeI, ne2, gam1);
-        const S yI1 = qdiv(rfma(rmul(rmul(y2, r2.alpha_HeII), ne2), hs, yI), rfma(D1, hs, S(1.0)));
+        const S yI1 = cdiv(rfma(rmul(rmul(y2, r2.alpha_HeII), ne2), hs, yI), rfma(D1, hs, S(1.0)), ctl);
         const S C2 = rfma(yI1, D1, rmul(rmul(y3, r2.alpha_HeIII), ne2));
         const S D2 = rfma(radd(r2.beta_HeII, r2.alpha_HeII), ne2, gam2);
-        y2n = qdiv(rfma(C2, hs, y2), rfma(D2, hs, S(1.0)));
+        y2n = cdiv(rfma(C2, hs, y2), rfma(D2, hs, S(1.0)), ctl);
         const S q1 = he_electrons(y2n, y3);
         const S ne3 = ne_of(nHII1, q1, nHe);
         HeRatesT<S> r3;
-        if (p.isothermal) {
+        if (isothermal) {
             r3 = iso.he;
         } else {
             TLevel L;
-            const double dT = level_mu(mu_den(p, x1, md_he(p, q1)), iT, Tmu1, L);
-            he3_rates<TS, MIX>(L, dT, p.case_b, r3);
+            const double dT = level_mu(mu_den(p, x1, md_he(p, q1)), iT, Tmu1, L, ctl);
+            he3_rates<TS, MIX>(L, dT, p.case_b, r3, ctl);
         }
         const S C3 = rmul(y2n, rfma(r3.beta_HeII, ne3, gam2));
         const S D3 = rmul(r3.alpha_HeIII, ne3);
-        y3n = qdiv(rfma(C3, hs, y3), rfma(D3, hs, S(1.0)));
+        y3n = cdiv(rfma(C3, hs, y3), rfma(D3, hs, S(1.0)), ctl);
         // conservation: lower the largest fraction (HeI largest: no change);
         // (the fractions are positive or zero: compared by their bits)
         const long long bI = dbits(val(yI1)), b2 = dbits(val(y2n)), b3 = dbits(val(y3n));
-        if (b2 >= bI && b2 >= b3) y2n = radd(radd(S(1.0), -yI1), -y3n);
-        else if (b3 >= bI && b3 > b2) y3n = radd(radd(S(1.0), -yI1), -y2n);
+        const bool two = b2 >= bI && b2 >= b3, three = !two && b3 >= bI;
+        const S rest = radd(radd(S(1.0), -yI1), two ? -y3n : -y2n);
+        y2n = two ? rest : y2n;
+        y3n = three ? rest : y3n;
         y2n = min0(max0(y2n, 0.0), 1.0);
         y3n = min0(max0(y3n, 0.0), 1.0);
     }
     const S q2 = he_electrons(y2n, y3n);
-    if (!change_ok(ne_of(nHII1, q2, nHe), ne, iso.nef, sm)) return false;
-    const S Tf = p.isothermal ? s.T : qdiv(Tmu1, mu_den(p, x1, md_he(p, q2)));
+    if (!change_ok(ne_of(nHII1, q2, nHe), ne, iso.nef, sm, ctl)) return false;
+    const S Tf = isothermal ? s.T : cdiv(Tmu1, mu_den(p, x1, md_he(p, q2)), ctl);
     o.x = x1;
     o.y2 = y2n;
     o.y3 = y3n;
@@ -639,8 +687,26 @@ __device__ __forceinline__ bool subcycle_once(const ThermoParams &p, const S &nH
     double h = (dbits(dt_tc) < dbits(t_left)) ? dt_tc : t_left;
     ++att;
     CellState<lane_groups<S>(G, TS), S> o;
-    bool small = false;
-    if (attempt<G, TS, MIX, S, SM>(p, nH, st, h, iso, cc, o, small)) {
+    bool small = false, ok = false, decided = false;
+    if constexpr (TS == 4 && std::is_same<S, double>::value) {
+        if (!p.isothermal && p.helium && !p.emit && !cc.valid) {
+            dfm::Fast f;
+            attempt<G, TS, MIX, S, SM>(p, nH, st, h, iso, cc, o, small, f);
+            const unsigned m = team_mask<TS>();
+            const bool odd = __any_sync(m, f.odd), reject = __any_sync(m, f.reject);
+            small = __all_sync(m, small);
+            // (a broken limit rejects whatever else was odd, but an odd value may itself have broken it)
+            decided = !odd;
+            ok = decided && !reject;
+            cc.valid = decided;   // the cooling at T(t), kept if rejected
+        }
+    }
+    if (!decided) {
+        dfm::Exact e;
+        small = false;
+        ok = attempt<G, TS, MIX, S, SM>(p, nH, st, h, iso, cc, o, small, e);
+    }
+    if (ok) {
         st = o;
         cc.valid = false;
         cc.rvalid = false;
