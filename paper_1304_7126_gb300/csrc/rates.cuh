@@ -29,19 +29,33 @@
 namespace rtgb {
 
 // Quotients and reciprocals of the thermochemistry (dfmath.cuh: three and
-// two FP64 instructions)
-__device__ __forceinline__ double qdiv(double a, double b) { return dfm::fast_div(a, b); }
-__device__ __forceinline__ double qrcp(double b) { return dfm::fast_rcp(b); }
-__device__ __forceinline__ Dual qdiv(const Dual &a, const Dual &b)
+// two FP64 instructions).
+// dual numbers: the derivative (a' - q b')/b takes the refined reciprocal that
+// the quotient's seed gives with one more instruction
+template <class CTL>
+__device__ __forceinline__ Dual cdiv(const Dual &a, const Dual &b, CTL &ctl)
 {
-    const double q = dfm::fast_div(a.v, b.v);
-    return Dual(q, dfm::fast_div(a.d - q * b.d, b.v));
+    const bool in = dfm::div_range(b.v);
+    if constexpr (CTL::fast) {
+        ctl.odd |= !in;
+    } else if (!in) {
+        const double q = dfm::ieee_div(a.v, b.v);
+        return Dual(q, dfm::ieee_div(a.d - q * b.d, b.v));
+    }
+    const double r = dfm::rcp_seed(b.v), q0 = __dmul_rn(a.v, r);
+    const double q = __fma_rn(__fma_rn(-q0, b.v, a.v), r, q0);
+    return Dual(q, __fma_rn(-q, b.d, a.d) * __fma_rn(__fma_rn(-b.v, r, 1.0), r, r));
 }
-__device__ __forceinline__ Dual qrcp(const Dual &b)
+template <class CTL>
+__device__ __forceinline__ Dual crcp(const Dual &b, CTL &ctl)
 {
-    const double q = dfm::fast_rcp(b.v);
+    const double q = dfm::rcp_c(b.v, ctl);
     return Dual(q, -q * q * b.d);
 }
+template <class CTL>
+__device__ __forceinline__ double cdiv(double a, double b, CTL &ctl) { return dfm::div_c(a, b, ctl); }
+template <class CTL>
+__device__ __forceinline__ double crcp(double b, CTL &ctl) { return dfm::rcp_c(b, ctl); }
 
 // exp arguments: exp(fma(a, ln T, fma(b, 1/T, c)))
 enum {
@@ -421,10 +435,11 @@ __device__ __forceinline__ double rate_df(const RateVal &r, const TLevel &L)
     return rate_df(r, L, e);
 }
 // d2f/dT2 = f w / T^2
-__device__ __forceinline__ double rate_d2f(const RateVal &r, const TLevel &L)
+template <class CTL>
+__device__ __forceinline__ double rate_d2f(const RateVal &r, const TLevel &L, CTL &ctl)
 {
     using namespace dfm;
-    return to_double_i(norm(mulu(mulu(r.y, L.invT), mulu(r.w, L.invT))), r.m);
+    return to_double_c(norm(mulu(mulu(r.y, L.invT), mulu(r.w, L.invT))), r.m, ctl);
 }
 
 // values (and derivatives) of several functions at one temperature
@@ -600,13 +615,13 @@ __device__ __forceinline__ HeRates he_rates_team(const TLevel &L, int case_b, CT
 // dual numbers, by a team of eight lanes that hold the same value and each
 // their own tangent (level L of the value, dT this lane's tangent of T): the
 // values are those above, f carries df/dT dT and df/dT carries d2f/dT2 dT
-static __device__ __noinline__ HRatesT<Dual> h_rates_dual(TLevel L, double dT, int case_b)
+template <class CTL>
+__device__ __forceinline__ HRatesT<Dual> h_rates_dual(const TLevel &L, double dT, int case_b, CTL &ctl)
 {
     const unsigned m = team_mask<8>();
     RateVal v;
-    dfm::Exact e;
-    rate_lane<false, 2>(case_b, team_lane<8>() == 0 ? RF_BETA_HI : RF_ALPHA_HII, L, v, e);
-    const double f = rate_f(v), df = rate_df(v, L), d2f = rate_d2f(v, L);
+    rate_lane<false, 2>(case_b, team_lane<8>() == 0 ? RF_BETA_HI : RF_ALPHA_HII, L, v, ctl);
+    const double f = rate_f(v, ctl), df = rate_df(v, L, ctl), d2f = rate_d2f(v, L, ctl);
     HRatesT<Dual> r;
     const double b1 = team_get<8>(m, df, 0), a1 = team_get<8>(m, df, 1);
     r.beta = Dual(team_get<8>(m, f, 0), b1 * dT);
@@ -615,13 +630,13 @@ static __device__ __noinline__ HRatesT<Dual> h_rates_dual(TLevel L, double dT, i
     r.dalpha = Dual(a1, team_get<8>(m, d2f, 1) * dT);
     return r;
 }
-static __device__ __noinline__ HeRatesT<Dual> he_rates_dual(TLevel L, double dT, int case_b)
+template <class CTL>
+__device__ __forceinline__ HeRatesT<Dual> he_rates_dual(const TLevel &L, double dT, int case_b, CTL &ctl)
 {
     const unsigned m = team_mask<8>();
     RateVal v;
-    dfm::Exact e;
-    rate_lane<false, 1>(case_b, RF_BETA_HEI + (team_lane<8>() & 3), L, v, e);
-    const double f = rate_f(v), df = rate_df(v, L);
+    rate_lane<false, 1>(case_b, RF_BETA_HEI + (team_lane<8>() & 3), L, v, ctl);
+    const double f = rate_f(v, ctl), df = rate_df(v, L, ctl);
     HeRatesT<Dual> r;
     r.beta_HeI = Dual(team_get<8>(m, f, 0), team_get<8>(m, df, 0) * dT);
     r.beta_HeII = Dual(team_get<8>(m, f, 1), team_get<8>(m, df, 1) * dT);
@@ -835,17 +850,17 @@ __device__ __forceinline__ double2 cooling_sums_team4(int case_b, bool helium, d
 // t and t + 8; the values as above.  With the sums over the species s of
 // F_s = sum f and their T-derivatives, the tangents are dL = sum F_s dn_s +
 // L_T dT and dL_T = sum F_s' dn_s + L_TT dT.
-static __device__ __noinline__ void cooling_dual(int case_b, double comp, double tg, bool helium, const Dual &T,
-                                                 const Dual &ne, const Dual &nHI, const Dual &nHII, const Dual &nHeI,
-                                                 const Dual &nHeII, const Dual &nHeIII, Dual &L, Dual &dL)
+template <class CTL>
+__device__ __forceinline__ void cooling_dual(int case_b, double comp, double tg, bool helium, const Dual &T,
+                                             const Dual &ne, const Dual &nHI, const Dual &nHII, const Dual &nHeI,
+                                             const Dual &nHeII, const Dual &nHeIII, Dual &L, Dual &dL, CTL &ctl)
 {
     using namespace dfm;
     const unsigned mask = team_mask<8>();
     const int t = team_lane<8>();
     const RateFn *R = g_rate_fn[case_b].f;
     TLevel Lv;
-    Exact e;
-    t_level(T.v, Lv, e);
+    t_level(T.v, Lv, ctl);
     Dual n[NSP];
     cool_densities(nHI, nHII, nHeI, nHeII, nHeIII, n);
     double nv[NSP];
@@ -857,13 +872,13 @@ static __device__ __noinline__ void cooling_dual(int case_b, double comp, double
     for (int r = 0; r < 2; ++r) {
         const int k = r ? (t < 4 ? g_cool_at[t + 8] : kNCool) : g_cool_at[t];
         F2 sig{0.0f, 0.0f}, l{0.0f, 0.0f};
-        if (r == 0) l = rate_softplus<false>(R[k], Lv, sig);   // (none in places 8 to 11)
+        if (r == 0) l = rate_softplus<false>(R[k], Lv, sig, ctl);   // (none in places 8 to 11)
         RateVal q;
         rate_val<false, 2>(R[k], Lv, l, sig, r ? 1u << kZeroC3 : 0u, false, q);
-        cool_term(q, split_density(pick(nv, g_cool_sp[k])), v[r], dv[r]);
+        cool_term(q, split_density(pick(nv, g_cool_sp[k]), ctl), v[r], dv[r]);
         d2[r] = mulu(v[r], q.w);
-        f[r] = rate_f(q);
-        df[r] = rate_df(q, Lv);
+        f[r] = rate_f(q, ctl);
+        df[r] = rate_df(q, Lv, ctl);
         if (k >= kNCool || (!helium && (cool_mask(1) >> k & 1))) {
             v[r] = dv[r] = d2[r] = F2{0.0f, 0.0f};
             f[r] = df[r] = 0.0;
@@ -876,9 +891,9 @@ static __device__ __noinline__ void cooling_dual(int case_b, double comp, double
         ds = team_add(mask, ds, m);
         d2s = team_add(mask, d2s, m);
     }
-    const double Ls = to_double_i(norm(s), -kCoolExp);
-    const double dLs = to_double_i(norm(mulu(norm(ds), Lv.invT)), -kCoolExp);
-    const double d2Ls = to_double_i(norm(mulu(mulu(d2s, Lv.invT), Lv.invT)), -kCoolExp);
+    const double Ls = to_double_c(norm(s), -kCoolExp, ctl);
+    const double dLs = to_double_c(norm(mulu(norm(ds), Lv.invT)), -kCoolExp, ctl);
+    const double d2Ls = to_double_c(norm(mulu(mulu(d2s, Lv.invT), Lv.invT)), -kCoolExp, ctl);
     double tL = dLs * T.d, tdL = d2Ls * T.d;
 #pragma unroll
     for (int p = 0; p < kNCool; ++p) {

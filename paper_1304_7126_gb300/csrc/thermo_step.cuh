@@ -57,7 +57,8 @@ template <typename S>
 __device__ __forceinline__ void cell_constants(const ThermoParams &p, const S &nH, IsoRates<S> &iso)
 {
     iso.nHe = nH * p.he_ratio;
-    iso.K = qdiv(S(p.kfac), nH);
+    dfm::Exact e;
+    iso.K = cdiv(S(p.kfac), nH, e);
     iso.nef = kNeFloor * nH;
 }
 
@@ -275,20 +276,20 @@ __device__ __forceinline__ void he3_rates(const TLevel &L, double, int case_b, H
 }
 // dual numbers, a team of eight: the level of the value, dT the tangent of T
 template <int TS, bool MIX, class CTL>
-__device__ __forceinline__ void h_rates(const TLevel &L, double dT, int case_b, HRatesT<Dual> &r, CTL &)
+__device__ __forceinline__ void h_rates(const TLevel &L, double dT, int case_b, HRatesT<Dual> &r, CTL &ctl)
 {
     static_assert(TS == 8 && !MIX, "dual rates: teams of eight, FP64");
-    r = h_rates_dual(L, dT, case_b);
+    r = h_rates_dual(L, dT, case_b, ctl);
 }
 template <int TS, bool MIX, class CTL>
-__device__ __forceinline__ void he_rates(const TLevel &L, double dT, int case_b, HeRatesT<Dual> &r, CTL &)
+__device__ __forceinline__ void he_rates(const TLevel &L, double dT, int case_b, HeRatesT<Dual> &r, CTL &ctl)
 {
-    r = he_rates_dual(L, dT, case_b);
+    r = he_rates_dual(L, dT, case_b, ctl);
 }
 template <int TS, bool MIX, class CTL>
-__device__ __forceinline__ void he3_rates(const TLevel &L, double dT, int case_b, HeRatesT<Dual> &r, CTL &)
+__device__ __forceinline__ void he3_rates(const TLevel &L, double dT, int case_b, HeRatesT<Dual> &r, CTL &ctl)
 {
-    r = he_rates_dual(L, dT, case_b);
+    r = he_rates_dual(L, dT, case_b, ctl);
 }
 
 // The level of T = (T/mu') mu_j given 1/mu_j = md and 1/(T/mu') = iT as a
@@ -321,7 +322,7 @@ template <class CTL>
 __device__ __forceinline__ double level_mu(const Dual &md, dfm::F2 iT, const Dual &Tmu1, TLevel &L, CTL &ctl)
 {
     t_level_inv(dfm::norm(dfm::mulu(md_pair(md.v, ctl), iT)), L, ctl);
-    return qdiv(Tmu1, md).d;
+    return cdiv(Tmu1, md, ctl).d;
 }
 template <class CTL>
 __device__ __forceinline__ double level_mu(double md, dfm::F2 iT, double, TLevel &L, CTL &ctl)
@@ -329,16 +330,6 @@ __device__ __forceinline__ double level_mu(double md, dfm::F2 iT, double, TLevel
     t_level_inv(dfm::norm(dfm::mulu(md_pair(md, ctl), iT)), L, ctl);
     return 0.0;
 }
-
-// quotient and reciprocal (dual numbers: always the exact way)
-template <class CTL>
-__device__ __forceinline__ double cdiv(double a, double b, CTL &ctl) { return dfm::div_c(a, b, ctl); }
-template <class CTL>
-__device__ __forceinline__ double crcp(double b, CTL &ctl) { return dfm::rcp_c(b, ctl); }
-template <class CTL>
-__device__ __forceinline__ Dual cdiv(const Dual &a, const Dual &b, CTL &) { return qdiv(a, b); }
-template <class CTL>
-__device__ __forceinline__ Dual crcp(const Dual &b, CTL &) { return qrcp(b); }
 
 // (alpha^A_j - alpha^B_j) n_j n_e of HII, HeII, HeIII at temperature T
 // (Eq. (cool_N_cr)); out of line: it only runs without the OTSA, and
@@ -360,6 +351,25 @@ static __device__ __noinline__ void recomb_rates(double T, double nHII, double n
     rj[0] = (aA[0] - aB[0]) * nHII * ne;
     rj[1] = (aA[1] - aB[1]) * nHeII * ne;
     rj[2] = (aA[2] - aB[2]) * nHeIII * ne;
+}
+
+// ... by a team: lane j species j, both cases; the same operations
+template <int TS, bool MIX>
+__device__ __forceinline__ void recomb_rates_team(double T, double nHII, double nHeII, double nHeIII, double ne,
+                                                  double *rj)
+{
+    const unsigned m = team_mask<TS>();
+    const int t = team_lane<TS>();
+    const int k = t == 0 ? RF_ALPHA_HII : t == 1 ? RF_ALPHA_HEII : RF_ALPHA_HEIII;
+    TLevel L;
+    dfm::Exact e;
+    t_level(T, L, e);
+    RateVal a, b;
+    rate_lane<MIX, 0>(0, k, L, a, e);
+    rate_lane<MIX, 0>(1, k, L, b, e);
+    const double r = (rate_f(a) - rate_f(b)) * (t == 0 ? nHII : t == 1 ? nHeII : nHeIII) * ne;
+#pragma unroll
+    for (int j = 0; j < 3; ++j) rj[j] = team_get<TS>(m, r, j);
 }
 
 // Photon update of one group, Eq. (SIE photons): N_i' = (N_i + h C_i)/(1 + h D_i)
@@ -437,7 +447,7 @@ __device__ __forceinline__ bool photons_team(const ThermoParams &p, const CellSt
         if (p.emit) {
 #pragma unroll
             for (int j = 0; j < 3; ++j)
-                if (p.rec_g[j] == gi) Crec += cc.rj[j];
+                if (mine && p.rec_g[j] == gi) Crec += cc.rj[j];
         }
         // (a lane without a group of this round runs group 0 on zeros, which changes nothing)
         photon_group<MIX, SM>(p, gi, s.N[r], s.Fs[r], s.Nd[r], s.Fb[r], Crec, nHI, nHeI, nHeII, h, pt[r], ctl);
@@ -470,11 +480,11 @@ __device__ __forceinline__ bool photons_team(const ThermoParams &p, const CellSt
     return ok;
 }
 
-template <int G, bool MIX, bool SM, typename S>
+template <int G, bool MIX, bool SM, typename S, class CTL>
 __device__ __forceinline__ bool photons_serial(const ThermoParams &p, const CellState<G, S> &s,
                                                const CoolCache<S> &cc, const S &nHI, const S &nHeI, const S &nHeII,
                                                double h, CellState<G, S> &o, S &gam0, S &gam1, S &gam2, S &heat,
-                                               bool &sm)
+                                               bool &sm, CTL &ctl)
 {
     PhotonTerms<S> pt;
 #pragma unroll
@@ -485,8 +495,7 @@ __device__ __forceinline__ bool photons_serial(const ThermoParams &p, const Cell
             for (int j = 0; j < 3; ++j)
                 if (p.rec_g[j] == i) Crec += cc.rj[j];
         }
-        dfm::Exact e;
-        photon_group<MIX, SM>(p, i, s.N[i], s.Fs[i], s.Nd[i], s.Fb[i], Crec, nHI, nHeI, nHeII, h, pt, e);
+        photon_group<MIX, SM>(p, i, s.N[i], s.Fs[i], s.Nd[i], s.Fb[i], Crec, nHI, nHeI, nHeII, h, pt, ctl);
         if (!pt.ok) return false;
         sm = sm && pt.small;
         o.N[i] = pt.Nn;
@@ -519,8 +528,9 @@ __device__ __forceinline__ bool photons_serial(const ThermoParams &p, const Cell
 // share its rate functions and each update their own photon groups; the same
 // operations in the same order, so the same bits.  Dual: teams of eight lanes
 // with the same values and a tangent each; they share the rate functions.
-// CTL: Exact, or Fast (teams, OTSA, evolving T, with helium): no branches; the
-// result counts unless ctl.odd or ctl.reject is set in a lane of the team.
+// CTL: Exact, or Fast (teams, evolving T, with helium): no branches but that of
+// the recombination photons; the result counts unless ctl.odd or ctl.reject is
+// set in a lane of the team.
 template <int G, int TS, bool MIX, typename S, bool SM, class CTL>
 __device__ __forceinline__ bool attempt(const ThermoParams &p, const S &nH, const CellState<lane_groups<S>(G, TS), S> &s,
                                         double h, const IsoRates<S> &iso, CoolCache<S> &cc,
@@ -550,16 +560,18 @@ __device__ __forceinline__ bool attempt(const ThermoParams &p, const S &nH, cons
     // photon update; kept over rejected attempts
     // recombination photons without the OTSA, Eq. (cool_N_cr), at T(t) with
     // the backward abundances; group i gains C_i = sum_j [rec_g[j] == i] rj[j]
-    if constexpr (!dual && !fast) {   // (the adjoint needs the OTSA)
+    if constexpr (!dual) {   // (the adjoint needs the OTSA)
         if (p.emit && !cc.rvalid) {
-            recomb_rates<MIX>(s.T, nHII, nHeII, nHeIII, ne, cc.rj);
+            if constexpr (TS > 1) recomb_rates_team<TS, MIX>(s.T, nHII, nHeII, nHeIII, ne, cc.rj);
+            else recomb_rates<MIX>(s.T, nHII, nHeII, nHeIII, ne, cc.rj);
             cc.rvalid = true;
         }
     }
 
     if (fast || (!isothermal && !cc.valid)) {
         if constexpr (dual) {
-            cooling_dual(p.case_b, p.comp, p.tg, helium, s.T, ne, nHI, nHII, nHeI, nHeII, nHeIII, cc.L, cc.dL);
+            cooling_dual(p.case_b, p.comp, p.tg, helium, s.T, ne, nHI, nHII, nHeI, nHeII, nHeIII, cc.L, cc.dL,
+                         ctl);
         } else if constexpr (TS > 1) {
             const double2 c = cooling_sums_team4<MIX>(p.case_b, helium, s.T, nHI, nHII, nHeI, nHeII, nHeIII, ctl);
             cooling_close(p.comp, p.tg, s.T, ne, c.x, c.y, cc.L, cc.dL);
@@ -578,7 +590,7 @@ __device__ __forceinline__ bool attempt(const ThermoParams &p, const S &nH, cons
         bool ok;
         if constexpr (TS > 1 && !dual)
             ok = photons_team<G, TS, MIX, SM>(p, s, cc, nHI, nHeI, nHeII, h, o, gam0, gam1, gam2, heat, sm, ctl);
-        else ok = photons_serial<G, MIX, SM>(p, s, cc, nHI, nHeI, nHeII, h, o, gam0, gam1, gam2, heat, sm);
+        else ok = photons_serial<G, MIX, SM>(p, s, cc, nHI, nHeI, nHeII, h, o, gam0, gam1, gam2, heat, sm, ctl);
         if (!ok) return false;
     }
 
@@ -688,8 +700,8 @@ __device__ __forceinline__ bool subcycle_once(const ThermoParams &p, const S &nH
     ++att;
     CellState<lane_groups<S>(G, TS), S> o;
     bool small = false, ok = false, decided = false;
-    if constexpr (TS == 4 && std::is_same<S, double>::value) {
-        if (!p.isothermal && p.helium && !p.emit && !cc.valid) {
+    if constexpr (TS > 1) {
+        if (!p.isothermal && p.helium && !cc.valid) {
             dfm::Fast f;
             attempt<G, TS, MIX, S, SM>(p, nH, st, h, iso, cc, o, small, f);
             const unsigned m = team_mask<TS>();
