@@ -43,7 +43,7 @@ LONG_ATTEMPTS = 134
 # DRAM bytes (read + write) per launch, from the ncu captures of the current
 # kernels summarised in profiles/ (128^3 x 3 groups, HLL)
 TRAFFIC = {"transport": 399187712 + 192541696,
-           # thermo_team
+           # thermo_team, both stages
            "thermo_drain": 325376}
 
 
@@ -218,8 +218,8 @@ def _config(w):
 
 
 # kernels each profiled phase of one RT step launches (the thermochemistry
-# drain phase: the team-per-cell kernel)
-KERNELS_PER_PHASE = {"inject": 1, "transport": 1, "thermo_pass1": 1, "thermo_drain": 1, "reduce": 1, "finalize": 1}
+# drain phase: the two stages of the team-per-cell kernel)
+KERNELS_PER_PHASE = {"inject": 1, "transport": 1, "thermo_pass1": 1, "thermo_drain": 2, "reduce": 1, "finalize": 1}
 
 
 def oracle_rate(w, nthreads, max_steps, seconds=30.0, boxes=None):
@@ -443,7 +443,7 @@ def main():
         roof = {"bound": "alu", "achieved": ach, "peak": fp64_peak, "unit": "GFLOP/s",
                 "frac": ach / fp64_peak,
                 "traffic": TRAFFIC.get(dominant) if w.name == "cosmo128_s7" else None,
-                "kernel": dominant + " (thermo_team, four lanes per cell)"
+                "kernel": dominant + " (thermo_team, two stages)"
                 if dominant == "thermo_drain" else dominant,
                 "peak_kind": "measured (cuBLAS DGEMM, FP64)",
                 "flop_per_attempt": fpa, "transcendental_calls_per_attempt":

@@ -500,14 +500,14 @@ __device__ __forceinline__ void rates_serial(const TLevel &L, int case_b, unsign
     }
 }
 
-// ---- teams: TS (4 or 8) adjacent lanes of a warp work on one cell, holding
+// ---- teams: TS (2, 4 or 8) adjacent lanes of a warp work on one cell, holding
 // the same state and sharing its rate functions ----
 template <int TS>
 __device__ __forceinline__ int team_lane() { return (int)(threadIdx.x & (TS - 1)); }
 template <int TS>
 __device__ __forceinline__ unsigned team_mask()
 {
-    static_assert(TS == 1 || TS == 4 || TS == 8, "team sizes");
+    static_assert(TS == 1 || TS == 2 || TS == 4 || TS == 8, "team sizes");
     return ((1u << TS) - 1u) << (threadIdx.x & 31u & ~(TS - 1u));
 }
 template <int TS>
@@ -580,8 +580,8 @@ static __device__ __noinline__ double2 he3_rates_serial(TLevel L, int case_b)
     rates_serial<MIX>(L, case_b, kNeedHe3, 0u, t);
     return make_double2(t.f[RF_BETA_HEII], t.f[RF_ALPHA_HEIII]);
 }
-// ... and by a team: lanes 0 and 1 the two hydrogen functions, lanes 0..3
-// the four helium ones, each then in every lane
+// ... and by a team: lanes 0 and 1 the two hydrogen functions, lanes 0..3 (a
+// team of two: twice lanes 0, 1) the four helium ones, each then in every lane
 template <int TS, bool MIX, class CTL>
 __device__ __forceinline__ HRates h_rates_team(const TLevel &L, int case_b, CTL &ctl)
 {
@@ -608,10 +608,33 @@ __device__ __forceinline__ HeRates he_rates_team(const TLevel &L, int case_b, CT
     HeRates r;
     r.beta_HeI = team_get<TS>(m, f, 0);
     r.beta_HeII = team_get<TS>(m, f, 1);
-    r.alpha_HeII = team_get<TS>(m, f, 2);
-    r.alpha_HeIII = team_get<TS>(m, f, 3);
+    if constexpr (TS >= 4) {
+        r.alpha_HeII = team_get<TS>(m, f, 2);
+        r.alpha_HeIII = team_get<TS>(m, f, 3);
+    } else {   // lanes 0, 1 once more
+        rate_lane<MIX, 0>(case_b, RF_BETA_HEI + 2 + team_lane<TS>(), L, v, ctl);
+        const double g = rate_f(v, ctl);
+        r.alpha_HeII = team_get<TS>(m, g, 0);
+        r.alpha_HeIII = team_get<TS>(m, g, 1);
+    }
     return r;
 }
+// only beta_HeII and alpha_HeIII
+template <int TS, bool MIX, class CTL>
+__device__ __forceinline__ void he3_rates_team(const TLevel &L, int case_b, HeRates &r, CTL &ctl)
+{
+    if constexpr (TS >= 4) {
+        r = he_rates_team<TS, MIX>(L, case_b, ctl);
+    } else {
+        const unsigned m = team_mask<TS>();
+        RateVal v;
+        rate_lane<MIX, 0>(case_b, team_lane<TS>() == 0 ? RF_BETA_HEII : RF_ALPHA_HEIII, L, v, ctl);
+        const double f = rate_f(v, ctl);
+        r.beta_HeII = team_get<TS>(m, f, 0);
+        r.alpha_HeIII = team_get<TS>(m, f, 1);
+    }
+}
+
 // dual numbers, by a team of eight lanes that hold the same value and each
 // their own tangent (level L of the value, dT this lane's tangent of T): the
 // values are those above, f carries df/dT dT and df/dT carries d2f/dT2 dT
@@ -733,10 +756,10 @@ __device__ __forceinline__ void cooling_close(double comp, double tg, const S &T
     dL = rmul(ne, radd(dLs, S(comp)));
 }
 
-// The terms' places in the sums: place t + 4 r is lane t's term of round r in
-// a team of four (t + 8 r in one of eight), the last place empty.  The order
-// gives round 0 the two terms with a softplus of their own beside the first
-// two of u, so a team evaluates one softplus per lane.
+// The terms' places in the sums: place t + TS r is lane t's term of round r in
+// a team of TS, the last place empty.  The order gives the two terms with a
+// softplus of their own places 2 and 3 beside the first two of u, so a team
+// of four or eight evaluates one softplus per lane, a team of two two.
 __host__ __device__ __forceinline__ constexpr int cool_at(int place)
 {
     constexpr int at[12] = {0, 1, 2, 10, 4, 5, 6, 7, 8, 9, 3, -1};
@@ -806,43 +829,62 @@ __device__ __forceinline__ void cooling_serial(int case_b, double comp, double t
     cooling_close(comp, tg, T, ne, s.x, s.y, L, dL);
 }
 
-// a team of four: places t, t + 4, t + 8, the last sums over shuffles, in the
-// order of tree_sum
+// a team of TS = 2 or 4: places t, t + TS, ..., the last sums over shuffles,
+// in the order of tree_sum
 __device__ __forceinline__ dfm::F2 team_add(unsigned mask, dfm::F2 a, int m)
 {
     return dfm::addu(a, dfm::F2{__shfl_xor_sync(mask, a.hi, m), __shfl_xor_sync(mask, a.lo, m)});
 }
-template <bool MIX, class CTL>
-__device__ __forceinline__ double2 cooling_sums_team4(int case_b, bool helium, double T, double nHI, double nHII,
-                                                          double nHeI, double nHeII, double nHeIII, CTL &ctl)
+template <int TS, bool MIX, class CTL>
+__device__ __forceinline__ double2 cooling_sums_team(int case_b, bool helium, double T, double nHI, double nHII,
+                                                     double nHeI, double nHeII, double nHeIII, CTL &ctl)
 {
     using namespace dfm;
-    const unsigned mask = team_mask<4>();
-    const int t = team_lane<4>();
+    static_assert(TS == 2 || TS == 4, "team sizes");
+    const unsigned mask = team_mask<TS>();
+    const int t = team_lane<TS>();
     const RateFn *R = g_rate_fn[case_b].f;
     TLevel L;
     t_level(T, L, ctl);
     double n[NSP];
     cool_densities(nHI, nHII, nHeI, nHeII, nHeIII, n);
-    // round 0: lanes 0, 1 with the softplus of u, lanes 2, 3 with their own
-    F2 sig;
-    const int k0 = g_cool_at[t];
-    const F2 l = rate_softplus<MIX>(R[k0], L, sig, ctl);
-    const F2 lu{__shfl_sync(mask, l.hi, 0, 4), __shfl_sync(mask, l.lo, 0, 4)};
-    const F2 su{__shfl_sync(mask, sig.hi, 0, 4), __shfl_sync(mask, sig.lo, 0, 4)};
-    F2 v[3], dv[3];
+    // the softplus of u: lane 0's of round 0 (a team of two: of both lanes);
+    // places 2 and 3 have their own, places 7 to 11 none (c3 = c3 c4 = 0)
+    F2 l, sig;
+    l = rate_softplus<MIX>(R[g_cool_at[t]], L, sig, ctl);
+    F2 lu = l, su = sig;
+    if constexpr (TS == 4) {
+        lu = F2{__shfl_sync(mask, l.hi, 0, TS), __shfl_sync(mask, l.lo, 0, TS)};
+        su = F2{__shfl_sync(mask, sig.hi, 0, TS), __shfl_sync(mask, sig.lo, 0, TS)};
+    }
+    constexpr int NR = 12 / TS;
+    F2 v[NR], dv[NR];
 #pragma unroll
-    for (int r = 0; r < 3; ++r) {
-        const int k = r ? g_cool_at[t + 4 * r] : k0;
+    for (int r = 0; r < NR; ++r) {
+        const int k = g_cool_at[t + TS * r];
+        const bool own = r * TS < 4;   // the round has a softplus of its own
+        if (own && r > 0) l = rate_softplus<MIX>(R[k], L, sig, ctl);
         RateVal q;
-        // (no softplus in round 2 nor in lane 3 of round 1: c3 = c3 c4 = 0)
-        rate_val<MIX, 1>(R[k], L, r ? lu : l, r ? su : sig, r == 2 ? 1u << kZeroC3 : 0u, false, q);
+        rate_val<MIX, 1>(R[k], L, own ? l : lu, own ? sig : su, r * TS >= 8 ? 1u << kZeroC3 : 0u, false, q);
         cool_term(q, split_density(pick(n, g_cool_sp[k]), ctl), v[r], dv[r]);
         if (k >= kNCool || (!helium && (cool_mask(1) >> k & 1))) v[r] = dv[r] = F2{0.0f, 0.0f};
     }
-    F2 s = addu(addu(v[0], v[2]), v[1]), ds = addu(addu(dv[0], dv[2]), dv[1]);
-    s = norm(team_add(mask, team_add(mask, s, 2), 1));
-    ds = norm(team_add(mask, team_add(mask, ds, 2), 1));
+    // places 8 apart, 4 apart, 2 and 1 apart
+#pragma unroll
+    for (int r = 0; r < 4 / TS; ++r) {
+        v[r] = addu(addu(v[r], v[r + 8 / TS]), v[r + 4 / TS]);
+        dv[r] = addu(addu(dv[r], dv[r + 8 / TS]), dv[r + 4 / TS]);
+    }
+    F2 s = v[0], ds = dv[0];
+    if constexpr (TS == 2) {
+        s = addu(s, v[1]);
+        ds = addu(ds, dv[1]);
+    } else {
+        s = team_add(mask, s, 2);
+        ds = team_add(mask, ds, 2);
+    }
+    s = norm(team_add(mask, s, 1));
+    ds = norm(team_add(mask, ds, 1));
     return make_double2(to_double_c(s, -kCoolExp, ctl), to_double_c(norm(mulu(ds, L.invT)), -kCoolExp, ctl));
 }
 

@@ -160,8 +160,8 @@ ThermoParams thermo_params(const rt_handle *h, double dt)
     p.case_b = h->opt.otsa ? 1 : 0;
     p.max_sub = h->opt.max_subcycles;
     p.pass1_attempts = h->routing.pass1_attempts;
-    p.lane_budget = h->routing.lane_budget;
-    p.lane_min = h->routing.lane_min;
+    p.bulk_budget = h->routing.bulk_budget;
+    p.bulk_min = h->routing.bulk_min;
     p.emit = h->opt.otsa ? 0 : 1;
     for (int j = 0; j < 3; ++j) {
         int r = h->opt.rec_group[j];
@@ -829,10 +829,10 @@ int rt_set_thermo_routing(rt_handle *h, int pass1_attempts, int drain_budget, in
     ThermoParams d{};
     default_routing(d);
     h->routing.pass1_attempts = pass1_attempts > 0 ? pass1_attempts : d.pass1_attempts;
-    const long long b = (long long)(drain_budget > 0 ? drain_budget : d.lane_budget / 2) +
-                        (drain2_budget > 0 ? drain2_budget : d.lane_budget / 2);
-    h->routing.lane_budget = (int)std::min<long long>(b, 1LL << 30);
-    h->routing.lane_min = drain2_min_cells >= 0 ? drain2_min_cells : d.lane_min;
+    const long long b = (long long)(drain_budget > 0 ? drain_budget : d.bulk_budget / 2) +
+                        (drain2_budget > 0 ? drain2_budget : d.bulk_budget / 2);
+    h->routing.bulk_budget = (int)std::min<long long>(b, 1LL << 30);
+    h->routing.bulk_min = drain2_min_cells >= 0 ? drain2_min_cells : d.bulk_min;
     invalidate_graph(h);   // the captured launches carry the old routing
     return RT_OK;
 }

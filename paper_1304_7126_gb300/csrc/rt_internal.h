@@ -66,8 +66,9 @@ struct ThermoParams {
     int case_b;
     int max_sub;
     int pass1_attempts;      // attempts before a cell is handed to the queue
-    int lane_budget;         // attempts a cell may spend in the lane-per-cell drain
-    long long lane_min;      // the drain runs only for queues of more cells than this
+    int bulk_budget;         // attempts between two looks of a stage-1 cell at whether the queue is empty
+    long long bulk_min;      // stage 1 runs only for queues of more cells than this (< 0: what two
+                             // blocks of teams per SM hold)
     int emit;                // no OTSA: recombination photons (Sec. 3.3.2)
     int rec_g[3];            // group receiving HII, HeII, HeIII recombination photons (-1: none)
     GroupConsts gc;
@@ -106,12 +107,12 @@ inline void derive_group_terms(ThermoParams &p)
 inline void default_routing(ThermoParams &p)
 {
     p.pass1_attempts = 6;
-    p.lane_budget = 256;
-    p.lane_min = 1LL << 40;
+    p.bulk_budget = 16;
+    p.bulk_min = -1;
 }
 
 // Device work queues of cells whose sub-cycling outlasted the first pass (a,
-// filled from both ends) and the lane-per-cell drain (b).
+// filled from both ends) and the first stage of the team kernel (b).
 constexpr int kQueueCounters = 8;
 
 struct QueueArrays {
@@ -123,7 +124,8 @@ struct QueueArrays {
 struct Queue {
     QueueArrays a, b;
     unsigned long long *counters;   // kQueueCounters: [0] a.count at the front, [1] at the back,
-                                    // [2] a.head, [3] b.count, [4] items taken after the first round
+                                    // [2] items taken after the first round in stage 1, [3] b.count,
+                                    // [4] items taken after the first round in stage 2
     long long capacity;             // items per queue
     double *fscale;                 // [2G][nc]: a queued cell's flux scale Fs_i (rows 0..G-1) and,
                                     // smoothed RT, its Fdot weight Fb_i (rows G..2G-1)

@@ -20,12 +20,13 @@
 //   thermo_pass1  one thread per cell (coalesced), up to 6 attempts; cells
 //                 still sub-cycling go to queue A with their partial state,
 //                 those with many sub-steps ahead to its front;
-//   thermo_team   persistent; a team of four lanes per queued cell, eight
-//                 cells per warp: the lanes share the cell's rate and cooling
-//                 functions (rates.cuh) and its photon groups while the scalar
-//                 update runs redundantly in all four;
-//   thermo_drain  between them, only when rt_set_thermo_routing asks for it:
-//                 persistent, one lane per cell.
+//   thermo_team   persistent, two stages: teams of two lanes per queued cell
+//                 while the queue lasts (only for queues longer than the
+//                 second stage holds at once), then teams of four for the
+//                 cells with many sub-steps left, on few warps: the lanes share
+//                 the cell's rate and cooling functions (rates.cuh) and its
+//                 photon groups while the scalar update runs redundantly in
+//                 all of them.
 // The arithmetic is the same in all of them, and a queued cell carries its
 // flux scale, so results do not depend on which kernel finished a cell.
 // Nothing waits on another thread; each kernel ends when its queue is empty.

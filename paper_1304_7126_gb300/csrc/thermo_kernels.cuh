@@ -1,5 +1,5 @@
-// Thermochemistry kernels (first pass, lane-per-cell drain, team-per-cell
-// kernel) and their launch sequence, templated on the group count G, the
+// Thermochemistry kernels (first pass, and the two stages of the
+// team-per-cell kernel) and their launch sequence, templated on the group count G, the
 // photon storage type P (double: RT_FP64; float: RT_MIXED), FP32 rate
 // transcendentals R32 (RT_MIXED32) and smoothed RT SM (Sec. 3.4).  Each
 // launcher translation unit instantiates one (P, R32) family, so the
@@ -25,8 +25,8 @@ namespace {
 using namespace thermo_detail;
 
 constexpr int kPass1Block = 128;
-constexpr int kTeam = 4;            // lanes per cell of thermo_team
 constexpr double kLongSteps = 32.0; // sub-steps ahead from which a queued cell is taken early
+constexpr double kHandSteps = 8.0;  // ... from which it moves to the second stage
 
 // first: the cell's first load in this RT step (thermo_pass1).  PT: 1, or the
 // lanes of the cell's team, each of which loads and stores its own groups
@@ -206,117 +206,95 @@ struct QueueView {
     }
 };
 
-// The lane-per-cell drain, for long queues only (more than lane_min cells):
-// cells of queue A sub-cycle here for at most lane_budget attempts, every
-// lane taking items one at a time; a cell still unfinished moves to queue B.
-template <int G, typename P, bool R32, bool SM>
+// A team of TS lanes per queued cell, 32 / TS cells per warp: the team's
+// lanes share the cell's rate functions and photon groups.  An attempt is a
+// chain of dependent FP32 pair and FP64 operations; on a warp alone it takes
+// 7.9 us with teams of four, whether the warp holds one cell or eight, and
+// two warps per SM sub-partition come close to filling the FP64 pipe.  (A
+// pair of warps per cell was no shorter and spent sixteen times the issue
+// slots and FP64 instructions per cell.)  The first items go to different
+// warps, spread over the SMs, then each team takes the next one.
+//
+// It runs twice.  Stage 1, for queues of more than bulk_min cells, fills the
+// SMs and is bound by the FP64 pipe, of which a team of two needs half as
+// much per cell as a team of four and takes longer per attempt.  Once the
+// queue has run empty its warps hold a few long cells each, whose attempts
+// cost a warp as much as full ones, so every 16th attempt (bulk_budget) a
+// cell with many sub-steps ahead then moves to queue B.  Stage 2, teams of
+// four, takes those, or a queue that was short, on few warps.
+template <int G, int TS, typename P, bool R32, bool SM>
 __global__ void __launch_bounds__(128)
-thermo_drain(ThermoParams p, const double *__restrict__ nH, double *xHII, double *xHeII, double *xHeIII,
-             double *T, P *N, P *F, P *Npre, P *Fpre, int32_t *subcycles, Queue q, unsigned *status)
+thermo_team(ThermoParams p, const double *__restrict__ nH, double *xHII, double *xHeII, double *xHeIII,
+            double *T, P *N, P *F, P *Npre, P *Fpre, int32_t *subcycles, Queue q, unsigned *status,
+            unsigned few_blocks)
 {
+    constexpr int stage = TS == 2 ? 1 : 2;
     const QueueView qv(q);
-    if ((long long)qv.total <= p.lane_min) return;
-    CellState<G> st;
+    const bool bulk = (long long)qv.total > p.bulk_min;
+    if (stage == 1 && !bulk) return;
+    const bool left = stage == 2 && bulk;   // queue B
+    unsigned long long count = left ? q.counters[3] : qv.total;
+    if (count > (unsigned long long)q.capacity) count = (unsigned long long)q.capacity;
+    const QueueArrays src = left ? q.b : q.a;
+    unsigned long long *taken = &q.counters[stage == 1 ? 2 : 4];
+    const unsigned per_block = blockDim.x / TS;
+    // stage 2 runs on one block per SM (few_blocks) for as many cells as those
+    // hold, else on two (more made the longest chains longer)
+    const unsigned blocks =
+        (stage == 2 && count <= (unsigned long long)few_blocks * per_block && few_blocks < gridDim.x) ? few_blocks
+                                                                                                      : gridDim.x;
+    if (blockIdx.x >= blocks) return;
+    const unsigned mask = team_mask<TS>();
+    const int t = team_lane<TS>();
+    // item order of the first round: warp 0 of every block, warp 1, ...
+    const unsigned long long warps = (unsigned long long)blocks * (blockDim.x >> 5);
+    const unsigned long long teams = (unsigned long long)blocks * per_block;
+    unsigned long long it = ((threadIdx.x & 31) / TS) * warps + (threadIdx.x >> 5) * blocks + blockIdx.x;
+    CellState<lane_groups<>(G, TS)> st;
     IsoRates<> iso;
     CoolCache<> cc;
     double t_left = 0.0, dt_tc = 0.0, n = 0.0;
     int att = 0, used = 0;
     long long c = -1;
-    bool have = false;
-    auto fetch = [&]() {
-        const unsigned long long it = atomicAdd(&q.counters[2], 1ULL);
-        have = it < qv.total;
-        if (have) {
-            const unsigned long long sl = qv.slot(q, it);
-            c = q.a.cell[sl];
-            t_left = q.a.t_left[sl];
-            dt_tc = q.a.dt_tc[sl];
-            att = q.a.attempts[sl];
-            n = nH[c];
-            used = 0;
-            load_cell<G, 1, P, R32, SM>(p, c, false, xHII, xHeII, xHeIII, T, N, Npre, q.fscale, st, iso, cc);
-            cell_constants(p, n, iso);
-        }
-    };
-    fetch();
-    while (have) {
-        bool done = subcycle_once<G, 1, R32, double, SM>(p, n, st, t_left, dt_tc, att, iso, cc);
-        if (!done && att >= p.max_sub) {
-            atomicOr(status, kStatusSubcycle);
-            done = true;
-        }
-        if (done) {
-            store_cell<G, 1, P, SM>(p, c, false, false, xHII, xHeII, xHeIII, T, N, F, Npre, Fpre, q.fscale, st, status);
-            subcycles[c] = att;
-            fetch();
-        } else if (++used >= p.lane_budget) {
-            // long sub-cycler: hand it to the team kernel
-            store_cell<G, 1, P, SM>(p, c, false, true, xHII, xHeII, xHeIII, T, N, F, Npre, Fpre, q.fscale, st, status);
-            const unsigned long long slot = atomicAdd(&q.counters[3], 1ULL);
-            push_item(q.b, slot, q.capacity, (uint32_t)c, t_left, dt_tc, att, status);
-            fetch();
-        }
-    }
-}
-
-// A team of four lanes per queued cell, eight cells per warp: the team's
-// lanes share the cell's rate functions (one softplus and exponential each
-// instead of four to eleven) and photon groups.  Bound by the length of an
-// attempt, a chain of dependent FP32 pair and FP64 operations in which a warp
-// of one cell and a warp of eight take the same time; a pair of warps per
-// cell, the kernel before, was no shorter and spent sixteen times the issue
-// slots and FP64 instructions per cell.  The first items go to different
-// warps, spread over the SMs, then each team takes the next one.
-template <int G, typename P, bool R32, bool SM>
-__global__ void __launch_bounds__(128)
-thermo_team(ThermoParams p, const double *__restrict__ nH, double *xHII, double *xHeII, double *xHeIII,
-            double *T, P *N, P *F, P *Npre, P *Fpre, int32_t *subcycles, Queue q, unsigned *status)
-{
-    const QueueView qv(q);
-    const bool drained = (long long)qv.total > p.lane_min;   // the cells left are in queue B
-    unsigned long long count = drained ? q.counters[3] : qv.total;
-    if (count > (unsigned long long)q.capacity) count = (unsigned long long)q.capacity;
-    const QueueArrays src = drained ? q.b : q.a;
-    const unsigned mask = team_mask<kTeam>();
-    const int t = team_lane<kTeam>();
-    // item order of the first round: warp 0 of every block, warp 1, ...
-    const unsigned long long warps = (unsigned long long)gridDim.x * (blockDim.x >> 5);
-    const unsigned long long first = ((threadIdx.x & 31) / kTeam) * warps + (threadIdx.x >> 5) * gridDim.x + blockIdx.x;
-    const unsigned long long teams = warps * (32 / kTeam);
-    CellState<lane_groups<>(G, kTeam)> st;
-    IsoRates<> iso;
-    CoolCache<> cc;
-    double t_left = 0.0, dt_tc = 0.0, n = 0.0;
-    int att = 0;
-    long long c = -1;
-    unsigned long long it = first;
     auto load = [&]() {
         if (it >= count) return false;
-        const unsigned long long sl = drained ? it : qv.slot(q, it);
+        const unsigned long long sl = left ? it : qv.slot(q, it);
         c = src.cell[sl];
         t_left = src.t_left[sl];
         dt_tc = src.dt_tc[sl];
         att = src.attempts[sl];
+        used = 0;
         n = nH[c];
-        load_cell<G, kTeam, P, R32, SM>(p, c, false, xHII, xHeII, xHeIII, T, N, Npre, q.fscale, st, iso, cc);
+        load_cell<G, TS, P, R32, SM>(p, c, false, xHII, xHeII, xHeIII, T, N, Npre, q.fscale, st, iso, cc);
         cell_constants(p, n, iso);
         return true;
     };
     bool have = load();
     while (have) {
-        bool done = subcycle_once<G, kTeam, R32, double, SM>(p, n, st, t_left, dt_tc, att, iso, cc);
+        bool done = subcycle_once<G, TS, R32, double, SM>(p, n, st, t_left, dt_tc, att, iso, cc);
         if (!done && att >= p.max_sub) {
             if (t == 0) atomicOr(status, kStatusSubcycle);
             done = true;
         }
-        if (done) {
-            store_cell<G, kTeam, P, SM>(p, c, false, false, xHII, xHeII, xHeIII, T, N, F, Npre, Fpre, q.fscale, st,
+        bool hand = false;
+        if (stage == 1 && !done && ++used >= p.bulk_budget) {
+            used = 0;
+            unsigned long long k = 0;
+            if (t == 0) k = teams + *(volatile unsigned long long *)taken;
+            k = __shfl_sync(mask, k, 0, TS);
+            hand = k >= count && t_left > kHandSteps * dt_tc;   // the queue is empty
+        }
+        if (done || hand) {
+            store_cell<G, TS, P, SM>(p, c, false, hand, xHII, xHeII, xHeIII, T, N, F, Npre, Fpre, q.fscale, st,
                                         status);
-            if (t == 0) subcycles[c] = att;
+            if (t == 0) {
+                if (done) subcycles[c] = att;
+                else push_item(q.b, atomicAdd(&q.counters[3], 1ULL), q.capacity, (uint32_t)c, t_left, dt_tc, att, status);
+            }
             it = count;
             if (count > teams) {
-                if (t == 0) it = teams + atomicAdd(&q.counters[4], 1ULL);
-                it = __shfl_sync(mask, it, 0, kTeam);
+                if (t == 0) it = teams + atomicAdd(taken, 1ULL);
+                it = __shfl_sync(mask, it, 0, TS);
             }
             have = load();
         }
@@ -335,27 +313,26 @@ cudaError_t launch_g(const ThermoParams &tp, const double *nH, double *xHII, dou
                                                           status);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    static int per_sm[2] = {0, 0};
-    if (per_sm[0] == 0) {
-        int a = 0, b = 0;
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&a, thermo_drain<G, P, R32, SM>, 128, 0);
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, thermo_team<G, P, R32, SM>, 128, 0);
-        per_sm[1] = b < 1 ? 1 : b;
-        per_sm[0] = a < 1 ? 1 : a;
+    static int per_sm = 0;
+    if (per_sm == 0) {
+        int k = 0;
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&k, thermo_team<G, 2, P, R32, SM>, 128, 0);
+        per_sm = k < 1 ? 1 : k;
     }
-    auto grid = [&](int k, long long cells_per_block) {
-        const long long g = (long long)per_sm[k] * n_sm, need = (tp.nc + cells_per_block - 1) / cells_per_block;
-        return (unsigned)(g < need ? g : need);
-    };
     if (ev) { cudaEventRecord(ev[1], s); cudaEventRecord(ev[2], s); }
-    if (tp.nc > tp.lane_min) {   // (otherwise the queue cannot hold that many)
-        thermo_drain<G, P, R32, SM><<<grid(0, 128), 128, 0, s>>>(tp, nH, xHII, xHeII, xHeIII, T, N, F, Npre, Fpre, sub,
-                                                                q, status);
+    ThermoParams p = tp;
+    // a queue that fits two blocks per SM needs no first stage
+    if (p.bulk_min < 0) p.bulk_min = 2LL * n_sm * (128 / 4);
+    if (p.nc > p.bulk_min) {   // (otherwise the queue cannot hold that many)
+        thermo_team<G, 2, P, R32, SM><<<(unsigned)(per_sm * n_sm), 128, 0, s>>>(p, nH, xHII, xHeII, xHeIII, T, N, F,
+                                                                              Npre, Fpre, sub, q, status, 0u);
         e = cudaGetLastError();
         if (e != cudaSuccess) return e;
     }
-    thermo_team<G, P, R32, SM><<<grid(1, 128 / kTeam), 128, 0, s>>>(tp, nH, xHII, xHeII, xHeIII, T, N, F, Npre, Fpre,
-                                                                   sub, q, status);
+    const long long g = 2LL * n_sm, need = (p.nc + 128 / 4 - 1) / (128 / 4);
+    thermo_team<G, 4, P, R32, SM><<<(unsigned)(g < need ? g : need), 128, 0, s>>>(p, nH, xHII, xHeII, xHeIII, T, N, F,
+                                                                                Npre, Fpre, sub, q, status,
+                                                                                (unsigned)n_sm);
     if (ev) cudaEventRecord(ev[3], s);
     return cudaGetLastError();
 }

@@ -267,7 +267,7 @@ template <int TS, bool MIX, class CTL>
 __device__ __forceinline__ void he3_rates(const TLevel &L, double, int case_b, HeRates &r, CTL &ctl)
 {
     if constexpr (TS > 1) {
-        r = he_rates_team<TS, MIX>(L, case_b, ctl);
+        he3_rates_team<TS, MIX>(L, case_b, r, ctl);
     } else {
         const double2 t = he3_rates_serial<MIX>(L, case_b);
         r.beta_HeII = t.x;
@@ -359,17 +359,21 @@ __device__ __forceinline__ void recomb_rates_team(double T, double nHII, double 
                                                   double *rj)
 {
     const unsigned m = team_mask<TS>();
-    const int t = team_lane<TS>();
-    const int k = t == 0 ? RF_ALPHA_HII : t == 1 ? RF_ALPHA_HEII : RF_ALPHA_HEIII;
     TLevel L;
     dfm::Exact e;
     t_level(T, L, e);
-    RateVal a, b;
-    rate_lane<MIX, 0>(0, k, L, a, e);
-    rate_lane<MIX, 0>(1, k, L, b, e);
-    const double r = (rate_f(a) - rate_f(b)) * (t == 0 ? nHII : t == 1 ? nHeII : nHeIII) * ne;
 #pragma unroll
-    for (int j = 0; j < 3; ++j) rj[j] = team_get<TS>(m, r, j);
+    for (int j0 = 0; j0 < 3; j0 += TS) {
+        const int j = j0 + team_lane<TS>();
+        const int k = j == 0 ? RF_ALPHA_HII : j == 1 ? RF_ALPHA_HEII : RF_ALPHA_HEIII;
+        RateVal a, b;
+        rate_lane<MIX, 0>(0, k, L, a, e);
+        rate_lane<MIX, 0>(1, k, L, b, e);
+        const double r = (rate_f(a) - rate_f(b)) * (j == 0 ? nHII : j == 1 ? nHeII : nHeIII) * ne;
+#pragma unroll
+        for (int i = 0; i < TS; ++i)
+            if (j0 + i < 3) rj[j0 + i] = team_get<TS>(m, r, i);
+    }
 }
 
 // Photon update of one group, Eq. (SIE photons): N_i' = (N_i + h C_i)/(1 + h D_i)
@@ -524,7 +528,7 @@ __device__ __forceinline__ bool photons_serial(const ThermoParams &p, const Cell
 //
 // S is double, or Dual for the adjoint's differentiated recomputation
 // (values bit-identical to the double path; MIX only with double).
-// TS: 1, one thread, or 4, a team of four lanes that hold the same cell,
+// TS: 1, one thread, or 2 or 4, a team of lanes that hold the same cell,
 // share its rate functions and each update their own photon groups; the same
 // operations in the same order, so the same bits.  Dual: teams of eight lanes
 // with the same values and a tangent each; they share the rate functions.
@@ -539,7 +543,7 @@ __device__ __forceinline__ bool attempt(const ThermoParams &p, const S &nH, cons
     constexpr bool fast = CTL::fast;
     const bool isothermal = !fast && p.isothermal, helium = fast || p.helium;
     constexpr bool dual = !std::is_same<S, double>::value;
-    static_assert(dual ? TS == 8 : TS == 1 || TS == 4, "team sizes");
+    static_assert(dual ? TS == 8 : TS == 1 || TS == 2 || TS == 4, "team sizes");
     static_assert(!MIX || sizeof(S) == sizeof(double), "the mixed path is not differentiated");
     const S nHe = iso.nHe;
     const S x = s.x, y2 = s.y2, y3 = s.y3;
@@ -573,7 +577,7 @@ __device__ __forceinline__ bool attempt(const ThermoParams &p, const S &nH, cons
             cooling_dual(p.case_b, p.comp, p.tg, helium, s.T, ne, nHI, nHII, nHeI, nHeII, nHeIII, cc.L, cc.dL,
                          ctl);
         } else if constexpr (TS > 1) {
-            const double2 c = cooling_sums_team4<MIX>(p.case_b, helium, s.T, nHI, nHII, nHeI, nHeII, nHeIII, ctl);
+            const double2 c = cooling_sums_team<TS, MIX>(p.case_b, helium, s.T, nHI, nHII, nHeI, nHeII, nHeIII, ctl);
             cooling_close(p.comp, p.tg, s.T, ne, c.x, c.y, cc.L, cc.dL);
         } else {
             cooling_serial<MIX>(p.case_b, p.comp, p.tg, helium, s.T, ne, nHI, nHII, nHeI, nHeII, nHeIII, cc.L,
@@ -701,7 +705,9 @@ __device__ __forceinline__ bool subcycle_once(const ThermoParams &p, const S &nH
     CellState<lane_groups<S>(G, TS), S> o;
     bool small = false, ok = false, decided = false;
     if constexpr (TS > 1) {
-        if (!p.isothermal && p.helium && !cc.valid) {
+        // (a retry evaluates the cooling again, to the same bits: beside teams
+        // that need theirs it takes no longer, and the warp stays together)
+        if (!p.isothermal && p.helium) {
             dfm::Fast f;
             attempt<G, TS, MIX, S, SM>(p, nH, st, h, iso, cc, o, small, f);
             const unsigned m = team_mask<TS>();
@@ -710,7 +716,7 @@ __device__ __forceinline__ bool subcycle_once(const ThermoParams &p, const S &nH
             // (a broken limit rejects whatever else was odd, but an odd value may itself have broken it)
             decided = !odd;
             ok = decided && !reject;
-            cc.valid = decided;   // the cooling at T(t), kept if rejected
+            cc.valid = decided;   // the cooling at T(t), kept for an attempt the exact way
         }
     }
     if (!decided) {
