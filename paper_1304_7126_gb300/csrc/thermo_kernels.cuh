@@ -223,7 +223,7 @@ struct QueueView {
 // cell with many sub-steps ahead then moves to queue B.  Stage 2, teams of
 // four, takes those, or a queue that was short, on few warps.
 template <int G, int TS, typename P, bool R32, bool SM>
-__global__ void __launch_bounds__(128)
+__global__ void __launch_bounds__(128, TS == 2 ? 4 : 2)
 thermo_team(ThermoParams p, const double *__restrict__ nH, double *xHII, double *xHeII, double *xHeIII,
             double *T, P *N, P *F, P *Npre, P *Fpre, int32_t *subcycles, Queue q, unsigned *status,
             unsigned few_blocks)
