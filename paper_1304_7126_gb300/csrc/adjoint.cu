@@ -85,41 +85,48 @@ thermo_vjp_kernel(ThermoParams p, const double *__restrict__ nH, const double *_
         }
     }
     __syncwarp();
-    if (!valid) return;   // (the lanes past NT stay: they share the team's rate functions)
+    // (the lanes past NT, and past the last cell, stay: whole warps run the
+    // attempts, and eight lanes share a cell's rate functions)
 
-    CellState<G, Dual> st;
-    st.x = Dual(xHII[c], j == G ? 1.0 : 0.0);
-    st.y2 = Dual(xHeII[c], j == G + 1 ? 1.0 : 0.0);
-    st.y3 = Dual(xHeIII[c], j == G + 2 ? 1.0 : 0.0);
-    st.T = Dual(T[c], j == G + 3 ? 1.0 : 0.0);
+    CellState<G, Dual> st{};
+    IsoRates<Dual> iso{};
+    CoolCache<Dual> cc{};
+    Dual n(0.0);
+    if (valid) {
+        st.x = Dual(xHII[c], j == G ? 1.0 : 0.0);
+        st.y2 = Dual(xHeII[c], j == G + 1 ? 1.0 : 0.0);
+        st.y3 = Dual(xHeIII[c], j == G + 2 ? 1.0 : 0.0);
+        st.T = Dual(T[c], j == G + 3 ? 1.0 : 0.0);
 #pragma unroll
-    for (int i = 0; i < G; ++i) {
-        st.N[i] = Dual(N[(long long)i * nc + c], j == i ? 1.0 : 0.0);
-        st.Fs[i] = Dual(1.0);
-    }
-    const Dual n(nH[c], j == G + 4 ? 1.0 : 0.0);
-    IsoRates<Dual> iso;
-    cell_constants(p, n, iso);
-    CoolCache<Dual> cc;
-    cc.valid = false;
-    cc.rvalid = false;
-    if (p.isothermal) {
-        TLevel L;
-        dfm::Exact e;
-        t_level(st.T.v, L, e);
-        h_rates<8, false>(L, st.T.d, p.case_b, iso.h, e);
-        if (p.helium) he_rates<8, false>(L, st.T.d, p.case_b, iso.he, e);
+        for (int i = 0; i < G; ++i) {
+            st.N[i] = Dual(N[(long long)i * nc + c], j == i ? 1.0 : 0.0);
+            st.Fs[i] = Dual(1.0);
+        }
+        n = Dual(nH[c], j == G + 4 ? 1.0 : 0.0);
+        cell_constants(p, n, iso);
+        cc.valid = false;
+        cc.rvalid = false;
+        if (p.isothermal) {
+            TLevel L;
+            dfm::Exact e;
+            t_level(st.T.v, L, e);
+            h_rates<8, false>(L, st.T.d, p.case_b, iso.h, e);
+            if (p.helium) he_rates<8, false>(L, st.T.d, p.case_b, iso.he, e);
+        }
     }
     double t_left = p.dt, dt_tc = p.dt;
     int att = 0;
-    bool done = false;
-    while (!done) {
-        done = subcycle_once<G, 8, false, Dual>(p, n, st, t_left, dt_tc, att, iso, cc);
+    bool done = !valid;
+    while (__any_sync(0xffffffffu, !done)) {
+        const bool fin = subcycle_once<G, 8, false, Dual>(p, n, st, t_left, dt_tc, att, iso, cc, !done);
+        if (done) continue;
+        done = fin;
         if (!done && att >= p.max_sub) {
             atomicOr(status, kStatusSubcycle);
             done = true;
         }
     }
+    if (!valid) return;
 
     double g = lxv * st.x.d + ly2v * st.y2.d + ly3v * st.y3.d + lTv * st.T.d;
 #pragma unroll

@@ -510,6 +510,19 @@ __device__ __forceinline__ unsigned team_mask()
     static_assert(TS == 1 || TS == 2 || TS == 4 || TS == 8, "team sizes");
     return ((1u << TS) - 1u) << (threadIdx.x & 31u & ~(TS - 1u));
 }
+// ... of the shuffles and votes of an attempt.  On the fast path of teams of
+// two and of the adjoint's teams of eight the whole warp runs it (teams
+// without a cell on whatever they hold), with a constant full mask.  Teams of
+// four, often one to a warp, run without the others (a lone cell's attempt
+// took 4% longer with the idle lanes' table reads).
+template <int TS>
+__host__ __device__ constexpr bool whole_warp() { return TS == 2 || TS == 8; }
+template <int TS, class CTL>
+__device__ __forceinline__ unsigned team_mask_c()
+{
+    if constexpr (CTL::fast && whole_warp<TS>()) return 0xffffffffu;
+    else return team_mask<TS>();
+}
 template <int TS>
 __device__ __forceinline__ double team_get(unsigned m, double v, int src) { return __shfl_sync(m, v, src, TS); }
 
@@ -585,7 +598,7 @@ static __device__ __noinline__ double2 he3_rates_serial(TLevel L, int case_b)
 template <int TS, bool MIX, class CTL>
 __device__ __forceinline__ HRates h_rates_team(const TLevel &L, int case_b, CTL &ctl)
 {
-    const unsigned m = team_mask<TS>();
+    const unsigned m = team_mask_c<TS, CTL>();
     RateVal v;
     rate_lane<MIX, 1>(case_b, team_lane<TS>() == 0 ? RF_BETA_HI : RF_ALPHA_HII, L, v, ctl);
     const double f = rate_f(v, ctl), df = rate_df(v, L, ctl);
@@ -601,7 +614,7 @@ static_assert(RF_BETA_HEII == RF_BETA_HEI + 1 && RF_ALPHA_HEII == RF_BETA_HEI + 
 template <int TS, bool MIX, class CTL>
 __device__ __forceinline__ HeRates he_rates_team(const TLevel &L, int case_b, CTL &ctl)
 {
-    const unsigned m = team_mask<TS>();
+    const unsigned m = team_mask_c<TS, CTL>();
     RateVal v;
     rate_lane<MIX, 0>(case_b, RF_BETA_HEI + (team_lane<TS>() & 3), L, v, ctl);
     const double f = rate_f(v, ctl);
@@ -626,7 +639,7 @@ __device__ __forceinline__ void he3_rates_team(const TLevel &L, int case_b, HeRa
     if constexpr (TS >= 4) {
         r = he_rates_team<TS, MIX>(L, case_b, ctl);
     } else {
-        const unsigned m = team_mask<TS>();
+        const unsigned m = team_mask_c<TS, CTL>();
         RateVal v;
         rate_lane<MIX, 0>(case_b, team_lane<TS>() == 0 ? RF_BETA_HEII : RF_ALPHA_HEIII, L, v, ctl);
         const double f = rate_f(v, ctl);
@@ -641,7 +654,7 @@ __device__ __forceinline__ void he3_rates_team(const TLevel &L, int case_b, HeRa
 template <class CTL>
 __device__ __forceinline__ HRatesT<Dual> h_rates_dual(const TLevel &L, double dT, int case_b, CTL &ctl)
 {
-    const unsigned m = team_mask<8>();
+    const unsigned m = team_mask_c<8, CTL>();
     RateVal v;
     rate_lane<false, 2>(case_b, team_lane<8>() == 0 ? RF_BETA_HI : RF_ALPHA_HII, L, v, ctl);
     const double f = rate_f(v, ctl), df = rate_df(v, L, ctl), d2f = rate_d2f(v, L, ctl);
@@ -656,7 +669,7 @@ __device__ __forceinline__ HRatesT<Dual> h_rates_dual(const TLevel &L, double dT
 template <class CTL>
 __device__ __forceinline__ HeRatesT<Dual> he_rates_dual(const TLevel &L, double dT, int case_b, CTL &ctl)
 {
-    const unsigned m = team_mask<8>();
+    const unsigned m = team_mask_c<8, CTL>();
     RateVal v;
     rate_lane<false, 1>(case_b, RF_BETA_HEI + (team_lane<8>() & 3), L, v, ctl);
     const double f = rate_f(v, ctl), df = rate_df(v, L, ctl);
@@ -841,7 +854,7 @@ __device__ __forceinline__ double2 cooling_sums_team(int case_b, bool helium, do
 {
     using namespace dfm;
     static_assert(TS == 2 || TS == 4, "team sizes");
-    const unsigned mask = team_mask<TS>();
+    const unsigned mask = team_mask_c<TS, CTL>();
     const int t = team_lane<TS>();
     const RateFn *R = g_rate_fn[case_b].f;
     TLevel L;
@@ -898,7 +911,7 @@ __device__ __forceinline__ void cooling_dual(int case_b, double comp, double tg,
                                              const Dual &nHeII, const Dual &nHeIII, Dual &L, Dual &dL, CTL &ctl)
 {
     using namespace dfm;
-    const unsigned mask = team_mask<8>();
+    const unsigned mask = team_mask_c<8, CTL>();
     const int t = team_lane<8>();
     const RateFn *R = g_rate_fn[case_b].f;
     TLevel Lv;

@@ -250,9 +250,9 @@ thermo_team(ThermoParams p, const double *__restrict__ nH, double *xHII, double 
     const unsigned long long warps = (unsigned long long)blocks * (blockDim.x >> 5);
     const unsigned long long teams = (unsigned long long)blocks * per_block;
     unsigned long long it = ((threadIdx.x & 31) / TS) * warps + (threadIdx.x >> 5) * blocks + blockIdx.x;
-    CellState<lane_groups<>(G, TS)> st;
-    IsoRates<> iso;
-    CoolCache<> cc;
+    CellState<lane_groups<>(G, TS)> st{};
+    IsoRates<> iso{};
+    CoolCache<> cc{};
     double t_left = 0.0, dt_tc = 0.0, n = 0.0;
     int att = 0, used = 0;
     long long c = -1;
@@ -270,8 +270,9 @@ thermo_team(ThermoParams p, const double *__restrict__ nH, double *xHII, double 
         return true;
     };
     bool have = load();
-    while (have) {
-        bool done = subcycle_once<G, TS, R32, double, SM>(p, n, st, t_left, dt_tc, att, iso, cc);
+    while (whole_warp<TS>() ? __any_sync(0xffffffffu, have) : have) {
+        bool done = subcycle_once<G, TS, R32, double, SM>(p, n, st, t_left, dt_tc, att, iso, cc, have);
+        if (!have) continue;
         if (!done && att >= p.max_sub) {
             if (t == 0) atomicOr(status, kStatusSubcycle);
             done = true;

@@ -354,22 +354,21 @@ static __device__ __noinline__ void recomb_rates(double T, double nHII, double n
 }
 
 // ... by a team: lane j species j, both cases; the same operations
-template <int TS, bool MIX>
+template <int TS, bool MIX, class CTL>
 __device__ __forceinline__ void recomb_rates_team(double T, double nHII, double nHeII, double nHeIII, double ne,
-                                                  double *rj)
+                                                  double *rj, CTL &ctl)
 {
-    const unsigned m = team_mask<TS>();
+    const unsigned m = team_mask_c<TS, CTL>();
     TLevel L;
-    dfm::Exact e;
-    t_level(T, L, e);
+    t_level(T, L, ctl);
 #pragma unroll
     for (int j0 = 0; j0 < 3; j0 += TS) {
         const int j = j0 + team_lane<TS>();
         const int k = j == 0 ? RF_ALPHA_HII : j == 1 ? RF_ALPHA_HEII : RF_ALPHA_HEIII;
         RateVal a, b;
-        rate_lane<MIX, 0>(0, k, L, a, e);
-        rate_lane<MIX, 0>(1, k, L, b, e);
-        const double r = (rate_f(a) - rate_f(b)) * (j == 0 ? nHII : j == 1 ? nHeII : nHeIII) * ne;
+        rate_lane<MIX, 0>(0, k, L, a, ctl);
+        rate_lane<MIX, 0>(1, k, L, b, ctl);
+        const double r = (rate_f(a, ctl) - rate_f(b, ctl)) * (j == 0 ? nHII : j == 1 ? nHeII : nHeIII) * ne;
 #pragma unroll
         for (int i = 0; i < TS; ++i)
             if (j0 + i < 3) rj[j0 + i] = team_get<TS>(m, r, i);
@@ -439,7 +438,7 @@ __device__ __forceinline__ bool photons_team(const ThermoParams &p, const CellSt
                                              double &gam2, double &heat, bool &sm, CTL &ctl)
 {
     constexpr int NG = lane_groups<>(G, PT);
-    const unsigned mask = team_mask<PT>();
+    const unsigned mask = team_mask_c<PT, CTL>();
     const int t = team_lane<PT>();
     bool ok = true, small = true;
     PhotonTerms<double> pt[NG];
@@ -565,8 +564,8 @@ __device__ __forceinline__ bool attempt(const ThermoParams &p, const S &nH, cons
     // recombination photons without the OTSA, Eq. (cool_N_cr), at T(t) with
     // the backward abundances; group i gains C_i = sum_j [rec_g[j] == i] rj[j]
     if constexpr (!dual) {   // (the adjoint needs the OTSA)
-        if (p.emit && !cc.rvalid) {
-            if constexpr (TS > 1) recomb_rates_team<TS, MIX>(s.T, nHII, nHeII, nHeIII, ne, cc.rj);
+        if (p.emit && (fast || !cc.rvalid)) {
+            if constexpr (TS > 1) recomb_rates_team<TS, MIX>(s.T, nHII, nHeII, nHeIII, ne, cc.rj, ctl);
             else recomb_rates<MIX>(s.T, nHII, nHeII, nHeIII, ne, cc.rj);
             cc.rvalid = true;
         }
@@ -694,14 +693,16 @@ __device__ __forceinline__ bool attempt(const ThermoParams &p, const S &nH, cons
 }
 
 // One attempt of the sub-cycling loop; returns true when the cell is done.
+// Teams of two and eight: called by whole warps; `have`: the lane's team has a
+// cell.
 template <int G, int TS, bool MIX, typename S = double, bool SM = false>
 __device__ __forceinline__ bool subcycle_once(const ThermoParams &p, const S &nH,
                                               CellState<lane_groups<S>(G, TS), S> &st, double &t_left, double &dt_tc,
-                                              int &att, const IsoRates<S> &iso, CoolCache<S> &cc)
+                                              int &att, const IsoRates<S> &iso, CoolCache<S> &cc, bool have = true)
 {
     // t_left, dt_tc > 0: compared through their bits
     double h = (dbits(dt_tc) < dbits(t_left)) ? dt_tc : t_left;
-    ++att;
+    att += have;
     CellState<lane_groups<S>(G, TS), S> o;
     bool small = false, ok = false, decided = false;
     if constexpr (TS > 1) {
@@ -710,15 +711,16 @@ __device__ __forceinline__ bool subcycle_once(const ThermoParams &p, const S &nH
         if (!p.isothermal && p.helium) {
             dfm::Fast f;
             attempt<G, TS, MIX, S, SM>(p, nH, st, h, iso, cc, o, small, f);
-            const unsigned m = team_mask<TS>();
-            const bool odd = __any_sync(m, f.odd), reject = __any_sync(m, f.reject);
-            small = __all_sync(m, small);
+            const unsigned m = team_mask<TS>(), all = team_mask_c<TS, dfm::Fast>();
+            const bool odd = (__ballot_sync(all, f.odd) & m) != 0, reject = (__ballot_sync(all, f.reject) & m) != 0;
+            small = (__ballot_sync(all, !small) & m) == 0;
             // (a broken limit rejects whatever else was odd, but an odd value may itself have broken it)
             decided = !odd;
             ok = decided && !reject;
             cc.valid = decided;   // the cooling at T(t), kept for an attempt the exact way
         }
     }
+    if (!have) return true;
     if (!decided) {
         dfm::Exact e;
         small = false;
