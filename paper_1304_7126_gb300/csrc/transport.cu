@@ -714,7 +714,7 @@ __device__ __noinline__ void transport_segment(PlaneSmem<S, TBX, TBY> &s, const 
 // planes (a launch of one CTA per tile chunk left a last, nearly empty wave);
 // a CTA walks its range one tile column segment at a time.  Budget partials:
 // [group][CTA], each the CTA's segments of that group summed in order.
-template <typename S, int FLUX>
+template <typename S, int FLUX, int TBY>
 __device__ __forceinline__ void transport_kernel_body(GridDev g, int G, S c, S dtdx, double area_dt,
                                                       const S *__restrict__ N0all, const S *__restrict__ F0all,
                                                       S *__restrict__ N1all, S *__restrict__ F1all,
@@ -722,7 +722,7 @@ __device__ __forceinline__ void transport_kernel_body(GridDev g, int G, S c, S d
                                                       double *__restrict__ part_inbox,
                                                       double *__restrict__ part_out, int tiles_x, int tiles_y)
 {
-    constexpr int TBX = 32, TBY = 8;
+    constexpr int TBX = 32;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     PlaneSmem<S, TBX, TBY> &s = *reinterpret_cast<PlaneSmem<S, TBX, TBY> *>(smem_raw);
     const long long tiles = (long long)tiles_x * tiles_y;
@@ -778,8 +778,23 @@ transport_kernel(GridDev g, int G, S c, S dtdx, double area_dt, const S *__restr
                  const Lam<S> *__restrict__ tab, const S *__restrict__ inflow, double *__restrict__ part_inbox,
                  double *__restrict__ part_out, int tiles_x, int tiles_y)
 {
-    transport_kernel_body<S, FLUX>(g, G, c, dtdx, area_dt, N0all, F0all, N1all, F1all, tab, inflow, part_inbox,
-                                   part_out, tiles_x, tiles_y);
+    transport_kernel_body<S, FLUX, 8>(g, G, c, dtdx, area_dt, N0all, F0all, N1all, F1all, tab, inflow, part_inbox,
+                                      part_out, tiles_x, tiles_y);
+}
+
+// Small boxes, where every CTA has one plane at most and the launch is as
+// long as one CTA's plane (two warps per SM sub-partition taking turns on the
+// FP64 pipe): tiles of 32 x 4, so twice as many CTAs of half the warps.
+// 32^3, one group, GLF, FP64: 43 -> 27 us.
+template <typename S, int FLUX>
+__global__ void __launch_bounds__(128, 2)
+transport_small_kernel(GridDev g, int G, S c, S dtdx, double area_dt, const S *__restrict__ N0all,
+                       const S *__restrict__ F0all, S *__restrict__ N1all, S *__restrict__ F1all,
+                       const Lam<S> *__restrict__ tab, const S *__restrict__ inflow, double *__restrict__ part_inbox,
+                       double *__restrict__ part_out, int tiles_x, int tiles_y)
+{
+    transport_kernel_body<S, FLUX, 4>(g, G, c, dtdx, area_dt, N0all, F0all, N1all, F1all, tab, inflow, part_inbox,
+                                      part_out, tiles_x, tiles_y);
 }
 
 template <int FLUX>
@@ -789,8 +804,8 @@ transport_kernel_f32(GridDev g, int G, float c, float dtdx, double area_dt, cons
                      const float *__restrict__ tab, const float *__restrict__ inflow,
                      double *__restrict__ part_inbox, double *__restrict__ part_out, int tiles_x, int tiles_y)
 {
-    transport_kernel_body<float, FLUX>(g, G, c, dtdx, area_dt, N0all, F0all, N1all, F1all, tab, inflow,
-                                       part_inbox, part_out, tiles_x, tiles_y);
+    transport_kernel_body<float, FLUX, 8>(g, G, c, dtdx, area_dt, N0all, F0all, N1all, F1all, tab, inflow,
+                                          part_inbox, part_out, tiles_x, tiles_y);
 }
 
 // Batched boxes: CTA i works on item i (box, group, tile, z range) of a
@@ -886,6 +901,11 @@ void transport_init()
     cudaFuncSetAttribute(transport_kernel<double, RT_GLF>, cudaFuncAttributeMaxDynamicSharedMemorySize, s8);
     cudaFuncSetAttribute(transport_kernel_f32<RT_HLL>, cudaFuncAttributeMaxDynamicSharedMemorySize, s4);
     cudaFuncSetAttribute(transport_kernel_f32<RT_GLF>, cudaFuncAttributeMaxDynamicSharedMemorySize, s4);
+    const int q8 = (int)sizeof(PlaneSmem<double, 32, 4>), q4 = (int)sizeof(PlaneSmem<float, 32, 4>);
+    cudaFuncSetAttribute(transport_small_kernel<double, RT_HLL>, cudaFuncAttributeMaxDynamicSharedMemorySize, q8);
+    cudaFuncSetAttribute(transport_small_kernel<double, RT_GLF>, cudaFuncAttributeMaxDynamicSharedMemorySize, q8);
+    cudaFuncSetAttribute(transport_small_kernel<float, RT_HLL>, cudaFuncAttributeMaxDynamicSharedMemorySize, q4);
+    cudaFuncSetAttribute(transport_small_kernel<float, RT_GLF>, cudaFuncAttributeMaxDynamicSharedMemorySize, q4);
     cudaFuncSetAttribute(transport_batch_all_kernel<double, RT_HLL>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                          batch_all_smem<double>());
     cudaFuncSetAttribute(transport_batch_all_kernel<double, RT_GLF>, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -910,6 +930,20 @@ static cudaError_t launch_t(const GridDev &g, int G, int flux, double cr, double
     const size_t smem = sizeof(PlaneSmem<S, 32, 8>);
     const S dtdx = (S)(dt / g.dx);
     const double area_dt = g.dx * g.dx * dt;
+    if (2LL * tiles_x * tiles_y * G * g.nz <= p.n_tr_blocks) {
+        const int tiles_y4 = (g.ny + 3) / 4;
+        const dim3 block4(32, 4);
+        const size_t smem4 = sizeof(PlaneSmem<S, 32, 4>);
+        if (flux == RT_HLL)
+            transport_small_kernel<S, RT_HLL><<<grid, block4, smem4, st>>>(g, G, (S)cr, dtdx, area_dt, N0, F0, N1, F1, tab,
+                                                                           inflow, p.tr_inbox, p.tr_outflow, tiles_x,
+                                                                           tiles_y4);
+        else
+            transport_small_kernel<S, RT_GLF><<<grid, block4, smem4, st>>>(g, G, (S)cr, dtdx, area_dt, N0, F0, N1, F1, tab,
+                                                                           inflow, p.tr_inbox, p.tr_outflow, tiles_x,
+                                                                           tiles_y4);
+        return cudaGetLastError();
+    }
     if constexpr (sizeof(S) == sizeof(float)) {
         if (flux == RT_HLL)
             transport_kernel_f32<RT_HLL><<<grid, block, smem, st>>>(g, G, (S)cr, dtdx, area_dt, N0, F0, N1, F1, tab,
