@@ -109,6 +109,24 @@ __global__ void batch_finalize_kernel(int k0, int nbg, int mode, const int *__re
     }
 }
 
+// rows of n values converted between arrays of different row lengths
+template <typename A, typename B>
+__global__ void __launch_bounds__(kRB)
+convert_rows_kernel(long long n, const A *__restrict__ in, long long in_row, B *__restrict__ out, long long out_row)
+{
+    const A *a = in + blockIdx.y * in_row;
+    B *b = out + blockIdx.y * out_row;
+    for (long long i = (long long)blockIdx.x * kRB + threadIdx.x; i < n; i += (long long)gridDim.x * kRB) b[i] = (B)a[i];
+}
+template <typename A, typename B>
+cudaError_t convert_rows(long long n, int rows, const A *in, long long in_row, B *out, long long out_row, cudaStream_t s)
+{
+    const long long need = (n + kRB - 1) / kRB;
+    convert_rows_kernel<A, B><<<dim3((unsigned)std::min<long long>(need, 128), (unsigned)rows), kRB, 0, s>>>(n, in, in_row,
+                                                                                                           out, out_row);
+    return cudaGetLastError();
+}
+
 __global__ void reset_counters_kernel(unsigned long long *c, int n)
 {
     if (threadIdx.x < n) c[threadIdx.x] = 0ULL;
@@ -624,24 +642,23 @@ int rt_batch_set_box_state(rt_batch *b, int box, const double *nH, const double 
     B_CUDA(b, cudaMemcpyAsync(c.xHeII + off, xHeII, bytes, k, b->stream));
     B_CUDA(b, cudaMemcpyAsync(c.xHeIII + off, xHeIII, bytes, k, b->stream));
     B_CUDA(b, cudaMemcpyAsync(c.T + off, T, bytes, k, b->stream));
-    for (int g = 0; g < G; ++g) {
-        for (int comp = -1; comp < 3; ++comp) {
-            const double *src = comp < 0 ? N + (size_t)g * nc : F + ((size_t)3 * g + comp) * nc;
-            long long dst_off = comp < 0 ? (long long)g * c.nc + off : (3LL * g + comp) * c.nc + off;
-            if (!b->mixed) {
-                double *dst = (double *)(comp < 0 ? c.N[b->cur] : c.F[b->cur]) + dst_off;
-                B_CUDA(b, cudaMemcpyAsync(dst, src, bytes, k, b->stream));
-            } else {
-                float *dst = (float *)(comp < 0 ? c.N[b->cur] : c.F[b->cur]) + dst_off;
-                if (device_ptrs) {
-                    cudaError_t e = launch_convert_d2f(nc, src, dst, b->stream);
-                    if (e != cudaSuccess) return bcuda(b, e, "convert");
-                } else {
-                    std::vector<float> tmp(src, src + nc);
-                    B_CUDA(b, cudaMemcpyAsync(dst, tmp.data(), nc * sizeof(float), cudaMemcpyHostToDevice, b->stream));
-                    B_CUDA(b, cudaStreamSynchronize(b->stream));
-                }
-            }
+    // N in G rows, F in 3 G rows, one copy or conversion each
+    const double *src[2] = {N, F};
+    void *dst[2] = {c.N[b->cur], c.F[b->cur]};
+    for (int f = 0; f < 2; ++f) {
+        const int rows = f ? 3 * G : G;
+        if (!b->mixed) {
+            B_CUDA(b, cudaMemcpy2DAsync((double *)dst[f] + off, (size_t)c.nc * sizeof(double), src[f], bytes, bytes, rows, k,
+                                        b->stream));
+        } else if (device_ptrs) {
+            cudaError_t e = convert_rows(nc, rows, src[f], nc, (float *)dst[f] + off, c.nc, b->stream);
+            if (e != cudaSuccess) return bcuda(b, e, "convert");
+        } else {
+            const size_t row = (size_t)nc * sizeof(float);
+            std::vector<float> tmp(src[f], src[f] + (size_t)rows * nc);
+            B_CUDA(b, cudaMemcpy2DAsync((float *)dst[f] + off, (size_t)c.nc * sizeof(float), tmp.data(), row, row, rows,
+                                        cudaMemcpyHostToDevice, b->stream));
+            B_CUDA(b, cudaStreamSynchronize(b->stream));
         }
     }
     if (!device_ptrs) B_CUDA(b, cudaStreamSynchronize(b->stream));
@@ -680,26 +697,24 @@ int rt_batch_get_box_state(rt_batch *b, int box, double *nH, double *xHII, doubl
     if (xHeII) B_CUDA(b, cudaMemcpyAsync(xHeII, c.xHeII + off, bytes, k, b->stream));
     if (xHeIII) B_CUDA(b, cudaMemcpyAsync(xHeIII, c.xHeIII + off, bytes, k, b->stream));
     if (T) B_CUDA(b, cudaMemcpyAsync(T, c.T + off, bytes, k, b->stream));
-    for (int g = 0; g < bx.G; ++g) {
-        for (int comp = -1; comp < 3; ++comp) {
-            double *dst = comp < 0 ? (N ? N + (size_t)g * nc : nullptr) : (F ? F + ((size_t)3 * g + comp) * nc : nullptr);
-            if (!dst) continue;
-            long long src_off = comp < 0 ? (long long)g * c.nc + off : (3LL * g + comp) * c.nc + off;
-            if (!b->mixed) {
-                const double *src = (const double *)(comp < 0 ? c.N[b->cur] : c.F[b->cur]) + src_off;
-                B_CUDA(b, cudaMemcpyAsync(dst, src, bytes, k, b->stream));
-            } else {
-                const float *src = (const float *)(comp < 0 ? c.N[b->cur] : c.F[b->cur]) + src_off;
-                if (device_ptrs) {
-                    cudaError_t e = launch_convert_f2d(nc, src, dst, b->stream);
-                    if (e != cudaSuccess) return bcuda(b, e, "convert");
-                } else {
-                    std::vector<float> tmp(nc);
-                    B_CUDA(b, cudaMemcpyAsync(tmp.data(), src, nc * sizeof(float), cudaMemcpyDeviceToHost, b->stream));
-                    B_CUDA(b, cudaStreamSynchronize(b->stream));
-                    for (long long i = 0; i < nc; ++i) dst[i] = tmp[i];
-                }
-            }
+    double *dst[2] = {N, F};
+    const void *src[2] = {c.N[b->cur], c.F[b->cur]};
+    for (int f = 0; f < 2; ++f) {
+        if (!dst[f]) continue;
+        const int rows = f ? 3 * bx.G : bx.G;
+        if (!b->mixed) {
+            B_CUDA(b, cudaMemcpy2DAsync(dst[f], bytes, (const double *)src[f] + off, (size_t)c.nc * sizeof(double), bytes,
+                                        rows, k, b->stream));
+        } else if (device_ptrs) {
+            cudaError_t e = convert_rows(nc, rows, (const float *)src[f] + off, c.nc, dst[f], nc, b->stream);
+            if (e != cudaSuccess) return bcuda(b, e, "convert");
+        } else {
+            const size_t row = (size_t)nc * sizeof(float);
+            std::vector<float> tmp((size_t)rows * nc);
+            B_CUDA(b, cudaMemcpy2DAsync(tmp.data(), row, (const float *)src[f] + off, (size_t)c.nc * sizeof(float), row, rows,
+                                        cudaMemcpyDeviceToHost, b->stream));
+            B_CUDA(b, cudaStreamSynchronize(b->stream));
+            for (size_t i = 0; i < tmp.size(); ++i) dst[f][i] = tmp[i];
         }
     }
     if (!device_ptrs) B_CUDA(b, cudaStreamSynchronize(b->stream));
