@@ -158,11 +158,11 @@ __device__ __forceinline__ void hll_lookup_fix(const long long *__restrict__ tab
                                                double mu, long long &lo, long long &hi)
 {
     const unsigned long long a = to_fix(mu);
-    long long v = (1LL << 62) + (tbits(mu) < 0 ? -(long long)a : (long long)a);   // (mu + 1) 2^62
-    if (tbits(mu) >= 0 && v < 0) v = 0x7fffffffffffffffLL;
-    if (v < 0) v = 0;
+    unsigned long long v = (1ULL << 62) + (tbits(mu) < 0 ? 0ULL - a : a);   // (mu + 1) 2^62, mod 2^64
+    const unsigned long long end = tbits(mu) < 0 ? 0ULL : 0x7fffffffffffffffULL;
+    v = (v >> 63) ? end : v;                                       // |mu| >= 1
     const int j = (int)(v >> 55);                                  // 0..255
-    const unsigned long long wm = (unsigned long long)v << 9;
+    const unsigned long long wm = v << 9;
     const longlong2 *t = reinterpret_cast<const longlong2 *>(tab) + k * kHllNMU + j;
     const longlong2 A = __ldg(t), B = __ldg(t + 1), C = __ldg(t + kHllNMU), D = __ldg(t + kHllNMU + 1);
     const long long lo0 = A.x + fix_mul(B.x - A.x, wm), lo1 = C.x + fix_mul(D.x - C.x, wm);
