@@ -7,9 +7,9 @@
 // Every rate coefficient and every cooling term is one function of T of
 // the form
 //     f(T) = Cc exp(c0 + c1 ln T + c2 / T - c3 softplus(c4 ln T + c5)),
-// softplus(z) = ln(1 + e^z) (see RateFn below).  A warp evaluates them all
-// at once, lane k function k; one thread evaluates the ones it needs.  The
-// argument is formed in the double-float arithmetic of dfmath.cuh (on the
+// softplus(z) = ln(1 + e^z) (see RateFn below).  The lanes of a team of two,
+// four or eight that share a cell take a function each; one thread evaluates
+// the ones it needs in turn.  The argument is formed in the double-float arithmetic of dfmath.cuh (on the
 // FP32 pipe), exponentiated by dfm::exp2d and scaled by Cc in FP64; both
 // paths run the same expressions and so give identical bits.
 //
@@ -632,22 +632,6 @@ __device__ __forceinline__ HeRates he_rates_team(const TLevel &L, int case_b, CT
     }
     return r;
 }
-// only beta_HeII and alpha_HeIII
-template <int TS, bool MIX, class CTL>
-__device__ __forceinline__ void he3_rates_team(const TLevel &L, int case_b, HeRates &r, CTL &ctl)
-{
-    if constexpr (TS >= 4) {
-        r = he_rates_team<TS, MIX>(L, case_b, ctl);
-    } else {
-        const unsigned m = team_mask_c<TS, CTL>();
-        RateVal v;
-        rate_lane<MIX, 0>(case_b, team_lane<TS>() == 0 ? RF_BETA_HEII : RF_ALPHA_HEIII, L, v, ctl);
-        const double f = rate_f(v, ctl);
-        r.beta_HeII = team_get<TS>(m, f, 0);
-        r.alpha_HeIII = team_get<TS>(m, f, 1);
-    }
-}
-
 // dual numbers, by a team of eight lanes that hold the same value and each
 // their own tangent (level L of the value, dT this lane's tangent of T): the
 // values are those above, f carries df/dT dT and df/dT carries d2f/dT2 dT
@@ -697,8 +681,8 @@ __device__ __forceinline__ void recomb_alphas(const RatesT<S> &t, S a[3])
 // terms, scaled by 2^kCoolExp, and their sums are float pairs (2^-46, the
 // accuracy of the functions themselves is 1e-14 to 1e-12): before, 11
 // functions and derivatives entered FP64 one by one, 90 of an attempt's FP64
-// instructions.  The one-thread sum and the warp sum (lane k term k) run the
-// same operations and give the same bits.
+// instructions.  The one-thread sum and the teams' sums run the same
+// operations and give the same bits.
 constexpr int kCoolExp = 80;
 
 // a[i] through selects (registers, not local memory, for a lane-dependent

@@ -209,12 +209,14 @@ struct QueueView {
 };
 
 // A team of TS lanes per queued cell, 32 / TS cells per warp: the team's
-// lanes share the cell's rate functions and photon groups.  An attempt is a
-// chain of dependent FP32 pair and FP64 operations; on a warp alone it takes
-// 7.9 us with teams of four, whether the warp holds one cell or eight, and
-// two warps per SM sub-partition come close to filling the FP64 pipe.  (A
-// pair of warps per cell was no shorter and spent sixteen times the issue
-// slots and FP64 instructions per cell.)  The first items go to different
+// lanes share the cell's rate functions and photon groups and, where they
+// can, its FP64 terms (one FP64 instruction with a term per lane).  An
+// attempt is a chain of dependent FP32 pair and FP64 operations; on a warp
+// alone it takes 7.1 us with teams of four (7.9 before the FP64 terms were
+// shared), whether the warp holds one cell or eight, and two warps per SM
+// sub-partition come close to filling the FP64 pipe.  (A pair of warps per
+// cell was no shorter and spent sixteen times the issue slots and FP64
+// instructions per cell.)  The first items go to different
 // warps, spread over the SMs, then each team takes the next one.
 //
 // It runs twice.  Stage 1, for queues of more than bulk_min cells, fills the

@@ -262,17 +262,120 @@ __device__ __forceinline__ void he_rates(const TLevel &L, double, int case_b, He
     if constexpr (TS > 1) r = he_rates_team<TS, MIX>(L, case_b, ctl);
     else r = he_rates_serial<MIX>(L, case_b);
 }
-// (only beta_HeII and alpha_HeIII)
+// (only beta_HeII and alpha_HeIII; one thread)
 template <int TS, bool MIX, class CTL>
 __device__ __forceinline__ void he3_rates(const TLevel &L, double, int case_b, HeRates &r, CTL &ctl)
 {
-    if constexpr (TS > 1) {
-        he3_rates_team<TS, MIX>(L, case_b, r, ctl);
+    const double2 t = he3_rates_serial<MIX>(L, case_b);
+    r.beta_HeII = t.x;
+    r.alpha_HeIII = t.y;
+}
+
+// What an attempt of a team makes of the rates at one temperature, each lane
+// from its own function before the shuffles: an FP64 instruction takes a warp
+// 64 cycles whatever its lanes hold, so the lanes' terms share one (each a
+// fused multiply-add with a factor 1 or an addend 0 where a lane has none:
+// the bits of the one-thread path).
+// With the sums of photons_team about 24 of an attempt's 135 FP64
+// instructions less: 128^3 with 16 bright sources, one lone cell's chain of
+// 2448 attempts 19.4 -> 17.3 ms; 48^3 without the OTSA 10.9 -> 10.2 ms; 256^3
+// 37.5 -> 34.4 ms.
+// The densities n_HI, n_HeI, n_HeII, n_HeIII:
+template <int TS, class CTL>
+__device__ __forceinline__ void densities_team(double nH, double nHe, double xI, double yI, double y2, double y3,
+                                               double &nHI, double &nHeI, double &nHeII, double &nHeIII)
+{
+    const unsigned m = team_mask_c<TS, CTL>();
+    const int t = team_lane<TS>();
+    const double n = t == 0 ? nH : nHe;
+    if constexpr (TS >= 4) {
+        const double d = rmul(n, t == 0 ? xI : t == 1 ? yI : t == 2 ? y2 : y3);
+        nHI = team_get<TS>(m, d, 0);
+        nHeI = team_get<TS>(m, d, 1);
+        nHeII = team_get<TS>(m, d, 2);
+        nHeIII = team_get<TS>(m, d, 3);
     } else {
-        const double2 t = he3_rates_serial<MIX>(L, case_b);
-        r.beta_HeII = t.x;
-        r.alpha_HeIII = t.y;
+        const double d = rmul(n, t == 0 ? xI : yI), e = rmul(nHe, t == 0 ? y2 : y3);
+        nHI = team_get<TS>(m, d, 0);
+        nHeI = team_get<TS>(m, d, 1);
+        nHeII = team_get<TS>(m, e, 0);
+        nHeIII = team_get<TS>(m, e, 1);
     }
+}
+// The cooling L and dL/dT of the sums (cooling_close):
+template <int TS, class CTL>
+__device__ __forceinline__ void cooling_close_team(double comp, double tg, double T, double ne, double Ls, double dLs,
+                                                   double &L, double &dL)
+{
+    const unsigned m = team_mask_c<TS, CTL>();
+    const bool l = team_lane<TS>() == 0;
+    const double z = rmul(ne, radd(l ? Ls : dLs, l ? rmul(radd(T, -tg), comp) : comp));
+    L = team_get<TS>(m, z, 0);
+    dL = team_get<TS>(m, z, 1);
+}
+// Hydrogen: beta, alpha, dC = n_H beta + f dbeta/dT, dD = n_H alpha + f dalpha/dT
+template <int TS, bool MIX, class CTL>
+__device__ __forceinline__ void h_terms_team(const TLevel &L, int case_b, double nH, double f, double &beta,
+                                             double &alpha, double &dC, double &dD, CTL &ctl)
+{
+    const unsigned m = team_mask_c<TS, CTL>();
+    RateVal v;
+    rate_lane<MIX, 1>(case_b, team_lane<TS>() == 0 ? RF_BETA_HI : RF_ALPHA_HII, L, v, ctl);
+    const double r = rate_f(v, ctl), d = rfma(f, rate_df(v, L, ctl), rmul(nH, r));
+    beta = team_get<TS>(m, r, 0);
+    alpha = team_get<TS>(m, r, 1);
+    dC = team_get<TS>(m, d, 0);
+    dD = team_get<TS>(m, d, 1);
+}
+// HeI and HeII: D1 = beta_HeI n_e + Gamma_1, P3 = y3 alpha_HeIII n_e, num1 =
+// yI + h y2 alpha_HeII n_e, den1 = 1 + h D1, den2 = 1 + h ((beta_HeII +
+// alpha_HeII) n_e + Gamma_2)
+template <int TS, bool MIX, class CTL>
+__device__ __forceinline__ void he_terms_team(const TLevel &L, int case_b, double y2, double y3, double yI, double ne,
+                                              double gam1, double gam2, double h, double &D1, double &P3,
+                                              double &num1, double &den1, double &den2, CTL &ctl)
+{
+    const unsigned m = team_mask_c<TS, CTL>();
+    const int t = team_lane<TS>();
+    RateVal v;
+    rate_lane<MIX, 0>(case_b, RF_BETA_HEI + t, L, v, ctl);
+    const double r = rate_f(v, ctl);
+    if constexpr (TS >= 4) {   // lanes beta_HeI, beta_HeII, alpha_HeII, alpha_HeIII
+        const double a2 = team_get<TS>(m, r, 2);
+        const double u = rfma(t < 2 ? 1.0 : t == 2 ? y2 : y3, r, t == 1 ? a2 : 0.0);
+        const double w = rfma(u, ne, t == 0 ? gam1 : t == 1 ? gam2 : 0.0);
+        const double z = rfma(w, h, t == 2 ? yI : 1.0);
+        D1 = team_get<TS>(m, w, 0);
+        P3 = team_get<TS>(m, w, 3);
+        den1 = team_get<TS>(m, z, 0);
+        den2 = team_get<TS>(m, z, 1);
+        num1 = team_get<TS>(m, z, 2);
+    } else {   // beta_HeI, beta_HeII, then alpha_HeII, alpha_HeIII
+        rate_lane<MIX, 0>(case_b, RF_BETA_HEI + 2 + t, L, v, ctl);
+        const double a = rate_f(v, ctl), a2 = team_get<TS>(m, a, 0);
+        const double w = rfma(radd(r, t == 0 ? 0.0 : a2), ne, t == 0 ? gam1 : gam2);
+        const double z = rfma(w, h, 1.0);
+        const double P = rmul(rmul(t == 0 ? y2 : y3, a), ne);
+        D1 = team_get<TS>(m, w, 0);
+        P3 = team_get<TS>(m, P, 1);
+        den1 = team_get<TS>(m, z, 0);
+        den2 = team_get<TS>(m, z, 1);
+        num1 = team_get<TS>(m, rfma(P, h, yI), 0);
+    }
+}
+// HeIII: C3 = y2 (beta_HeII n_e + Gamma_2), den3 = 1 + h alpha_HeIII n_e
+template <int TS, bool MIX, class CTL>
+__device__ __forceinline__ void he3_terms_team(const TLevel &L, int case_b, double y2, double ne, double gam2,
+                                               double h, double &C3, double &den3, CTL &ctl)
+{
+    const unsigned m = team_mask_c<TS, CTL>();
+    const bool b = team_lane<TS>() == 0;
+    RateVal v;
+    rate_lane<MIX, 0>(case_b, b ? RF_BETA_HEII : RF_ALPHA_HEIII, L, v, ctl);
+    const double w = rfma(rate_f(v, ctl), ne, b ? gam2 : 0.0);
+    const double z = rfma(w, b ? y2 : h, b ? 0.0 : 1.0);
+    C3 = team_get<TS>(m, z, 0);
+    den3 = team_get<TS>(m, z, 1);
 }
 // dual numbers, a team of eight: the level of the value, dT the tangent of T
 template <int TS, bool MIX, class CTL>
@@ -378,13 +481,13 @@ __device__ __forceinline__ void recomb_rates_team(double T, double nHII, double 
 // Photon update of one group, Eq. (SIE photons): N_i' = (N_i + h C_i)/(1 + h D_i)
 // (C_i = 0 under the OTSA; smoothed RT adds the rate Ndot_i), F_i scaled by
 // 1/(1 + h D_i), D_i = c_r sum_j sigma^N_ij n_j with the backward absorber
-// densities; with the group's 10% and 5% checks on N_i and its terms of the
-// photo-ionisation rates sigma^N_ij c_r N_i' (t0..t2) and of the
-// photoheating c_r N_i' sum_j n_j (egy_i sigma^E_ij - eps_j sigma^N_ij)
-// (tq).  Products and sums are rounded as written.
+// densities; with the group's 10% and 5% checks on N_i and the factors of its
+// terms of the photo-ionisation rates c_r N_i' sigma^N_ij and of the
+// photoheating c_r N_i' q, q = sum_j n_j (egy_i sigma^E_ij - eps_j sigma^N_ij).
+// Products and sums are rounded as written.
 template <typename S>
 struct PhotonTerms {
-    S Nn, Fs, Fb, t0, t1, t2, tq;
+    S Nn, Fs, Fb, crN, q;
     bool ok, small;
 };
 
@@ -419,16 +522,14 @@ __device__ __forceinline__ void photon_group(const ThermoParams &p, int i, const
     o.Nn = Nn;
     o.Fs = rmul(Fs, inv);
     if constexpr (SM) o.Fb = rmul(radd(Fb, S(h)), inv);
-    const S crN = rmul(Nn, p.cr);
-    o.t0 = rmul(crN, p.gc.sigN[i][0]);
-    o.t1 = rmul(crN, p.gc.sigN[i][1]);
-    o.t2 = rmul(crN, p.gc.sigN[i][2]);
-    o.tq = rmul(crN, rfma(p.hq[i][2], nHeII, rfma(p.hq[i][1], nHeI, rmul(nHI, p.hq[i][0]))));
+    o.crN = rmul(Nn, p.cr);
+    o.q = rfma(p.hq[i][2], nHeII, rfma(p.hq[i][1], nHeI, rmul(nHI, p.hq[i][0])));
 }
 
 // The photon stage of an attempt by a team of PT lanes (each with its own
 // groups), filling the lanes' new N_i and flux scales and, in every lane, the
-// photo-ionisation rates gam_j and the photoheating; false when a group
+// photo-ionisation rates gam_j and the photoheating, each summed over the
+// groups in one lane (a team of two: two in each); false when a group
 // breaks the 10% rule.  The recombination photons C_i (without the OTSA) come
 // from cc.rj.
 template <int G, int PT, bool MIX, bool SM, class CTL>
@@ -469,17 +570,22 @@ __device__ __forceinline__ bool photons_team(const ThermoParams &p, const CellSt
         ok = __all_sync(mask, ok);
         sm = sm && (__all_sync(mask, small) != 0);
     }
+    constexpr int NS = 4 / PT;   // sums per lane: t NS, t NS + 1, ... of gam0, gam1, gam2, heat
+    double sum[NS];
 #pragma unroll
     for (int i = 0; i < G; ++i) {
-        const PhotonTerms<double> &q = pt[i / PT];
-        const double t0 = team_get<PT>(mask, q.t0, i % PT), t1 = team_get<PT>(mask, q.t1, i % PT),
-                     t2 = team_get<PT>(mask, q.t2, i % PT), tq = team_get<PT>(mask, q.tq, i % PT);
-        if (i == 0) {
-            gam0 = t0; gam1 = t1; gam2 = t2; heat = tq;
-        } else {
-            gam0 = radd(gam0, t0); gam1 = radd(gam1, t1); gam2 = radd(gam2, t2); heat = radd(heat, tq);
+        const double crN = team_get<PT>(mask, pt[i / PT].crN, i % PT), q = team_get<PT>(mask, pt[i / PT].q, i % PT);
+#pragma unroll
+        for (int k = 0; k < NS; ++k) {
+            const int j = t * NS + k;
+            const double v = rmul(crN, j == 3 ? q : p.gc.sigN[i][j < 3 ? j : 2]);
+            sum[k] = i == 0 ? v : radd(sum[k], v);
         }
     }
+    gam0 = team_get<PT>(mask, sum[0], 0);
+    gam1 = team_get<PT>(mask, sum[1 % NS], 1 / NS);
+    gam2 = team_get<PT>(mask, sum[2 % NS], 2 / NS);
+    heat = team_get<PT>(mask, sum[3 % NS], 3 / NS);
     return ok;
 }
 
@@ -507,11 +613,12 @@ __device__ __forceinline__ bool photons_serial(const ThermoParams &p, const Cell
             o.Fb[i] = pt.Fb;
             o.Nd[i] = s.Nd[i];
         }
+        const S t0 = rmul(pt.crN, p.gc.sigN[i][0]), t1 = rmul(pt.crN, p.gc.sigN[i][1]),
+                t2 = rmul(pt.crN, p.gc.sigN[i][2]), tq = rmul(pt.crN, pt.q);
         if (i == 0) {
-            gam0 = pt.t0; gam1 = pt.t1; gam2 = pt.t2; heat = pt.tq;
+            gam0 = t0; gam1 = t1; gam2 = t2; heat = tq;
         } else {
-            gam0 = radd(gam0, pt.t0); gam1 = radd(gam1, pt.t1); gam2 = radd(gam2, pt.t2);
-            heat = radd(heat, pt.tq);
+            gam0 = radd(gam0, t0); gam1 = radd(gam1, t1); gam2 = radd(gam2, t2); heat = radd(heat, tq);
         }
     }
     return true;
@@ -547,12 +654,19 @@ __device__ __forceinline__ bool attempt(const ThermoParams &p, const S &nH, cons
     const S nHe = iso.nHe;
     const S x = s.x, y2 = s.y2, y3 = s.y3;
     const S q0 = he_electrons(y2, y3);
-    const S nHI = rmul(nH, radd(S(1.0), -x));
+    const S xI = radd(S(1.0), -x);
     const S nHII = rmul(nH, x);
     const S yI = radd(radd(S(1.0), -y2), -y3);
-    const S nHeI = rmul(nHe, yI);
-    const S nHeII = rmul(nHe, y2);
-    const S nHeIII = rmul(nHe, y3);
+    S nHI, nHeI, nHeII, nHeIII;
+    constexpr bool team = TS > 1 && !dual;
+    if constexpr (team) {
+        densities_team<TS, CTL>(nH, nHe, xI, yI, y2, y3, nHI, nHeI, nHeII, nHeIII);
+    } else {
+        nHI = rmul(nH, xI);
+        nHeI = rmul(nHe, yI);
+        nHeII = rmul(nHe, y2);
+        nHeIII = rmul(nHe, y3);
+    }
     const S ne = ne_of(nHII, q0, nHe);
     const S mhe = md_he(p, q0);
     bool sm = true;
@@ -577,7 +691,7 @@ __device__ __forceinline__ bool attempt(const ThermoParams &p, const S &nH, cons
                          ctl);
         } else if constexpr (TS > 1) {
             const double2 c = cooling_sums_team<TS, MIX>(p.case_b, helium, s.T, nHI, nHII, nHeI, nHeII, nHeIII, ctl);
-            cooling_close(p.comp, p.tg, s.T, ne, c.x, c.y, cc.L, cc.dL);
+            cooling_close_team<TS, CTL>(p.comp, p.tg, s.T, ne, c.x, c.y, cc.L, cc.dL);
         } else {
             cooling_serial<MIX>(p.case_b, p.comp, p.tg, helium, s.T, ne, nHI, nHII, nHeI, nHeII, nHeIII, cc.L,
                                 cc.dL);
@@ -614,27 +728,51 @@ __device__ __forceinline__ bool attempt(const ThermoParams &p, const S &nH, cons
     // 1/(T/mu') as a pair, for the temperatures (T/mu') mu_j of steps 3 and 4
     const dfm::F2 iT = isothermal ? dfm::F2{0.0f, 0.0f} : inv_pair(val(Tmu1), ctl);
 
-    // 3. hydrogen
-    HRatesT<S> hr;
-    if (isothermal) {
-        hr = iso.h;
+    // 3. hydrogen: C = beta n_e + Gamma, D = alpha n_e and their derivatives
+    S beta, alpha, dC, dD;
+    // - n_e (T/mu') mu^2 X d/dT
+    const S f = isothermal ? S(0.0) : rmul(rmul(ne, rmul(Tmu1, mu)), rmul(-mu, p.X));
+    if (team && !isothermal) {
+        if constexpr (team) {
+            TLevel L;
+            level_mu(mden, iT, Tmu1, L, ctl);
+            h_terms_team<TS, MIX>(L, p.case_b, nH, f, beta, alpha, dC, dD, ctl);
+        }
     } else {
-        TLevel L;
-        const double dT = level_mu(mden, iT, Tmu1, L, ctl);
-        h_rates<TS, MIX>(L, dT, p.case_b, hr, ctl);
+        HRatesT<S> hr;
+        if (isothermal) {
+            hr = iso.h;
+        } else {
+            TLevel L;
+            const double dT = level_mu(mden, iT, Tmu1, L, ctl);
+            h_rates<TS, MIX>(L, dT, p.case_b, hr, ctl);
+        }
+        beta = hr.beta;
+        alpha = hr.alpha;
+        dC = rmul(nH, hr.beta);
+        dD = rmul(nH, hr.alpha);
+        if (!isothermal) {
+            dC = rfma(f, hr.dbeta, dC);
+            dD = rfma(f, hr.dalpha, dD);
+        }
     }
-    const S C = rfma(hr.beta, ne, gam0);
-    const S CD = rfma(hr.alpha, ne, C);   // C + D, D = alpha n_e
-    S dC = rmul(nH, hr.beta), dD = rmul(nH, hr.alpha);
-    if (!isothermal) {
-        // - n_e (T/mu') mu^2 X d/dT
-        const S f = rmul(rmul(ne, rmul(Tmu1, mu)), rmul(-mu, p.X));
-        dC = rfma(f, hr.dbeta, dC);
-        dD = rfma(f, hr.dalpha, dD);
+    const S C = rfma(beta, ne, gam0);
+    const S CD = rfma(alpha, ne, C);   // C + D
+    // h (C - x (C + D)) and 1 - h J, J = dC - C - D - x (dC + dD)
+    S hx, den;
+    if constexpr (team) {
+        const unsigned m = team_mask_c<TS, CTL>();
+        const bool j = team_lane<TS>() == 0;
+        const double v = rfma(-x, j ? radd(dC, dD) : CD, j ? radd(dC, -CD) : C);
+        const double z = rfma(j ? -v : v, h, j ? 1.0 : 0.0);
+        den = team_get<TS>(m, z, 0);
+        hx = team_get<TS>(m, z, 1);
+    } else {
+        const S J = rfma(-x, radd(dC, dD), radd(dC, -CD));
+        hx = rmul(rfma(-x, CD, C), h);
+        den = rfma(-J, S(h), S(1.0));
     }
-    const S J = rfma(-x, radd(dC, dD), radd(dC, -CD));
-    const S hx = rmul(rfma(-x, CD, C), h);
-    S x1 = radd(x, cdiv(hx, rfma(-J, S(h), S(1.0)), ctl));
+    S x1 = radd(x, cdiv(hx, den, ctl));
     x1 = min0(max0(x1, kXMin), 1.0);
     if (!change_ok(x1, x, S(kXMin), sm, ctl)) return false;
     if (!term_ok(hx, max0(x, kXMin), ctl)) return false;
@@ -644,33 +782,54 @@ __device__ __forceinline__ bool attempt(const ThermoParams &p, const S &nH, cons
     const S nHII1 = rmul(x1, nH);
     if (helium) {
         const S ne2 = ne_of(nHII1, q0, nHe);
-        HeRatesT<S> r2;
-        if (isothermal) {
-            r2 = iso.he;
-        } else {
-            TLevel L;
-            const double dT = level_mu(mu_den(p, x1, mhe), iT, Tmu1, L, ctl);
-            he_rates<TS, MIX>(L, dT, p.case_b, r2, ctl);
-        }
         const S hs(h);
-        const S D1 = rfma(r2.beta_HeI, ne2, gam1);
-        const S yI1 = cdiv(rfma(rmul(rmul(y2, r2.alpha_HeII), ne2), hs, yI), rfma(D1, hs, S(1.0)), ctl);
-        const S C2 = rfma(yI1, D1, rmul(rmul(y3, r2.alpha_HeIII), ne2));
-        const S D2 = rfma(radd(r2.beta_HeII, r2.alpha_HeII), ne2, gam2);
-        y2n = cdiv(rfma(C2, hs, y2), rfma(D2, hs, S(1.0)), ctl);
+        S D1, P3, num1, den1, den2;
+        if (team && !isothermal) {
+            if constexpr (team) {
+                TLevel L;
+                level_mu(mu_den(p, x1, mhe), iT, Tmu1, L, ctl);
+                he_terms_team<TS, MIX>(L, p.case_b, y2, y3, yI, ne2, gam1, gam2, h, D1, P3, num1, den1, den2, ctl);
+            }
+        } else {
+            HeRatesT<S> r2;
+            if (isothermal) {
+                r2 = iso.he;
+            } else {
+                TLevel L;
+                const double dT = level_mu(mu_den(p, x1, mhe), iT, Tmu1, L, ctl);
+                he_rates<TS, MIX>(L, dT, p.case_b, r2, ctl);
+            }
+            D1 = rfma(r2.beta_HeI, ne2, gam1);
+            P3 = rmul(rmul(y3, r2.alpha_HeIII), ne2);
+            num1 = rfma(rmul(rmul(y2, r2.alpha_HeII), ne2), hs, yI);
+            den1 = rfma(D1, hs, S(1.0));
+            den2 = rfma(rfma(radd(r2.beta_HeII, r2.alpha_HeII), ne2, gam2), hs, S(1.0));
+        }
+        const S yI1 = cdiv(num1, den1, ctl);
+        const S C2 = rfma(yI1, D1, P3);
+        y2n = cdiv(rfma(C2, hs, y2), den2, ctl);
         const S q1 = he_electrons(y2n, y3);
         const S ne3 = ne_of(nHII1, q1, nHe);
-        HeRatesT<S> r3;
-        if (isothermal) {
-            r3 = iso.he;
+        S C3, den3;
+        if (team && !isothermal) {
+            if constexpr (team) {
+                TLevel L;
+                level_mu(mu_den(p, x1, md_he(p, q1)), iT, Tmu1, L, ctl);
+                he3_terms_team<TS, MIX>(L, p.case_b, y2n, ne3, gam2, h, C3, den3, ctl);
+            }
         } else {
-            TLevel L;
-            const double dT = level_mu(mu_den(p, x1, md_he(p, q1)), iT, Tmu1, L, ctl);
-            he3_rates<TS, MIX>(L, dT, p.case_b, r3, ctl);
+            HeRatesT<S> r3;
+            if (isothermal) {
+                r3 = iso.he;
+            } else {
+                TLevel L;
+                const double dT = level_mu(mu_den(p, x1, md_he(p, q1)), iT, Tmu1, L, ctl);
+                he3_rates<TS, MIX>(L, dT, p.case_b, r3, ctl);
+            }
+            C3 = rmul(y2n, rfma(r3.beta_HeII, ne3, gam2));
+            den3 = rfma(rmul(r3.alpha_HeIII, ne3), hs, S(1.0));
         }
-        const S C3 = rmul(y2n, rfma(r3.beta_HeII, ne3, gam2));
-        const S D3 = rmul(r3.alpha_HeIII, ne3);
-        y3n = cdiv(rfma(C3, hs, y3), rfma(D3, hs, S(1.0)), ctl);
+        y3n = cdiv(rfma(C3, hs, y3), den3, ctl);
         // conservation: lower the largest fraction (HeI largest: no change);
         // (the fractions are positive or zero: compared by their bits)
         const long long bI = dbits(val(yI1)), b2 = dbits(val(y2n)), b3 = dbits(val(y3n));
