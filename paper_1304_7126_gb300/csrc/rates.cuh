@@ -705,7 +705,7 @@ __device__ __forceinline__ void cool_densities(const S &nHI, const S &nHII, cons
     n[SP_HEI] = nHeI;
     n[SP_HEII] = nHeII;
     n[SP_HEIII] = nHeIII;
-    n[SP_FF] = radd(radd(nHII, nHeII), rmul(nHeIII, 4.0));
+    n[SP_FF] = rfma(4.0, nHeIII, radd(nHII, nHeII));
 }
 
 // a density as a pair (below 2^-70, 1e-21 of the smallest electron density
@@ -748,8 +748,7 @@ template <typename S>
 __device__ __forceinline__ void cooling_close(double comp, double tg, const S &T, const S &ne, const S &Ls,
                                               const S &dLs, S &L, S &dL)
 {
-    const S vp = rmul(radd(T, S(-tg)), comp);
-    L = rmul(ne, radd(Ls, vp));
+    L = rmul(ne, rfma(comp, radd(T, S(-tg)), Ls));
     dL = rmul(ne, radd(dLs, S(comp)));
 }
 

@@ -74,7 +74,7 @@ struct ThermoParams {
     GroupConsts gc;
     // derived per-group terms of the photon update (derive_group_terms):
     double crs[kMaxG][3];    // c_r sigma^N_ij, the absorption coefficient per absorber
-    double hq[kMaxG][3];     // egy_i sigma^E_ij - eps_j sigma^N_ij, photoheating per absorber
+    double hq[kMaxG][3];     // c_r (egy_i sigma^E_ij - eps_j sigma^N_ij), photoheating per absorber
     double mu_0, mu_w;       // 1/mu = X x + mu_0 + mu_w (y2 + 2 y3): X + (1 - X)/4, (1 - X)/4
     double tg;               // T_gamma = 2.727 / a, the Compton temperature
     double comp;             // 1.017e-37 T_gamma^4, Compton exchange per (T - T_gamma) n_e
@@ -92,7 +92,7 @@ inline void derive_group_terms(ThermoParams &p)
     for (int i = 0; i < kMaxG; ++i)
         for (int j = 0; j < 3; ++j) {
             p.crs[i][j] = p.cr * p.gc.sigN[i][j];
-            p.hq[i][j] = p.gc.egy[i] * p.gc.sigE[i][j] - eps[j] * p.gc.sigN[i][j];
+            p.hq[i][j] = p.cr * (p.gc.egy[i] * p.gc.sigE[i][j] - eps[j] * p.gc.sigN[i][j]);
         }
     // Compton cooling/heating of the rate appendix, varpi = 1.017e-37 T_g^4 (T - T_g)
     p.mu_w = 0.25 * (1.0 - p.X);
