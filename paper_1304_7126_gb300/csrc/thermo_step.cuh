@@ -313,7 +313,8 @@ __device__ __forceinline__ void cooling_close_team(double comp, double tg, doubl
     L = team_get<TS>(m, z, 0);
     dL = team_get<TS>(m, z, 1);
 }
-// Hydrogen: beta, alpha, dC = n_H beta + f dbeta/dT, dD = n_H alpha + f dalpha/dT
+// Hydrogen: beta, alpha, dC = n_H beta + f T dbeta/dT, dD = n_H alpha + f T
+// dalpha/dT
 template <int TS, bool MIX, class CTL>
 __device__ __forceinline__ void h_terms_team(const TLevel &L, int case_b, double nH, double f, double &beta,
                                              double &alpha, double &dC, double &dD, CTL &ctl)
@@ -321,7 +322,7 @@ __device__ __forceinline__ void h_terms_team(const TLevel &L, int case_b, double
     const unsigned m = team_mask_c<TS, CTL>();
     RateVal v;
     rate_lane<MIX, 1>(case_b, team_lane<TS>() == 0 ? RF_BETA_HI : RF_ALPHA_HII, L, v, ctl);
-    const double r = rate_f(v, ctl), d = rfma(f, rate_df(v, L, ctl), rmul(nH, r));
+    const double r = rate_f(v, ctl), d = rfma(f, rate_tdf(v, ctl), rmul(nH, r));
     beta = team_get<TS>(m, r, 0);
     alpha = team_get<TS>(m, r, 1);
     dC = team_get<TS>(m, d, 0);
@@ -736,8 +737,9 @@ __device__ __forceinline__ bool attempt(const ThermoParams &p, const S &nH, cons
 
     // 3. hydrogen: C = beta n_e + Gamma, D = alpha n_e and their derivatives
     S beta, alpha, dC, dD;
-    // - n_e (T/mu') mu^2 X d/dT
-    const S f = isothermal ? S(0.0) : rmul(rmul(ne, rmul(Tmu1, mu)), rmul(-mu, p.X));
+    // d/dx at constant T/mu' through T = (T/mu') mu: - n_e (T/mu') mu^2 X d/dT =
+    // - n_e mu X (T d/dT)
+    const S f = isothermal ? S(0.0) : rmul(rmul(ne, mu), -p.X);
     if (team && !isothermal) {
         if constexpr (team) {
             TLevel L;
@@ -758,8 +760,8 @@ __device__ __forceinline__ bool attempt(const ThermoParams &p, const S &nH, cons
         dC = rmul(nH, hr.beta);
         dD = rmul(nH, hr.alpha);
         if (!isothermal) {
-            dC = rfma(f, hr.dbeta, dC);
-            dD = rfma(f, hr.dalpha, dD);
+            dC = rfma(f, hr.tbeta, dC);
+            dD = rfma(f, hr.talpha, dD);
         }
     }
     const S C = rfma(beta, ne, gam0);
