@@ -42,9 +42,9 @@ PASS1_ATTEMPTS = 6
 LONG_ATTEMPTS = 134
 # DRAM bytes (read + write) per launch, from the ncu captures of the current
 # kernels summarised in profiles/ (128^3 x 3 groups, HLL)
-TRAFFIC = {"transport": 399187712 + 192541696,
+TRAFFIC = {"transport": 395040768 + 185719808,
            # thermo_team, both stages
-           "thermo_drain": 325376}
+           "thermo_drain": 65536 + 812288 + 256}
 
 
 def _op_counts():

@@ -212,7 +212,7 @@ struct QueueView {
 // lanes share the cell's rate functions and photon groups and, where they
 // can, its FP64 terms (one FP64 instruction with a term per lane).  An
 // attempt is a chain of dependent FP32 pair and FP64 operations; on a warp
-// alone it takes 7.1 us with teams of four (7.9 before the FP64 terms were
+// alone it takes 7.0 us with teams of four (7.9 before the FP64 terms were
 // shared), whether the warp holds one cell or eight, and two warps per SM
 // sub-partition come close to filling the FP64 pipe.  (A pair of warps per
 // cell was no shorter and spent sixteen times the issue slots and FP64

@@ -30,7 +30,8 @@
 // 64-bit fixed point (2^-62) from the table to the face, where they enter
 // FP64 as the two weights of Eq. (hll); reciprocals and square roots start
 // from float pairs (dfmath.cuh) and take two or three FP64 instructions.
-// About 150 FP64 instructions per cell and group (302 before): 3.44 -> 2.0 ms
+// 151 FP64 instructions per cell and group (302 before): 3.72 -> 2.06 ms
+// with photons in every cell, 3.44 -> 1.58 ms with a third of them empty,
 // at 128^3 x 3 groups, HLL.
 #include <cuda_runtime.h>
 
