@@ -569,9 +569,9 @@ int rt_batch_create(int n_boxes, const rt_grid *grids, const int *n_groups, cons
         std::vector<double> tab((size_t)kHllNF * kHllNMU * 2);
         rtgb::hll_table(kHllNF, kHllNMU, tab.data());
         if (!b->mixed) {
-            const std::vector<long long> tq = hll_fix_table(tab);
-            if ((rc = balloc(b, &b->hllq, tq.size()))) goto bad;
-            cudaMemcpy(b->hllq, tq.data(), tq.size() * sizeof(long long), cudaMemcpyHostToDevice);
+            hll_fix_table(tab);
+            if ((rc = balloc(b, &b->hllq, tab.size()))) goto bad;
+            cudaMemcpy(b->hllq, tab.data(), tab.size() * sizeof(long long), cudaMemcpyHostToDevice);
         } else {
             std::vector<float> tf(tab.begin(), tab.end());
             if ((rc = balloc(b, &b->hllf, tf.size()))) goto bad;

@@ -502,9 +502,9 @@ int rt_create(const rt_grid *grid, int n_groups, const rt_options *opt, double c
             rc = cuda_fail(h, e, "hll copy"); goto bad;
         }
         if (!h->mixed) {
-            const std::vector<long long> tabq = hll_fix_table(tab);
-            if ((rc = dalloc(h, &h->hllq, tabq.size()))) goto bad;
-            if ((e = cudaMemcpy(h->hllq, tabq.data(), tabq.size() * sizeof(long long), cudaMemcpyHostToDevice)) !=
+            hll_fix_table(tab);
+            if ((rc = dalloc(h, &h->hllq, tab.size()))) goto bad;
+            if ((e = cudaMemcpy(h->hllq, tab.data(), tab.size() * sizeof(long long), cudaMemcpyHostToDevice)) !=
                 cudaSuccess) {
                 rc = cuda_fail(h, e, "hll copy"); goto bad;
             }
