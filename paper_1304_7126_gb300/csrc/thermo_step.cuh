@@ -556,7 +556,7 @@ __device__ __forceinline__ bool photons_team(const ThermoParams &p, const CellSt
             for (int j = 0; j < 3; ++j)
                 if (mine && p.rec_g[j] == gi) Crec += cc.rj[j];
         }
-        // (a lane without a group of this round runs group 0 on zeros, which changes nothing)
+        // (a lane without a group here runs group 0 on zeros, which changes nothing)
         photon_group<MIX, SM>(p, gi, s.N[r], s.Fs[r], s.Nd[r], s.Fb[r], Crec, nHI, nHeI, nHeII, h, pt[r], ctl);
         ok = ok && (pt[r].ok || !mine);
         small = small && (pt[r].small || !mine);
