@@ -242,9 +242,11 @@ int rt_hll_table(int nf, int nmu, double *out);
  * of four lanes per cell for the rest.  Routing decides which kernel runs
  * which attempts of a cell, never the arithmetic of an attempt: x_HII,
  * x_HeII, x_HeIII, T, N, F and the attempt counts are identical for every
- * routing (a queued cell carries its flux scale prod 1/(1 + h D_i), and F is
- * formed once, when the cell finishes).  Values <= 0 (drain2_min_cells < 0) restore the defaults: 6,
- * 8, 8 and 64 cells per SM.  Takes effect at the next step. */
+ * routing (a queued cell carries its N in FP64 and its flux scale
+ * prod 1/(1 + h D_i); N is rounded to the precision of the photon state, and
+ * F formed, once, when the cell finishes), and repeated runs give the same
+ * bits.  Values <= 0 (drain2_min_cells < 0) restore the defaults: 6, 8, 8 and
+ * 64 cells per SM.  Takes effect at the next step. */
 int rt_set_thermo_routing(rt_handle *h, int pass1_attempts, int drain_budget, int drain2_budget,
                           long long drain2_min_cells);
 

@@ -326,6 +326,7 @@ int enqueue_batch_step(rt_batch *b, double dt)
     b->cur = nxt;
     for (ClassData &c : b->cls) {
         ThermoParams tp = class_params(b, c, dt);
+        c.q.N = (double *)c.F[1 - b->cur];
         if (f32)
             e = launch_thermo_mixed(tp, c.G, b->opt.precision == RT_MIXED32, c.nH, c.xHII, c.xHeII, c.xHeIII, c.T,
                                     (float *)c.N[b->cur], (float *)c.F[b->cur], nullptr, nullptr, c.sub, c.q,

@@ -235,6 +235,7 @@ int enqueue_step(rt_handle *h, double dt, bool capturing = false)
     if (prof) cudaEventRecord(b, h->stream);
     h->cur = nxt;
     ThermoParams tp = thermo_params(h, dt);
+    h->q.N = h->mixed ? reinterpret_cast<double *>(h->Ff[1 - h->cur]) : h->F[1 - h->cur];
     cudaEvent_t tev[4];
     if (prof) {
         prof_pair(h, 2, &tev[0], &tev[1]);

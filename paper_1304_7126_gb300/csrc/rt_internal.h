@@ -129,6 +129,9 @@ struct Queue {
     long long capacity;             // items per queue
     double *fscale;                 // [2G][nc]: a queued cell's flux scale Fs_i (rows 0..G-1) and,
                                     // smoothed RT, its Fdot weight Fb_i (rows G..2G-1)
+    double *N;                      // [G][nc]: a queued cell's N_i in FP64 (RT_MIXED and smoothed RT; memory
+                                    // that is free during the thermochemistry: the flux buffer of the state
+                                    // before transport, 12 bytes or more per cell and group)
 };
 
 // Per-block partial sums of the photon budget.

@@ -28,7 +28,8 @@
 //                 photon groups while the scalar update runs redundantly in
 //                 all of them.
 // The arithmetic is the same in all of them, and a queued cell carries its
-// flux scale, so results do not depend on which kernel finished a cell.
+// photon densities in FP64 and its flux scale, so results do not depend on
+// which kernel ran which of a cell's attempts.
 // Nothing waits on another thread; each kernel ends when its queue is empty.
 // The kernels live in thermo_kernels.cuh, instantiated per precision family
 // in thermo_f64.cu, thermo_mix.cu, thermo_mix32.cu and their smoothed-RT

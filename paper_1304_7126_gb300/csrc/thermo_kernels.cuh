@@ -6,14 +6,20 @@
 // families compile in parallel.
 //
 // Smoothed RT: on entry N, F hold the result N', F' of injection and
-// transport and Npre, Fpre the state before them.  The first pass loads
-// N^t = Npre and Ndot = (N' - N^t)/dt per group; a cell's flux is kept as
-// F = Fs F_base + Fb Fdot with Fs = prod 1/(1 + h D), Fb = sum h prod
-// 1/(1 + h D) over its accepted sub-steps.  A cell handed to a queue
-// leaves its partial N, F in N, F and its Ndot, Fdot in Npre, Fpre.
+// transport and Npre, Fpre the state before them.  A cell starts from
+// N^t = Npre with Ndot = (N' - N^t)/dt per group; its flux is kept as
+// F = Fs Fpre + Fb Fdot, Fdot = (F' - Fpre)/dt, with Fs = prod 1/(1 + h D),
+// Fb = sum h prod 1/(1 + h D) over its accepted sub-steps.
+//
+// A cell handed to a queue keeps its N in FP64 beside its flux scales (N
+// itself is rounded to P once, when the cell finishes), and N', F', Npre,
+// Fpre stay as they are until then: which kernel runs which of its attempts
+// depends on timing and must not show in the result.
 #pragma once
 
 #include <cuda_runtime.h>
+
+#include <type_traits>
 
 #include "rates.cuh"
 #include "rt_internal.h"
@@ -28,12 +34,19 @@ constexpr int kPass1Block = 128;
 constexpr double kLongSteps = 32.0; // sub-steps ahead from which a queued cell is taken early
 constexpr double kHandSteps = 8.0;  // ... from which it moves to the second stage
 
+// a queued cell's N in Queue::N; else (RT_FP64 without smoothing) in N, exactly
+template <typename P, bool SM>
+__host__ __device__ constexpr bool queue_keeps_N()
+{
+    return SM || !std::is_same<P, double>::value;
+}
+
 // first: the cell's first load in this RT step (thermo_pass1).  PT: 1, or the
 // lanes of the cell's team, each of which loads and stores its own groups
 template <int G, int PT, typename P, bool R32, bool SM>
 __device__ __forceinline__ void load_cell(const ThermoParams &p, long long c, bool first, const double *xHII,
                                           const double *xHeII, const double *xHeIII, const double *T,
-                                          const P *N, const P *Npre, const double *fscale,
+                                          const P *N, const P *Npre, const Queue &q,
                                           CellState<lane_groups<>(G, PT)> &st, IsoRates<> &iso, CoolCache<> &cc)
 {
     st.x = xHII[c];
@@ -49,19 +62,16 @@ __device__ __forceinline__ void load_cell(const ThermoParams &p, long long c, bo
         if (PT > 1 && i >= G) continue;
         const long long k = (long long)i * p.nc + c;
         if constexpr (SM) {
-            if (first) {
-                const double n0 = (double)Npre[k];
-                st.Nd[r] = ((double)N[k] - n0) / p.dt;   // Eq. (smoothrate1)
-                st.N[r] = n0;
-            } else {
-                st.N[r] = (double)N[k];
-                st.Nd[r] = (double)Npre[k];
-            }
-            st.Fb[r] = first ? 0.0 : fscale[(long long)(G + i) * p.nc + c];
+            const double n0 = (double)Npre[k];
+            st.Nd[r] = ((double)N[k] - n0) / p.dt;   // Eq. (smoothrate1)
+            st.N[r] = first ? n0 : q.N[k];
+            st.Fb[r] = first ? 0.0 : q.fscale[(long long)(G + i) * p.nc + c];
+        } else if constexpr (queue_keeps_N<P, SM>()) {
+            st.N[r] = first ? (double)N[k] : q.N[k];
         } else {
             st.N[r] = (double)N[k];
         }
-        st.Fs[r] = first ? 1.0 : fscale[k];
+        st.Fs[r] = first ? 1.0 : q.fscale[k];
     }
     cc.valid = false;
     cc.rvalid = false;
@@ -74,14 +84,14 @@ __device__ __forceinline__ void load_cell(const ThermoParams &p, long long c, bo
     }
 }
 
-// handoff: the cell goes to a queue unfinished.  Its flux scale (and Fdot
-// weight) then goes to fscale and F keeps F_base: the flux is formed once,
-// when the cell finishes, so it does not depend on where it sub-cycled.
+// handoff: the cell goes to a queue unfinished.  Its N, flux scale and (smoothed
+// RT) Fdot weight then go to the queue's arrays, and the flux is formed once,
+// when the cell finishes, so neither depends on where it sub-cycled.
 template <int G, int PT, typename P, bool SM>
-__device__ __forceinline__ void store_cell(const ThermoParams &p, long long c, bool first, bool handoff,
-                                           double *xHII, double *xHeII, double *xHeIII, double *T, P *N, P *F,
-                                           P *Npre, P *Fpre, double *fscale,
-                                           const CellState<lane_groups<>(G, PT)> &st, unsigned *status)
+__device__ __forceinline__ void store_cell(const ThermoParams &p, long long c, bool handoff, double *xHII,
+                                           double *xHeII, double *xHeIII, double *T, P *N, P *F, const P *Fpre,
+                                           const Queue &q, const CellState<lane_groups<>(G, PT)> &st,
+                                           unsigned *status)
 {
     if (team_lane<PT>() == 0) {
         xHII[c] = st.x;
@@ -94,34 +104,25 @@ __device__ __forceinline__ void store_cell(const ThermoParams &p, long long c, b
     for (int r = 0; r < lane_groups<>(G, PT); ++r) {
         const int i = r * PT + team_lane<PT>();
         if (PT > 1 && i >= G) continue;
-        N[(long long)i * p.nc + c] = (P)st.N[r];
+        const long long k = (long long)i * p.nc + c;
         bad |= !isfinite(st.N[r]);
         if (handoff) {
-            fscale[(long long)i * p.nc + c] = st.Fs[r];
-            if constexpr (SM) fscale[(long long)(G + i) * p.nc + c] = st.Fb[r];
+            if constexpr (queue_keeps_N<P, SM>()) q.N[k] = st.N[r];
+            else N[k] = st.N[r];
+            q.fscale[k] = st.Fs[r];
+            if constexpr (SM) q.fscale[(long long)(G + i) * p.nc + c] = st.Fb[r];
+            continue;
         }
+        N[k] = (P)st.N[r];
         if constexpr (SM) {
-            if (handoff && !first) continue;
 #pragma unroll
             for (int d = 0; d < 3; ++d) {
                 const long long b = (3LL * i + d) * p.nc + c;
-                double base, fd;
-                if (first) {
-                    base = (double)Fpre[b];
-                    fd = ((double)F[b] - base) / p.dt;   // Eq. (smoothrate2)
-                } else {
-                    base = (double)F[b];
-                    fd = (double)Fpre[b];
-                }
-                if (handoff) {
-                    F[b] = Fpre[b];
-                    Fpre[b] = (P)fd;
-                } else {
-                    F[b] = (P)(st.Fs[r] * base + st.Fb[r] * fd);
-                }
+                const double base = (double)Fpre[b];
+                const double fd = ((double)F[b] - base) / p.dt;   // Eq. (smoothrate2)
+                F[b] = (P)(st.Fs[r] * base + st.Fb[r] * fd);
             }
-            if (handoff) Npre[(long long)i * p.nc + c] = (P)st.Nd[r];
-        } else if (!handoff && st.Fs[r] != 1.0) {
+        } else if (st.Fs[r] != 1.0) {
             long long b = 3LL * i * p.nc + c;
             const P f = (P)st.Fs[r];
             F[b] *= f;
@@ -150,7 +151,7 @@ __device__ __forceinline__ void push_item(const QueueArrays &a, unsigned long lo
 template <int G, typename P, bool R32, bool SM>
 __global__ void __launch_bounds__(kPass1Block, 4)
 thermo_pass1(ThermoParams p, const double *__restrict__ nH, double *xHII, double *xHeII, double *xHeIII,
-             double *T, P *N, P *F, P *Npre, P *Fpre, int32_t *subcycles, Queue q, unsigned *status)
+             double *T, P *N, P *F, const P *Npre, const P *Fpre, int32_t *subcycles, Queue q, unsigned *status)
 {
     long long c = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     bool valid = c < p.nc;
@@ -161,7 +162,7 @@ thermo_pass1(ThermoParams p, const double *__restrict__ nH, double *xHII, double
         CellState<G> st;
         IsoRates<> iso;
         CoolCache<> cc;
-        load_cell<G, 1, P, R32, SM>(p, c, true, xHII, xHeII, xHeIII, T, N, Npre, q.fscale, st, iso, cc);
+        load_cell<G, 1, P, R32, SM>(p, c, true, xHII, xHeII, xHeIII, T, N, Npre, q, st, iso, cc);
         double n = nH[c];
         cell_constants(p, n, iso);
         bool done = false;
@@ -172,7 +173,7 @@ thermo_pass1(ThermoParams p, const double *__restrict__ nH, double *xHII, double
             atomicOr(status, kStatusSubcycle);
             done = true;
         }
-        store_cell<G, 1, P, SM>(p, c, true, !done, xHII, xHeII, xHeIII, T, N, F, Npre, Fpre, q.fscale, st, status);
+        store_cell<G, 1, P, SM>(p, c, !done, xHII, xHeII, xHeIII, T, N, F, Fpre, q, st, status);
         if (done) subcycles[c] = att;
         else push = true;
     }
@@ -233,7 +234,7 @@ struct QueueView {
 template <int G, int TS, typename P, bool R32, bool SM>
 __global__ void __launch_bounds__(128, TS == 2 ? 4 : 2)
 thermo_team(ThermoParams p, const double *__restrict__ nH, double *xHII, double *xHeII, double *xHeIII,
-            double *T, P *N, P *F, P *Npre, P *Fpre, int32_t *subcycles, Queue q, unsigned *status,
+            double *T, P *N, P *F, const P *Npre, const P *Fpre, int32_t *subcycles, Queue q, unsigned *status,
             unsigned few_blocks)
 {
     constexpr int stage = TS == 2 ? 1 : 2;
@@ -273,7 +274,7 @@ thermo_team(ThermoParams p, const double *__restrict__ nH, double *xHII, double 
         att = src.attempts[sl];
         used = 0;
         n = nH[c];
-        load_cell<G, TS, P, R32, SM>(p, c, false, xHII, xHeII, xHeIII, T, N, Npre, q.fscale, st, iso, cc);
+        load_cell<G, TS, P, R32, SM>(p, c, false, xHII, xHeII, xHeIII, T, N, Npre, q, st, iso, cc);
         cell_constants(p, n, iso);
         return true;
     };
@@ -294,8 +295,7 @@ thermo_team(ThermoParams p, const double *__restrict__ nH, double *xHII, double 
             hand = k >= count && t_left > kHandSteps * dt_tc;   // the queue is empty
         }
         if (done || hand) {
-            store_cell<G, TS, P, SM>(p, c, false, hand, xHII, xHeII, xHeIII, T, N, F, Npre, Fpre, q.fscale, st,
-                                        status);
+            store_cell<G, TS, P, SM>(p, c, hand, xHII, xHeII, xHeIII, T, N, F, Fpre, q, st, status);
             if (t == 0) {
                 if (done) subcycles[c] = att;
                 else push_item(q.b, atomicAdd(&q.counters[3], 1ULL), q.capacity, (uint32_t)c, t_left, dt_tc, att, status);
