@@ -405,7 +405,10 @@ __device__ __noinline__ void rescale_flux(double nw[4], double c, double sc0)
 }
 __device__ __forceinline__ void realisable(double nw[4], double c)
 {
-    if (tbits(nw[0]) < 0) nw[0] = nw[1] = nw[2] = nw[3] = 0.0;   // (-0 included: its |F| <= c N is 0)
+    // bits from -0 (whose |F| <= c N is 0) to -infinity; those above are NaN and stay, for the
+    // thermochemistry to report (inf - inf and the like set a NaN's sign bit)
+    if ((unsigned long long)tbits(nw[0]) - (1ULL << 63) <= 0x7ff0000000000000ULL)
+        nw[0] = nw[1] = nw[2] = nw[3] = 0.0;
     const double cn = tmul(c, nw[0]);
     const long long m = max(max(tbits(tabs_(nw[1])), tbits(tabs_(nw[2]))), max(tbits(tabs_(nw[3])), tbits(cn)));
     const double F2 = tfma(nw[3], nw[3], tfma(nw[2], nw[2], tmul(nw[1], nw[1])));
