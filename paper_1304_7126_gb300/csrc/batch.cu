@@ -127,6 +127,22 @@ cudaError_t convert_rows(long long n, int rows, const A *in, long long in_row, B
     return cudaGetLastError();
 }
 
+// Rows of `width` bytes between arrays of different row lengths: one 2-D copy, or a
+// copy per row where a row length is above the limit that CUDA states for 2-D
+// copies (cudaDevAttrMaxPitch, 2^31 - 1 bytes: 2^28 cells of a class in FP64.
+// Driver 580.159 takes longer rows all the same.)
+cudaError_t copy_rows(size_t max_pitch, void *dst, size_t dst_pitch, const void *src, size_t src_pitch, size_t width,
+                      int rows, cudaMemcpyKind k, cudaStream_t s)
+{
+    if (dst_pitch <= max_pitch && src_pitch <= max_pitch)
+        return cudaMemcpy2DAsync(dst, dst_pitch, src, src_pitch, width, rows, k, s);
+    cudaError_t e = cudaSuccess;
+    for (int r = 0; r < rows && e == cudaSuccess; ++r)
+        e = cudaMemcpyAsync(static_cast<char *>(dst) + r * dst_pitch, static_cast<const char *>(src) + r * src_pitch, width,
+                            k, s);
+    return e;
+}
+
 __global__ void reset_counters_kernel(unsigned long long *c, int n)
 {
     if (threadIdx.x < n) c[threadIdx.x] = 0ULL;
@@ -140,6 +156,7 @@ struct rt_batch {
     rt_options opt{};
     bool mixed = false;
     int device = 0, n_sm = 1;
+    size_t max_pitch = 0;           // of 2-D copies, bytes
     cudaStream_t own_stream = nullptr, stream = nullptr;
     std::vector<BoxHost> box;
     std::vector<ClassData> cls;
@@ -493,15 +510,17 @@ int rt_batch_create(int n_boxes, const rt_grid *grids, const int *n_groups, cons
         bx.zc = 16;
         b->box.push_back(bx);
     }
-    int rc = RT_OK;
+    int rc = RT_OK, pitch = 0;
     cudaError_t e;
     if ((e = cudaGetDevice(&b->device)) != cudaSuccess ||
         (e = cudaDeviceGetAttribute(&b->n_sm, cudaDevAttrMultiProcessorCount, b->device)) != cudaSuccess ||
+        (e = cudaDeviceGetAttribute(&pitch, cudaDevAttrMaxPitch, b->device)) != cudaSuccess ||
         (e = cudaStreamCreateWithFlags(&b->own_stream, cudaStreamNonBlocking)) != cudaSuccess) {
         rc = bcuda(b, e, "setup");
         goto bad;
     }
     b->stream = b->own_stream;
+    b->max_pitch = (size_t)pitch;
     transport_init();
     {
         const size_t pb = b->mixed ? sizeof(float) : sizeof(double);
@@ -649,16 +668,16 @@ int rt_batch_set_box_state(rt_batch *b, int box, const double *nH, const double 
     for (int f = 0; f < 2; ++f) {
         const int rows = f ? 3 * G : G;
         if (!b->mixed) {
-            B_CUDA(b, cudaMemcpy2DAsync((double *)dst[f] + off, (size_t)c.nc * sizeof(double), src[f], bytes, bytes, rows, k,
-                                        b->stream));
+            B_CUDA(b, copy_rows(b->max_pitch, (double *)dst[f] + off, (size_t)c.nc * sizeof(double), src[f], bytes,
+                                bytes, rows, k, b->stream));
         } else if (device_ptrs) {
             cudaError_t e = convert_rows(nc, rows, src[f], nc, (float *)dst[f] + off, c.nc, b->stream);
             if (e != cudaSuccess) return bcuda(b, e, "convert");
         } else {
             const size_t row = (size_t)nc * sizeof(float);
             std::vector<float> tmp(src[f], src[f] + (size_t)rows * nc);
-            B_CUDA(b, cudaMemcpy2DAsync((float *)dst[f] + off, (size_t)c.nc * sizeof(float), tmp.data(), row, row, rows,
-                                        cudaMemcpyHostToDevice, b->stream));
+            B_CUDA(b, copy_rows(b->max_pitch, (float *)dst[f] + off, (size_t)c.nc * sizeof(float), tmp.data(), row,
+                                row, rows, cudaMemcpyHostToDevice, b->stream));
             B_CUDA(b, cudaStreamSynchronize(b->stream));
         }
     }
@@ -704,16 +723,16 @@ int rt_batch_get_box_state(rt_batch *b, int box, double *nH, double *xHII, doubl
         if (!dst[f]) continue;
         const int rows = f ? 3 * bx.G : bx.G;
         if (!b->mixed) {
-            B_CUDA(b, cudaMemcpy2DAsync(dst[f], bytes, (const double *)src[f] + off, (size_t)c.nc * sizeof(double), bytes,
-                                        rows, k, b->stream));
+            B_CUDA(b, copy_rows(b->max_pitch, dst[f], bytes, (const double *)src[f] + off,
+                                (size_t)c.nc * sizeof(double), bytes, rows, k, b->stream));
         } else if (device_ptrs) {
             cudaError_t e = convert_rows(nc, rows, (const float *)src[f] + off, c.nc, dst[f], nc, b->stream);
             if (e != cudaSuccess) return bcuda(b, e, "convert");
         } else {
             const size_t row = (size_t)nc * sizeof(float);
             std::vector<float> tmp((size_t)rows * nc);
-            B_CUDA(b, cudaMemcpy2DAsync(tmp.data(), row, (const float *)src[f] + off, (size_t)c.nc * sizeof(float), row, rows,
-                                        cudaMemcpyDeviceToHost, b->stream));
+            B_CUDA(b, copy_rows(b->max_pitch, tmp.data(), row, (const float *)src[f] + off,
+                                (size_t)c.nc * sizeof(float), row, rows, cudaMemcpyDeviceToHost, b->stream));
             B_CUDA(b, cudaStreamSynchronize(b->stream));
             for (size_t i = 0; i < tmp.size(); ++i) dst[f][i] = tmp[i];
         }
