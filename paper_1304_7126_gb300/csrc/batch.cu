@@ -143,6 +143,13 @@ cudaError_t copy_rows(size_t max_pitch, void *dst, size_t dst_pitch, const void 
     return e;
 }
 
+// rows of nc floats to stage in host memory at a time, of those left: 64 MB of them (a box of
+// 64^3 in one go), or one
+int staged_rows(long long nc, int left)
+{
+    return (int)std::max<long long>(1, std::min<long long>(left, (16LL << 20) / nc));
+}
+
 __global__ void reset_counters_kernel(unsigned long long *c, int n)
 {
     if (threadIdx.x < n) c[threadIdx.x] = 0ULL;
@@ -675,10 +682,14 @@ int rt_batch_set_box_state(rt_batch *b, int box, const double *nH, const double 
             if (e != cudaSuccess) return bcuda(b, e, "convert");
         } else {
             const size_t row = (size_t)nc * sizeof(float);
-            std::vector<float> tmp(src[f], src[f] + (size_t)rows * nc);
-            B_CUDA(b, copy_rows(b->max_pitch, (float *)dst[f] + off, (size_t)c.nc * sizeof(float), tmp.data(), row,
-                                row, rows, cudaMemcpyHostToDevice, b->stream));
-            B_CUDA(b, cudaStreamSynchronize(b->stream));
+            std::vector<float> tmp;
+            for (int r = 0, n; r < rows; r += n) {
+                n = staged_rows(nc, rows - r);
+                tmp.assign(src[f] + (size_t)r * nc, src[f] + (size_t)(r + n) * nc);
+                B_CUDA(b, copy_rows(b->max_pitch, (float *)dst[f] + off + (size_t)r * c.nc, (size_t)c.nc * sizeof(float),
+                                    tmp.data(), row, row, n, cudaMemcpyHostToDevice, b->stream));
+                B_CUDA(b, cudaStreamSynchronize(b->stream));
+            }
         }
     }
     if (!device_ptrs) B_CUDA(b, cudaStreamSynchronize(b->stream));
@@ -730,11 +741,14 @@ int rt_batch_get_box_state(rt_batch *b, int box, double *nH, double *xHII, doubl
             if (e != cudaSuccess) return bcuda(b, e, "convert");
         } else {
             const size_t row = (size_t)nc * sizeof(float);
-            std::vector<float> tmp((size_t)rows * nc);
-            B_CUDA(b, copy_rows(b->max_pitch, tmp.data(), row, (const float *)src[f] + off,
-                                (size_t)c.nc * sizeof(float), row, rows, cudaMemcpyDeviceToHost, b->stream));
-            B_CUDA(b, cudaStreamSynchronize(b->stream));
-            for (size_t i = 0; i < tmp.size(); ++i) dst[f][i] = tmp[i];
+            std::vector<float> tmp((size_t)staged_rows(nc, rows) * nc);
+            for (int r = 0, n; r < rows; r += n) {
+                n = staged_rows(nc, rows - r);
+                B_CUDA(b, copy_rows(b->max_pitch, tmp.data(), row, (const float *)src[f] + off + (size_t)r * c.nc,
+                                    (size_t)c.nc * sizeof(float), row, n, cudaMemcpyDeviceToHost, b->stream));
+                B_CUDA(b, cudaStreamSynchronize(b->stream));
+                std::copy(tmp.begin(), tmp.begin() + (size_t)n * nc, dst[f] + (size_t)r * nc);
+            }
         }
     }
     if (!device_ptrs) B_CUDA(b, cudaStreamSynchronize(b->stream));

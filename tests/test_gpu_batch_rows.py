@@ -33,3 +33,45 @@ def test_box_state_in_a_class_beyond_the_pitch_limit(prec, nbig, device):
         for k in s:
             assert np.array_equal(got[k], s[k]), (i, k)
     bt.close()
+
+
+STAGING = """
+import resource
+import numpy as np
+from paper_1304_7126_gb300 import rt as R
+from paper_1304_7126_gb300 import workloads as W
+w = W.stromgren32(152)                      # a row of 13.4 MB as float
+w.G = 8
+w.sigN, w.sigE, w.egy = np.repeat(w.sigN, 8, 0), np.repeat(w.sigE, 8, 0), np.repeat(w.egy, 8)
+bt = R.RTBatch([w], precision=R.RT_MIXED)
+rng = np.random.default_rng(2)
+s = w.state()
+for k in "NF":
+    rng.random(out=s[k])
+now = lambda: int([l for l in open("/proc/self/status") if l.startswith("VmRSS")][0].split()[1]) / 1024.0
+peak = lambda: resource.getrusage(resource.RUSAGE_SELF).ru_maxrss / 1024.0
+a = now()
+bt.set_box_state(0, s)
+b = peak()
+c = now()
+got = bt.get_box_state(0)
+d = peak()
+for k in s:
+    assert np.array_equal(got[k], s[k].astype(np.float32).astype(np.float64) if k in "NF" else s[k]), k
+print(b - a, d - c - sum(v.nbytes for v in got.values()) / 2**20)
+"""
+
+
+def test_host_staging_is_bounded():
+    """RT_MIXED through host memory: N and F are rounded to float in chunks of
+    rows (several here, the last one shorter), 64 MB of staging, not in a copy of
+    all rows of F (322 MB); the process's memory peak says so."""
+    import os
+    import subprocess
+    import sys
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    r = subprocess.run([sys.executable, "-c", STAGING], cwd=root, capture_output=True, text=True)
+    assert r.returncode == 0, r.stderr
+    put, get = map(float, r.stdout.split())
+    print("MB beyond the state's own arrays: set %.0f, get %.0f" % (put, get))
+    assert put < 160 and get < 160, (put, get)
