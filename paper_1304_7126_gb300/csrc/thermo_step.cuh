@@ -884,7 +884,10 @@ __device__ __forceinline__ bool subcycle_once(const ThermoParams &p, const S &nH
             // (a broken limit rejects whatever else was odd, but an odd value may itself have broken it)
             decided = !odd;
             ok = decided && !reject;
-            cc.valid = decided;   // the cooling at T(t), kept for an attempt the exact way
+            // the cooling and recombination rates at T(t) for an attempt the exact way: only what
+            // was in range counts
+            cc.valid = decided;
+            cc.rvalid = decided;
         }
     }
     if (!have) return true;
