@@ -687,6 +687,12 @@ __device__ __forceinline__ void recomb_alphas(const RatesT<S> &t, S a[3])
 // instructions.  The one-thread sum and the teams' sums run the same
 // operations and give the same bits.
 constexpr int kCoolExp = 80;
+// Terms whose function is below 2^kCoolCut on this scale (6e-55 erg cm^3 s^-1) count
+// as zero: with n_HII >= 1e-6 n_H, the floor of x_HII, they are below 2^-48 of the
+// bremsstrahlung whatever the densities they are multiplied by.  (At -60 the
+// excitation cooling of neutral gas near 2000 K was lost, up to 1e-11 of it.)
+// Above it the low floats stay clear of float subnormals.
+constexpr int kCoolCut = -100;
 
 // a[i] through selects (registers, not local memory, for a lane-dependent
 // i; a plain a[i] once unrolled with a constant i)
@@ -739,8 +745,7 @@ __device__ __forceinline__ void cool_term(const RateVal &r, dfm::F2 n, dfm::F2 &
 {
     using namespace dfm;
     const int e = r.m + kCoolExp;
-    // (terms below 2^-60 of this scale, e-42 erg, are below 2^-48 of the bremsstrahlung)
-    const float sc = e < -60 ? 0.0f : pow2f(e > 100 ? 100 : e);
+    const float sc = e < kCoolCut ? 0.0f : pow2f(e > 100 ? 100 : e);
     v = mulu(F2{r.y.hi * sc, r.y.lo * sc}, n);
     dv = mulu(v, r.g);
 }
