@@ -884,14 +884,13 @@ __device__ __forceinline__ bool subcycle_once(const ThermoParams &p, const S &nH
             // (a broken limit rejects whatever else was odd, but an odd value may itself have broken it)
             decided = !odd;
             ok = decided && !reject;
-            // the cooling and recombination rates at T(t) for an attempt the exact way: only what
-            // was in range counts
-            cc.valid = decided;
-            cc.rvalid = decided;
         }
     }
     if (!have) return true;
     if (!decided) {
+        // (nothing of an undecided fast attempt is kept for the exact one)
+        if constexpr (TS > 1)
+            if (!p.isothermal && p.helium) cc.valid = cc.rvalid = false;
         dfm::Exact e;
         small = false;
         ok = attempt<G, TS, MIX, S, SM>(p, nH, st, h, iso, cc, o, small, e);
