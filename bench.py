@@ -36,8 +36,9 @@ UNIT = "cell-group updates/s"
 # (oracle/make_counts.py writes tests/golden/op_counts.json): FP64 flops per
 # thermochemistry attempt and per transport cell-group, as the oracle states
 # the method.  Transport bytes: N, F read and written once per cell-group.
-# the library's default routing: attempts of the first pass; cells past
-# LONG_ATTEMPTS in all are reported as long sub-cyclers
+# the library's default routing: attempts of the first pass.  LONG_ATTEMPTS: cells
+# with more are reported as long sub-cyclers (a number of the report, at which the
+# library does nothing)
 PASS1_ATTEMPTS = 6
 LONG_ATTEMPTS = 134
 # DRAM bytes (read + write) per launch, from the ncu captures of the current

@@ -2,20 +2,22 @@
 // coefficients (collisional ionisation: Cen 1992; recombination and
 // recombination cooling: Hui & Gnedin 1997; collisional excitation: Cen
 // 1992; bremsstrahlung; Compton: Haiman et al. 1996; dielectronic: Black
-// 1981), each with its analytic temperature derivative, in FP64.
+// 1981), each with its analytic temperature derivative, in float pairs (48 bits)
+// up to the FP64 update.
 //
 // Every rate coefficient and every cooling term is one function of T of
 // the form
 //     f(T) = Cc exp(c0 + c1 ln T + c2 / T - c3 softplus(c4 ln T + c5)),
 // softplus(z) = ln(1 + e^z) (see RateFn below).  The lanes of a team of two,
 // four or eight that share a cell take a function each; one thread evaluates
-// the ones it needs in turn.  The argument is formed in the double-float arithmetic of dfmath.cuh (on the
-// FP32 pipe), exponentiated by dfm::exp2d and scaled by Cc in FP64; both
-// paths run the same expressions and so give identical bits.
+// the ones it needs in turn.  The argument, its exponential (dfm::exp_pair) and
+// the product with the factor (Cm, with the reference's share of the argument)
+// are formed in the double-float arithmetic of dfmath.cuh, on the FP32 pipe;
+// both paths run the same expressions and so give identical bits.
 //
 // What bounds them: the FP64 pipe, of which a warp gets one instruction per
 // 64 cycles (so the count of FP64 instructions sets both the length of a lone
-// cell's chain of attempts and the throughput of the lane-per-cell kernels).
+// cell's chain of attempts and the throughput of the kernels).
 // The functions, their T-derivatives and the cooling sums therefore stay
 // float pairs until they enter the FP64 update, and enter it through integer
 // operations (dfm::combine) instead of an FP64 addition each.
@@ -180,7 +182,7 @@ enum {
     RF_BETA_HI = 16, RF_ALPHA_HII, RF_BETA_HEI, RF_BETA_HEII, RF_ALPHA_HEII, RF_ALPHA_HEIII,
     NRF
 };
-static_assert(kNCool <= 16 && NRF <= 32, "function slots are warp lanes");
+static_assert(kNCool <= 16 && NRF <= 32, "function slots fit the tables and the masks of slots");
 
 // The kernels take ln T relative to 2^14 K, the middle of the range that
 // matters: |ln(T / 2^14 K)| is a few units where |ln T| is 9, and so are the
@@ -463,7 +465,6 @@ __host__ __device__ constexpr unsigned cool_mask(int he)
         if (cool_row(k).he == he) m |= rf_bit(RF_COOL0 + k);
     return m;
 }
-constexpr unsigned kNeedCoolH = cool_mask(0), kNeedCoolHe = cool_mask(1);
 
 // one thread: slot k (a constant once unrolled) at level L, given the
 // softplus of u

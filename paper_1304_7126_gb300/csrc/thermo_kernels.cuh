@@ -146,8 +146,11 @@ __device__ __forceinline__ void push_item(const QueueArrays &a, unsigned long lo
     }
 }
 
-// Four blocks per SM (128 registers, a few spilled): 128^3 x 3 groups 1.18,
-// 1.08 and 1.14 ms with three, four and five.
+// Four blocks per SM (128 registers, some spilled): 128^3 x 3 groups 1.18,
+// 1.08 and 1.14 ms with three, four and five.  The more groups, the more is
+// spilled and the less the fourth block gives: 96^3, three against four blocks,
+// 1, 3, 5 and 8 groups 0.39, 0.84, 0.99 and 1.39 against 0.36, 0.76, 0.91 and 1.39
+// ms; smoothed 0.57, 0.95, 1.33 and 1.99 against 0.54, 0.92, 1.37 and 2.00 ms.
 template <int G, typename P, bool R32, bool SM>
 __global__ void __launch_bounds__(kPass1Block, 4)
 thermo_pass1(ThermoParams p, const double *__restrict__ nH, double *xHII, double *xHeII, double *xHeIII,
@@ -230,7 +233,10 @@ struct QueueView {
 // Two stages instead of teams of four alone: 256^3 48.1 -> 39.7 ms, 128^3 with
 // grown fronts 21.1 -> 17.9 ms; a queue that stage 2 holds at once gains
 // nothing from stage 1.  Stage 1 at 128 registers and four blocks per SM,
-// stage 2 at up to 255 (both at 128: 256^3 39.7 instead of 37.6 ms).
+// stage 2 at up to 255 (both at 128: 256^3 39.7 instead of 37.6 ms).  From five
+// groups on stage 1 spills (340 bytes at eight): 96^3 with fronts in progress and
+// 24000 to 31000 queued cells, both stages: 17.2 ms at three groups, 22.1 at five,
+// 22.3 at eight.
 template <int G, int TS, typename P, bool R32, bool SM>
 __global__ void __launch_bounds__(128, TS == 2 ? 4 : 2)
 thermo_team(ThermoParams p, const double *__restrict__ nH, double *xHII, double *xHeII, double *xHeIII,

@@ -636,7 +636,7 @@ __device__ __forceinline__ bool photons_serial(const ThermoParams &p, const Cell
 // The checks |dX| / den > 0.1 go through ratio_gt / ratio_lt (a division
 // only near the threshold).
 // MIX (RT_MIXED32): the rates' softplus corrections and exponentials and
-// the absorption coefficients in FP32 (rates.cuh, rate_value_f); the
+// the absorption coefficients in FP32 (rates.cuh, rate_softplus, rate_val); the
 // photon, T/mu, x_HII and helium updates and 1 - x in FP64.
 //
 // S is double, or Dual for the adjoint's differentiated recomputation

@@ -683,7 +683,11 @@ transport_kernel(GridDev g, int G, S c, S dtdx, double area_dt, const S *__restr
 // Small boxes, where every CTA has one plane at most and the launch is as
 // long as one CTA's plane (two warps per SM sub-partition taking turns on the
 // FP64 pipe): tiles of 32 x 4, so twice as many CTAs of half the warps.
-// 32^3, one group, GLF, FP64: 43 -> 27 us.
+// 32^3, one group, GLF, FP64: 43 -> 27 us.  24^3, two groups, HLL: FP64 53 -> 33
+// us, FP32 27 -> 17 us.  FP32 HLL holds three of these CTAs per SM where the rule
+// lets up to four per SM in (as many as the large tiles' grid); the few that come
+// second cost less than the large tiles do: 32^2 x 30 and x 37, two groups (480 and
+// 592 planes of tiles): 25.5 -> 22.4 and 26.0 -> 24.2 us.
 template <typename S, int FLUX>
 __global__ void __launch_bounds__(128, 2)
 transport_small_kernel(GridDev g, int G, S c, S dtdx, double area_dt, const S *__restrict__ N0all,

@@ -131,8 +131,9 @@ def test_full_step_parity_cosmo128(oracle_mod, R):
     the GPU restarted from the oracle's state before the second, against the
     oracle on all host cores; the same per-cell attempt counts outside
     oracle-reported ties and 1e-10 on every other cell, which must be at
-    least 99% of them.  The source cells take hundreds of attempts, so all
-    four thermochemistry kernels run."""
+    least 99% of them.  The source cells take hundreds of attempts, so they
+    finish in the team kernel (test_gpu_routing.py has queues that take both of
+    its stages)."""
     import os
     from paper_1304_7126_gb300 import workloads as W
     w = W.cosmo128()
@@ -156,13 +157,15 @@ def test_full_step_parity_cosmo128(oracle_mod, R):
 
 @pytest.mark.parametrize("flux", [1, 0])
 def test_routing_reaches_every_kernel(oracle_mod, R, flux):
-    """The cells of a small box routed through all four thermochemistry
-    kernels (one first-pass attempt, two attempts in the first drain, three
-    in the second, which is forced to run, then a warp per cell): against
-    the oracle as above, and against the default routing, which must give
-    identical bits for x_HII, x_HeII, x_HeIII, T, N, F and the attempt
-    counts: routing never changes the arithmetic, and a queued cell carries
-    its flux scale, so its F is formed once, when it finishes."""
+    """The cells of a small box routed through the first pass (one attempt),
+    the first stage of the team kernel, which is forced to run, and the second,
+    to which a cell may move after every five attempts: against
+    the oracle as above, and against the default routing (six first-pass
+    attempts, then the second stage), which must give identical bits for
+    x_HII, x_HeII, x_HeIII, T, N, F and the attempt counts: routing never
+    changes the arithmetic, and a queued cell carries its flux scale, so its F
+    is formed once, when it finishes.  (The teams hold this whole queue at
+    once; test_gpu_routing.py has one several times as long.)"""
     from paper_1304_7126_gb300 import workloads as W
     w = W.small_cosmo(16, seed=3, nsrc=4, flux=flux, nx=21, ny=13)
     forced = R.RT.from_workload(w)
@@ -179,7 +182,7 @@ def test_routing_reaches_every_kernel(oracle_mod, R, flux):
         st, b, sub_o, mg = p.step(ref, dt, w.src_ijk, w.src_L)
         assert st == 0
         sub_f = forced.subcycles().reshape(-1)
-        assert np.sum(sub_f > 6) > 0, "some cells must reach the warp-per-cell kernel"
+        assert np.sum(sub_f > 6) > 0, "some cells must be queued by the first pass of both"
         differ = sub_f != sub_o.reshape(-1)
         assert np.all(mg.reshape(-1)[differ] < 1e-9), (step, int(differ.sum()))
         gf = forced.get_state()
