@@ -36,7 +36,6 @@ def test_box_state_in_a_class_beyond_the_pitch_limit(prec, nbig, device):
 
 
 STAGING = """
-import resource
 import numpy as np
 from paper_1304_7126_gb300 import rt as R
 from paper_1304_7126_gb300 import workloads as W
@@ -48,8 +47,8 @@ rng = np.random.default_rng(2)
 s = w.state()
 for k in "NF":
     rng.random(out=s[k])
-now = lambda: int([l for l in open("/proc/self/status") if l.startswith("VmRSS")][0].split()[1]) / 1024.0
-peak = lambda: resource.getrusage(resource.RUSAGE_SELF).ru_maxrss / 1024.0
+mb = lambda key: int([l for l in open("/proc/self/status") if l.startswith(key)][0].split()[1]) / 1024.0
+now, peak = lambda: mb("VmRSS"), lambda: mb("VmHWM")   # (getrusage's peak starts at the parent's)
 a = now()
 bt.set_box_state(0, s)
 b = peak()
